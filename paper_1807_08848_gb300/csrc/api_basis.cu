@@ -24,7 +24,11 @@ extern "C" msp_status msp_extract_basis(msp_medium m, double tau, int precision,
     return MSP_OK;
 }
 
-extern "C" void msp_basis_destroy(msp_basis b) { delete b; }
+extern "C" void msp_basis_destroy(msp_basis b) {
+    if (!b) return;
+    wait_for_device();
+    delete b;
+}
 
 extern "C" msp_status msp_basis_info(msp_basis b, int patch, int* k, double* sigma_host) {
     clear_error();

@@ -52,6 +52,8 @@ int num_sms() {
     return n;
 }
 
+void wait_for_device() { cudaDeviceSynchronize(); }
+
 static msp_status need_device() {
     int n = 0;
     cudaError_t e = cudaGetDeviceCount(&n);
@@ -245,6 +247,7 @@ extern "C" msp_status msp_build_medium_full(const msp_medium_desc* d, const msp_
 
 extern "C" void msp_medium_destroy(msp_medium m) {
     if (!m) return;
+    wait_for_device();
     for (auto& g : m->M.graph)
         if (g) cudaGraphExecDestroy(g);
     if (m->M.capture_stream) cudaStreamDestroy(m->M.capture_stream);

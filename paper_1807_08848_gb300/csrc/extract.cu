@@ -751,6 +751,7 @@ msp_status svd_bases(const double* snaps, long long snap_elems, const std::vecto
     // ---- SVD of the triangular factor
     MSP_TRY(W.alloc(mo, s));
     MSP_TRY(V.alloc(mo, s));
+    DevBuf<SmallMat> d_by_size;   // read by the sweeps until the synchronisation below
     if (maxc > 2 * kJacMaxPairs) {
         set_error("basis extraction: more than " + std::to_string(2 * kJacMaxPairs) + " snapshot columns on a patch");
         return MSP_ERR_INVALID_ARG;
@@ -764,7 +765,6 @@ msp_status svd_bases(const double* snaps, long long snap_elems, const std::vecto
         // the largest blocks first (their sweeps cost the most), so the last wave is short
         std::vector<SmallMat> by_size(mats);
         std::stable_sort(by_size.begin(), by_size.end(), [](const SmallMat& a, const SmallMat& b) { return a.c > b.c; });
-        DevBuf<SmallMat> d_by_size;
         MSP_TRY(upload(d_by_size, by_size, s));
         if (svd_mixed()) {
             // FP32 sweeps on (float) T^T from V = I, then V re-orthogonalised in FP64

@@ -32,6 +32,12 @@ msp_status cuda_fail(cudaError_t e, const char* what, const char* file, int line
 #define MSP_TRY(call)                                                               \
     do { msp_status s_ = (call); if (s_ != MSP_OK) return s_; } while (0)
 
+// Waits for every kernel of the current device: called before a handle's buffers
+// go back to the pool.  cudaFree of a stream-ordered allocation takes its accesses
+// to be complete and waits for nothing, while a call that only enqueues (a solve
+// without iteration counts, a snapshot copy) may still be running.
+void wait_for_device();
+
 // Stream-ordered device buffer owned by a handle.
 template <class T>
 struct DevBuf {

@@ -730,7 +730,11 @@ extern "C" msp_status msp_kinetic_build_hg(int n_cells, double eps, double g, in
     return MSP_OK;
 }
 
-extern "C" void msp_kinetic_destroy(msp_kmedium k) { delete k; }
+extern "C" void msp_kinetic_destroy(msp_kmedium k) {
+    if (!k) return;
+    wait_for_device();
+    delete k;
+}
 
 extern "C" msp_status msp_kinetic_velocities(msp_kmedium k, double* v_host, double* w_host) {
     clear_error();
@@ -875,7 +879,11 @@ extern "C" msp_status msp_kinetic_extract(msp_kmedium km, double tau, void* stre
     return MSP_OK;
 }
 
-extern "C" void msp_kinetic_basis_destroy(msp_kbasis b) { delete b; }
+extern "C" void msp_kinetic_basis_destroy(msp_kbasis b) {
+    if (!b) return;
+    wait_for_device();
+    delete b;
+}
 
 extern "C" msp_status msp_kinetic_basis_info(msp_kbasis b, int patch, int* k, double* sigma_host) {
     clear_error();
