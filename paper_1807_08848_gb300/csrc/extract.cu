@@ -12,6 +12,7 @@
 #include "internal.h"
 #include "dense.cuh"
 #include "device_util.cuh"
+#include "patch_dense.h"
 
 #include <algorithm>
 #include <cmath>
@@ -27,100 +28,6 @@ struct SmallMat {
     int n;           // rows of the tall matrix
     int idx;         // patch index (the Jacobi kernels run the blocks largest first)
 };
-
-// Cholesky of (G + shift I) = L L^T in global memory (one CTA per matrix),
-// then F = L^T and Fi = L^{-T} (upper triangular), column-major order c.
-// shift0 > 0 requests a shifted factorisation; on a non-positive pivot the
-// shift grows (to 1e-14 trace if it was zero, else x100) up to 6 tries.
-// status[b]: number of tries used, or -1 on failure.
-__global__ void __launch_bounds__(256) chol_factor_kernel(const SmallMat* mats, const double* G, double* L,
-                                                          double* F, double* Fi, const double* shift_scale,
-                                                          int shifted, int* status) {
-    const SmallMat S = mats[blockIdx.x];
-    const int c = S.c;
-    if (c <= 0) return;
-    const double* g = G + S.off;
-    double* l = L + S.off;
-    double* f = F + S.off;
-    double* fi = Fi + S.off;
-    __shared__ double s_trace;
-    __shared__ int s_ok;
-    if (threadIdx.x == 0) {
-        double t = 0.0;
-        for (int i = 0; i < c; ++i) t += g[i + (long long)i * c];
-        s_trace = t;
-    }
-    __syncthreads();
-    const double trace = s_trace;
-    double shift = 0.0;
-    if (shifted) shift = shift_scale[blockIdx.x] * trace;
-    int tries = 0;
-    bool ok = false;
-    for (; tries < 6 && !ok; ++tries) {
-        for (long long e = threadIdx.x; e < (long long)c * c; e += blockDim.x) {
-            const int i = (int)(e % c), j = (int)(e / c);
-            l[e] = (i >= j) ? g[e] + (i == j ? shift : 0.0) : 0.0;
-        }
-        __syncthreads();
-        ok = true;
-        for (int k = 0; k < c; ++k) {
-            if (threadIdx.x == 0) {
-                const double d = l[k + (long long)k * c];
-                s_ok = (d > 0.0 && isfinite(d)) ? 1 : 0;
-                if (s_ok) l[k + (long long)k * c] = sqrt(d);
-            }
-            __syncthreads();
-            if (!s_ok) { ok = false; break; }
-            const double piv = l[k + (long long)k * c];
-            for (int i = k + 1 + threadIdx.x; i < c; i += blockDim.x) l[i + (long long)k * c] /= piv;
-            __syncthreads();
-            // trailing update of the lower triangle: a warp per column j, lanes along
-            // the rows i >= j (contiguous in the column-major block)
-            {
-                const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-                for (int j = k + 1 + (threadIdx.x >> 5); j < c; j += nw) {
-                    const double ljk = l[j + (long long)k * c];
-                    double* lj = l + (long long)j * c;
-                    const double* lk = l + (long long)k * c;
-                    for (int i = j + lane; i < c; i += 32) lj[i] -= lk[i] * ljk;
-                }
-            }
-            __syncthreads();
-        }
-        __syncthreads();
-        if (!ok) shift = (shift == 0.0) ? 1e-14 * trace : shift * 100.0;
-    }
-    if (!ok) {
-        if (threadIdx.x == 0) status[blockIdx.x] = -1;
-        return;
-    }
-    if (threadIdx.x == 0) status[blockIdx.x] = tries;
-    // F = L^T
-    for (long long e = threadIdx.x; e < (long long)c * c; e += blockDim.x) {
-        const int i = (int)(e % c), j = (int)(e / c);
-        f[e] = (i <= j) ? l[j + (long long)i * c] : 0.0;
-    }
-    // Fi = (L^{-1})^T, X = L^{-1} with X(i, j) stored at Fi(j, i) = fi[j + i c]: row i
-    // of X, X(i, j) = (delta_ij - sum_{q<i} l_iq X(q, j)) / l_ii, for all j <= i at
-    // once -- one barrier per row, a warp per column j, lanes along q, the partial
-    // sums of a warp combined by shuffles in a fixed order
-    for (long long e = threadIdx.x; e < (long long)c * c; e += blockDim.x) fi[e] = 0.0;
-    __syncthreads();
-    {
-        const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-        for (int i = 0; i < c; ++i) {
-            const double rli = 1.0 / l[i + (long long)i * c];
-            const double* li = l + i;   // l_iq at li[q c]
-            for (int j = threadIdx.x >> 5; j <= i; j += nw) {
-                double a = 0.0;
-                for (int q = j + lane; q < i; q += 32) a += li[(long long)q * c] * fi[j + (long long)q * c];
-                a = warp_sum(a);
-                if (lane == 0) fi[j + (long long)i * c] = ((i == j ? 1.0 : 0.0) - a) * rli;
-            }
-            __syncthreads();
-        }
-    }
-}
 
 // W = T^T, V = I (per patch, order c).
 __global__ void jacobi_init_kernel(const SmallMat* mats, const double* T, double* W, double* V) {
@@ -648,20 +555,28 @@ msp_status svd_bases(const double* snaps, long long snap_elems, const std::vecto
     MSP_TRY(phase_mark(marks, s));
     // ---- small-matrix layout
     std::vector<SmallMat> mats(np);
-    std::vector<long long> sig_off(np);
+    std::vector<long long> sig_off(np), mat_off(np);
     long long mo = 0, so = 0;
     int maxc = 0, maxn = 0;
     for (int m = 0; m < np; ++m) {
         mats[m] = SmallMat{mo, cols[m], n_rows[m], m};
+        mat_off[m] = mo;
         mo += (long long)cols[m] * cols[m];
         sig_off[m] = so;
         so += cols[m];
         maxc = std::max(maxc, cols[m]);
         maxn = std::max(maxn, n_rows[m]);
     }
+    if (maxc > 2 * kJacMaxPairs) {
+        set_error("basis extraction: more than " + std::to_string(2 * kJacMaxPairs) + " snapshot columns on a patch");
+        return MSP_ERR_INVALID_ARG;
+    }
+    const PatchClasses classes = classify_patches(cols, mat_off);
     DevBuf<SmallMat> d_mats;
+    DevBuf<PatchBlock> d_blocks;
     DevBuf<long long> d_sig_off;
     MSP_TRY(upload(d_mats, mats, s));
+    MSP_TRY(upload(d_blocks, classes.blocks, s));
     MSP_TRY(upload(d_sig_off, sig_off, s));
     DevBuf<double> G, L, F, Fi, T0, T1, W, V, ping, pong, sig_tmp, sig;
     DevBuf<int> order, kdev, status, sweeps, sweeps32;
@@ -713,9 +628,7 @@ msp_status svd_bases(const double* snaps, long long snap_elems, const std::vecto
             gd[m].lower = 1;   // the Cholesky reads the lower triangle only
         }
         MSP_TRY(run_gemm(true, maxc, maxc, kGemmStructured));
-        chol_factor_kernel<<<np, 256, 0, s>>>(d_mats.p, G.p, L.p, F.p, Fi.p, shift_scale.p, pass == 0, status.p);
-        count_launches(1);
-        MSP_CUDA(cudaGetLastError());
+        MSP_TRY(patch_cholesky(classes, d_blocks.p, G.p, L.p, F.p, Fi.p, shift_scale.p, pass == 0, status.p, s));
         MSP_CUDA(cudaMemcpyAsync(hstat.data(), status.p, sizeof(int) * np, cudaMemcpyDeviceToHost, s));
         MSP_CUDA(cudaStreamSynchronize(s));
         for (int m = 0; m < np; ++m) max_tries = std::max(max_tries, hstat[m]);
@@ -752,10 +665,6 @@ msp_status svd_bases(const double* snaps, long long snap_elems, const std::vecto
     MSP_TRY(W.alloc(mo, s));
     MSP_TRY(V.alloc(mo, s));
     DevBuf<SmallMat> d_by_size;   // read by the sweeps until the synchronisation below
-    if (maxc > 2 * kJacMaxPairs) {
-        set_error("basis extraction: more than " + std::to_string(2 * kJacMaxPairs) + " snapshot columns on a patch");
-        return MSP_ERR_INVALID_ARG;
-    }
     {
         int dev = 0, optin = 0;
         MSP_CUDA(cudaGetDevice(&dev));
@@ -1064,8 +973,10 @@ msp_status finish_basis(Basis& B, const double* aE_dev, const double* aN_dev, cu
     precond_block_kernel<<<np, 256, 0, s>>>(B.d_k.p, B.d_ne.p, B.d_e_off.p, B.E.p, B.d_slot_off.p, B.tr_ptr.p,
                                             d_kmats.p, G.p);
     count_launches(1);
-    chol_factor_kernel<<<np, 256, 0, s>>>(d_kmats.p, G.p, L.p, F.p, Fi.p, shift_scale.p, 0, status.p);
-    count_launches(1);
+    const PatchClasses classes = classify_patches(B.k, B.binv_off);
+    DevBuf<PatchBlock> d_blocks;
+    MSP_TRY(upload(d_blocks, classes.blocks, s));
+    MSP_TRY(patch_cholesky(classes, d_blocks.p, G.p, L.p, F.p, Fi.p, shift_scale.p, false, status.p, s));
     precond_inverse_kernel<<<np, 256, 0, s>>>(d_kmats.p, Fi.p, B.d_binv_off.p, B.Binv.p);
     // keep L_m^{-T} of every patch block: the scaling of the online factor
     MSP_TRY(B.bt_Fi.alloc(std::max<long long>(ko, 1), s));

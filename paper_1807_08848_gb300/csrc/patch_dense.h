@@ -1,0 +1,33 @@
+// Dense factorisations of the patches' small symmetric and square blocks on
+// thread-block clusters: one patch on one CTA, or on eight when it would otherwise
+// keep a single SM busy after the others have finished.
+#pragma once
+#include "internal.h"
+
+namespace msp {
+
+// One patch's c x c block (column-major, leading dimension c) in the stacked arrays.
+struct PatchBlock {
+    long long off;
+    int c;
+    int idx;      // patch
+};
+
+constexpr int kPatchCluster = 8;   // CTAs of a patch that takes a cluster (the portable limit)
+
+// Patches that take a cluster each, then those that take one CTA, both largest first.
+struct PatchClasses {
+    std::vector<PatchBlock> blocks;
+    int n_big = 0;
+    int max_c[2] = {0, 0};         // largest order of either class
+};
+PatchClasses classify_patches(const std::vector<int>& cols, const std::vector<long long>& off);
+
+// Cholesky of every block G (lower triangle read) + shift I, shift = shift_scale[patch]
+// trace(G) (shifted != 0; else 0), on a non-positive pivot a growing shift (1e-14 trace
+// if it was zero, else x 100), at most six tries: status[patch] = tries, or -1.
+// F = L^T and Fi = L^{-T}; L is overwritten.  `blocks` is C.blocks on the device.
+msp_status patch_cholesky(const PatchClasses& C, const PatchBlock* blocks, const double* G, double* L, double* F,
+                          double* Fi, const double* shift_scale, bool shifted, int* status, cudaStream_t s);
+
+}  // namespace msp
