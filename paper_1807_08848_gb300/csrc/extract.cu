@@ -664,7 +664,8 @@ msp_status svd_bases(const double* snaps, long long snap_elems, const std::vecto
     // ---- SVD of the triangular factor
     MSP_TRY(W.alloc(mo, s));
     MSP_TRY(V.alloc(mo, s));
-    DevBuf<SmallMat> d_by_size;   // read by the sweeps until the synchronisation below
+    DevBuf<SmallMat> d_by_size, d_rest;   // read by the sweeps until the synchronisation below
+    DevBuf<PatchBlock> d_jac;
     {
         int dev = 0, optin = 0;
         MSP_CUDA(cudaGetDevice(&dev));
@@ -743,6 +744,15 @@ msp_status svd_bases(const double* snaps, long long snap_elems, const std::vecto
             MSP_CUDA(cudaGetLastError());
         }
         MSP_TRY(phase_mark(marks, s));
+        // a cluster per patch; the blocks too large for one (above about 450 columns) on
+        // one CTA each
+        std::vector<PatchBlock> rest_blocks;
+        std::vector<PatchBlock> sorted(classes.blocks);
+        std::stable_sort(sorted.begin(), sorted.end(), [](const PatchBlock& a, const PatchBlock& b) { return a.c > b.c; });
+        MSP_TRY(patch_jacobi(sorted, W.p, V.p, 40, maxc * 1.12e-16, small_rel, sweeps.p, d_jac, rest_blocks, s));
+        std::vector<SmallMat> rest;
+        for (const PatchBlock& b : rest_blocks) rest.push_back(mats[b.idx]);
+        MSP_TRY(upload(d_rest, rest, s));
         // largest order whose W is held in shared memory: the opt-in limit per
         // block less the kernel's static shared memory
         cudaFuncAttributes fa{};
@@ -753,9 +763,12 @@ msp_status svd_bases(const double* snaps, long long snap_elems, const std::vecto
         c64 = std::min(c64, maxc);
         const size_t sm64 = (size_t)c64 * (c64 + 1) * sizeof(double);
         MSP_CUDA(cudaFuncSetAttribute(jacobi_svd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm64));
-        jacobi_svd_kernel<<<np, 512, sm64, s>>>(d_by_size.p, W.p, V.p, 40, maxc * 1.12e-16, small_rel, c64, sweeps.p);
-        count_launches(1);
-        MSP_CUDA(cudaGetLastError());
+        if (!rest.empty()) {
+            jacobi_svd_kernel<<<(int)rest.size(), 512, sm64, s>>>(d_rest.p, W.p, V.p, 40, maxc * 1.12e-16, small_rel, c64,
+                                                                  sweeps.p);
+            count_launches(1);
+            MSP_CUDA(cudaGetLastError());
+        }
         MSP_TRY(phase_mark(marks, s));
     }
     sort_truncate_kernel<<<np, 256, 0, s>>>(d_mats.p, W.p, tau, sig_tmp.p, sig.p, d_sig_off.p, order.p, kdev.p);

@@ -221,6 +221,328 @@ __global__ void __launch_bounds__(32 * kInvWarps) patch_inverse_kernel(const Pat
     }
 }
 
+// ------------------------------------------------------------------ Jacobi
+constexpr int kJacThreads = 256;
+constexpr int kJacLanes = 8;                           // threads per column pair
+constexpr int kJacPairs = kJacThreads / kJacLanes;     // pairs per CTA at most
+constexpr int kJacCluster = 16;                        // CTAs of a patch at most (beyond the portable eight)
+static_assert(kJacPairs == 32, "one warp takes the angles of a CTA's pairs");
+constexpr size_t kJacSmem = 76 * 1024;                 // three CTAs per SM
+
+struct JacShape {
+    int m;        // pairs of a round (positions of the tournament)
+    int slots;    // column slots of a CTA: its pairs' columns and two to receive into
+    int ld;
+    bool v_smem;  // V beside W in shared memory, else in global memory
+    size_t bytes;
+};
+
+__host__ __device__ inline JacShape jac_shape(int c, int nc) {
+    JacShape s;
+    s.m = (c + 1) / 2;
+    s.slots = 2 * ((s.m + nc - 1) / nc) + (nc > 1 ? 2 : 0);
+    s.ld = c | 1;
+    const size_t w = (size_t)s.slots * s.ld * sizeof(double);
+    s.v_smem = 2 * w <= kJacSmem;
+    s.bytes = s.v_smem ? 2 * w : w;
+    return s;
+}
+
+struct JacArgs {
+    const PatchBlock* blocks;
+    double* W;
+    double* V;
+    int* sweeps_out;
+    int max_sweeps;
+    double tol, small_rel;
+};
+
+// One-sided (Hestenes) Jacobi on the columns of W (c x c), V accumulating the same
+// rotations, one patch per cluster.  Column pairs follow the round-robin tournament:
+// in round r position 0 plays (r, np - 1) and position i plays ((r + i), (r - i)) mod
+// (np - 1), np = c rounded up to even.  From one round to the next the first player of
+// a position comes from the position above, the second from the one below, so each
+// CTA holds a range of positions, its columns in shared memory, and passes one
+// column to each neighbour per round through distributed shared memory; a cluster
+// barrier ends the round.  Phases of a round: groups of eight threads form a pair's
+// inner products; one thread per pair decides and takes the angle; the CTA applies
+// the rotations.  A column's squared norm is kept until the column is rotated.
+// Skips: columns below u |W|_F are numerically zero; a pair orthogonal to the
+// rounding floor of its inner product is left alone; and a pair whose columns are
+// both below small_rel |W|_F (far under the truncation level) is left alone, since
+// rotating it only mixes directions that are dropped.
+// Every pair, sum and rotation is that of the one-CTA form (jacobi_svd_kernel), in
+// the same order: the result does not depend on the cluster size.
+// Bound: the FP64 pipe (3 c products and 8 c for the two rotations per pair, about
+// 1.75 FMA per clock and SM); the three CTAs of an SM hide each other's angles and
+// barriers, and a large patch no longer runs on one SM alone.
+__global__ void __launch_bounds__(kJacThreads, 3) patch_jacobi_kernel(JacArgs A) {
+    extern __shared__ __align__(16) double jsm[];
+    constexpr int kSlots = 2 * kJacPairs + 2;
+    __shared__ double s_red[16];
+    __shared__ double2 s_ab[kJacPairs];                // squared norms, then cos and sin
+    __shared__ double s_ga[kJacPairs];
+    __shared__ int4 s_at[kJacPairs];                   // slots and columns of the pair (x < 0: none)
+    __shared__ double s_nrm[kSlots];
+    __shared__ int s_have[kSlots];                     // s_nrm is the norm of the column held
+    __shared__ int s_col[kSlots];                      // column in a slot
+    __shared__ short s_top[2][kJacPairs], s_bot[2][kJacPairs], s_free[2][2];   // by round parity
+    __shared__ int s_rot, s_all[2][kJacCluster];
+    cg::cluster_group cl = cg::this_cluster();
+    const int nc = (int)cl.num_blocks(), rank = (int)cl.block_rank();
+    const PatchBlock P = A.blocks[blockIdx.x / nc];
+    const int c = P.c, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
+    if (c <= 1) {                                      // the whole cluster
+        if (rank == 0 && tid == 0) A.sweeps_out[P.idx] = 0;
+        return;
+    }
+    const JacShape S = jac_shape(c, nc);
+    const int np = c + (c & 1), m = S.m, ld = S.ld;
+    const int lo = rank * m / nc, hi = (rank + 1) * m / nc, n = hi - lo;
+    double* Wg = A.W + P.off;
+    double* Vg = A.V + P.off;
+    double* w = jsm;
+    double* vs = jsm + (size_t)S.slots * ld;
+    // |W|_F^2 in the order of a block of 512 threads: thread t takes the elements of
+    // threads t and t + 256, the sixteen warp sums are added in order
+    double fro2 = 0.0;
+    {
+        double a0 = 0.0, a1 = 0.0;
+        const long long cc = (long long)c * c;
+        for (long long e = tid; e < cc; e += 512) {
+            const double x = Wg[e];
+            a0 += x * x;
+            if (e + 256 < cc) {
+                const double y = Wg[e + 256];
+                a1 += y * y;
+            }
+        }
+        a0 = warp_sum(a0);
+        a1 = warp_sum(a1);
+        if (lane == 0) {
+            s_red[warp] = a0;
+            s_red[warp + 8] = a1;
+        }
+        __syncthreads();
+        for (int k = 0; k < 16; ++k) fro2 += s_red[k];
+    }
+    // positions lo .. hi - 1 of round 0 in slots 2 i (first player) and 2 i + 1
+    for (int i = tid; i < n; i += blockDim.x) {
+        const int pr = lo + i;
+        s_col[2 * i] = pr == 0 ? 0 : pr % (np - 1);
+        s_col[2 * i + 1] = pr == 0 ? np - 1 : (np - 1 - pr) % (np - 1);
+        s_top[0][i] = (short)(2 * i);
+        s_bot[0][i] = (short)(2 * i + 1);
+    }
+    for (int i = tid; i < kSlots; i += blockDim.x) s_have[i] = 0;
+    if (tid == 0) {
+        s_free[0][0] = (short)(2 * n);
+        s_free[0][1] = (short)(2 * n + 1);
+        s_rot = 0;
+    }
+    __syncthreads();
+    for (int k = warp; k < 2 * n; k += nw) {
+        const int col = s_col[k];
+        if (col >= c) continue;                        // the dummy player of an odd c
+        for (int i = lane; i < c; i += 32) w[(size_t)k * ld + i] = Wg[(size_t)col * c + i];
+        if (S.v_smem)
+            for (int i = lane; i < c; i += 32) vs[(size_t)k * ld + i] = Vg[(size_t)col * c + i];
+    }
+    cl.sync();   // W is read before any CTA stores to it; every CTA runs before its slots are written to
+    constexpr double u = 1.1102230246251565e-16;
+    const double tol = A.tol, small_rel = A.small_rel;
+    const double negligible = u * u * fro2;
+    const double floor_abs = 2.0 * c * u * sqrt(fro2);
+    const double small2 = small_rel * small_rel * fro2;
+    const double inv_fro2 = 1.0 / fro2;
+    const float floor_rel = 2.0f * c * (float)u;
+    const int g = tid & (kJacLanes - 1), pr = tid / kJacLanes;
+    int par = 0, sweep = 0;
+    for (; sweep < A.max_sweeps; ++sweep) {
+        for (int r = 0; r < np - 1; ++r) {
+            // phase 1
+            int kp = 0, kq = 0;
+            bool real = false;
+            if (pr < n) {
+                kp = s_top[par][pr];
+                kq = s_bot[par][pr];
+                if (s_col[kp] > s_col[kq]) { const int t = kp; kp = kq; kq = t; }
+                real = s_col[kq] < c;
+            }
+            double al = 0, be = 0, ga = 0;
+            const bool have = !real || (s_have[kp] && s_have[kq]);
+            if (__all_sync(0xffffffffu, have)) {
+                // norms kept: the inner product alone, and not for pairs the norms already skip
+                if (real) {
+                    al = s_nrm[kp];
+                    be = s_nrm[kq];
+                }
+                const bool skip = al <= negligible || be <= negligible || (al < small2 && be < small2);
+                if (real && !skip) {
+                    const double* wp = w + (size_t)kp * ld;
+                    const double* wq = w + (size_t)kq * ld;
+                    for (int i = g; i < c; i += kJacLanes) ga = fma(wp[i], wq[i], ga);
+                }
+#pragma unroll
+                for (int o = kJacLanes / 2; o > 0; o >>= 1) ga += __shfl_xor_sync(0xffffffffu, ga, o);
+            } else {
+                if (real) {
+                    const double* wp = w + (size_t)kp * ld;
+                    const double* wq = w + (size_t)kq * ld;
+                    for (int i = g; i < c; i += kJacLanes) {
+                        const double x = wp[i], y = wq[i];
+                        al = fma(x, x, al);
+                        be = fma(y, y, be);
+                        ga = fma(x, y, ga);
+                    }
+                }
+#pragma unroll
+                for (int o = kJacLanes / 2; o > 0; o >>= 1) {
+                    al += __shfl_xor_sync(0xffffffffu, al, o);
+                    be += __shfl_xor_sync(0xffffffffu, be, o);
+                    ga += __shfl_xor_sync(0xffffffffu, ga, o);
+                }
+                if (real && g == 0) {
+                    s_nrm[kp] = al;
+                    s_nrm[kq] = be;
+                    s_have[kp] = s_have[kq] = 1;
+                }
+            }
+            if (pr < n && g == 0) {
+                s_at[pr] = real ? make_int4(kp, kq, s_col[kp], s_col[kq]) : make_int4(-1, 0, 0, 0);
+                s_ab[pr] = make_double2(al, be);
+                s_ga[pr] = ga;
+            }
+            __syncthreads();
+            // phase 2, by one warp, another each round (a warp's FP64 instructions all go to
+            // its quarter of the SM): the decision in FP32 on values scaled by 1 / |W|_F^2
+            // where it is clear by a percent, else as stated; then the angle
+            if (warp == (r & (nw - 1)) && lane < n && s_at[lane].x >= 0) {
+                const double a = s_ab[lane].x, b = s_ab[lane].y, gg = s_ga[lane];
+                bool go = !(a <= negligible || b <= negligible || (a < small2 && b < small2));
+                if (go) {
+                    const float af = sqrtf((float)(a * inv_fro2)), bf = sqrtf((float)(b * inv_fro2));
+                    const float gf = fabsf((float)(gg * inv_fro2));
+                    const float bound = (float)tol * af * bf + floor_rel * (af + bf);
+                    if (!(gf > 1.01f * bound)) {
+                        if (gf < 0.99f * bound) {
+                            go = false;
+                        } else {
+                            const double na = sqrt(a), nb = sqrt(b);
+                            go = !(fabs(gg) <= tol * na * nb + floor_abs * (na + nb));
+                        }
+                    }
+                }
+                if (!go) {
+                    s_at[lane].x = -1;
+                } else {
+                    const double zeta = (b - a) / (2.0 * gg);
+                    const double t = (zeta >= 0.0 ? 1.0 : -1.0) / (fabs(zeta) + sqrt(1.0 + zeta * zeta));
+                    const double cs = 1.0 / sqrt(1.0 + t * t);
+                    s_ab[lane] = make_double2(cs, cs * t);
+                    s_have[s_top[par][lane]] = s_have[s_bot[par][lane]] = 0;
+                    s_rot = 1;
+                }
+            }
+            __syncthreads();
+            // phase 3: rows fastest over the pairs
+            for (int e = tid; e < n * c; e += blockDim.x) {
+                const int k = e / c, i = e - k * c;
+                const int4 at = s_at[k];
+                if (at.x < 0) continue;
+                const double2 rot = s_ab[k];
+                const double cs = rot.x, sn = rot.y;
+                double xv, yv;
+                double *vp, *vq;
+                if (S.v_smem) {
+                    vp = vs + at.x * ld + i;
+                    vq = vs + at.y * ld + i;
+                    xv = *vp;
+                    yv = *vq;
+                } else {                               // other CTAs held these columns: past the L1
+                    vp = Vg + at.z * c + i;
+                    vq = Vg + at.w * c + i;
+                    xv = __ldcg(vp);
+                    yv = __ldcg(vq);
+                }
+                double* xp = w + at.x * ld + i;
+                double* xq = w + at.y * ld + i;
+                const double x = *xp, y = *xq;
+                *xp = cs * x - sn * y;
+                *xq = sn * x + cs * y;
+                const double rv = cs * xv - sn * yv, ru = sn * xv + cs * yv;
+                if (S.v_smem) {
+                    *vp = rv;
+                    *vq = ru;
+                } else {
+                    __stcg(vp, rv);
+                    __stcg(vq, ru);
+                }
+            }
+            __syncthreads();
+            // next round's positions; the columns leaving the CTA go to the slots their
+            // neighbours keep free
+            const int nxt = par ^ 1;
+            for (int i = tid; i < n; i += blockDim.x) {
+                short nt, nb;
+                if (i + 1 < n) nt = s_top[par][i + 1];
+                else nt = hi < m ? s_free[par][0] : s_bot[par][i];
+                if (lo + i == 0) nb = s_bot[par][0];
+                else if (i == 0) nb = s_free[par][1];
+                else nb = lo + i == 1 ? s_top[par][0] : s_bot[par][i - 1];
+                if (m == 1) { nt = s_top[par][0]; nb = s_bot[par][0]; }
+                s_top[nxt][i] = nt;
+                s_bot[nxt][i] = nb;
+            }
+            if (tid == 0) {
+                s_free[nxt][0] = lo > 0 ? s_top[par][0] : s_bot[par][n - 1];
+                s_free[nxt][1] = hi < m ? s_bot[par][n - 1] : s_top[par][0];
+            }
+            for (int dir = 0; dir < 2; ++dir) {
+                if (dir == 0 ? lo == 0 : hi == m) continue;
+                const int to = dir == 0 ? rank - 1 : rank + 1;
+                const int k = dir == 0 ? s_top[par][0] : s_bot[par][n - 1];
+                const int dst = cl.map_shared_rank(&s_free[par][0], to)[dir == 0 ? 0 : 1];
+                double* rw = cl.map_shared_rank(w, to) + (size_t)dst * ld;
+                const int half = blockDim.x / 2, t = tid - dir * half;
+                if (t >= 0 && t < half) {
+                    for (int i = t; i < c; i += half) rw[i] = w[(size_t)k * ld + i];
+                    if (S.v_smem) {
+                        double* rv = cl.map_shared_rank(vs, to) + (size_t)dst * ld;
+                        for (int i = t; i < c; i += half) rv[i] = vs[(size_t)k * ld + i];
+                    }
+                    if (t == 0) {
+                        cl.map_shared_rank(s_col, to)[dst] = s_col[k];
+                        cl.map_shared_rank(s_nrm, to)[dst] = s_nrm[k];
+                        cl.map_shared_rank(s_have, to)[dst] = s_have[k];
+                    }
+                }
+            }
+            if (r == np - 2 && tid < nc) cl.map_shared_rank(&s_all[sweep & 1][0], tid)[rank] = s_rot;
+            if (nc > 1) {
+                if (!S.v_smem) __threadfence();
+                cl.sync();
+            } else {
+                __syncthreads();
+            }
+            par = nxt;
+        }
+        int rot = 0;
+        for (int k = 0; k < nc; ++k) rot |= s_all[sweep & 1][k];
+        if (rot == 0) break;
+        if (tid == 0) s_rot = 0;     // set again only after the next round's first barrier
+    }
+    for (int k = warp; k < 2 * n; k += nw) {
+        const int slot = (k & 1) ? s_bot[par][k >> 1] : s_top[par][k >> 1];
+        const int col = s_col[slot];
+        if (col >= c) continue;
+        for (int i = lane; i < c; i += 32) Wg[(size_t)col * c + i] = w[(size_t)slot * ld + i];
+        if (S.v_smem)
+            for (int i = lane; i < c; i += 32) Vg[(size_t)col * c + i] = vs[(size_t)slot * ld + i];
+    }
+    if (rank == 0 && tid == 0) A.sweeps_out[P.idx] = sweep;
+}
+
 template <class... KArgs, class... Args>
 msp_status launch_cluster(void (*kernel)(KArgs...), int patches, int nc, int threads, size_t smem, cudaStream_t s,
                           Args... args) {
@@ -304,6 +626,134 @@ msp_status patch_cholesky(const PatchClasses& C, const PatchBlock* blocks, const
             count_launches(1);
         }
         MSP_CUDA(cudaGetLastError());
+    }
+    return MSP_OK;
+}
+
+// Cluster sizes of the sweeps.  A warp's FP64 instructions go to its quarter of the SM
+// at 64 to 76 clocks each, whatever its lanes hold, so a CTA does best with pairs for four
+// or eight full warps of inner products: 5 and 10 CTAs put 29 and 15 pairs of a 289-column
+// patch on a CTA where 4 and 8 put 37 (too many) and 19 (a fifth warp on one quarter).
+constexpr int kJacSizes = 7;
+constexpr int kJacNc[kJacSizes] = {16, 10, 8, 5, 4, 2, 1};
+
+// Cluster size of one patch: enough CTAs that it takes about its share of the GPU (twice
+// its work over the work per SM: up to three CTAs share an SM), as far as its columns
+// need them (32 pairs a CTA, W in shared memory) and as long as each has six pairs (below
+// that a round is shorter than its barriers); one below 48 columns; 0 when no cluster
+// holds W.
+static int jac_cluster(int c, double share, size_t room, int max_nc) {
+    auto fits = [&](int nc) {
+        const JacShape s = jac_shape(c, nc);
+        return s.bytes <= (nc > kPatchCluster ? kJacSmem : room) && (s.m + nc - 1) / nc <= kJacPairs;
+    };
+    if (c < 48) return fits(1) ? 1 : 0;
+    const double want = 2.0 * c * c * c / share;
+    int best = 0;
+    for (int q = kJacSizes - 2; q >= 0; --q) {         // ascending from 2
+        const int nc = kJacNc[q];
+        if (nc > max_nc || (best && (c + 1) / 2 < 6 * nc)) break;
+        if (!fits(nc)) continue;
+        best = nc;
+        if (nc >= want) break;
+    }
+    return best;
+}
+
+// Streams beside the caller's for launches that may overlap; on every way out the
+// caller's stream waits for them.
+struct ForkedStreams {
+    cudaStream_t main = nullptr;
+    cudaStream_t st[kJacSizes] = {};
+    cudaEvent_t fork = nullptr, join[kJacSizes] = {};
+    int n = 0;
+    msp_status open(cudaStream_t s) {
+        main = s;
+        MSP_CUDA(cudaEventCreateWithFlags(&fork, cudaEventDisableTiming));
+        MSP_CUDA(cudaEventRecord(fork, s));
+        return MSP_OK;
+    }
+    msp_status next(cudaStream_t* out) {
+        MSP_CUDA(cudaStreamCreateWithFlags(&st[n], cudaStreamNonBlocking));
+        const int k = n++;
+        MSP_CUDA(cudaEventCreateWithFlags(&join[k], cudaEventDisableTiming));
+        MSP_CUDA(cudaStreamWaitEvent(st[k], fork, 0));
+        *out = st[k];
+        return MSP_OK;
+    }
+    ~ForkedStreams() {
+        for (int k = 0; k < n; ++k) {
+            if (join[k]) {
+                cudaEventRecord(join[k], st[k]);
+                cudaStreamWaitEvent(main, join[k], 0);
+                cudaEventDestroy(join[k]);
+            }
+            cudaStreamDestroy(st[k]);                  // released when its work is done
+        }
+        if (fork) cudaEventDestroy(fork);
+    }
+};
+
+msp_status patch_jacobi(const std::vector<PatchBlock>& all, double* W, double* V, int max_sweeps, double tol,
+                        double small_rel, int* sweeps, DevBuf<PatchBlock>& d_blocks, std::vector<PatchBlock>& rest,
+                        cudaStream_t s) {
+    size_t room = 0;
+    MSP_TRY(smem_room(&room));
+    room -= 4096;                                      // the kernel's tables
+    double total = 0.0;
+    for (const PatchBlock& b : all) total += (double)b.c * b.c * b.c;
+    const double share = total / num_sms();
+    // more than 8 CTAs in a cluster are an option of the device: ask whether one can be resident
+    int max_nc = kPatchCluster;
+    MSP_CUDA(cudaFuncSetAttribute(patch_jacobi_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+    MSP_CUDA(cudaFuncSetAttribute(patch_jacobi_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)room));
+    for (int q = 0; q < kJacSizes && kJacNc[q] > max_nc; ++q) {
+        cudaLaunchConfig_t cfg{};
+        cfg.gridDim = dim3((unsigned)kJacNc[q]);
+        cfg.blockDim = dim3(kJacThreads);
+        cfg.dynamicSmemBytes = kJacSmem;
+        cudaLaunchAttribute at{};
+        at.id = cudaLaunchAttributeClusterDimension;
+        at.val.clusterDim.x = (unsigned)kJacNc[q];
+        at.val.clusterDim.y = at.val.clusterDim.z = 1;
+        cfg.attrs = &at;
+        cfg.numAttrs = 1;
+        int clusters = 0;
+        if (cudaOccupancyMaxActiveClusters(&clusters, patch_jacobi_kernel, &cfg) == cudaSuccess && clusters > 0)
+            max_nc = kJacNc[q];
+        else
+            (void)cudaGetLastError();
+    }
+    std::vector<PatchBlock> list;
+    rest.clear();
+    int first[kJacSizes + 1] = {};
+    size_t bytes[kJacSizes] = {};
+    for (int q = 0; q < kJacSizes; ++q) {
+        first[q] = (int)list.size();
+        for (const PatchBlock& b : all) {
+            const int nc = jac_cluster(b.c, share, room, max_nc);
+            if (nc == kJacNc[q]) {
+                list.push_back(b);
+                bytes[q] = std::max(bytes[q], jac_shape(b.c, nc).bytes);
+            } else if (nc == 0 && q == 0) {
+                rest.push_back(b);
+            }
+        }
+    }
+    first[kJacSizes] = (int)list.size();
+    MSP_TRY(upload(d_blocks, list, s));
+    // the largest patches first, the other sizes beside them
+    ForkedStreams fs;
+    MSP_TRY(fs.open(s));
+    bool on_main = true;
+    for (int q = 0; q < kJacSizes; ++q) {
+        const int count = first[q + 1] - first[q];
+        if (!count) continue;
+        cudaStream_t ss = s;
+        if (!on_main) MSP_TRY(fs.next(&ss));
+        on_main = false;
+        const JacArgs a{d_blocks.p + first[q], W, V, sweeps, max_sweeps, tol, small_rel};
+        MSP_TRY(launch_cluster(patch_jacobi_kernel, count, kJacNc[q], kJacThreads, bytes[q], ss, a));
     }
     return MSP_OK;
 }

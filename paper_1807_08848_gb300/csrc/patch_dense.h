@@ -30,4 +30,12 @@ PatchClasses classify_patches(const std::vector<int>& cols, const std::vector<lo
 msp_status patch_cholesky(const PatchClasses& C, const PatchBlock* blocks, const double* G, double* L, double* F,
                           double* Fi, const double* shift_scale, bool shifted, int* status, cudaStream_t s);
 
+// FP64 one-sided Jacobi sweeps of every block (W rotated to U S, V accumulating) with
+// each patch on a cluster; `all` largest first.  Blocks whose columns a cluster's
+// shared memory does not hold are returned in `rest`.  d_blocks is read until the
+// stream has passed the launches.
+msp_status patch_jacobi(const std::vector<PatchBlock>& all, double* W, double* V, int max_sweeps, double tol,
+                        double small_rel, int* sweeps, DevBuf<PatchBlock>& d_blocks, std::vector<PatchBlock>& rest,
+                        cudaStream_t s);
+
 }  // namespace msp
