@@ -265,152 +265,6 @@ __global__ void newton_schulz_kernel(const SmallMat* mats, double* G) {
 }
 
 
-// Householder QR with column pivoting of T (c x c, column-major; one CTA of 512
-// threads per patch), the preconditioner of the one-sided Jacobi SVD in the
-// manner of Drmac and Veselic (2008): with T P = Q R, the Jacobi sweeps run on
-// the columns of W = R^T, whose rows decay with the pivots, and V starts at Q, so
-// that the rotations J of the sweeps leave V = Q J, the left singular vectors of
-// T (the permutation only acts on the right).  Step j: squared norms of the
-// trailing columns over rows j.. (recomputed, no downdating), the largest swapped
-// into place, the reflector H_j = I - tau v v^T (v_0 = 1) that maps it onto
-// R(j, j) e_0, applied to the trailing columns.  Q = H_0 H_1 ... H_{c-1} is then
-// formed backwards in V.  A lives in shared memory (leading dimension c + 1) when
-// c <= smem_c, else in W, which is overwritten by R^T at the end either way.
-__global__ void __launch_bounds__(512) qrcp_kernel(const SmallMat* mats, const double* Tm, double* W, double* V,
-                                                   int smem_c) {
-    extern __shared__ __align__(16) unsigned char qr_smem[];
-    __shared__ double s_nrm[2 * kJacMaxPairs];
-    __shared__ double s_tau[2 * kJacMaxPairs];
-    __shared__ int s_piv;
-    const SmallMat S = mats[blockIdx.x];
-    const int c = S.c;
-    if (c < 1 || c > 2 * kJacMaxPairs) return;
-    const bool in_smem = c <= smem_c;
-    const int lda = in_smem ? c + 1 : c;
-    double* a = in_smem ? reinterpret_cast<double*>(qr_smem) : W + S.off;
-    double* q = V + S.off;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    for (long long e = threadIdx.x; e < (long long)c * c; e += blockDim.x) {
-        const int i = (int)(e % c), j = (int)(e / c);
-        a[i + (long long)j * lda] = Tm[S.off + e];
-    }
-    __syncthreads();
-    for (int j = 0; j < c; ++j) {
-        // squared norms of columns j.. over rows j..
-        for (int col = j + warp; col < c; col += nw) {
-            const double* ac = a + (long long)col * lda;
-            double t = 0.0;
-            for (int i = j + lane; i < c; i += 32) t = fma(ac[i], ac[i], t);
-            t = warp_sum(t);
-            if (lane == 0) s_nrm[col] = t;
-        }
-        __syncthreads();
-        if (warp == 0) {
-            double best = -1.0;
-            int bi = j;
-            for (int col = j + lane; col < c; col += 32)
-                if (s_nrm[col] > best) { best = s_nrm[col]; bi = col; }
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                const double ob = __shfl_xor_sync(0xffffffffu, best, o);
-                const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-                if (ob > best || (ob == best && oi < bi)) { best = ob; bi = oi; }
-            }
-            if (lane == 0) s_piv = bi;
-        }
-        __syncthreads();
-        const int p = s_piv;
-        if (p != j) {
-            for (int i = threadIdx.x; i < c; i += blockDim.x) {
-                const double x = a[i + (long long)j * lda];
-                a[i + (long long)j * lda] = a[i + (long long)p * lda];
-                a[i + (long long)p * lda] = x;
-            }
-        }
-        __syncthreads();
-        // reflector of column j: beta = -sign(alpha) |x|, tau = (beta - alpha) / beta,
-        // v = x(1:) / (alpha - beta) below the diagonal, R(j, j) = beta; the squared
-        // norm below the diagonal is summed afresh (a difference of the column norm
-        // and alpha^2 could cancel, and tau must match v for H_j to be orthogonal)
-        double* aj = a + (long long)j * lda;
-        if (warp == 0) {
-            double t = 0.0;
-            for (int i = j + 1 + lane; i < c; i += 32) t = fma(aj[i], aj[i], t);
-            t = warp_sum(t);
-            if (lane == 0) s_nrm[j] = t;
-        }
-        __syncthreads();
-        const double alpha = aj[j];
-        const double xn2 = s_nrm[j];
-        double tau = 0.0, scal = 0.0, beta = alpha;
-        if (xn2 > 0.0) {
-            beta = -copysign(sqrt(alpha * alpha + xn2), alpha);
-            tau = (beta - alpha) / beta;
-            scal = 1.0 / (alpha - beta);
-        }
-        __syncthreads();
-        if (tau != 0.0) {
-            for (int i = j + 1 + threadIdx.x; i < c; i += blockDim.x) aj[i] *= scal;
-        }
-        if (threadIdx.x == 0) {
-            aj[j] = beta;
-            s_tau[j] = tau;
-        }
-        __syncthreads();
-        if (tau != 0.0) {
-            // A(j:, col) -= tau v (v^T A(j:, col)) for the trailing columns, a warp each
-            for (int col = j + 1 + warp; col < c; col += nw) {
-                double* ac = a + (long long)col * lda;
-                double t = (lane == 0) ? ac[j] : 0.0;
-                for (int i = j + 1 + lane; i < c; i += 32) t = fma(aj[i], ac[i], t);
-                t = warp_sum(t) * tau;
-                if (lane == 0) ac[j] -= t;
-                for (int i = j + 1 + lane; i < c; i += 32) ac[i] = fma(-t, aj[i], ac[i]);
-            }
-        }
-        __syncthreads();
-    }
-    // Q = H_0 ... H_{c-1}: from the identity, H_j applied to rows j.. of columns j..
-    for (long long e = threadIdx.x; e < (long long)c * c; e += blockDim.x) {
-        const int i = (int)(e % c), j = (int)(e / c);
-        q[e] = (i == j) ? 1.0 : 0.0;
-    }
-    __syncthreads();
-    for (int j = c - 1; j >= 0; --j) {
-        const double tau = s_tau[j];
-        if (tau != 0.0) {
-            const double* aj = a + (long long)j * lda;
-            for (int col = j + warp; col < c; col += nw) {
-                double* qc = q + (long long)col * c;
-                double t = (lane == 0) ? qc[j] : 0.0;
-                for (int i = j + 1 + lane; i < c; i += 32) t = fma(aj[i], qc[i], t);
-                t = warp_sum(t) * tau;
-                if (lane == 0) qc[j] -= t;
-                for (int i = j + 1 + lane; i < c; i += 32) qc[i] = fma(-t, aj[i], qc[i]);
-            }
-        }
-        __syncthreads();
-    }
-    // W = R^T (lower triangular); in the global case R is read before W is written
-    // over it, column by column of W = row by row of R, through registers
-    if (in_smem) {
-        for (long long e = threadIdx.x; e < (long long)c * c; e += blockDim.x) {
-            const int i = (int)(e % c), j = (int)(e / c);
-            W[S.off + e] = (i >= j) ? a[j + (long long)i * lda] : 0.0;
-        }
-    } else {
-        // transpose in place: swap (i, j) and (j, i) for i > j, zero the upper part
-        for (long long e = threadIdx.x; e < (long long)c * c; e += blockDim.x) {
-            const int i = (int)(e % c), j = (int)(e / c);
-            if (i > j) {
-                const double r = a[j + (long long)i * lda];   // R(j, i), upper part
-                a[i + (long long)j * lda] = r;                // W(i, j)
-                a[j + (long long)i * lda] = 0.0;
-            }
-        }
-    }
-}
-
 // Column norms of W = singular values; sort descending (rank by comparison);
 // keep k = #{s_i > tau s_1}.  Writes sigma (sorted), order, k.
 __global__ void sort_truncate_kernel(const SmallMat* mats, const double* W, double tau, double* sig_tmp,
@@ -497,36 +351,60 @@ __global__ void edge_ops_kernel(int N, const double* aE, const double* aN, const
     }
 }
 
-// Patch block of the normal equations: B_m = sum_s cnt_s E[s]^T E[s] (k x k).
-__global__ void precond_block_kernel(const int* kk, const int* ne, const long long* e_off, const double* E,
-                                     const int* slot_off, const int* tr_ptr, const SmallMat* mats, double* Bm) {
-    const int m = blockIdx.x;
+// Patch block of the normal equations: B_m = sum_s cnt_s E[s]^T E[s] (k x k), its tiles on
+// and below the diagonal (the Cholesky reads the lower triangle).  32 x 32 outputs per CTA,
+// 2 x 2 per thread, 32 rows of E staged at a time, the left factor scaled by cnt_s as it is
+// staged; each output is one chain of FMAs over the rows in order.  FP64-bound
+// (k^2 n_s / 2 FMA); as one thread per output reading E from the cache it took 12.6 ms at
+// 513^2 and 30 ms at 2049^2.
+constexpr int kPbTile = 32, kPbRows = 32;
+__global__ void __launch_bounds__(256) precond_block_kernel(const int* kk, const int* ne, const long long* e_off,
+                                                            const double* E, const int* slot_off, const int* tr_ptr,
+                                                            const SmallMat* mats, double* Bm) {
+    __shared__ double As[kPbRows][kPbTile], Bs[kPbRows][kPbTile];
+    const int m = blockIdx.y;
     const int k = kk[m], ns = 2 * ne[m];
+    // tile (ti, tj), tj <= ti, numbered row by row
+    int ti = 0, rem = blockIdx.x;
+    while (rem > ti) rem -= ++ti;
+    const int i0 = ti * kPbTile, j0 = rem * kPbTile;
+    if (i0 >= k) return;
     const double* e = E + e_off[m];
-    for (long long w = threadIdx.x; w < (long long)k * k; w += blockDim.x) {
-        const int i = (int)(w % k), j = (int)(w / k);
-        double a = 0.0;
-        for (int s = 0; s < ns; ++s) {
-            const int g = slot_off[m] + s;
-            const int cnt = tr_ptr[g + 1] - tr_ptr[g];
-            if (cnt) a += cnt * e[(long long)s * k + i] * e[(long long)s * k + j];
+    const int* tp = tr_ptr + slot_off[m];
+    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+    double acc[2][2] = {};
+    for (int s0 = 0; s0 < ns; s0 += kPbRows) {
+        for (int q = threadIdx.x; q < kPbRows * kPbTile; q += 256) {
+            const int r = q / kPbTile, x = q % kPbTile, s = s0 + r;
+            double va = 0.0, vb = 0.0;
+            if (s < ns) {
+                const int cnt = tp[s + 1] - tp[s];
+                if (cnt) {
+                    if (i0 + x < k) va = cnt * e[(long long)s * k + i0 + x];
+                    if (j0 + x < k) vb = e[(long long)s * k + j0 + x];
+                }
+            }
+            As[r][x] = va;
+            Bs[r][x] = vb;
         }
-        Bm[mats[m].off + w] = a;
+        __syncthreads();
+#pragma unroll 8
+        for (int r = 0; r < kPbRows; ++r) {
+            const double a0 = As[r][tx], a1 = As[r][tx + 16], b0 = Bs[r][ty], b1 = Bs[r][ty + 16];
+            acc[0][0] = fma(a0, b0, acc[0][0]);
+            acc[1][0] = fma(a1, b0, acc[1][0]);
+            acc[0][1] = fma(a0, b1, acc[0][1]);
+            acc[1][1] = fma(a1, b1, acc[1][1]);
+        }
+        __syncthreads();
     }
-}
-
-// Binv = Fi Fi^T (Fi = L^{-T}, so Binv = (L L^T)^{-1}); stored at binv_off.
-__global__ void precond_inverse_kernel(const SmallMat* mats, const double* Fi, const long long* binv_off,
-                                       double* Binv) {
-    const SmallMat S = mats[blockIdx.x];
-    const int c = S.c;
-    const double* f = Fi + S.off;
-    for (long long w = threadIdx.x; w < (long long)c * c; w += blockDim.x) {
-        const int i = (int)(w % c), j = (int)(w / c);
-        double a = 0.0;
-        for (int l = max(i, j); l < c; ++l) a += f[i + (long long)l * c] * f[j + (long long)l * c];
-        Binv[binv_off[blockIdx.x] + w] = a;
-    }
+#pragma unroll
+    for (int u = 0; u < 2; ++u)
+#pragma unroll
+        for (int v = 0; v < 2; ++v) {
+            const int i = i0 + tx + 16 * u, j = j0 + ty + 16 * v;
+            if (i < k && j < k) Bm[mats[m].off + i + (long long)j * k] = acc[u][v];
+        }
 }
 
 }  // namespace
@@ -673,10 +551,10 @@ msp_status svd_bases(const double* snaps, long long snap_elems, const std::vecto
         // pairs of columns both below 1e-3 tau sigma_1 (|T|_F / sqrt(c) <= sigma_1) are not rotated
         const double small_rel = 1e-3 * tau / std::sqrt((double)std::max(maxc, 1));
         // the largest blocks first (their sweeps cost the most), so the last wave is short
-        std::vector<SmallMat> by_size(mats);
-        std::stable_sort(by_size.begin(), by_size.end(), [](const SmallMat& a, const SmallMat& b) { return a.c > b.c; });
-        MSP_TRY(upload(d_by_size, by_size, s));
         if (svd_mixed()) {
+            std::vector<SmallMat> by_size(mats);
+            std::stable_sort(by_size.begin(), by_size.end(), [](const SmallMat& a, const SmallMat& b) { return a.c > b.c; });
+            MSP_TRY(upload(d_by_size, by_size, s));
             // FP32 sweeps on (float) T^T from V = I, then V re-orthogonalised in FP64
             // by two Newton-Schulz steps (orthogonal to ~1e-6 -> ~1e-12 -> rounding),
             // W = T^T V; the FP64 sweeps below then start from nearly orthogonal
@@ -727,17 +605,7 @@ msp_status svd_bases(const double* snaps, long long snap_elems, const std::vecto
             }
             MSP_TRY(run_gemm(true, maxc, maxc));
         } else if (svd_qr()) {
-            cudaFuncAttributes fq{};
-            MSP_CUDA(cudaFuncGetAttributes(&fq, qrcp_kernel));
-            const long long dyn_max = (long long)optin - (long long)fq.sharedSizeBytes - 1024;
-            int cq = 0;
-            while ((long long)(cq + 1) * (cq + 2) * (long long)sizeof(double) <= dyn_max) ++cq;
-            cq = std::min(cq, maxc);
-            const size_t smq = (size_t)cq * (cq + 1) * sizeof(double);
-            MSP_CUDA(cudaFuncSetAttribute(qrcp_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smq));
-            qrcp_kernel<<<np, 512, smq, s>>>(d_by_size.p, Tacc, W.p, V.p, cq);
-            count_launches(1);
-            MSP_CUDA(cudaGetLastError());
+            MSP_TRY(patch_qrcp(classes, d_blocks.p, Tacc, W.p, V.p, L.p, G.p, s));
         } else {
             jacobi_init_kernel<<<np, 256, 0, s>>>(d_mats.p, Tacc, W.p, V.p);
             count_launches(1);
@@ -983,14 +851,34 @@ msp_status finish_basis(Basis& B, const double* aE_dev, const double* aN_dev, cu
     MSP_TRY(upload(d_kmats, kmats, s));
     MSP_TRY(upload(B.d_binv_off, B.binv_off, s));
     MSP_TRY(B.Binv.alloc(std::max<long long>(ko, 1), s));
-    precond_block_kernel<<<np, 256, 0, s>>>(B.d_k.p, B.d_ne.p, B.d_e_off.p, B.E.p, B.d_slot_off.p, B.tr_ptr.p,
-                                            d_kmats.p, G.p);
-    count_launches(1);
+    {
+        int maxk = 1;
+        for (int m = 0; m < np; ++m) maxk = std::max(maxk, B.k[m]);
+        const int tl = (maxk + kPbTile - 1) / kPbTile;
+        for (int m0 = 0; m0 < np; m0 += 65535) {
+            precond_block_kernel<<<dim3(tl * (tl + 1) / 2, std::min(65535, np - m0)), 256, 0, s>>>(
+                B.d_k.p + m0, B.d_ne.p + m0, B.d_e_off.p + m0, B.E.p, B.d_slot_off.p + m0, B.tr_ptr.p, d_kmats.p + m0,
+                G.p);
+            count_launches(1);
+        }
+    }
     const PatchClasses classes = classify_patches(B.k, B.binv_off);
     DevBuf<PatchBlock> d_blocks;
     MSP_TRY(upload(d_blocks, classes.blocks, s));
     MSP_TRY(patch_cholesky(classes, d_blocks.p, G.p, L.p, F.p, Fi.p, shift_scale.p, false, status.p, s));
-    precond_inverse_kernel<<<np, 256, 0, s>>>(d_kmats.p, Fi.p, B.d_binv_off.p, B.Binv.p);
+    // Binv = Fi Fi^T (Fi = L^{-T} upper triangular, so Binv = (L L^T)^{-1})
+    std::vector<GemmDesc> ig;
+    int maxk = 1;
+    for (int m = 0; m < np; ++m) {
+        const int k = B.k[m];
+        if (k == 0) continue;
+        ig.push_back(GemmDesc{Fi.p + B.binv_off[m], Fi.p + B.binv_off[m], B.Binv.p + B.binv_off[m], k, k, k, k, k, k, 1.0, 0.0});
+        ig.back().b_lower = 1;
+        maxk = std::max(maxk, k);
+    }
+    DevBuf<GemmDesc> d_ig;
+    MSP_TRY(upload(d_ig, ig, s));
+    gemm_batched<double>(d_ig.p, (int)ig.size(), maxk, maxk, false, true, s, kGemmStructured);
     // keep L_m^{-T} of every patch block: the scaling of the online factor
     MSP_TRY(B.bt_Fi.alloc(std::max<long long>(ko, 1), s));
     if (ko > 0) MSP_CUDA(cudaMemcpyAsync(B.bt_Fi.p, Fi.p, sizeof(double) * ko, cudaMemcpyDeviceToDevice, s));

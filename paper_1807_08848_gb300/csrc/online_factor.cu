@@ -42,33 +42,56 @@ struct PairBlock {
     int ld;              // leading dimension of that dense block
 };
 
-__global__ void assemble_kernel(const PairBlock* pb, const int* list_sa, const int* list_sb, const signed char* list_sg,
-                                const int* k, const long long* e_off, const int* slot_off, const double* E,
-                                double* dst_base) {
-    // one warp per (column j, 128 rows): lanes own rows i, i + 32, i + 64, i + 96 and
-    // accumulate them from one broadcast E_b value per list entry, in list order
+// H_ab(i, j) = sum over the pair's list of +- E_a[sa][i] E_b[sb][j]: 32 x 32 outputs per CTA
+// (blockIdx.y: tile), 2 x 2 per thread, 32 list entries staged at a time with the sign on
+// the right factor; each output is one chain of FMAs in list order.  FP64-bound (k_a k_b
+// FMA per entry); as one warp per column and CTA per pair it took 9.8 ms at 513^2 and
+// 43 ms at 2049^2.
+constexpr int kAsTile = 32, kAsRows = 32;
+__global__ void __launch_bounds__(256) assemble_kernel(const PairBlock* pb, const int* list_sa, const int* list_sb,
+                                                       const signed char* list_sg, const int* k, const long long* e_off,
+                                                       const int* slot_off, const double* E, double* dst_base) {
+    __shared__ double As[kAsRows][kAsTile], Bs[kAsRows][kAsTile];
     const PairBlock b = pb[blockIdx.x];
     const int ka = k[b.ma], kb = k[b.mb];
+    const int ta = (ka + kAsTile - 1) / kAsTile, tb = (kb + kAsTile - 1) / kAsTile;
+    if ((int)blockIdx.y >= ta * tb) return;
+    const int i0 = (int)(blockIdx.y % ta) * kAsTile, j0 = (int)(blockIdx.y / ta) * kAsTile;
     const double* Ea = E + e_off[b.ma];
     const double* Eb = E + e_off[b.mb];
     const int ga = slot_off[b.ma], gb = slot_off[b.mb];
-    const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-    const int nib = (ka + 127) / 128;
-    for (int task = threadIdx.x >> 5; task < kb * nib; task += nw) {
-        const int j = task / nib, i0 = (task - j * nib) * 128 + lane;
-        double a[4] = {0.0, 0.0, 0.0, 0.0};
-        for (int t = b.list_begin; t < b.list_end; ++t) {
-            const double* ea = Ea + (long long)(list_sa[t] - ga) * ka;
-            double e = Eb[(long long)(list_sb[t] - gb) * kb + j];
-            if (list_sg[t] < 0) e = -e;
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-                if (i0 + 32 * u < ka) a[u] = fma(ea[i0 + 32 * u], e, a[u]);
+    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+    double acc[2][2] = {};
+    for (int t0 = b.list_begin; t0 < b.list_end; t0 += kAsRows) {
+        for (int q = threadIdx.x; q < kAsRows * kAsTile; q += 256) {
+            const int r = q / kAsTile, x = q % kAsTile, t = t0 + r;
+            double va = 0.0, vb = 0.0;
+            if (t < b.list_end) {
+                if (i0 + x < ka) va = Ea[(long long)(list_sa[t] - ga) * ka + i0 + x];
+                if (j0 + x < kb) vb = Eb[(long long)(list_sb[t] - gb) * kb + j0 + x];
+                if (list_sg[t] < 0) vb = -vb;
+            }
+            As[r][x] = va;
+            Bs[r][x] = vb;
         }
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-            if (i0 + 32 * u < ka) dst_base[b.dst + (i0 + 32 * u) + (long long)j * b.ld] = a[u];
+        __syncthreads();
+#pragma unroll 8
+        for (int r = 0; r < kAsRows; ++r) {
+            const double a0 = As[r][tx], a1 = As[r][tx + 16], b0 = Bs[r][ty], b1 = Bs[r][ty + 16];
+            acc[0][0] = fma(a0, b0, acc[0][0]);
+            acc[1][0] = fma(a1, b0, acc[1][0]);
+            acc[0][1] = fma(a0, b1, acc[0][1]);
+            acc[1][1] = fma(a1, b1, acc[1][1]);
+        }
+        __syncthreads();
     }
+#pragma unroll
+    for (int u = 0; u < 2; ++u)
+#pragma unroll
+        for (int v = 0; v < 2; ++v) {
+            const int i = i0 + tx + 16 * u, j = j0 + ty + 16 * v;
+            if (i < ka && j < kb) dst_base[b.dst + i + (long long)j * b.ld] = acc[u][v];
+        }
 }
 
 // FP32 copy of one dense block of the scaled matrix, plus a shift on the diagonal
@@ -936,7 +959,10 @@ msp_status build_online_factor(Basis& B, const std::vector<int>& row_ptr, const 
     MSP_TRY(H64.alloc(std::max<long long>(total, 1), s));
     MSP_CUDA(cudaMemsetAsync(H64.p, 0, sizeof(double) * std::max<long long>(total, 1), s));
     if (!pb.empty()) {
-        assemble_kernel<<<(int)pb.size(), 256, 0, s>>>(d_pb.p, d_lsa.p, d_lsb.p, d_lsg.p, B.d_k.p, B.d_e_off.p,
+        int tiles = 1;
+        for (const PairBlock& p : pb)
+            tiles = std::max(tiles, ((B.k[p.ma] + kAsTile - 1) / kAsTile) * ((B.k[p.mb] + kAsTile - 1) / kAsTile));
+        assemble_kernel<<<dim3((unsigned)pb.size(), (unsigned)tiles), 256, 0, s>>>(d_pb.p, d_lsa.p, d_lsb.p, d_lsg.p, B.d_k.p, B.d_e_off.p,
                                                        B.d_slot_off.p, B.E.p, H64.p);
         count_launches(1);
     }
@@ -961,13 +987,15 @@ msp_status build_online_factor(Basis& B, const std::vector<int>& row_ptr, const 
             const double* Fb = B.bt_Fi.p + B.binv_off[pb[t].mb];
             g1[t] = GemmDesc{H64.p + pb[t].dst, Fb, Tp.p + toff[t], ka, kb, kb, pb[t].ld, kb, ka, 1.0, 0.0};
             g2[t] = GemmDesc{Fa, Tp.p + toff[t], Hs64.p + pb[t].dst, ka, kb, ka, ka, ka, pb[t].ld, 1.0, 0.0};
+            g1[t].b_upper = 1;   // F = L^{-T} is upper triangular
+            g2[t].a_lower = 1;
         }
         DevBuf<GemmDesc> d1, d2;
         MSP_TRY(upload(d1, g1, s));
         MSP_TRY(upload(d2, g2, s));
         if (!pb.empty()) {
-            gemm_batched<double>(d1.p, (int)pb.size(), maxk, maxk, false, false, s);
-            gemm_batched<double>(d2.p, (int)pb.size(), maxk, maxk, true, false, s);
+            gemm_batched<double>(d1.p, (int)pb.size(), maxk, maxk, false, false, s, kGemmStructured);
+            gemm_batched<double>(d2.p, (int)pb.size(), maxk, maxk, true, false, s, kGemmStructured);
         }
         MSP_CUDA(cudaGetLastError());
         MSP_CUDA(cudaStreamSynchronize(s));   // descriptor buffers go out of scope

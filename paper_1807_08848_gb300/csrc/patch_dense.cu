@@ -221,6 +221,197 @@ __global__ void __launch_bounds__(32 * kInvWarps) patch_inverse_kernel(const Pat
     }
 }
 
+// ------------------------------------------------------------------ pivoted QR
+constexpr int kQrThreads = 512;
+constexpr int kFormWarps = 8;       // columns of Q per CTA
+
+// Householder QR with column pivoting of T (c x c), one patch per cluster: column r lives
+// with CTA r mod nc, in shared memory (or in R, in_smem = 0).  Step j: the CTAs publish
+// their largest remaining partial norm, every CTA picks the same pivot, its owner forms
+// the reflector H_j = I - tau v v^T (v_0 = 1) that maps the column onto R(j, j) e_0 and
+// sends v to all, and every CTA applies it to its remaining columns; the squared norms over
+// the rows below are summed afresh in the same pass (no downdating).  Columns are not
+// moved: a table holds the column at each position of the permuted order.
+// W = R^T (lower triangular); R holds the reflectors, v below the diagonal and tau on it,
+// for patch_form_q_kernel.
+struct QrShared {
+    double cand[2][kPatchCluster];   // published candidates, by step parity
+    int cand_pos[2][kPatchCluster];
+    double tau[2], xn2;
+};
+
+__host__ __device__ inline size_t qr_head(int c, int nc) {   // bytes before the columns
+    const size_t l = (size_t)(c + nc - 1) / nc;
+    return ((2 * (size_t)c + l) * sizeof(double) + (l + (size_t)c) * sizeof(int) + 15) / 16 * 16;
+}
+
+__global__ void __launch_bounds__(kQrThreads) patch_qrcp_kernel(const PatchBlock* blocks, const double* T, double* W,
+                                                                double* R, double* cols, int in_smem) {
+    extern __shared__ __align__(16) double qsm[];
+    __shared__ QrShared S;
+    cg::cluster_group cl = cg::this_cluster();
+    const int nc = (int)cl.num_blocks(), rank = (int)cl.block_rank();
+    const PatchBlock P = blocks[blockIdx.x / nc];
+    const int c = P.c, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
+    if (c < 1) return;                                       // the whole cluster
+    const int nl = (c - rank + nc - 1) / nc, ml = (c + nc - 1) / nc;   // local columns
+    const int lda = c | 1;
+    double* vb = qsm;                                        // two reflectors, by step parity
+    double* nrm = vb + 2 * (size_t)c;                        // partial norms, < 0 when taken
+    int* pos = reinterpret_cast<int*>(nrm + ml);             // position of a local column
+    int* perm = pos + ml;                                    // column at a position
+    double* A = reinterpret_cast<double*>(reinterpret_cast<char*>(qsm) + qr_head(c, nc));
+    auto col = [&](int l) { return in_smem ? A + (size_t)l * lda : cols + P.off + (size_t)(rank + l * nc) * c; };
+    const double* Tm = T + P.off;
+    double* Rm = R + P.off;
+    for (int i = tid; i < c; i += blockDim.x) perm[i] = i;
+    for (int l = warp; l < nl; l += nw) {
+        double* a = col(l);
+        const double* src = Tm + (size_t)(rank + l * nc) * c;
+        double s = 0.0;
+        for (int i = lane; i < c; i += 32) {
+            const double x = src[i];
+            a[i] = x;
+            s = fma(x, x, s);
+        }
+        s = warp_sum(s);
+        if (lane == 0) {
+            nrm[l] = s;
+            pos[l] = rank + l * nc;
+        }
+    }
+    cl.sync();   // every CTA runs before its shared memory is written to
+    for (int j = 0; j < c; ++j) {
+        const int par = j & 1;
+        if (warp == 0) {                                     // local candidate, to every CTA
+            double best = -1.0;
+            int bp = c;
+            for (int l = lane; l < nl; l += 32) {
+                const double x = nrm[l];
+                if (x > best || (x == best && x >= 0.0 && pos[l] < bp)) { best = x; bp = pos[l]; }
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                const double ob = __shfl_xor_sync(0xffffffffu, best, o);
+                const int op = __shfl_xor_sync(0xffffffffu, bp, o);
+                if (ob > best || (ob == best && op < bp)) { best = ob; bp = op; }
+            }
+            if (lane < nc) {
+                QrShared* to = cl.map_shared_rank(&S, lane);
+                to->cand[par][rank] = best;
+                to->cand_pos[par][rank] = bp;
+            }
+        }
+        cl.sync();
+        double best = -1.0;
+        int bp = j;                                          // no candidate (NaN): the column in place
+        for (int q = 0; q < nc; ++q) {
+            const double b = S.cand[par][q];
+            const int p = S.cand_pos[par][q];
+            if (p < c && (b > best || (b == best && p < bp))) { best = b; bp = p; }
+        }
+        const int pc = perm[bp], moved = perm[j];            // pivot; the column it swaps with
+        if (pc % nc == rank) {
+            // beta = -sign(alpha) |x|, tau = (beta - alpha) / beta, v = x(1:) / (alpha - beta);
+            // the squared norm below the diagonal is summed by itself (a difference of
+            // the column norm and alpha^2 could cancel, and tau must match v)
+            double* a = col(pc / nc);
+            if (warp == 0) {
+                double s = 0.0;
+                for (int i = j + 1 + lane; i < c; i += 32) s = fma(a[i], a[i], s);
+                s = warp_sum(s);
+                if (lane == 0) S.xn2 = s;
+            }
+            __syncthreads();
+            const double alpha = a[j], xn2 = S.xn2;
+            double tau = 0.0, scal = 0.0, beta = alpha;
+            if (xn2 > 0.0) {
+                beta = -copysign(sqrt(alpha * alpha + xn2), alpha);
+                tau = (beta - alpha) / beta;
+                scal = 1.0 / (alpha - beta);
+            }
+            for (int i = j + 1 + tid; i < c; i += blockDim.x) {
+                const double v = tau != 0.0 ? a[i] * scal : a[i];
+                for (int q = 0; q < nc; ++q) cl.map_shared_rank(vb, q)[(size_t)par * c + i] = v;
+                Rm[(size_t)j * c + i] = v;
+            }
+            if (tid < nc) cl.map_shared_rank(&S, tid)->tau[par] = tau;
+            __syncthreads();
+            if (tid == 0) {
+                a[j] = beta;
+                Rm[(size_t)j * c + j] = tau;
+                nrm[pc / nc] = -1.0;
+                pos[pc / nc] = j;
+            }
+        }
+        cl.sync();
+        if (tid == 0) {
+            perm[j] = pc;
+            perm[bp] = moved;
+            if (moved != pc && moved % nc == rank) pos[moved / nc] = bp;
+        }
+        const double tau = S.tau[par];
+        const double* v = vb + (size_t)par * c;
+        // A(j:, l) -= tau v (v^T A(j:, l)) on the remaining local columns, a warp each
+        for (int l = warp; l < nl; l += nw) {
+            if (nrm[l] < 0.0) continue;
+            double* a = col(l);
+            double s = 0.0;
+            if (tau != 0.0) {
+                double t = (lane == 0) ? a[j] : 0.0;
+                for (int i = j + 1 + lane; i < c; i += 32) t = fma(v[i], a[i], t);
+                t = warp_sum(t) * tau;
+                if (lane == 0) a[j] -= t;
+                for (int i = j + 1 + lane; i < c; i += 32) {
+                    const double x = fma(-t, v[i], a[i]);
+                    a[i] = x;
+                    s = fma(x, x, s);
+                }
+            } else {
+                for (int i = j + 1 + lane; i < c; i += 32) s = fma(a[i], a[i], s);
+            }
+            s = warp_sum(s);
+            if (lane == 0) nrm[l] = s;
+        }
+        __syncthreads();
+    }
+    // W(p, j) = R(j, p) for j <= p: the column at position p, transposed
+    for (int l = warp; l < nl; l += nw) {
+        const int p = pos[l];
+        const double* a = col(l);
+        for (int j = lane; j < c; j += 32) W[P.off + p + (size_t)j * c] = j <= p ? a[j] : 0.0;
+    }
+    cl.sync();   // no CTA leaves while another may write its shared memory
+}
+
+// Q = H_0 H_1 ... H_{c-1} from the reflectors: column k of Q takes H_k, ..., H_0 applied to
+// e_k, a warp per column and every column by itself, so a patch takes c / 8 CTAs.
+__global__ void __launch_bounds__(32 * kFormWarps) patch_form_q_kernel(const PatchBlock* blocks, const double* R,
+                                                                       double* Q) {
+    extern __shared__ __align__(16) double fsm[];
+    const PatchBlock P = blocks[blockIdx.y];
+    const int c = P.c, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int k = (int)(blockIdx.x * kFormWarps) + warp;
+    if (k >= c) return;                                      // a whole warp; no block barrier follows
+    double* q = fsm + (size_t)warp * c;
+    const double* Rm = R + P.off;
+    for (int i = lane; i < c; i += 32) q[i] = (i == k) ? 1.0 : 0.0;
+    __syncwarp();
+    for (int j = k; j >= 0; --j) {
+        const double* v = Rm + (size_t)j * c;
+        const double tau = v[j];
+        if (tau != 0.0) {
+            double t = (lane == 0) ? q[j] : 0.0;
+            for (int i = j + 1 + lane; i < c; i += 32) t = fma(v[i], q[i], t);
+            t = warp_sum(t) * tau;
+            if (lane == 0) q[j] -= t;
+            for (int i = j + 1 + lane; i < c; i += 32) q[i] = fma(-t, v[i], q[i]);
+        }
+        __syncwarp();
+    }
+    for (int i = lane; i < c; i += 32) Q[P.off + (size_t)k * c + i] = q[i];
+}
+
 // ------------------------------------------------------------------ Jacobi
 constexpr int kJacThreads = 256;
 constexpr int kJacLanes = 8;                           // threads per column pair
@@ -623,6 +814,33 @@ msp_status patch_cholesky(const PatchClasses& C, const PatchBlock* blocks, const
             const unsigned nb = (unsigned)std::min<size_t>(65535, C.blocks.size() - b0);
             patch_inverse_kernel<<<dim3((c + kInvWarps - 1) / kInvWarps, nb), 32 * kInvWarps, bytes(tr), s>>>(
                 blocks + b0, L, F, Fi, status, tr);
+            count_launches(1);
+        }
+        MSP_CUDA(cudaGetLastError());
+    }
+    return MSP_OK;
+}
+
+msp_status patch_qrcp(const PatchClasses& C, const PatchBlock* blocks, const double* T, double* W, double* Q, double* R,
+                      double* cols, cudaStream_t s) {
+    size_t room = 0;
+    MSP_TRY(smem_room(&room));
+    const int count[2] = {C.n_big, (int)C.blocks.size() - C.n_big};
+    for (int cls = 0; cls < 2; ++cls) {
+        if (!count[cls] || C.max_c[cls] <= 0) continue;
+        const int nc = cls == 0 ? kPatchCluster : 1, c = C.max_c[cls];
+        const size_t own = sizeof(double) * ((size_t)(c + nc - 1) / nc) * (c | 1), head = qr_head(c, nc);
+        const int in_smem = head + own <= room ? 1 : 0;
+        MSP_TRY(launch_cluster(patch_qrcp_kernel, count[cls], nc, kQrThreads, in_smem ? head + own : head, s,
+                               blocks + (cls == 0 ? 0 : C.n_big), T, W, R, cols, in_smem));
+    }
+    const int c = std::max(C.max_c[0], C.max_c[1]);
+    if (c > 0) {
+        const size_t bytes = sizeof(double) * (size_t)kFormWarps * c;
+        MSP_CUDA(cudaFuncSetAttribute(patch_form_q_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+        for (size_t b0 = 0; b0 < C.blocks.size(); b0 += 65535) {
+            const unsigned nb = (unsigned)std::min<size_t>(65535, C.blocks.size() - b0);
+            patch_form_q_kernel<<<dim3((c + kFormWarps - 1) / kFormWarps, nb), 32 * kFormWarps, bytes, s>>>(blocks + b0, R, Q);
             count_launches(1);
         }
         MSP_CUDA(cudaGetLastError());

@@ -30,6 +30,14 @@ PatchClasses classify_patches(const std::vector<int>& cols, const std::vector<lo
 msp_status patch_cholesky(const PatchClasses& C, const PatchBlock* blocks, const double* G, double* L, double* F,
                           double* Fi, const double* shift_scale, bool shifted, int* status, cudaStream_t s);
 
+// Householder QR with column pivoting T P = Q R of every block: W = R^T and Q, the
+// preconditioner of the Jacobi sweeps in the manner of Drmac and Veselic (2008): the
+// sweeps run on the columns of R^T, whose rows decay with the pivots, with V started at Q,
+// so that their rotations J leave V = Q J, the left singular vectors of T (the
+// permutation only acts on the right).  R and cols are work blocks as large as T.
+msp_status patch_qrcp(const PatchClasses& C, const PatchBlock* blocks, const double* T, double* W, double* Q, double* R,
+                      double* cols, cudaStream_t s);
+
 // FP64 one-sided Jacobi sweeps of every block (W rotated to U S, V accumulating) with
 // each patch on a cluster; `all` largest first.  Blocks whose columns a cluster's
 // shared memory does not hold are returned in `rest`.  d_blocks is read until the
