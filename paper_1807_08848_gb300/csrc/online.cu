@@ -40,21 +40,70 @@ struct OnArgs {
     const int* row_bnd;
     const int* tr_ptr;
     const int* tr_ent;
+    // the same tables from patch m0 on (launches of at most 65535 patches)
+    OnArgs from(int m0) const {
+        OnArgs P = *this;
+        P.c_off += m0;
+        P.k += m0;
+        P.slot_off += m0;
+        P.ne += m0;
+        P.e_off += m0;
+        return P;
+    }
 };
 
-// e[slot][b] = sum_j E_m[slot][j] x_m[j][b] for every slot of patch m (one CTA per patch)
-__global__ void edge_apply_kernel(OnArgs A, const double* x, double* e) {
-    const int m = blockIdx.x, k = A.k[m], ns = 2 * A.ne[m], B = A.B;
+// Tiles of the per-patch products: kOpRows outputs (slots, coefficients or nodes) by up to
+// 4 kOpBatch data sets per CTA of 256 threads, the operator staged through shared memory
+// kOpK terms at a time.  A thread takes one output and BT data sets (group tid / 64), each a
+// chain of FMAs in the order of the terms, so no result depends on the tiling or the batch.
+// These products are bound by the FP64 pipe in batches and by the chain's latency for one
+// data set; as one CTA per patch they kept 64 of 152 SMs busy at 513^2 and read the operator
+// once per data set.
+constexpr int kOpRows = 64, kOpK = 32, kOpBatch = 8;
+
+__host__ __device__ inline int op_bt(int B) { return B <= 4 ? 1 : kOpBatch; }
+inline unsigned op_groups(int B) { return (unsigned)((B + 4 * op_bt(B) - 1) / (4 * op_bt(B))); }
+
+// e[slot][b] = sum_j E_m[slot][j] x_m[j][b]: blockIdx (slot tile, patch, data-set group)
+template <int BT>
+__global__ void __launch_bounds__(256) edge_apply_kernel(OnArgs A, const double* x, double* e) {
+    __shared__ double Es[kOpRows][kOpK + 1];
+    __shared__ double xs[kOpK][4 * BT];
+    const int m = blockIdx.y, k = A.k[m], ns = 2 * A.ne[m], B = A.B;
+    const int s0 = blockIdx.x * kOpRows, b0 = blockIdx.z * 4 * BT;
+    if (s0 >= ns) return;
     const double* Em = A.E + A.e_off[m];
     const double* xm = x + (long long)A.c_off[m] * B;
     double* em = e + (long long)A.slot_off[m] * B;
-    for (int w = threadIdx.x; w < ns * B; w += blockDim.x) {
-        const int s = w / B, b = w - s * B;
-        const double* er = Em + (long long)s * k;
-        double a = 0.0;
-        for (int j = 0; j < k; ++j) a += er[j] * xm[(long long)j * B + b];
-        em[w] = a;
+    const int row = threadIdx.x & (kOpRows - 1), grp = threadIdx.x / kOpRows;
+    const int s = s0 + row, bg = b0 + grp * BT;
+    const bool live = s < ns && bg < B;
+    double acc[BT];
+#pragma unroll
+    for (int t = 0; t < BT; ++t) acc[t] = 0.0;
+    for (int j0 = 0; j0 < k; j0 += kOpK) {
+        const int jn = min(kOpK, k - j0);
+        for (int q = threadIdx.x; q < kOpRows * kOpK; q += 256) {
+            const int r = q / kOpK, j = q % kOpK;
+            if (j < jn && s0 + r < ns) Es[r][j] = Em[(long long)(s0 + r) * k + j0 + j];
+        }
+        for (int q = threadIdx.x; q < kOpK * 4 * BT; q += 256) {
+            const int j = q / (4 * BT), b = q % (4 * BT);
+            if (j < jn && b0 + b < B) xs[j][b] = xm[(long long)(j0 + j) * B + b0 + b];
+        }
+        __syncthreads();
+        if (live)
+            for (int j = 0; j < jn; ++j) {
+                const double v = Es[row][j];
+#pragma unroll
+                for (int t = 0; t < BT; ++t) acc[t] += v * xs[j][grp * BT + t];
+            }
+        __syncthreads();
     }
+    if (live)
+#pragma unroll
+        for (int t = 0; t < BT; ++t)
+            if (bg + t < B) em[(long long)s * B + bg + t] = acc[t];
 }
 
 __device__ __forceinline__ double row_value(const OnArgs& A, const double* e, int r, int b) {
@@ -182,48 +231,90 @@ __global__ void normal_precond_kernel(OnArgs A, const double* r, double* z, doub
     }
 }
 
-// s = P~^T r per patch (gather the rows of every edge slot, then E_m^T); [element][B]
-__global__ void normal_rhs_kernel(OnArgs A, const double* r, double* sout) {
-    extern __shared__ double sm[];
-    const int m = blockIdx.x, k = A.k[m], ns = 2 * A.ne[m], B = A.B;
-    double* t = sm;   // [ns][B]
-    const int g0 = A.slot_off[m];
-    for (int w = threadIdx.x; w < ns * B; w += blockDim.x) {
-        const int s = w / B, b = w - s * B;
+// s = P~^T r in two passes: t[slot][b] = the signed sum of the rows that read the slot,
+// then s = E_m^T t per patch; [element][B]
+__global__ void __launch_bounds__(256) gather_rows_kernel(OnArgs A, const double* r, double* t, long long n) {
+    const int B = A.B;
+    for (long long w = blockIdx.x * 256LL + threadIdx.x; w < n; w += 256LL * gridDim.x) {
+        const int s = (int)(w / B), b = (int)(w - (long long)s * B);
         double a = 0.0;
-        for (int u = A.tr_ptr[g0 + s]; u < A.tr_ptr[g0 + s + 1]; ++u) {
+        for (int u = A.tr_ptr[s]; u < A.tr_ptr[s + 1]; ++u) {
             const unsigned v = (unsigned)A.tr_ent[u];
             const double x = r[(long long)(v & 0x7fffffffu) * B + b];
             a += (v & 0x80000000u) ? -x : x;
         }
         t[w] = a;
     }
-    __syncthreads();
-    const double* Em = A.E + A.e_off[m];
-    double* so = sout + (long long)A.c_off[m] * B;
-    for (int w = threadIdx.x; w < k * B; w += blockDim.x) {
-        const int j = w / B, b = w - j * B;
-        double a = 0.0;
-        for (int s = 0; s < ns; ++s) a += Em[(long long)s * k + j] * t[s * B + b];
-        so[w] = a;
-    }
 }
 
-// per-patch partial sums (s.z, s.s), fixed order over the patch's unknowns
-__global__ void dots_kernel(OnArgs A, const double* sv, const double* z, double* part) {
+template <int BT>
+__global__ void __launch_bounds__(256) normal_rhs_kernel(OnArgs A, const double* t, double* sout) {
+    __shared__ double Es[kOpK][kOpRows];
+    __shared__ double ts[kOpK][4 * BT];
+    const int m = blockIdx.y, k = A.k[m], ns = 2 * A.ne[m], B = A.B;
+    const int j0 = blockIdx.x * kOpRows, b0 = blockIdx.z * 4 * BT;
+    if (j0 >= k) return;
+    const double* Em = A.E + A.e_off[m];
+    const double* tm = t + (long long)A.slot_off[m] * B;
+    double* so = sout + (long long)A.c_off[m] * B;
+    const int row = threadIdx.x & (kOpRows - 1), grp = threadIdx.x / kOpRows;
+    const int j = j0 + row, bg = b0 + grp * BT;
+    const bool live = j < k && bg < B;
+    double acc[BT];
+#pragma unroll
+    for (int u = 0; u < BT; ++u) acc[u] = 0.0;
+    for (int s0 = 0; s0 < ns; s0 += kOpK) {
+        const int sn = min(kOpK, ns - s0);
+        for (int q = threadIdx.x; q < kOpRows * kOpK; q += 256) {
+            const int s = q / kOpRows, c = q % kOpRows;
+            if (s < sn && j0 + c < k) Es[s][c] = Em[(long long)(s0 + s) * k + j0 + c];
+        }
+        for (int q = threadIdx.x; q < kOpK * 4 * BT; q += 256) {
+            const int s = q / (4 * BT), b = q % (4 * BT);
+            if (s < sn && b0 + b < B) ts[s][b] = tm[(long long)(s0 + s) * B + b0 + b];
+        }
+        __syncthreads();
+        if (live)
+            for (int s = 0; s < sn; ++s) {
+                const double v = Es[s][row];
+#pragma unroll
+                for (int u = 0; u < BT; ++u) acc[u] += v * ts[s][grp * BT + u];
+            }
+        __syncthreads();
+    }
+    if (live)
+#pragma unroll
+        for (int u = 0; u < BT; ++u)
+            if (bg + u < B) so[(long long)j * B + bg + u] = acc[u];
+}
+
+// per-patch partial sums (s.z, s.s), fixed order over the patch's unknowns: the vectors
+// staged through shared memory, one thread per data set and sum
+__global__ void __launch_bounds__(128) dots_kernel(OnArgs A, const double* sv, const double* z, double* part) {
+    constexpr int kElems = 1024;
+    __shared__ double ss[kElems], zs[kElems];
     const int m = blockIdx.x, k = A.k[m], B = A.B;
     const double* sm_ = sv + (long long)A.c_off[m] * B;
     const double* zm = z + (long long)A.c_off[m] * B;
-    for (int b = threadIdx.x; b < B; b += blockDim.x) {
-        double sz = 0.0, ss = 0.0;
-        for (int j = 0; j < k; ++j) {
-            sz += sm_[(long long)j * B + b] * zm[(long long)j * B + b];
-            ss += sm_[(long long)j * B + b] * sm_[(long long)j * B + b];
+    const int rows = kElems / B;                       // B <= kMaxBatch
+    const int b = threadIdx.x >> 1, which = threadIdx.x & 1;
+    double a = 0.0;
+    for (int j0 = 0; j0 < k; j0 += rows) {
+        const int n = min(rows, k - j0) * B;
+        for (int e = threadIdx.x; e < n; e += 128) {
+            ss[e] = sm_[(long long)j0 * B + e];
+            zs[e] = zm[(long long)j0 * B + e];
         }
-        part[((long long)m * B + b) * 2 + 0] = sz;
-        part[((long long)m * B + b) * 2 + 1] = ss;
+        __syncthreads();
+        if (b < B) {
+            const double* o = which ? ss : zs;
+            for (int e = b; e < n; e += B) a += ss[e] * o[e];
+        }
+        __syncthreads();
     }
+    if (b < B) part[((long long)m * B + b) * 2 + which] = a;
 }
+static_assert(2 * kMaxBatch <= 128, "dots_kernel takes two threads per data set");
 
 // gamma' = sum_m s.z, |s| = sqrt(sum_m s.s); convergence; beta.  mode 0: first
 // call (sets gamma and |P^T d|), mode 1: iteration.  beta goes to scal[7].
@@ -278,33 +369,62 @@ __global__ void update_p_kernel(OnArgs A, double* p, const double* z, const doub
     }
 }
 
-// interior nodes of every K_m: u = Q_m c_m (one CTA per patch); Q in FP64, or in
-// FP32 for the map-based serving path (FP32 products, FP32 accumulation)
-template <class TQ, class TC>
-__global__ void recon_interior_kernel(OnArgs A, const PatchDev* patches, const long long* q_off, const TQ* Q,
-                                      const TC* c, double* u, int N) {
-    const int m = blockIdx.x, B = A.B, k = A.k[m];
+// interior nodes of every K_m: u = Q_m c_m; Q in FP64, or in FP32 for the map-based
+// serving path.  Products and partial sums of 16 terms in TQ, the partial sums added in
+// FP64.  A thread takes one node and BT data sets, so that a column of Q is read once,
+// coalesced, for all of them, and u is written along the rows; blockIdx (data-set group,
+// node tile, patch).  FP64: bound by the FP64 pipe in batches (n_k k B FMA), by the reading
+// of Q for one data set; FP32: by Q.
+template <class TQ, class TC, int BT>
+__global__ void __launch_bounds__(256) recon_interior_kernel(OnArgs A, const PatchDev* patches, const long long* q_off,
+                                                             const TQ* Q, const TC* c, double* u, int N) {
+    __shared__ TQ cs[16 * 16][BT];
+    const int m = blockIdx.z, B = A.B, k = A.k[m];
     const PatchDev P = patches[m];
     const int wi = P.x1 - P.x0 - 1, hi = P.y1 - P.y0 - 1;
-    if (wi <= 0 || hi <= 0) return;
-    const int wk = P.x1 - P.x0 + 1;
-    const TQ* q = Q + q_off[m];
+    const int b0 = blockIdx.x * BT, node0 = blockIdx.y * 256;
+    if (wi <= 0 || hi <= 0 || node0 >= wi * hi) return;
+    const int node = node0 + threadIdx.x;
+    const bool live = node < wi * hi;
+    const int ii = live ? node % wi + 1 : 0, jj = live ? node / wi + 1 : 0;
+    const TQ* q = Q + q_off[m] + ii + jj * (P.x1 - P.x0 + 1);
     const TC* cm = c + (long long)A.c_off[m] * B;
     const long long nn = (long long)(N + 1) * (N + 1);
-    for (long long w = threadIdx.x; w < (long long)wi * hi * B; w += blockDim.x) {
-        const int b = (int)(w % B);
-        const long long node = w / B;
-        const int ii = (int)(node % wi) + 1, jj = (int)(node / wi) + 1;
-        const int loc = ii + jj * wk;
-        // products and partial sums of 16 terms in TQ, the partial sums added in FP64
-        double a = 0.0;
-        for (int j0 = 0; j0 < k; j0 += 16) {
-            TQ part = TQ(0);
-            const int j1 = min(k, j0 + 16);
-            for (int j = j0; j < j1; ++j) part += q[loc + (long long)j * P.n_k] * (TQ)cm[(long long)j * B + b];
-            a += (double)part;
+    double a[BT];
+#pragma unroll
+    for (int t = 0; t < BT; ++t) a[t] = 0.0;
+    for (int k0 = 0; k0 < k; k0 += 256) {
+        const int kn = min(256, k - k0);
+        __syncthreads();
+        for (int e = threadIdx.x; e < kn * BT; e += 256) {
+            const int j = e / BT, t = e % BT;
+            cs[j][t] = b0 + t < B ? (TQ)cm[(long long)(k0 + j) * B + b0 + t] : TQ(0);
         }
-        u[(long long)b * nn + (long long)(P.y0 + jj) * (N + 1) + (P.x0 + ii)] = a;
+        __syncthreads();
+        if (live)
+            for (int j0 = 0; j0 < kn; j0 += 16) {
+                const int jn = min(16, kn - j0);
+                TQ part[BT], qv[16];
+#pragma unroll
+                for (int t = 0; t < BT; ++t) part[t] = TQ(0);
+#pragma unroll
+                for (int j = 0; j < 16; ++j)
+                    if (j < jn) qv[j] = q[(long long)(k0 + j0 + j) * P.n_k];
+#pragma unroll
+                for (int j = 0; j < 16; ++j)
+                    if (j < jn) {
+#pragma unroll
+                        for (int t = 0; t < BT; ++t) part[t] += qv[j] * cs[j0 + j][t];
+                    }
+#pragma unroll
+                for (int t = 0; t < BT; ++t) a[t] += (double)part[t];
+            }
+    }
+    if (live) {
+        double* un = u + (long long)(P.y0 + jj) * (N + 1) + (P.x0 + ii);
+#pragma unroll
+        for (int t = 0; t < BT; ++t)
+            if (b0 + t < B) un[(long long)(b0 + t) * nn] = a[t];
     }
 }
 
@@ -424,23 +544,54 @@ __global__ void __launch_bounds__(256) map_gemm_kernel(const float* G, const flo
 // Value slots of the edge operators for the map path: e[slot][b] for the even
 // (value) slots of every patch, from FP32 operators and coefficients, partial
 // sums of 16 terms in FP32 added in FP64.  Only the skeleton averages read them.
-__global__ void edge_values_map_kernel(OnArgs A, const float* E32, const float* c32, double* e) {
-    const int m = blockIdx.x, k = A.k[m], nt = A.ne[m], B = A.B;
+// Tiled like edge_apply_kernel: 64 ring nodes and up to 32 data sets per CTA.
+template <int BT>
+__global__ void __launch_bounds__(256) edge_values_map_kernel(OnArgs A, const float* E32, const float* c32, double* e) {
+    __shared__ float Es[kOpRows][kOpK + 1];
+    __shared__ float xs[kOpK][4 * BT];
+    const int m = blockIdx.y, k = A.k[m], nt = A.ne[m], B = A.B;
+    const int t0 = blockIdx.x * kOpRows, b0 = blockIdx.z * 4 * BT;
+    if (t0 >= nt) return;
     const float* Em = E32 + A.e_off[m];
     const float* xm = c32 + (long long)A.c_off[m] * B;
     double* em = e + (long long)A.slot_off[m] * B;
-    for (int w = threadIdx.x; w < nt * B; w += blockDim.x) {
-        const int t = w / B, b = w - t * B;
-        const float* er = Em + (long long)(2 * t) * k;
-        double a = 0.0;
-        for (int j0 = 0; j0 < k; j0 += 16) {
-            float part = 0.f;
-            const int j1 = min(k, j0 + 16);
-            for (int j = j0; j < j1; ++j) part = fmaf(er[j], xm[(long long)j * B + b], part);
-            a += (double)part;
+    const int row = threadIdx.x & (kOpRows - 1), grp = threadIdx.x / kOpRows;
+    const int bg = b0 + grp * BT;
+    const bool live = t0 + row < nt && bg < B;
+    double acc[BT];
+#pragma unroll
+    for (int t = 0; t < BT; ++t) acc[t] = 0.0;
+    for (int j0 = 0; j0 < k; j0 += kOpK) {
+        const int jn = min(kOpK, k - j0);
+        for (int q = threadIdx.x; q < kOpRows * kOpK; q += 256) {
+            const int r = q / kOpK, j = q % kOpK;
+            if (j < jn && t0 + r < nt) Es[r][j] = Em[(long long)(2 * (t0 + r)) * k + j0 + j];
         }
-        em[(long long)(2 * t) * B + b] = a;
+        for (int q = threadIdx.x; q < kOpK * 4 * BT; q += 256) {
+            const int j = q / (4 * BT), b = q % (4 * BT);
+            if (j < jn && b0 + b < B) xs[j][b] = xm[(long long)(j0 + j) * B + b0 + b];
+        }
+        __syncthreads();
+        if (live)
+            for (int h = 0; h < jn; h += 16) {
+                float part[BT];
+#pragma unroll
+                for (int t = 0; t < BT; ++t) part[t] = 0.f;
+                const int h1 = min(jn, h + 16);
+                for (int j = h; j < h1; ++j) {
+                    const float v = Es[row][j];
+#pragma unroll
+                    for (int t = 0; t < BT; ++t) part[t] = fmaf(v, xs[j][grp * BT + t], part[t]);
+                }
+#pragma unroll
+                for (int t = 0; t < BT; ++t) acc[t] += (double)part[t];
+            }
+        __syncthreads();
     }
+    if (live)
+#pragma unroll
+        for (int t = 0; t < BT; ++t)
+            if (bg + t < B) em[(long long)(2 * (t0 + row)) * B + bg + t] = acc[t];
 }
 
 }  // namespace
@@ -458,16 +609,75 @@ static OnArgs make_args(const Basis& Bs, int B) {
     return A;
 }
 
+// e = E x, s = E^T (gathered r) and the interior reconstruction for the batch of A
+static void launch_edge_apply(const Basis& Bs, const OnArgs& A, const double* x, double* e, cudaStream_t s) {
+    int ns = 1;
+    for (int n : Bs.n_e) ns = std::max(ns, 2 * n);
+    for (int m0 = 0; m0 < A.np; m0 += 65535) {
+        const OnArgs P = A.from(m0);
+        const dim3 g((ns + kOpRows - 1) / kOpRows, std::min(65535, A.np - m0), op_groups(A.B));
+        if (op_bt(A.B) == 1) edge_apply_kernel<1><<<g, 256, 0, s>>>(P, x, e);
+        else edge_apply_kernel<kOpBatch><<<g, 256, 0, s>>>(P, x, e);
+        count_launches(1);
+    }
+}
+
+// t is scratch of n_slots x B
+static void launch_normal_rhs(const Basis& Bs, const OnArgs& A, const double* r, double* t, double* sout, cudaStream_t s) {
+    int k = 1;
+    for (int v : Bs.k) k = std::max(k, v);
+    const long long n = (long long)Bs.n_slots * A.B;
+    gather_rows_kernel<<<(int)std::max<long long>(1, std::min<long long>((n + 255) / 256, num_sms() * 32LL)), 256, 0, s>>>(
+        A, r, t, n);
+    count_launches(1);
+    for (int m0 = 0; m0 < A.np; m0 += 65535) {
+        const OnArgs P = A.from(m0);
+        const dim3 g((k + kOpRows - 1) / kOpRows, std::min(65535, A.np - m0), op_groups(A.B));
+        if (op_bt(A.B) == 1) normal_rhs_kernel<1><<<g, 256, 0, s>>>(P, t, sout);
+        else normal_rhs_kernel<kOpBatch><<<g, 256, 0, s>>>(P, t, sout);
+        count_launches(1);
+    }
+}
+
+static void launch_edge_values_map(const Basis& Bs, const OnArgs& A, const float* E32, const float* c32, double* e,
+                                   cudaStream_t s) {
+    int nt = 1;
+    for (int n : Bs.n_e) nt = std::max(nt, n);
+    for (int m0 = 0; m0 < A.np; m0 += 65535) {
+        const OnArgs P = A.from(m0);
+        const dim3 g((nt + kOpRows - 1) / kOpRows, std::min(65535, A.np - m0), op_groups(A.B));
+        if (op_bt(A.B) == 1) edge_values_map_kernel<1><<<g, 256, 0, s>>>(P, E32, c32, e);
+        else edge_values_map_kernel<kOpBatch><<<g, 256, 0, s>>>(P, E32, c32, e);
+        count_launches(1);
+    }
+}
+
+template <class TQ, class TC>
+static void launch_recon_interior(const Basis& Bs, const OnArgs& A, const TQ* Q, const TC* c, double* u, cudaStream_t s) {
+    int nodes = 0;
+    for (const PatchDev& P : Bs.patches) nodes = std::max(nodes, (P.x1 - P.x0 - 1) * (P.y1 - P.y0 - 1));
+    if (nodes <= 0) return;
+    const int bt = op_bt(A.B);
+    for (int m0 = 0; m0 < A.np; m0 += 65535) {
+        const OnArgs P = A.from(m0);
+        const dim3 g((A.B + bt - 1) / bt, (nodes + 255) / 256, std::min(65535, A.np - m0));
+        if (bt == 1)
+            recon_interior_kernel<TQ, TC, 1><<<g, 256, 0, s>>>(P, Bs.d_patches.p + m0, Bs.d_q_off.p + m0, Q, c, u, Bs.N);
+        else
+            recon_interior_kernel<TQ, TC, kOpBatch><<<g, 256, 0, s>>>(P, Bs.d_patches.p + m0, Bs.d_q_off.p + m0, Q, c, u,
+                                                                      Bs.N);
+        count_launches(1);
+    }
+}
+
 // reconstruction u = sum_m chi_m Q_m c_m (interior of the patches, then the
 // skeleton from the edge values, phi on the domain boundary) for coefficients c
 // in the [coefficient][B] layout; e is scratch of n_slots x B
 static void reconstruct(const Basis& Bs, const OnArgs& A, const double* c, double* e, const double* phi, int n4,
                         double* u, cudaStream_t s) {
-    const int np = (int)Bs.patches.size(), N = Bs.N, B = A.B;
-    recon_interior_kernel<double, double><<<np, 256, 0, s>>>(A, Bs.d_patches.p, Bs.d_q_off.p, Bs.Q.p, c, u, N);
-    count_launches(1);
-    edge_apply_kernel<<<np, 256, 0, s>>>(A, c, e);
-    count_launches(1);
+    const int N = Bs.N, B = A.B;
+    launch_recon_interior(Bs, A, (const double*)Bs.Q.p, c, u, s);
+    launch_edge_apply(Bs, A, c, e, s);
     const int sk_grid = std::max(1, std::min<int>((int)(((long long)Bs.n_skel * B + 255) / 256), num_sms() * 8));
     recon_skeleton_kernel<<<sk_grid, 256, 0, s>>>(A, Bs.n_skel, Bs.sk_ptr.p, Bs.sk_slot.p, Bs.sk_node.p, Bs.sk_ring.p,
                                                   e, phi, n4, u, N);
@@ -508,17 +718,16 @@ static msp_status online_batch(Basis& Bs, const double* phi, int B, double tol, 
     const size_t smem = sizeof(double) * ((size_t)max_ns * B + (size_t)max_k * B);
     if (smem > 48 * 1024) {
         MSP_CUDA(cudaFuncSetAttribute(normal_precond_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        MSP_CUDA(cudaFuncSetAttribute(normal_rhs_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     }
     if (Bs.w_s.n < (size_t)nc) MSP_TRY(Bs.w_s.alloc((size_t)std::max(Bs.Np, 1) * kMaxBatch, s));
     // z = M^{-1} P~^T r and the partial sums (s.z, s.s): block-row factor when built,
     // patch-block (additive Schwarz) inverses otherwise
     auto precondition = [&]() -> msp_status {
         if (Bs.bt_q > 0 && !Bs.use_block_jacobi) {
-            normal_rhs_kernel<<<np, 256, smem, s>>>(A, Bs.w_r.p, Bs.w_s.p);
-            count_launches(1);
+            // the edge values e are read out by now: their buffer takes the gathered rows
+            launch_normal_rhs(Bs, A, Bs.w_r.p, Bs.w_e.p, Bs.w_s.p, s);
             MSP_TRY(apply_online_factor(Bs, Bs.w_s.p, Bs.w_z.p, B, s));
-            dots_kernel<<<np, 64, 0, s>>>(A, Bs.w_s.p, Bs.w_z.p, Bs.w_part.p);
+            dots_kernel<<<np, 128, 0, s>>>(A, Bs.w_s.p, Bs.w_z.p, Bs.w_part.p);
             count_launches(1);
         } else {
             normal_precond_kernel<<<np, 256, smem, s>>>(A, Bs.w_r.p, Bs.w_z.p, Bs.w_part.p);
@@ -541,8 +750,7 @@ static msp_status online_batch(Basis& Bs, const double* phi, int B, double tol, 
     std::vector<double> scal(8 * (size_t)B);
     const int check_every = (Bs.bt_q > 0 && !Bs.use_block_jacobi) ? 2 : 16;
     for (int it = 0; it < max_iter; ++it) {
-        edge_apply_kernel<<<np, 256, 0, s>>>(A, Bs.w_p.p, Bs.w_e.p);
-        count_launches(1);
+        launch_edge_apply(Bs, A, Bs.w_p.p, Bs.w_e.p, s);
         rows_apply_kernel<<<A.n_chunks, kRowChunk, 0, s>>>(A, Bs.w_e.p, Bs.w_q.p, Bs.w_part.p, phi, n4, Bs.w_r.p, 0);
         count_launches(1);
         finalize_alpha_kernel<<<1, 1024, 0, s>>>(A, Bs.w_part.p, Bs.w_scal.p);
@@ -653,8 +861,7 @@ msp_status online_solve_constrained(Basis& Bs, const double* phi, int batch, dou
         const double* ph = phi + (long long)b0 * n4;
         const OnArgs AB = make_args(Bs, B), AR = make_args(R, B);
         cons_particular(Bs, C, ph, n4, B, C.cp.p, s);
-        edge_apply_kernel<<<np, 256, 0, s>>>(AB, C.cp.p, C.ep.p);
-        count_launches(1);
+        launch_edge_apply(Bs, AB, C.cp.p, C.ep.p, s);
         rows_apply_kernel<<<AR.n_chunks, kRowChunk, 0, s>>>(AR, C.ep.p, C.dq.p, C.part.p, ph, n4, nullptr, 0);
         count_launches(1);
         MSP_CUDA(cudaGetLastError());
@@ -814,10 +1021,8 @@ msp_status online_solve_map(const Basis& Bs, const double* phi, int batch, doubl
         }
         OnArgs A = make_args(Bs, B);
         double* ub = u + (long long)b0 * nn;
-        recon_interior_kernel<float, float><<<np, 256, 0, s>>>(A, Bs.d_patches.p, Bs.d_q_off.p, Bs.Q32.p, work->c32, ub, N);
-        count_launches(1);
-        edge_values_map_kernel<<<np, 256, 0, s>>>(A, Bs.E32.p, work->c32, work->e);
-        count_launches(1);
+        launch_recon_interior(Bs, A, (const float*)Bs.Q32.p, (const float*)work->c32, ub, s);
+        launch_edge_values_map(Bs, A, Bs.E32.p, work->c32, work->e, s);
         const int sk_grid = std::max(1, std::min<int>((int)(((long long)Bs.n_skel * B + 255) / 256), num_sms() * 8));
         recon_skeleton_kernel<<<sk_grid, 256, 0, s>>>(A, Bs.n_skel, Bs.sk_ptr.p, Bs.sk_slot.p, Bs.sk_node.p,
                                                       Bs.sk_ring.p, work->e, ph, n4, ub, N);

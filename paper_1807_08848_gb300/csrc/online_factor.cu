@@ -113,34 +113,89 @@ __global__ void round_kernel(const double* src, float* dst, long long n) {
 }
 
 // per-patch products with R_m^{-1} = F_m (upper, k x k column-major):
-// y = F^T s (FP64 in, FP32 out) before the sweeps, z = F x (FP32 in, FP64 out) after
-template <class T>
-__global__ void patch_pre_kernel(const double* F, const long long* f_off, const int* k, const int* c_off,
-                                 const double* s, T* y, int B) {
-    const int m = blockIdx.x, km = k[m];
+// y = F^T s (FP64 in, T out) before the sweeps, z = F x (T in, FP64 out) after.
+// 64 coefficients by up to 32 data sets per CTA, F staged 32 terms at a time, every
+// output one chain of FMAs in the order of the terms; blockIdx (tile, patch, data sets)
+constexpr int kPpRows = 64, kPpK = 32;
+template <class T, int BT>
+__global__ void __launch_bounds__(256) patch_pre_kernel(const double* F, const long long* f_off, const int* k,
+                                                        const int* c_off, const double* s, T* y, int B) {
+    __shared__ double Fs[kPpRows][kPpK + 1];
+    __shared__ double ss[kPpK][4 * BT];
+    const int m = blockIdx.y, km = k[m], i0 = blockIdx.x * kPpRows, b0 = blockIdx.z * 4 * BT;
+    if (i0 >= km) return;
     const double* Fm = F + f_off[m];
     const double* sm = s + (long long)c_off[m] * B;
     T* ym = y + (long long)c_off[m] * B;
-    for (int w = threadIdx.x; w < km * B; w += blockDim.x) {
-        const int i = w / B, b = w - i * B;
-        double a = 0.0;
-        for (int j = 0; j <= i; ++j) a += Fm[j + (long long)i * km] * sm[(long long)j * B + b];
-        ym[w] = (T)a;
+    const int row = threadIdx.x & (kPpRows - 1), grp = threadIdx.x / kPpRows;
+    const int i = i0 + row, bg = b0 + grp * BT;
+    const bool live = i < km && bg < B;
+    double acc[BT];
+#pragma unroll
+    for (int t = 0; t < BT; ++t) acc[t] = 0.0;
+    for (int j0 = 0; j0 < min(km, i0 + kPpRows); j0 += kPpK) {
+        for (int q = threadIdx.x; q < kPpRows * kPpK; q += 256) {
+            const int r = q / kPpK, j = q % kPpK;
+            if (i0 + r < km && j0 + j < km) Fs[r][j] = Fm[j0 + j + (long long)(i0 + r) * km];
+        }
+        for (int q = threadIdx.x; q < kPpK * 4 * BT; q += 256) {
+            const int j = q / (4 * BT), b = q % (4 * BT);
+            if (j0 + j < km && b0 + b < B) ss[j][b] = sm[(long long)(j0 + j) * B + b0 + b];
+        }
+        __syncthreads();
+        const int jn = min(kPpK, i - j0 + 1);          // terms j <= i
+        if (live)
+            for (int j = 0; j < jn; ++j) {
+                const double v = Fs[row][j];
+#pragma unroll
+                for (int t = 0; t < BT; ++t) acc[t] += v * ss[j][grp * BT + t];
+            }
+        __syncthreads();
     }
+    if (live)
+#pragma unroll
+        for (int t = 0; t < BT; ++t)
+            if (bg + t < B) ym[(long long)i * B + bg + t] = (T)acc[t];
 }
-template <class T>
-__global__ void patch_post_kernel(const double* F, const long long* f_off, const int* k, const int* c_off,
-                                  const T* x, double* z, int B) {
-    const int m = blockIdx.x, km = k[m];
+template <class T, int BT>
+__global__ void __launch_bounds__(256) patch_post_kernel(const double* F, const long long* f_off, const int* k,
+                                                         const int* c_off, const T* x, double* z, int B) {
+    __shared__ double Fs[kPpK][kPpRows];
+    __shared__ double xs[kPpK][4 * BT];
+    const int m = blockIdx.y, km = k[m], i0 = blockIdx.x * kPpRows, b0 = blockIdx.z * 4 * BT;
+    if (i0 >= km) return;
     const double* Fm = F + f_off[m];
     const T* xm = x + (long long)c_off[m] * B;
     double* zm = z + (long long)c_off[m] * B;
-    for (int w = threadIdx.x; w < km * B; w += blockDim.x) {
-        const int i = w / B, b = w - i * B;
-        double a = 0.0;
-        for (int j = i; j < km; ++j) a += Fm[i + (long long)j * km] * (double)xm[(long long)j * B + b];
-        zm[w] = a;
+    const int row = threadIdx.x & (kPpRows - 1), grp = threadIdx.x / kPpRows;
+    const int i = i0 + row, bg = b0 + grp * BT;
+    const bool live = i < km && bg < B;
+    double acc[BT];
+#pragma unroll
+    for (int t = 0; t < BT; ++t) acc[t] = 0.0;
+    for (int j0 = i0; j0 < km; j0 += kPpK) {
+        const int jn = min(kPpK, km - j0);
+        for (int q = threadIdx.x; q < kPpRows * kPpK; q += 256) {
+            const int j = q / kPpRows, r = q % kPpRows;
+            if (i0 + r < km && j < jn) Fs[j][r] = Fm[i0 + r + (long long)(j0 + j) * km];
+        }
+        for (int q = threadIdx.x; q < kPpK * 4 * BT; q += 256) {
+            const int j = q / (4 * BT), b = q % (4 * BT);
+            if (j < jn && b0 + b < B) xs[j][b] = (double)xm[(long long)(j0 + j) * B + b0 + b];
+        }
+        __syncthreads();
+        if (live)
+            for (int j = max(0, i - j0); j < jn; ++j) {   // terms j >= i
+                const double v = Fs[j][row];
+#pragma unroll
+                for (int t = 0; t < BT; ++t) acc[t] += v * xs[j][grp * BT + t];
+            }
+        __syncthreads();
     }
+    if (live)
+#pragma unroll
+        for (int t = 0; t < BT; ++t)
+            if (bg + t < B) zm[(long long)i * B + bg + t] = acc[t];
 }
 
 // Cholesky of one <= 64 x 64 diagonal tile in shared memory; writes L (lower,
@@ -355,6 +410,8 @@ struct SweepArgs {
     const T* F;
     T* y;
     T* x;
+    const int* row_lo;         // per unknown of block q: first nonzero column of its row of C_{q-1}
+    const int* col_hi;         // per unknown of block q: end of the nonzero rows of its column of C_q
     unsigned int* bar;         // [0] arrivals, [1] generation
     int* err;
     long long spin_limit;      // polls of the generation word before a CTA gives up
@@ -395,19 +452,33 @@ __device__ __forceinline__ bool grid_barrier(unsigned int* bar, unsigned int nbl
 }
 
 // Y[j][b] = alpha sum_k M[k][j] X[k][b] + beta Y[j][b] for b < B, spread over the
-// whole grid: one output column per warp and round, lanes along K.  The rows of X
-// needed by a K chunk are staged in shared memory by every CTA (all CTAs run the
-// same rounds and chunks, so the block barriers are uniform).
+// whole grid: one output column and BT data sets per warp and round, lanes along K.
+// range(j) bounds the nonzeros of column j (the triangle of L^{-1}, the coupled patches
+// of C): the blocks of 32 terms outside it are exact zeros and are skipped.  The CTAs are
+// dealt to the groups of BT data sets, and consecutive columns to different CTAs, so that
+// the long and the short columns of a triangle spread evenly over the SMs (FP64 products
+// are bound by the FP64 pipe of each).  The rows of X needed by a K chunk are staged in
+// shared memory by every CTA that has a column (its block barriers are uniform).
 constexpr int kSweepKC = 1024;
-template <class T, int BT>
+template <class T, int BT, class Range>
 __device__ __forceinline__ void sweep_product(const T* X, const T* M, int ldm, T* Y, int K, int ncols, int B, T alpha,
-                                              T beta, int gw, int nw, int lane, T* xs) {
-    for (int j0 = 0; j0 < ncols; j0 += nw) {
-        const int j = j0 + gw;
-        const bool live = j < ncols;
-        const T* mj = M + (long long)(live ? j : 0) * ldm;
-        for (int b0 = 0; b0 < B; b0 += BT) {
-            const int bt = min(BT, B - b0);
+                                              T beta, int lane, T* xs, Range range) {
+    const int nbc = (B + BT - 1) / BT, ng = min(nbc, (int)gridDim.x);
+    const int group = blockIdx.x % ng, cta = blockIdx.x / ng;
+    const int nctas = ((int)gridDim.x - group + ng - 1) / ng;   // CTAs of this group
+    const int warp = threadIdx.x >> 5, wpb = blockDim.x >> 5;
+    for (int bc = group; bc < nbc; bc += ng) {
+        const int b0 = bc * BT, bt = min(BT, B - b0);
+        for (int j0 = 0; j0 + cta < ncols; j0 += wpb * nctas) {
+            const int j = j0 + warp * nctas + cta;
+            const bool live = j < ncols;
+            const T* mj = M + (long long)(live ? j : 0) * ldm;
+            int lo = 0, hi = 0;
+            if (live) {
+                const int2 r = range(j);
+                lo = r.x;
+                hi = min(K, r.y);
+            }
             T acc[BT];
 #pragma unroll
             for (int t = 0; t < BT; ++t) acc[t] = T(0);
@@ -419,13 +490,12 @@ __device__ __forceinline__ void sweep_product(const T* X, const T* M, int ldm, T
                     xs[t * kSweepKC + kk] = __ldcg(X + (long long)(kc + kk) * B + b0 + t);
                 }
                 __syncthreads();
-                if (live) {
+                const int k1 = min(kn, hi - kc);
 #pragma unroll 8
-                    for (int kk = lane; kk < kn; kk += 32) {
-                        const T m = mj[kc + kk];
+                for (int kk = max(0, lo - kc) / 32 * 32 + lane; kk < k1; kk += 32) {
+                    const T m = mj[kc + kk];
 #pragma unroll
-                        for (int t = 0; t < BT; ++t) acc[t] = fma(m, xs[t * kSweepKC + kk], acc[t]);
-                    }
+                    for (int t = 0; t < BT; ++t) acc[t] = fma(m, xs[t * kSweepKC + kk], acc[t]);
                 }
             }
 #pragma unroll
@@ -445,8 +515,6 @@ __global__ void __launch_bounds__(512) sweep_kernel(SweepArgs<T> A) {
     extern __shared__ __align__(16) unsigned char sweep_smem[];
     T* xs = reinterpret_cast<T*>(sweep_smem);   // kSweepKC x BT
     const int lane = threadIdx.x & 31;
-    const int wpb = blockDim.x >> 5;
-    const int gw = blockIdx.x * wpb + (threadIdx.x >> 5), nw = gridDim.x * wpb;
     unsigned int gen = atomicAdd(&A.bar[1], 0u);
     const int B = A.B;
     // forward: y_q -= x_{q-1} C_{q-1}^T;  x_q = y_q Li_q^T
@@ -457,12 +525,12 @@ __global__ void __launch_bounds__(512) sweep_kernel(SweepArgs<T> A) {
             const int o0 = A.off[q - 1], n0 = o - o0;
             if (n0 > 0) {
                 sweep_product<T, BT>(A.x + (long long)o0 * B, A.FT + A.e_off[q - 1], n0, A.y + (long long)o * B, n0, nq,
-                                     B, T(-1), T(1), gw, nw, lane, xs);
+                                     B, T(-1), T(1), lane, xs, [&](int j) { return make_int2(A.row_lo[o + j], n0); });
                 if (!grid_barrier(A.bar, gridDim.x, gen, A.err, A.spin_limit)) return;
             }
         }
         sweep_product<T, BT>(A.y + (long long)o * B, A.LiT + A.d_off[q], nq, A.x + (long long)o * B, nq, nq, B, T(1),
-                             T(0), gw, nw, lane, xs);
+                             T(0), lane, xs, [&](int j) { return make_int2(0, j + 1); });
         if (!grid_barrier(A.bar, gridDim.x, gen, A.err, A.spin_limit)) return;
     }
     // backward: x_q -= z_{q+1} C_q;  z_q = x_q Li_q   (z into y)
@@ -473,12 +541,12 @@ __global__ void __launch_bounds__(512) sweep_kernel(SweepArgs<T> A) {
             const int o1 = A.off[q + 1], n1 = A.off[q + 2] - o1;
             if (n1 > 0) {
                 sweep_product<T, BT>(A.y + (long long)o1 * B, A.F + A.e_off[q], n1, A.x + (long long)o * B, n1, nq, B,
-                                     T(-1), T(1), gw, nw, lane, xs);
+                                     T(-1), T(1), lane, xs, [&](int j) { return make_int2(0, A.col_hi[o + j]); });
                 if (!grid_barrier(A.bar, gridDim.x, gen, A.err, A.spin_limit)) return;
             }
         }
         sweep_product<T, BT>(A.x + (long long)o * B, A.Li + A.d_off[q], nq, A.y + (long long)o * B, nq, nq, B, T(1), T(0),
-                             gw, nw, lane, xs);
+                             lane, xs, [&](int j) { return make_int2(j, nq); });
         if (!grid_barrier(A.bar, gridDim.x, gen, A.err, A.spin_limit)) return;
     }
 }
@@ -1016,6 +1084,18 @@ msp_status build_online_factor(Basis& B, const std::vector<int>& row_ptr, const 
             for (int r = B.bt_off[q + 1] - 2; r >= B.bt_off[q]; --r) rowlo[r] = std::min(rowlo[r], rowlo[r + 1]);
         }
         MSP_TRY(upload(B.d_bt_rowlo, rowlo, s));
+        // end of the nonzero rows of each column of C_q: rows (of block q + 1) whose first
+        // nonzero column is at most it
+        std::vector<int> colhi(std::max(B.Np, 1), 0);
+        for (int q = 0; q + 1 < Qn; ++q) {
+            int r = B.bt_off[q + 1];
+            for (int c = B.bt_off[q]; c < B.bt_off[q + 1]; ++c) {
+                while (r < B.bt_off[q + 2] && rowlo[r] <= c - B.bt_off[q]) ++r;
+                colhi[c] = r - B.bt_off[q + 1];
+            }
+        }
+        MSP_TRY(upload(B.d_bt_colhi, colhi, s));
+        MSP_CUDA(cudaStreamSynchronize(s));   // the host tables go out of scope
     }
     // factorise in FP32; if a pivot fails, in FP64
     int fail = 0;
@@ -1059,7 +1139,7 @@ msp_status build_online_factor(Basis& B, const std::vector<int>& row_ptr, const 
 // The grid size and the shared-memory attribute are set up once per device and
 // instance, under a lock (several host threads may make their first call at once).
 template <class T, int BT>
-msp_status launch_sweeps_bt(SweepArgs<T> A, cudaStream_t s) {
+msp_status launch_sweeps_bt(SweepArgs<T> A, int max_n, cudaStream_t s) {
     static std::mutex mu;
     static std::vector<int> grids;   // per device; 0 = not set up yet
     const size_t smem = sizeof(T) * kSweepKC * BT;
@@ -1080,6 +1160,8 @@ msp_status launch_sweeps_bt(SweepArgs<T> A, cudaStream_t s) {
         }
         grid = grids[dev];
     }
+    // no more CTAs than four columns each: a smaller grid has cheaper barriers
+    grid = (int)std::max<long long>(1, std::min<long long>(grid, ((long long)max_n * ((A.B + BT - 1) / BT) + 3) / 4));
     A.spin_limit = wait_limit();
     void* params[] = {&A};
     MSP_CUDA(cudaLaunchCooperativeKernel((const void*)sweep_kernel<T, BT>, dim3(grid), dim3(512), params, smem, s));
@@ -1111,12 +1193,16 @@ msp_status launch_sweeps(Basis& B, BtStore<T>& S, T* y, T* x, int Bsz, cudaStrea
     A.F = S.F.p;
     A.y = y;
     A.x = x;
+    A.row_lo = B.d_bt_rowlo.p;
+    A.col_hi = B.d_bt_colhi.p;
     A.bar = B.d_bt_bar.p;
     A.err = reinterpret_cast<int*>(B.d_bt_bar.p + 2);
-    if (Bsz <= 1) return launch_sweeps_bt<T, 1>(A, s);
-    if (Bsz <= 2) return launch_sweeps_bt<T, 2>(A, s);
-    if (Bsz <= 4) return launch_sweeps_bt<T, 4>(A, s);
-    return launch_sweeps_bt<T, 8>(A, s);
+    int max_n = 1;
+    for (int q = 0; q < B.bt_q; ++q) max_n = std::max(max_n, B.bt_off[q + 1] - B.bt_off[q]);
+    if (Bsz <= 1) return launch_sweeps_bt<T, 1>(A, max_n, s);
+    if (Bsz <= 2) return launch_sweeps_bt<T, 2>(A, max_n, s);
+    if (Bsz <= 4) return launch_sweeps_bt<T, 4>(A, max_n, s);
+    return launch_sweeps_bt<T, 8>(A, max_n, s);
 }
 
 template <class T>
@@ -1130,11 +1216,31 @@ msp_status apply_factor(Basis& B, BtStore<T>& S, const double* s_in, double* z_o
     T* y = S.w1.p;   // right-hand side, then the forward sweep's result
     T* x = S.w2.p;   // backward sweep's result
     const int np = (int)B.patches.size();
-    patch_pre_kernel<T><<<np, 256, 0, s>>>(B.bt_Fi.p, B.d_binv_off.p, B.d_k.p, B.d_c_off.p, s_in, y, Bsz);
-    count_launches(1);
+    int maxk = 1;
+    for (int v : B.k) maxk = std::max(maxk, v);
+    const int bt = Bsz <= 4 ? 1 : 8;
+    auto grid = [&](int m0) {
+        return dim3((maxk + kPpRows - 1) / kPpRows, std::min(65535, np - m0), (Bsz + 4 * bt - 1) / (4 * bt));
+    };
+    for (int m0 = 0; m0 < np; m0 += 65535) {
+        if (bt == 1)
+            patch_pre_kernel<T, 1><<<grid(m0), 256, 0, s>>>(B.bt_Fi.p, B.d_binv_off.p + m0, B.d_k.p + m0,
+                                                            B.d_c_off.p + m0, s_in, y, Bsz);
+        else
+            patch_pre_kernel<T, 8><<<grid(m0), 256, 0, s>>>(B.bt_Fi.p, B.d_binv_off.p + m0, B.d_k.p + m0,
+                                                            B.d_c_off.p + m0, s_in, y, Bsz);
+        count_launches(1);
+    }
     MSP_TRY(launch_sweeps<T>(B, S, y, x, Bsz, s));
-    patch_post_kernel<T><<<np, 256, 0, s>>>(B.bt_Fi.p, B.d_binv_off.p, B.d_k.p, B.d_c_off.p, y, z_out, Bsz);
-    count_launches(1);
+    for (int m0 = 0; m0 < np; m0 += 65535) {
+        if (bt == 1)
+            patch_post_kernel<T, 1><<<grid(m0), 256, 0, s>>>(B.bt_Fi.p, B.d_binv_off.p + m0, B.d_k.p + m0,
+                                                             B.d_c_off.p + m0, y, z_out, Bsz);
+        else
+            patch_post_kernel<T, 8><<<grid(m0), 256, 0, s>>>(B.bt_Fi.p, B.d_binv_off.p + m0, B.d_k.p + m0,
+                                                             B.d_c_off.p + m0, y, z_out, Bsz);
+        count_launches(1);
+    }
     MSP_CUDA(cudaGetLastError());
     return MSP_OK;
 }
