@@ -451,103 +451,194 @@ __device__ __forceinline__ bool grid_barrier(unsigned int* bar, unsigned int nbl
     return s_ok != 0;
 }
 
-// Y[j][b] = alpha sum_k M[k][j] X[k][b] + beta Y[j][b] for b < B, spread over the
-// whole grid: one output column and BT data sets per warp and round, lanes along K.
-// range(j) bounds the nonzeros of column j (the triangle of L^{-1}, the coupled patches
-// of C): the blocks of 32 terms outside it are exact zeros and are skipped.  The CTAs are
-// dealt to the groups of BT data sets, and consecutive columns to different CTAs, so that
-// the long and the short columns of a triangle spread evenly over the SMs (FP64 products
-// are bound by the FP64 pipe of each).  The rows of X needed by a K chunk are staged in
-// shared memory by every CTA that has a column (its block barriers are uniform).
-constexpr int kSweepKC = 1024;
-template <class T, int BT, class Range>
-__device__ __forceinline__ void sweep_product(const T* X, const T* M, int ldm, T* Y, int K, int ncols, int B, T alpha,
-                                              T beta, int lane, T* xs, Range range) {
-    const int nbc = (B + BT - 1) / BT, ng = min(nbc, (int)gridDim.x);
-    const int group = blockIdx.x % ng, cta = blockIdx.x / ng;
-    const int nctas = ((int)gridDim.x - group + ng - 1) / ng;   // CTAs of this group
-    const int warp = threadIdx.x >> 5, wpb = blockDim.x >> 5;
-    for (int bc = group; bc < nbc; bc += ng) {
-        const int b0 = bc * BT, bt = min(BT, B - b0);
-        for (int j0 = 0; j0 + cta < ncols; j0 += wpb * nctas) {
-            const int j = j0 + warp * nctas + cta;
-            const bool live = j < ncols;
-            const T* mj = M + (long long)(live ? j : 0) * ldm;
-            int lo = 0, hi = 0;
-            if (live) {
-                const int2 r = range(j);
-                lo = r.x;
-                hi = min(K, r.y);
-            }
-            T acc[BT];
-#pragma unroll
-            for (int t = 0; t < BT; ++t) acc[t] = T(0);
-            for (int kc = 0; kc < K; kc += kSweepKC) {
-                const int kn = min(kSweepKC, K - kc);
-                __syncthreads();
-                for (int e = threadIdx.x; e < kn * bt; e += blockDim.x) {
-                    const int kk = e / bt, t = e - kk * bt;
-                    xs[t * kSweepKC + kk] = __ldcg(X + (long long)(kc + kk) * B + b0 + t);
-                }
-                __syncthreads();
-                const int k1 = min(kn, hi - kc);
-#pragma unroll 8
-                for (int kk = max(0, lo - kc) / 32 * 32 + lane; kk < k1; kk += 32) {
-                    const T m = mj[kc + kk];
-#pragma unroll
-                    for (int t = 0; t < BT; ++t) acc[t] = fma(m, xs[t * kSweepKC + kk], acc[t]);
-                }
-            }
-#pragma unroll
-            for (int t = 0; t < BT; ++t) {
-                const T v = warp_sum(acc[t]);
-                if (live && lane == 0 && t < bt) {
-                    T* yp = Y + (long long)j * B + b0 + t;
-                    *yp = (beta == T(0)) ? alpha * v : alpha * v + beta * __ldcg(yp);
-                }
-            }
-        }
-    }
-}
+// One product of a sweep: Y[j][b] = alpha sum_k M[k][j] X[k][b] + beta Y[j][b], b < B,
+// columns j of M (K long) with nonzeros in rows lo(j) .. hi(j).  kind 0: rows from
+// row_lo[j] on (C^T); 1: rows up to j (L^{-T}); 2: rows up to col_hi[j] (C); 3: rows from j
+// on (L^{-1}).
+template <class T>
+struct SweepStep {
+    const T* X;
+    const T* M;
+    T* Y;
+    const int* bound;
+    int K, ncols, kind;
+    T alpha, beta;
+};
+
+// What a warp reads for its first column before the barrier that completes X: none of
+// it depends on the step before.
+template <class T, int BT>
+struct SweepAhead {
+    static constexpr int kN = BT == 1 ? 16 : 4;
+    T m[kN];
+    T y;                     // Y of the warp's column for data set b0 + lane
+    int lo, hi;
+};
+
+// Products are spread over the whole grid: one output column and BT data sets per warp
+// and round, lanes along K.  The CTAs are dealt to the groups of BT data sets, and
+// consecutive columns to different CTAs, so that the long and the short columns of a
+// triangle spread evenly over the SMs (FP64 products are bound by the FP64 pipe of each).
+// Outside a column's nonzeros (the triangle of L^{-1}, the coupled patches of C) lie
+// exact zeros, skipped in blocks of 32.  The rows of X are staged in shared memory by
+// every CTA that has a column (its block barriers are uniform), kSweepElems / BT at a time.
+constexpr int kSweepElems = 8192;
+template <class T, int BT>
+__host__ __device__ constexpr int sweep_kc() { return (sizeof(T) == 8 ? kSweepElems / 2 : kSweepElems) / BT; }
 
 template <class T, int BT>
-__global__ void __launch_bounds__(512) sweep_kernel(SweepArgs<T> A) {
+struct SweepLayout {
+    int B, nbc, ng, group, cta, nctas, warp, wpb, lane;
+    __device__ explicit SweepLayout(int B_) : B(B_) {
+        nbc = (B + BT - 1) / BT;
+        ng = min(nbc, (int)gridDim.x);
+        group = blockIdx.x % ng;
+        cta = blockIdx.x / ng;
+        nctas = ((int)gridDim.x - group + ng - 1) / ng;   // CTAs of this group
+        warp = threadIdx.x >> 5;
+        wpb = blockDim.x >> 5;
+        lane = threadIdx.x & 31;
+    }
+    __device__ void range(const SweepStep<T>& S, int j, int& lo, int& hi) const {
+        lo = S.kind == 0 ? S.bound[j] : S.kind == 3 ? j : 0;
+        hi = S.kind == 1 ? j + 1 : S.kind == 2 ? min(S.K, S.bound[j]) : S.K;
+    }
+    __device__ void ahead(const SweepStep<T>& S, SweepAhead<T, BT>& P) const {
+        const int j = warp * nctas + cta, b0 = group * BT;
+        P.lo = P.hi = 0;
+        if (j >= S.ncols) return;
+        range(S, j, P.lo, P.hi);
+        const T* mj = S.M + (long long)j * S.K;
+        const int k0 = P.lo / 32 * 32;
+#pragma unroll
+        for (int i = 0; i < SweepAhead<T, BT>::kN; ++i) {
+            const int kk = k0 + 32 * i + lane;
+            P.m[i] = kk < P.hi ? mj[kk] : T(0);
+        }
+        P.y = (S.beta != T(0) && lane < BT && b0 + lane < B) ? __ldcg(S.Y + (long long)j * B + b0 + lane) : T(0);
+        // the rest of the column into the L2: one 128-byte line per lane
+        constexpr int kLine = 128 / (int)sizeof(T);
+        for (int kk = k0 + 32 * SweepAhead<T, BT>::kN + lane * kLine; kk < P.hi; kk += 32 * kLine)
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(mj + kk));
+    }
+    __device__ void product(const SweepStep<T>& S, const SweepAhead<T, BT>& P, T* xs) const {
+        constexpr int KC = sweep_kc<T, BT>(), kN = SweepAhead<T, BT>::kN;
+        for (int bc = group; bc < nbc; bc += ng) {
+            const int b0 = bc * BT, bt = min(BT, B - b0);
+            for (int j0 = 0; j0 + cta < S.ncols; j0 += wpb * nctas) {
+                const int j = j0 + warp * nctas + cta;
+                const bool live = j < S.ncols, first = j0 == 0 && bc == group;
+                const T* mj = S.M + (long long)(live ? j : 0) * S.K;
+                int lo = 0, hi = 0;
+                if (first) {
+                    lo = P.lo;
+                    hi = P.hi;
+                } else if (live) {
+                    range(S, j, lo, hi);
+                }
+                const int k0 = lo / 32 * 32;
+                T acc[BT];
+#pragma unroll
+                for (int t = 0; t < BT; ++t) acc[t] = T(0);
+                for (int kc = 0; kc < S.K; kc += KC) {
+                    const int kn = min(KC, S.K - kc);
+                    __syncthreads();
+                    for (int e = threadIdx.x; e < kn * bt; e += blockDim.x) {
+                        const int kk = e / bt, t = e - kk * bt;
+                        xs[t * KC + kk] = __ldcg(S.X + (long long)(kc + kk) * B + b0 + t);
+                    }
+                    __syncthreads();
+                    const int k1 = min(kn, hi - kc);
+                    int kk = max(0, k0 - kc) + lane;
+                    if (first) {
+                        // the terms read ahead (the block of 32 k0 + 32 i), those of this chunk
+#pragma unroll
+                        for (int i = 0; i < kN; ++i) {
+                            const int ka = k0 + 32 * i - kc;
+                            if (ka >= 0 && ka < k1) {
+                                if (ka + lane < k1) {
+#pragma unroll
+                                    for (int t = 0; t < BT; ++t) acc[t] = fma(P.m[i], xs[t * KC + ka + lane], acc[t]);
+                                }
+                                kk = ka + 32 + lane;
+                            }
+                        }
+                    }
+#pragma unroll 8
+                    for (; kk < k1; kk += 32) {
+                        const T m = mj[kc + kk];
+#pragma unroll
+                        for (int t = 0; t < BT; ++t) acc[t] = fma(m, xs[t * KC + kk], acc[t]);
+                    }
+                }
+#pragma unroll
+                for (int t = 0; t < BT; ++t) {
+                    const T v = warp_sum(acc[t]);
+                    const T y = first ? __shfl_sync(0xffffffffu, P.y, t) : T(0);
+                    if (live && lane == 0 && t < bt) {
+                        T* yp = S.Y + (long long)j * B + b0 + t;
+                        *yp = (S.beta == T(0)) ? S.alpha * v : S.alpha * v + S.beta * (first ? y : __ldcg(yp));
+                    }
+                }
+            }
+        }
+    }
+};
+
+template <class T, int BT>
+__global__ void __launch_bounds__(512, BT >= 4 ? 2 : 1) sweep_kernel(SweepArgs<T> A) {
     extern __shared__ __align__(16) unsigned char sweep_smem[];
-    T* xs = reinterpret_cast<T*>(sweep_smem);   // kSweepKC x BT
-    const int lane = threadIdx.x & 31;
+    T* xs = reinterpret_cast<T*>(sweep_smem);   // BT x sweep_kc
     unsigned int gen = atomicAdd(&A.bar[1], 0u);
     const int B = A.B;
-    // forward: y_q -= x_{q-1} C_{q-1}^T;  x_q = y_q Li_q^T
-    for (int q = 0; q < A.Qn; ++q) {
+    const SweepLayout<T, BT> Lay(B);
+    // the products in order, as steps 2 q and 2 q + 1 of either sweep:
+    // forward  y_q -= x_{q-1} C_{q-1}^T, x_q = y_q Li_q^T;
+    // backward x_q -= z_{q+1} C_q, z_q = x_q Li_q (z into y), q descending
+    auto step = [&](int i, SweepStep<T>& S) -> bool {   // false: no such product
+        const bool fwd = i < 2 * A.Qn;
+        const int q = fwd ? i / 2 : A.Qn - 1 - (i - 2 * A.Qn) / 2;
         const int o = A.off[q], nq = A.off[q + 1] - o;
-        if (nq == 0) continue;
-        if (q > 0) {
-            const int o0 = A.off[q - 1], n0 = o - o0;
-            if (n0 > 0) {
-                sweep_product<T, BT>(A.x + (long long)o0 * B, A.FT + A.e_off[q - 1], n0, A.y + (long long)o * B, n0, nq,
-                                     B, T(-1), T(1), lane, xs, [&](int j) { return make_int2(A.row_lo[o + j], n0); });
-                if (!grid_barrier(A.bar, gridDim.x, gen, A.err, A.spin_limit)) return;
-            }
+        if (nq == 0) return false;
+        S.ncols = nq;
+        if ((i & 1) == 0) {
+            const int qn = fwd ? q - 1 : q + 1;
+            if (qn < 0 || qn >= A.Qn) return false;
+            const int on = A.off[qn], n = A.off[qn + 1] - on;
+            if (n == 0) return false;
+            S.K = n;
+            S.alpha = T(-1);
+            S.beta = T(1);
+            S.X = (fwd ? A.x : A.y) + (long long)on * B;
+            S.Y = (fwd ? A.y : A.x) + (long long)o * B;
+            S.M = fwd ? A.FT + A.e_off[qn] : A.F + A.e_off[q];
+            S.kind = fwd ? 0 : 2;
+            S.bound = (fwd ? A.row_lo : A.col_hi) + o;
+        } else {
+            S.K = nq;
+            S.alpha = T(1);
+            S.beta = T(0);
+            S.X = (fwd ? A.y : A.x) + (long long)o * B;
+            S.Y = (fwd ? A.x : A.y) + (long long)o * B;
+            S.M = (fwd ? A.LiT : A.Li) + A.d_off[q];
+            S.kind = fwd ? 1 : 3;
+            S.bound = nullptr;
         }
-        sweep_product<T, BT>(A.y + (long long)o * B, A.LiT + A.d_off[q], nq, A.x + (long long)o * B, nq, nq, B, T(1),
-                             T(0), lane, xs, [&](int j) { return make_int2(0, j + 1); });
+        return true;
+    };
+    const int steps = 4 * A.Qn;
+    SweepStep<T> S;
+    SweepAhead<T, BT> P;
+    int i = 0;
+    while (i < steps && !step(i, S)) ++i;
+    if (i < steps) Lay.ahead(S, P);
+    while (i < steps) {
+        Lay.product(S, P, xs);
+        int n = i + 1;
+        while (n < steps && !step(n, S)) ++n;
+        if (n < steps) Lay.ahead(S, P);
         if (!grid_barrier(A.bar, gridDim.x, gen, A.err, A.spin_limit)) return;
-    }
-    // backward: x_q -= z_{q+1} C_q;  z_q = x_q Li_q   (z into y)
-    for (int q = A.Qn - 1; q >= 0; --q) {
-        const int o = A.off[q], nq = A.off[q + 1] - o;
-        if (nq == 0) continue;
-        if (q + 1 < A.Qn) {
-            const int o1 = A.off[q + 1], n1 = A.off[q + 2] - o1;
-            if (n1 > 0) {
-                sweep_product<T, BT>(A.y + (long long)o1 * B, A.F + A.e_off[q], n1, A.x + (long long)o * B, n1, nq, B,
-                                     T(-1), T(1), lane, xs, [&](int j) { return make_int2(0, A.col_hi[o + j]); });
-                if (!grid_barrier(A.bar, gridDim.x, gen, A.err, A.spin_limit)) return;
-            }
-        }
-        sweep_product<T, BT>(A.x + (long long)o * B, A.Li + A.d_off[q], nq, A.y + (long long)o * B, nq, nq, B, T(1), T(0),
-                             lane, xs, [&](int j) { return make_int2(j, nq); });
-        if (!grid_barrier(A.bar, gridDim.x, gen, A.err, A.spin_limit)) return;
+        i = n;
     }
 }
 
@@ -1142,7 +1233,7 @@ template <class T, int BT>
 msp_status launch_sweeps_bt(SweepArgs<T> A, int max_n, cudaStream_t s) {
     static std::mutex mu;
     static std::vector<int> grids;   // per device; 0 = not set up yet
-    const size_t smem = sizeof(T) * kSweepKC * BT;
+    const size_t smem = sizeof(T) * sweep_kc<T, BT>() * BT;
     int dev = 0, grid = 0;
     MSP_CUDA(cudaGetDevice(&dev));
     {
