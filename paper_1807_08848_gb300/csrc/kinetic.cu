@@ -15,6 +15,7 @@
 // patches: factorised once (FP64 block Cholesky), solved per data set with two
 // corrected-semi-normal-equation refinement steps.
 #include "kinetic_internal.h"
+#include "kinetic_online.h"
 #include "device_util.cuh"
 
 #include <algorithm>
@@ -36,10 +37,12 @@ struct KBasis {
     DevBuf<int> d_k, d_c_off;
     DevBuf<long long> d_q_off;
     DevBuf<double> d_v;
-    // block-tridiagonal factor of H = P^T P: L_m (k_m x k_m, lower) and C_m (k_{m+1} x k_m)
+    // block-tridiagonal factor of H = P^T P as the online solve applies it: L_m^{-T}
+    // (k_m x k_m), L_{m+1}^{-1} C_m and L_m^{-T} C_m^T (k_{m+1} x k_m blocks)
     std::vector<long long> l_off, c_blk_off;
-    DevBuf<double> Lf, Cf;
+    DevBuf<double> Fi, Tf, Tb;
     DevBuf<long long> d_l_off, d_c_blk_off;
+    int k_max = 0;
     int max_sweeps = 0, max_tries = 0;
 };
 
@@ -381,260 +384,6 @@ __global__ void kinetic_si_mixed_kernel(KSolveArgs A) {
     }
 }
 
-// ---- online: block-tridiagonal normal equations along the chain of patches
-// rows of Q_m at the first (left) and last (right) node of K_m
-__device__ __forceinline__ const double* qrow(const double* Q, const KPatchDev& P, int node, int l, int nv) {
-    return Q + (long long)node * nv + l;   // column j at + j * n_k
-}
-
-// one CTA, sequential over patches: assemble H blocks and factorise
-__global__ void kinetic_factor_kernel(int M, int nv, const double* v, const KPatchDev* patches, const int* k,
-                                      const long long* q_off, const double* Q, const long long* l_off,
-                                      const long long* c_off, double* Lf, double* Cf, double* work, int* fail) {
-    // work: D (kmax x kmax) scratch
-    __shared__ int s_ok;
-    if (threadIdx.x == 0) { s_ok = 1; *fail = 0; }
-    __syncthreads();
-    for (int m = 0; m < M; ++m) {
-        const int km = k[m];
-        const KPatchDev P = patches[m];
-        const double* Qm = Q + q_off[m];
-        const int last = P.x1 - P.x0;
-        double* D = Lf + l_off[m];
-        // D = H_mm: right-interface rows (m < M-1), left-interface rows (m > 0), incoming rows
-        for (int e = threadIdx.x; e < km * km; e += blockDim.x) {
-            const int i = e % km, j = e / km;
-            double a = 0.0;
-            for (int l = 0; l < nv; ++l) {
-                const bool right = (m < M - 1) || (v[l] < 0.0);
-                const bool left = (m > 0) || (v[l] > 0.0);
-                if (right) a += Qm[(long long)last * nv + l + (long long)i * P.n_k] * Qm[(long long)last * nv + l + (long long)j * P.n_k];
-                if (left) a += Qm[l + (long long)i * P.n_k] * Qm[l + (long long)j * P.n_k];
-            }
-            D[e] = a;
-        }
-        __syncthreads();
-        if (m > 0) {   // D -= C_{m-1} C_{m-1}^T
-            const int kp = k[m - 1];
-            const double* Cp = Cf + c_off[m - 1];
-            for (int e = threadIdx.x; e < km * km; e += blockDim.x) {
-                const int i = e % km, j = e / km;
-                double a = 0.0;
-                for (int q = 0; q < kp; ++q) a += Cp[i + (long long)q * km] * Cp[j + (long long)q * km];
-                D[e] -= a;
-            }
-            __syncthreads();
-        }
-        // Cholesky D = L L^T in place (lower)
-        for (int c = 0; c < km; ++c) {
-            if (threadIdx.x == 0) {
-                const double d = D[c + (long long)c * km];
-                if (!(d > 0.0)) { s_ok = 0; D[c + (long long)c * km] = 1.0; }
-                else D[c + (long long)c * km] = sqrt(d);
-            }
-            __syncthreads();
-            const double piv = D[c + (long long)c * km];
-            for (int i = c + 1 + threadIdx.x; i < km; i += blockDim.x) D[i + (long long)c * km] /= piv;
-            __syncthreads();
-            const int R = km - c - 1;
-            for (int e = threadIdx.x; e < R * R; e += blockDim.x) {
-                const int i = c + 1 + e % R, j = c + 1 + e / R;
-                if (i >= j) D[i + (long long)j * km] -= D[i + (long long)c * km] * D[j + (long long)c * km];
-            }
-            __syncthreads();
-        }
-        for (int e = threadIdx.x; e < km * km; e += blockDim.x) {
-            const int i = e % km, j = e / km;
-            if (i < j) D[e] = 0.0;
-        }
-        __syncthreads();
-        if (m + 1 < M) {
-            // E = H_{m+1,m} = -Vl_{m+1}^T Vr_m ; C_m = E L_m^{-T}: row i of C solves L_m c = E_i^T
-            const int kn = k[m + 1];
-            const KPatchDev Pn = patches[m + 1];
-            const double* Qn = Q + q_off[m + 1];
-            double* Cm = Cf + c_off[m];
-            for (int e = threadIdx.x; e < kn * km; e += blockDim.x) {
-                const int i = e % kn, j = e / kn;
-                double a = 0.0;
-                for (int l = 0; l < nv; ++l)
-                    a -= Qn[l + (long long)i * Pn.n_k] * Qm[(long long)last * nv + l + (long long)j * P.n_k];
-                work[e] = a;
-            }
-            __syncthreads();
-            for (int i = threadIdx.x; i < kn; i += blockDim.x) {
-                for (int j = 0; j < km; ++j) {   // forward substitution on row i
-                    double a = work[i + (long long)j * kn];
-                    for (int q = 0; q < j; ++q) a -= D[j + (long long)q * km] * Cm[i + (long long)q * kn];
-                    Cm[i + (long long)j * kn] = a / D[j + (long long)j * km];
-                }
-            }
-            __syncthreads();
-        }
-    }
-    if (threadIdx.x == 0 && !s_ok) *fail = 1;
-}
-
-// Pieces of one data set's solve, one CTA per data set.
-struct KOnArgs {
-    int M, nv, N;
-    const double* v;
-    const KPatchDev* patches;
-    const int* k;
-    const int* c_off;
-    const long long* q_off;
-    const double* Q;
-    const long long* l_off;
-    const long long* cb_off;
-    const double* Lf;
-    const double* Cf;
-};
-
-// value of u_m at node `node`, velocity l for coefficients c_m
-__device__ double kval(const KOnArgs& A, int m, int node, int l, const double* c) {
-    const KPatchDev P = A.patches[m];
-    const double* Qm = A.Q + A.q_off[m];
-    double a = 0.0;
-    for (int j = 0; j < A.k[m]; ++j) a += Qm[(long long)node * A.nv + l + (long long)j * P.n_k] * c[A.c_off[m] + j];
-    return a;
-}
-
-// g = P^T r for the residual rows r (interfaces then incoming rows) -- rows evaluated
-// from the residual vector stored per row.  Row layout: interface m (m < M-1): nv rows;
-// then nv/2 left incoming rows (positive v, ascending), then nv/2 right incoming rows.
-__device__ void kinetic_normal_rhs(const KOnArgs& A, const double* r, double* g) {
-    const int nv = A.nv, M = A.M;
-    for (int m = 0; m < M; ++m) {
-        const KPatchDev P = A.patches[m];
-        const double* Qm = A.Q + A.q_off[m];
-        const int last = P.x1 - P.x0;
-        for (int j = threadIdx.x; j < A.k[m]; j += blockDim.x) {
-            double a = 0.0;
-            for (int l = 0; l < nv; ++l) {
-                if (m < M - 1) a += Qm[(long long)last * nv + l + (long long)j * P.n_k] * r[m * nv + l];
-                if (m > 0) a -= Qm[l + (long long)j * P.n_k] * r[(m - 1) * nv + l];
-            }
-            if (m == 0)
-                for (int t = 0; t < nv / 2; ++t) a += Qm[(nv / 2 + t) + (long long)j * P.n_k] * r[(M - 1) * nv + t];
-            if (m == M - 1)
-                for (int t = 0; t < nv / 2; ++t)
-                    a += Qm[(long long)last * nv + t + (long long)j * P.n_k] * r[(M - 1) * nv + nv / 2 + t];
-            g[A.c_off[m] + j] = a;
-        }
-    }
-    __syncthreads();
-}
-
-// solve H x = g in place with the block factor
-__device__ void kinetic_factor_solve(const KOnArgs& A, double* x) {
-    const int M = A.M;
-    for (int m = 0; m < M; ++m) {   // forward: L_m y_m = g_m - C_{m-1} y_{m-1}
-        const int km = A.k[m];
-        double* xm = x + A.c_off[m];
-        if (m > 0) {
-            const int kp = A.k[m - 1];
-            const double* C = A.Cf + A.cb_off[m - 1];
-            const double* xp = x + A.c_off[m - 1];
-            for (int i = threadIdx.x; i < km; i += blockDim.x) {
-                double a = 0.0;
-                for (int q = 0; q < kp; ++q) a += C[i + (long long)q * km] * xp[q];
-                xm[i] -= a;
-            }
-            __syncthreads();
-        }
-        if (threadIdx.x == 0) {
-            const double* L = A.Lf + A.l_off[m];
-            for (int i = 0; i < km; ++i) {
-                double a = xm[i];
-                for (int q = 0; q < i; ++q) a -= L[i + (long long)q * km] * xm[q];
-                xm[i] = a / L[i + (long long)i * km];
-            }
-        }
-        __syncthreads();
-    }
-    for (int m = M - 1; m >= 0; --m) {   // backward: L_m^T x_m = y_m - C_m^T x_{m+1}
-        const int km = A.k[m];
-        double* xm = x + A.c_off[m];
-        if (m + 1 < M) {
-            const int kn = A.k[m + 1];
-            const double* C = A.Cf + A.cb_off[m];
-            const double* xn = x + A.c_off[m + 1];
-            for (int j = threadIdx.x; j < km; j += blockDim.x) {
-                double a = 0.0;
-                for (int q = 0; q < kn; ++q) a += C[q + (long long)j * kn] * xn[q];
-                xm[j] -= a;
-            }
-            __syncthreads();
-        }
-        if (threadIdx.x == 0) {
-            const double* L = A.Lf + A.l_off[m];
-            for (int i = km - 1; i >= 0; --i) {
-                double a = xm[i];
-                for (int q = i + 1; q < km; ++q) a -= L[q + (long long)i * km] * xm[q];
-                xm[i] = a / L[i + (long long)i * km];
-            }
-        }
-        __syncthreads();
-    }
-}
-
-// residual rows r = d - P c
-__device__ void kinetic_residual(const KOnArgs& A, const double* c, const double* inl, const double* inr, double* r) {
-    const int nv = A.nv, M = A.M;
-    for (int t = threadIdx.x; t < (M - 1) * nv; t += blockDim.x) {
-        const int m = t / nv, l = t - m * nv;
-        const int last = A.patches[m].x1 - A.patches[m].x0;
-        r[t] = -(kval(A, m, last, l, c) - kval(A, m + 1, 0, l, c));
-    }
-    for (int t = threadIdx.x; t < nv / 2; t += blockDim.x) {
-        r[(M - 1) * nv + t] = inl[nv / 2 + t] - kval(A, 0, 0, nv / 2 + t, c);
-        const int last = A.patches[M - 1].x1 - A.patches[M - 1].x0;
-        r[(M - 1) * nv + nv / 2 + t] = inr[t] - kval(A, M - 1, last, t, c);
-    }
-    __syncthreads();
-}
-
-// c = argmin |P c - d| by the factorised normal equations and two refinement
-// steps (corrected semi-normal equations); then the reconstruction.
-__global__ void kinetic_online_kernel(KOnArgs A, const double* inflow, double* work, double* f_out, double* c_out,
-                                      int Np) {
-    const int b = blockIdx.x;
-    const int nv = A.nv, M = A.M, N = A.N;
-    const double* inl = inflow + (long long)b * 2 * nv;
-    const double* inr = inl + nv;
-    const int nrows = (M - 1) * nv + nv;
-    double* c = work + (long long)b * (2 * Np + nrows);
-    double* g = c + Np;
-    double* r = g + Np;
-    for (int j = threadIdx.x; j < Np; j += blockDim.x) c[j] = 0.0;
-    __syncthreads();
-    for (int pass = 0; pass < 3; ++pass) {
-        kinetic_residual(A, c, inl, inr, r);
-        kinetic_normal_rhs(A, r, g);
-        kinetic_factor_solve(A, g);
-        for (int j = threadIdx.x; j < Np; j += blockDim.x) c[j] += g[j];
-        __syncthreads();
-    }
-    if (c_out)
-        for (int j = threadIdx.x; j < Np; j += blockDim.x) c_out[(long long)b * Np + j] = c[j];
-    // reconstruction: patch interiors, interface averages, incoming data at the ends
-    double* fo = f_out + (long long)b * (N + 1) * nv;
-    for (long long t = threadIdx.x; t < (long long)(N + 1) * nv; t += blockDim.x) {
-        const int i = (int)(t / nv), l = (int)(t % nv);
-        const int W = A.patches[0].x1 - A.patches[0].x0;
-        int m = min(i / W, M - 1);
-        double val;
-        if (i == A.patches[m].x0 && m > 0) {
-            val = 0.5 * (kval(A, m - 1, A.patches[m - 1].x1 - A.patches[m - 1].x0, l, c) + kval(A, m, 0, l, c));
-        } else {
-            val = kval(A, m, i - A.patches[m].x0, l, c);
-        }
-        if (i == 0 && A.v[l] > 0.0) val = inl[l];
-        if (i == N && A.v[l] < 0.0) val = inr[l];
-        fo[t] = val;
-    }
-}
-
 // Per-sample iteration counts and flags to the caller's stats (optional; reading
 // them synchronises the stream).
 msp_status kinetic_stats(const KMedium& K, bool mixed, cudaStream_t s, msp_solve_stats* stats, const char* what) {
@@ -813,6 +562,14 @@ extern "C" msp_status msp_kinetic_get_snapshots(msp_kmedium k, int patch, double
     return MSP_OK;
 }
 
+static KOnArgs online_args(const KBasis& B) {
+    KOnArgs A{};
+    A.M = B.M; A.nv = B.n_v; A.N = B.N; A.k_max = B.k_max; A.v = B.d_v.p; A.patches = B.d_patches.p; A.k = B.d_k.p;
+    A.c_off = B.d_c_off.p; A.q_off = B.d_q_off.p; A.Q = B.Q.p; A.l_off = B.d_l_off.p; A.cb_off = B.d_c_blk_off.p;
+    A.Fi = B.Fi.p; A.Tf = B.Tf.p; A.Tb = B.Tb.p;
+    return A;
+}
+
 extern "C" msp_status msp_kinetic_extract(msp_kmedium km, double tau, void* stream, msp_kbasis* out) {
     clear_error();
     MSP_CHECK_ARG(km && out, "msp_kinetic_extract: NULL argument");
@@ -840,35 +597,29 @@ extern "C" msp_status msp_kinetic_extract(msp_kmedium km, double tau, void* stre
     B.l_off.assign(K.M, 0);
     B.c_blk_off.assign(std::max(K.M - 1, 1), 0);
     long long lo = 0, co = 0;
-    int kmax = 1;
     for (int m = 0; m < K.M; ++m) {
         B.l_off[m] = lo;
         lo += (long long)B.k[m] * B.k[m];
-        kmax = std::max(kmax, B.k[m]);
         if (m + 1 < K.M) {
             B.c_blk_off[m] = co;
             co += (long long)B.k[m + 1] * B.k[m];
         }
     }
-    DevBuf<double> work;
-    DevBuf<int> fail;
+    B.k_max = *std::max_element(B.k.begin(), B.k.end());
+    DevBuf<double> Lf, Cf;
     if ((st = upload(B.d_patches, B.patches, s)) || (st = upload(B.d_k, B.k, s)) || (st = upload(B.d_c_off, B.c_off, s)) ||
         (st = upload(B.d_q_off, B.q_off, s)) || (st = upload(B.d_v, B.v, s)) || (st = upload(B.d_l_off, B.l_off, s)) ||
-        (st = upload(B.d_c_blk_off, B.c_blk_off, s)) || (st = B.Lf.alloc(std::max<long long>(lo, 1), s)) ||
-        (st = B.Cf.alloc(std::max<long long>(co, 1), s)) || (st = work.alloc((size_t)kmax * kmax, s)) ||
-        (st = fail.alloc(1, s))) {
+        (st = upload(B.d_c_blk_off, B.c_blk_off, s)) || (st = Lf.alloc(std::max<long long>(lo, 1), s)) ||
+        (st = Cf.alloc(std::max<long long>(co, 1), s)) || (st = B.Fi.alloc(std::max<long long>(lo, 1), s)) ||
+        (st = B.Tf.alloc(std::max<long long>(co, 1), s)) || (st = B.Tb.alloc(std::max<long long>(co, 1), s))) {
         delete h;
         return st;
     }
-    kinetic_factor_kernel<<<1, 256, 0, s>>>(K.M, K.n_v, B.d_v.p, B.d_patches.p, B.d_k.p, B.d_q_off.p, B.Q.p, B.d_l_off.p,
-                                            B.d_c_blk_off.p, B.Lf.p, B.Cf.p, work.p, fail.p);
-    count_launches(1);
     int hf = 0;
-    if (cudaMemcpyAsync(&hf, fail.p, sizeof(int), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-        cudaStreamSynchronize(s) != cudaSuccess) {
+    st = kinetic_factor(online_args(B), B.k, B.l_off, B.c_blk_off, Lf.p, Cf.p, B.Fi.p, B.Tf.p, B.Tb.p, &hf, s);
+    if (st != MSP_OK) {
         delete h;
-        set_error("msp_kinetic_extract: CUDA failure in the online factorisation");
-        return MSP_ERR_CUDA;
+        return st;
     }
     if (hf) {
         delete h;
@@ -906,15 +657,5 @@ extern "C" msp_status msp_kinetic_online_solve(msp_kbasis b, const double* inflo
     if (batch == 0) return MSP_OK;
     KBasis& B = b->B;
     cudaStream_t s = (cudaStream_t)stream;
-    const int nrows = B.M * B.n_v;
-    DevBuf<double> work;
-    MSP_TRY(work.alloc((size_t)batch * (2 * std::max(B.Np, 1) + nrows), s));
-    KOnArgs A{};
-    A.M = B.M; A.nv = B.n_v; A.N = B.N; A.v = B.d_v.p; A.patches = B.d_patches.p; A.k = B.d_k.p; A.c_off = B.d_c_off.p;
-    A.q_off = B.d_q_off.p; A.Q = B.Q.p; A.l_off = B.d_l_off.p; A.cb_off = B.d_c_blk_off.p; A.Lf = B.Lf.p; A.Cf = B.Cf.p;
-    kinetic_online_kernel<<<batch, 256, 0, s>>>(A, inflow_dev, work.p, f_dev, c_dev, B.Np);
-    count_launches(1);
-    MSP_CUDA(cudaGetLastError());
-    MSP_CUDA(cudaStreamSynchronize(s));   // the work buffer is released on return
-    return MSP_OK;
+    return kinetic_online(online_args(B), B.Np, inflow_dev, batch, f_dev, c_dev, s);
 }

@@ -173,7 +173,7 @@ __global__ void __launch_bounds__(32 * kInvWarps) patch_inverse_kernel(const Pat
     extern __shared__ __align__(16) double ism[];
     const PatchBlock P = blocks[blockIdx.y];
     const int c = P.c, j0 = blockIdx.x * kInvWarps;
-    if (j0 >= c || status[P.idx] < 0) return;
+    if (j0 >= c || (status && status[P.idx] < 0)) return;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int j = j0 + warp;
     const double* l = L + P.off;
@@ -209,7 +209,7 @@ __global__ void __launch_bounds__(32 * kInvWarps) patch_inverse_kernel(const Pat
                 if (lane == 0) out[r * kInvWarps + warp] = v;
             }
         }
-        if (blockIdx.x == 0)
+        if (blockIdx.x == 0 && F)
             for (int r = warp; r < rows; r += kInvWarps)
                 for (int q = lane; q < c; q += 32) f[q + (size_t)(i0 + r) * c] = q <= i0 + r ? Ls[(size_t)r * c + q] : 0.0;
         __syncthreads();
@@ -791,19 +791,10 @@ PatchClasses classify_patches(const std::vector<int>& cols, const std::vector<lo
     return C;
 }
 
-msp_status patch_cholesky(const PatchClasses& C, const PatchBlock* blocks, const double* G, double* L, double* F,
-                          double* Fi, const double* shift_scale, bool shifted, int* status, cudaStream_t s) {
+static msp_status launch_inverse(const PatchClasses& C, const PatchBlock* blocks, const double* L, double* F, double* Fi,
+                                 const int* status, cudaStream_t s) {
     size_t room = 0;
     MSP_TRY(smem_room(&room));
-    const int count[2] = {C.n_big, (int)C.blocks.size() - C.n_big};
-    for (int cls = 0; cls < 2; ++cls) {
-        if (!count[cls] || C.max_c[cls] <= 0) continue;
-        const int nc = cls == 0 ? kPatchCluster : 1, c = C.max_c[cls];
-        const size_t head = sizeof(double) * (size_t)kPan * c, own = sizeof(double) * panel_elems(c, 0, nc);
-        const int in_smem = head + own <= room ? 1 : 0;
-        MSP_TRY(launch_cluster(patch_chol_kernel, count[cls], nc, kCholThreads, in_smem ? head + own : head, s,
-                               blocks + (cls == 0 ? 0 : C.n_big), G, L, shift_scale, shifted ? 1 : 0, status, in_smem));
-    }
     const int c = std::max(C.max_c[0], C.max_c[1]);
     if (c > 0) {
         int tr = 16;
@@ -819,6 +810,27 @@ msp_status patch_cholesky(const PatchClasses& C, const PatchBlock* blocks, const
         MSP_CUDA(cudaGetLastError());
     }
     return MSP_OK;
+}
+
+msp_status patch_triangular_inverse(const PatchClasses& C, const PatchBlock* blocks, const double* L, double* Fi,
+                                    cudaStream_t s) {
+    return launch_inverse(C, blocks, L, nullptr, Fi, nullptr, s);
+}
+
+msp_status patch_cholesky(const PatchClasses& C, const PatchBlock* blocks, const double* G, double* L, double* F,
+                          double* Fi, const double* shift_scale, bool shifted, int* status, cudaStream_t s) {
+    size_t room = 0;
+    MSP_TRY(smem_room(&room));
+    const int count[2] = {C.n_big, (int)C.blocks.size() - C.n_big};
+    for (int cls = 0; cls < 2; ++cls) {
+        if (!count[cls] || C.max_c[cls] <= 0) continue;
+        const int nc = cls == 0 ? kPatchCluster : 1, c = C.max_c[cls];
+        const size_t head = sizeof(double) * (size_t)kPan * c, own = sizeof(double) * panel_elems(c, 0, nc);
+        const int in_smem = head + own <= room ? 1 : 0;
+        MSP_TRY(launch_cluster(patch_chol_kernel, count[cls], nc, kCholThreads, in_smem ? head + own : head, s,
+                               blocks + (cls == 0 ? 0 : C.n_big), G, L, shift_scale, shifted ? 1 : 0, status, in_smem));
+    }
+    return launch_inverse(C, blocks, L, F, Fi, status, s);
 }
 
 msp_status patch_qrcp(const PatchClasses& C, const PatchBlock* blocks, const double* T, double* W, double* Q, double* R,

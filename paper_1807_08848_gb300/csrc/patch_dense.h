@@ -30,6 +30,10 @@ PatchClasses classify_patches(const std::vector<int>& cols, const std::vector<lo
 msp_status patch_cholesky(const PatchClasses& C, const PatchBlock* blocks, const double* G, double* L, double* F,
                           double* Fi, const double* shift_scale, bool shifted, int* status, cudaStream_t s);
 
+// Fi = L^{-T} of every lower triangular block
+msp_status patch_triangular_inverse(const PatchClasses& C, const PatchBlock* blocks, const double* L, double* Fi,
+                                    cudaStream_t s);
+
 // Householder QR with column pivoting T P = Q R of every block: W = R^T and Q, the
 // preconditioner of the Jacobi sweeps in the manner of Drmac and Veselic (2008): the
 // sweeps run on the columns of R^T, whose rows decay with the pivots, with V started at Q,
