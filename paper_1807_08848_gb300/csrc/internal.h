@@ -166,7 +166,10 @@ struct Medium {
         DevBuf<long long> w_off, s_off, x_off, r_off, k_off;   // per patch
         DevBuf<int> col_base;                                   // per patch: first global column
         DevBuf<int2> cols;                                      // global column -> (patch, column)
-        DevBuf<int4> chunks;                                    // (patch, first column, columns, -)
+        DevBuf<int4> chunks;                                    // (patch, first column, columns, chunk of the patch)
+        DevBuf<int4> ctas;                                      // the sweeps' CTAs: one chunk or two (wide) each
+        bool wide = false;
+        int n_ctas = 0;
         DevBuf<int> stat_idx;                                   // global column -> statistics slot
         DevBuf<float> W, D, R, K;
         DevBuf<double> s, X, b2, r2;

@@ -12,20 +12,21 @@
 //                          W_j = Z_j^{-1}  (Gauss-Jordan; Z_j is SPD).
 //   Solve A~ d = g:        forward  y_0 = g_0,  w_j = W_j y_j,  y_{j+1} = g_{j+1} + c_j o w_j;
 //                          backward d_{ny-1} = w_{ny-1},  d_j = w_j + W_j (c_j o d_{j+1}).
-// Every step of both sweeps is a product of the nx x nx block W_j with the
-// nx x 32 block of one chunk of 32 columns, so the sweeps are dense contractions
-// that the CTA of a chunk runs out of shared memory.
+// Every step of both sweeps is a product of the nx x nx block W_j with an nx x 64 or
+// nx x 32 block of columns, so the sweeps are dense contractions that a CTA runs out of
+// shared memory.
 // Accuracy comes from FP64 iterative refinement: r = b - A x in FP64 (b from
 // the ring data: x holds the ring values), g = S r rounded to FP32, x += S d,
 // until |r| <= tol |b| per column (a few passes: the FP32 factor reduces the
 // residual by about 1e-5 per pass on the workloads' media).
 //
 // Storage (per patch, offsets in the Direct tables):
-//   W  ny x ld x ld floats, W_j transposed (ld = nx rounded up to 4, zero padding)
+//   W  ny x ld x ld floats (ld = nx rounded up to 4, zero padding), W_j(i, k) at
+//      [k / 4][i][k mod 4]: four terms of a row are one 16-byte load
 //   s  ny x nx doubles; D  ny x nx floats (row j: c_j, zero on the last row)
 //   X  cols x (ny+2) x (nx+2) doubles: the FP64 iterate with its ring values
 //   R  chunks x ny x 32 x nx floats: the scaled residual g, column-major per row
-//   K  chunks x ny x ld x 32 floats: the forward sweep's w_j
+//   K  chunks x ny x 32 x ld floats: the forward sweep's w_j, a column's row contiguous
 #include "internal.h"
 #include "device_util.cuh"
 
@@ -52,6 +53,7 @@ struct DirArgs {
     const int* col_base;
     const int2* cols;
     const int4* chunks;
+    const int4* ctas;
     const int* stat_idx;
     float* W;
     float* D;
@@ -82,21 +84,20 @@ __host__ __device__ inline Geo geo(const PatchDev& P) {
     return g;
 }
 
-// Position of element (k, c), c < 32, in a swizzled k x 32 block: the 16-byte
-// group of c is xor-ed with k mod 8, so that 8 consecutive k of 4 consecutive c
-// (the transposing stores) and 32 consecutive k of one group (the GEMM's stores)
-// hit distinct banks, while each group of 4 columns stays one aligned float4.
-__device__ __forceinline__ int swz(int k, int c) { return k * kCB + ((((c >> 2) ^ (k & 7))) << 2) + (c & 3); }
-
 // ------------------------------------------------------------------ factor
 // One CTA per patch: s, the couplings c_j, and W_j = Z_j^{-1} row by row.  The
 // block lives in registers: thread (tr, tc) of a 16 x 16 layout holds the TS x TS
 // sub-block of rows tr TS .., columns tc TS .. (TS = ceil(ld / 16), one value for the
 // launch).  Z_j = T_j - C_{j-1} W_{j-1} C_{j-1} is formed elementwise from the
 // registers holding W_{j-1}; Gauss-Jordan inversion in place without pivoting (Z_j
-// is SPD), one barrier per pivot: after updating, the owners of row and column k+1
-// publish them to double-buffered shared rows for the next pivot.  W_j^T goes to
-// global memory through a padded shared copy (coalesced stores).
+// is SPD), TS pivots at a time: the thread of the diagonal sub-block runs its own pivots
+// and publishes the multipliers, the threads of its rows and columns apply them to
+// theirs and publish the pivot rows and column multipliers, all others apply the TS
+// rank-one updates out of shared memory -- two barriers for TS pivots, every element the
+// same operations in the same order as one pivot at a time.  W_j goes to global memory
+// through a padded shared copy (coalesced stores).  Bound: the latency of the pivot
+// chain, one CTA per patch.  One pivot per barrier took 50 ms on 1024 patches of 95
+// interior nodes a row.
 template <int TS>
 __global__ void __launch_bounds__(kDirThreads) direct_factor_kernel(DirArgs A) {
     extern __shared__ __align__(16) float fsm[];
@@ -107,8 +108,9 @@ __global__ void __launch_bounds__(kDirThreads) direct_factor_kernel(DirArgs A) {
     const int n = g.nx, ld = g.ld, N = A.N;
     constexpr int kW = 16 * TS;    // rows (and columns) the thread layout covers
     float* Zs = fsm;               // ld x (ld + 1): staging of W_j for the transposed store
-    float* rb = Zs + ld * (ld + 1);   // 2 x kW: row k of the current block
-    float* cb = rb + 2 * kW;          // 2 x kW: column k
+    float* RK = Zs + ld * (ld + 1);   // TS x kW: pivot rows before their scaling
+    float* FR = RK + TS * kW;         // TS x kW: column multipliers
+    __shared__ float s_inv[TS], s_fr[TS][TS], s_rk[TS][TS];   // diagonal sub-block: 1 / pivot, multipliers, rows
     double* sv = A.s + A.s_off[m];
     float* Dv = A.D + A.s_off[m];
     float* Wout = A.W + A.w_off[m];
@@ -158,53 +160,86 @@ __global__ void __launch_bounds__(kDirThreads) direct_factor_kernel(DirArgs A) {
                 z[a][b] = v;
             }
         }
-        // publish row 0 and column 0
-        if (r0 == 0)
+        const int tr = threadIdx.x >> 4, tc = threadIdx.x & 15;
+        for (int kb = 0; kb * TS < n; ++kb) {
+            const int nb = min(TS, n - kb * TS);
+            if (tr == kb && tc == kb) {
 #pragma unroll
-            for (int b = 0; b < TS; ++b) rb[c0 + b] = z[0][b];
-        if (c0 == 0)
+                for (int k = 0; k < TS; ++k) {
+                    if (k >= nb) break;
+                    const float inv = 1.f / z[k][k];
+                    s_inv[k] = inv;
+                    float rk[TS];
 #pragma unroll
-            for (int a = 0; a < TS; ++a) cb[r0 + a] = z[a][0];
-        __syncthreads();
-        for (int k = 0; k < n; ++k) {
-            const int p = (k & 1) * kW, q = kW - p;
-            const float inv = 1.f / cb[p + k];
-            float fr[TS], rk[TS];
+                    for (int b = 0; b < TS; ++b) {
+                        rk[b] = z[k][b];
+                        s_rk[k][b] = rk[b];
+                    }
 #pragma unroll
-            for (int a = 0; a < TS; ++a) fr[a] = cb[p + r0 + a] * inv;
+                    for (int a = 0; a < TS; ++a) {
+                        if (a == k) continue;
+                        const float fr = z[a][k] * inv;
+                        s_fr[k][a] = fr;
 #pragma unroll
-            for (int b = 0; b < TS; ++b) rk[b] = rb[p + c0 + b];
+                        for (int b = 0; b < TS; ++b)
+                            if (b != k) z[a][b] = fmaf(-fr, rk[b], z[a][b]);
+                        z[a][k] = -fr;
+                    }
 #pragma unroll
-            for (int a = 0; a < TS; ++a) {
-                const int r = r0 + a;
-#pragma unroll
-                for (int b = 0; b < TS; ++b) {
-                    const int c = c0 + b;
-                    float v = z[a][b];
-                    if (r != k && c != k) v = fmaf(-fr[a], rk[b], v);
-                    else if (r == k && c != k) v = rk[b] * inv;
-                    else if (r != k) v = -fr[a];
-                    else v = inv;
-                    z[a][b] = v;
+                    for (int b = 0; b < TS; ++b) z[k][b] = b == k ? inv : rk[b] * inv;
                 }
             }
-            // publish row k+1 and column k+1 of the updated block for the next pivot
-            const int k1 = k + 1;
-            if (k1 < n) {
+            __syncthreads();
+            if (tc == kb && tr != kb) {
 #pragma unroll
-                for (int a = 0; a < TS; ++a)
-                    if (r0 + a == k1)
+                for (int k = 0; k < TS; ++k) {
+                    if (k >= nb) break;
+                    const float inv = s_inv[k];
 #pragma unroll
-                        for (int b = 0; b < TS; ++b) rb[q + c0 + b] = z[a][b];
+                    for (int a = 0; a < TS; ++a) {
+                        const float fr = z[a][k] * inv;
+                        FR[k * kW + r0 + a] = fr;
 #pragma unroll
-                for (int b = 0; b < TS; ++b)
-                    if (c0 + b == k1)
+                        for (int b = 0; b < TS; ++b)
+                            if (b != k) z[a][b] = fmaf(-fr, s_rk[k][b], z[a][b]);
+                        z[a][k] = -fr;
+                    }
+                }
+            } else if (tr == kb && tc != kb) {
 #pragma unroll
-                        for (int a = 0; a < TS; ++a) cb[q + r0 + a] = z[a][b];
+                for (int k = 0; k < TS; ++k) {
+                    if (k >= nb) break;
+                    const float inv = s_inv[k];
+#pragma unroll
+                    for (int b = 0; b < TS; ++b) {
+                        const float rk = z[k][b];
+                        RK[k * kW + c0 + b] = rk;
+#pragma unroll
+                        for (int a = 0; a < TS; ++a)
+                            if (a != k) z[a][b] = fmaf(-s_fr[k][a], rk, z[a][b]);
+                        z[k][b] = rk * inv;
+                    }
+                }
             }
             __syncthreads();
+            if (tr != kb && tc != kb) {
+#pragma unroll
+                for (int k = 0; k < TS; ++k) {
+                    if (k >= nb) break;
+                    float fr[TS], rk[TS];
+#pragma unroll
+                    for (int a = 0; a < TS; ++a) fr[a] = FR[k * kW + r0 + a];
+#pragma unroll
+                    for (int b = 0; b < TS; ++b) rk[b] = RK[k * kW + c0 + b];
+#pragma unroll
+                    for (int a = 0; a < TS; ++a)
+#pragma unroll
+                        for (int b = 0; b < TS; ++b) z[a][b] = fmaf(-fr[a], rk[b], z[a][b]);
+                }
+            }
         }
-        // W_j^T to global (padding zero) through the padded shared copy
+        __syncthreads();
+        // W_j to global (padding zero) through the padded shared copy
 #pragma unroll
         for (int a = 0; a < TS; ++a)
 #pragma unroll
@@ -215,8 +250,8 @@ __global__ void __launch_bounds__(kDirThreads) direct_factor_kernel(DirArgs A) {
         __syncthreads();
         float* wj = Wout + (long long)j * ld * ld;
         for (int t = threadIdx.x; t < ld * ld; t += blockDim.x) {
-            const int r = t / ld, c = t - r * ld;
-            wj[t] = Zs[c * (ld + 1) + r];
+            const int k4 = t / (4 * ld), i = (t >> 2) - k4 * ld;
+            wj[t] = Zs[i * (ld + 1) + 4 * k4 + (t & 3)];
         }
         __syncthreads();
     }
@@ -322,127 +357,187 @@ __global__ void __launch_bounds__(kDirThreads) direct_residual_kernel(DirArgs A,
 }
 
 // ------------------------------------------------------------------ solve
-// d = Z^{-1} g by the two sweeps for one chunk of columns, then x += S d.
-// GEMM mapping: warp w owns the 4 columns 4w..4w+3, lane l the rows l + 32 q.
-template <int G>
-__device__ __forceinline__ void chunk_gemm(const float* Ws, const float* Ys, int n, int ld, int lane, int warp,
-                                           float (&acc)[G][4]) {
-#pragma unroll
-    for (int q = 0; q < G; ++q) acc[q][0] = acc[q][1] = acc[q][2] = acc[q][3] = 0.f;
-#pragma unroll 2
-    for (int k = 0; k < n; ++k) {
-        const float4 y = *reinterpret_cast<const float4*>(Ys + k * kCB + ((warp ^ (k & 7)) << 2));
-        const float* wk = Ws + k * ld + lane;
-#pragma unroll
-        for (int q = 0; q < G; ++q) {
-            const float w = wk[32 * q];
-            acc[q][0] = fmaf(w, y.x, acc[q][0]);
-            acc[q][1] = fmaf(w, y.y, acc[q][1]);
-            acc[q][2] = fmaf(w, y.z, acc[q][2]);
-            acc[q][3] = fmaf(w, y.w, acc[q][3]);
-        }
-    }
+// d = Z^{-1} g by the two sweeps for the columns of one CTA, then x += S d.  8 CPW columns
+// (two chunks of 32, or one): warp w owns columns CPW w .., lane l the rows l + 32 q, so a
+// thread keeps its w_j or d_{j+1} in registers and writes the next product's input y
+// straight from them.  W_j streams through a ring of slabs of 32 terms (cp.async, three
+// ahead, one barrier per slab); the product reads it four terms at a time (16-byte loads,
+// conflict-free) against broadcast loads of y, 4 G CPW FMAs for G + CPW loads, each output
+// one chain of FMAs over the terms in order.  R of the next row (forward) or w_j (backward)
+// is read before the product that hides it.  Bound: the FP32 pipe (2 nx^2 FMA per row and
+// column) with the shared-memory loads close behind; a warp whose columns have all
+// converged skips its products.
+constexpr int kSlabRows = 32;
+constexpr int kSlabs = 4;
+
+__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+
+// floats of shared memory: the slabs (and slack for the padded rows' reads), y
+__host__ __device__ inline int solve_smem_floats(int ld, int cw) {
+    return kSlabs * kSlabRows * ld + 128 + (ld + 3) / 4 * 4 * cw;
 }
 
-__device__ __forceinline__ void stage_block(float* dst, const float* src, int count) {
-    for (int t = threadIdx.x * 4; t < count; t += blockDim.x * 4)
-        *reinterpret_cast<float4*>(dst + t) = __ldg(reinterpret_cast<const float4*>(src + t));
-}
-
-template <int G>
-__global__ void __launch_bounds__(kDirThreads) direct_solve_kernel(DirArgs A) {
+template <int G, int CPW>
+__global__ void __launch_bounds__(kDirThreads, G * CPW <= 24 ? 2 : 1) direct_solve_kernel(DirArgs A) {
     extern __shared__ __align__(16) float ssm[];
-    const int4 ch = A.chunks[blockIdx.x];
+    constexpr int CW = 8 * CPW;                         // columns of the CTA
+    const int4 ch = A.ctas[blockIdx.x];                 // patch, first column, columns, first chunk
     const int m = ch.x, c0 = ch.y, nc = ch.z, chunk = ch.w;
-    const int gbase = A.col_base[m] + c0;
-    __shared__ int s_act[kCB];
-    __shared__ int s_any;
-    if (threadIdx.x == 0) s_any = 0;
-    __syncthreads();
-    if (threadIdx.x < kCB) {
-        const int a = threadIdx.x < nc ? A.active[gbase + threadIdx.x] : 0;
-        s_act[threadIdx.x] = a;
-        if (a) atomicOr(&s_any, 1);
-    }
-    __syncthreads();
-    if (!s_any) return;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int* active = A.active + A.col_base[m] + c0;
+    unsigned act = 0;                                   // the warp's active columns
+#pragma unroll
+    for (int c = 0; c < CPW; ++c)
+        if (CPW * warp + c < nc && active[CPW * warp + c]) act |= 1u << c;
+    if (!__syncthreads_or((int)act)) return;
     const PatchDev P = A.patches[m];
     const Geo g = geo(P);
     const int n = g.nx, ld = g.ld, ny = g.ny;
     if (n < 1 || ny < 1) return;
-    float* Ws = ssm;                                    // ld x ld (+ slack for the padded rows' reads)
-    float* Ys = Ws + ld * ld + 32 * G;                  // swizzled ld x 32
-    float* Ps = Ys + ld * kCB;                          // swizzled ld x 32: w_{j-1} / d_{j+1}
+    float* Ws = ssm;
+    float* Ys = Ws + kSlabs * kSlabRows * ld + 128;     // [k][CW], 16-byte groups xor-ed with k mod 8
     const float* Wg = A.W + A.w_off[m];
     const float* Dg = A.D + A.s_off[m];
     const double* sv = A.s + A.s_off[m];
     const float* Rc = A.R + A.r_off[m] + (long long)chunk * ny * kCB * n;
+    const long long r_chunk = (long long)ny * kCB * n;
+    const int kw = nc > kCB ? 2 * kCB : kCB;            // columns the CTA's part of K holds per row
     float* Kc = A.K + A.k_off[m] + (long long)chunk * ny * ld * kCB;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int nkb = (n + 7) >> 3;
-    float acc[G][4];
-    // ---- forward sweep
-    for (int j = 0; j < ny; ++j) {
-        stage_block(Ws, Wg + (long long)j * ld * ld, ld * ld);
-        // y_j = g_j + c_{j-1} o w_{j-1}: lanes take 8 rows x 4 columns
-        for (int p = warp; p < nkb * 8; p += 8) {
-            const int k = 8 * (p >> 3) + (lane & 7), c = 4 * (p & 7) + (lane >> 3);
-            if (k < n) {
-                float v = 0.f;
-                if (s_act[c]) {
-                    v = Rc[((long long)j * kCB + c) * n + k];
-                    if (j > 0) v = fmaf(Dg[(j - 1) * n + k], Ps[swz(k, c)], v);
-                }
-                Ys[swz(k, c)] = v;
-            }
+    const int nks = (n + kSlabRows - 1) / kSlabRows, total = (2 * ny - 1) * nks;
+    auto row_of = [&](int t) { return t < ny ? t : 2 * ny - 2 - t; };
+    auto issue = [&](int f) {                           // slab f of the stream over both sweeps
+        if (f < total) {
+            const int t = f / nks, ks = f - t * nks;
+            const float* src = Wg + (long long)row_of(t) * ld * ld + ks * kSlabRows * ld;
+            float* dst = Ws + (f % kSlabs) * kSlabRows * ld;
+            const int count = min(kSlabRows, ld - ks * kSlabRows) * ld;
+            for (int e = threadIdx.x * 4; e < count; e += kDirThreads * 4) cp_async16(dst + e, src + e);
         }
-        __syncthreads();
-        chunk_gemm<G>(Ws, Ys, n, ld, lane, warp, acc);
-        __syncthreads();   // Ps (w_{j-1}) and Ws no longer read
+        cp_async_commit();
+    };
+    auto put_y = [&](int i, const float (&v)[CPW]) {
+        float* y = Ys + i * CW;
+#pragma unroll
+        for (int c = 0; c < CPW; c += 4)
+            *reinterpret_cast<float4*>(y + ((((CPW * warp + c) >> 2) ^ (i & 7)) << 2)) =
+                make_float4(v[c], v[c + 1], v[c + 2], v[c + 3]);
+    };
+    // R of row j or w of row j for this thread's rows and columns
+    float pre[G][CPW];
+    auto load_r = [&](int j) {
 #pragma unroll
         for (int q = 0; q < G; ++q) {
             const int i = lane + 32 * q;
-            if (i < n) {
-                const float4 v = make_float4(acc[q][0], acc[q][1], acc[q][2], acc[q][3]);
-                *reinterpret_cast<float4*>(Ps + i * kCB + ((warp ^ (i & 7)) << 2)) = v;
-                *reinterpret_cast<float4*>(Kc + ((long long)j * ld + i) * kCB + 4 * warp) = v;
+#pragma unroll
+            for (int c = 0; c < CPW; ++c) {
+                const int col = CPW * warp + c;
+                pre[q][c] = (i < n && (act >> c & 1u))
+                                ? Rc[(col / kCB) * r_chunk + ((long long)j * kCB + col % kCB) * n + i] : 0.f;
             }
         }
-        __syncthreads();
+    };
+    for (int f = 0; f < kSlabs - 1; ++f) issue(f);
+    load_r(0);
+#pragma unroll
+    for (int q = 0; q < G; ++q) {
+        const int i = lane + 32 * q;
+        if (i < (ld + 3) / 4 * 4) {                     // rows n .. of y stay zero
+            float v[CPW];
+#pragma unroll
+            for (int c = 0; c < CPW; ++c) v[c] = i < n ? pre[q][c] : 0.f;
+            put_y(i, v);
+        }
     }
-    // ---- backward sweep and x += S d
-    for (int j = ny - 1; j >= 0; --j) {
-        if (j < ny - 1) {
-            stage_block(Ws, Wg + (long long)j * ld * ld, ld * ld);
-            for (int p = warp; p < nkb * 8; p += 8) {
-                const int k = 8 * (p >> 3) + (lane & 7), c = 4 * (p & 7) + (lane >> 3);
-                if (k < n) Ys[swz(k, c)] = Dg[j * n + k] * Ps[swz(k, c)];
-            }
-            __syncthreads();
-            chunk_gemm<G>(Ws, Ys, n, ld, lane, warp, acc);
+    int f = 0;
+    for (int t = 0; t < 2 * ny - 1; ++t) {
+        const int j = row_of(t);
+        const bool fwd = t < ny, turn = t == ny - 1;
+        if (fwd) {
+            if (!turn) load_r(j + 1);
         } else {
 #pragma unroll
-            for (int q = 0; q < G; ++q) acc[q][0] = acc[q][1] = acc[q][2] = acc[q][3] = 0.f;
+            for (int q = 0; q < G; ++q) {
+                const int i = lane + 32 * q;
+#pragma unroll
+                for (int c = 0; c < CPW; ++c)
+                    pre[q][c] = (i < n && (act >> c & 1u)) ? Kc[((long long)j * kw + CPW * warp + c) * ld + i] : 0.f;
+            }
         }
-        __syncthreads();   // Ps (d_{j+1}) and Ws no longer read
+        float acc[G][CPW];
+#pragma unroll
+        for (int q = 0; q < G; ++q)
+#pragma unroll
+            for (int c = 0; c < CPW; ++c) acc[q][c] = 0.f;
+        for (int ks = 0; ks < nks; ++ks, ++f) {
+            cp_async_wait<kSlabs - 2>();
+            __syncthreads();                            // slab f (and y) visible, slab f - 1 no longer read
+            issue(f + kSlabs - 1);
+            if (!act) continue;
+            const float* Wk = Ws + (f % kSlabs) * kSlabRows * ld;
+            const int kn4 = min(kSlabRows, ld - ks * kSlabRows) / 4;
+            for (int k4 = 0; k4 < kn4; ++k4) {
+                float4 w[G];
+#pragma unroll
+                for (int q = 0; q < G; ++q) w[q] = *reinterpret_cast<const float4*>(Wk + (k4 * ld + lane + 32 * q) * 4);
+#pragma unroll
+                for (int kk = 0; kk < 4; ++kk) {
+                    const int k = ks * kSlabRows + 4 * k4 + kk;
+                    float y[CPW];
+#pragma unroll
+                    for (int c = 0; c < CPW; c += 4) {
+                        const float4 v = *reinterpret_cast<const float4*>(
+                            Ys + k * CW + ((((CPW * warp + c) >> 2) ^ (k & 7)) << 2));
+                        y[c] = v.x; y[c + 1] = v.y; y[c + 2] = v.z; y[c + 3] = v.w;
+                    }
+#pragma unroll
+                    for (int q = 0; q < G; ++q) {
+                        const float wv = kk == 0 ? w[q].x : kk == 1 ? w[q].y : kk == 2 ? w[q].z : w[q].w;
+#pragma unroll
+                        for (int c = 0; c < CPW; ++c) acc[q][c] = fmaf(wv, y[c], acc[q][c]);
+                    }
+                }
+            }
+        }
+        __syncthreads();                                // y no longer read
+        // forward: w_j = acc; backward: d_j = acc + w_j (at the turn 0 + w_j)
 #pragma unroll
         for (int q = 0; q < G; ++q) {
             const int i = lane + 32 * q;
-            if (i < n) {
-                const float4 w = *reinterpret_cast<const float4*>(Kc + ((long long)j * ld + i) * kCB + 4 * warp);
-                const float4 v = make_float4(acc[q][0] + w.x, acc[q][1] + w.y, acc[q][2] + w.z, acc[q][3] + w.w);
-                *reinterpret_cast<float4*>(Ps + i * kCB + ((warp ^ (i & 7)) << 2)) = v;
+            if (i >= n || !act) continue;
+            const bool next = fwd ? true : j > 0;
+            float dn = 0.f;                             // coupling of the next product's row
+            if (fwd && !turn) dn = Dg[j * n + i];
+            else if (j > 0) dn = Dg[(j - 1) * n + i];
+            float v[CPW];
+            if (fwd && !turn) {
+#pragma unroll
+                for (int c = 0; c < CPW; ++c) {
+                    const float w = acc[q][c];
+                    if (act >> c & 1u) Kc[((long long)j * kw + CPW * warp + c) * ld + i] = w;
+                    v[c] = (act >> c & 1u) ? fmaf(dn, w, pre[q][c]) : 0.f;
+                }
+            } else {
+                const double s = sv[j * n + i];
+#pragma unroll
+                for (int c = 0; c < CPW; ++c) {
+                    const float dv = turn ? 0.f + acc[q][c] : acc[q][c] + pre[q][c];
+                    if (act >> c & 1u) {
+                        double* x = A.X + A.x_off[m] + (long long)(c0 + CPW * warp + c) * g.hd * g.wd + (j + 1) * g.wd + 1 + i;
+                        *x += s * (double)dv;
+                    }
+                    v[c] = (act >> c & 1u) ? dn * dv : 0.f;
+                }
             }
-        }
-        __syncthreads();
-        // x_j += S d_j on the active columns: warp w takes columns w, w+8, w+16, w+24
-        for (int q = 0; q < 4; ++q) {
-            const int c = warp + 8 * q;
-            if (c >= nc || !s_act[c]) continue;
-            double* x = A.X + A.x_off[m] + (long long)(c0 + c) * g.hd * g.wd + (j + 1) * g.wd + 1;
-            for (int k = lane; k < n; k += 32) x[k] += sv[j * n + k] * (double)Ps[swz(k, c)];
+            if (next) put_y(i, v);
         }
     }
+    cp_async_wait<0>();
 }
 
 // ------------------------------------------------------------------ finish
@@ -479,7 +574,7 @@ msp_status direct_plan(Medium& M, cudaStream_t s) {
     std::vector<int2> cols;
     std::vector<int4> chunks;
     long long w = 0, sv = 0, x = 0, r = 0, k = 0;
-    int max_ld = 0, fsm = 0, csm = 0;
+    int max_ld = 0;
     for (int m = 0; m < np; ++m) {
         const PatchDev& P = M.patches[m];
         const Geo g = geo(P);
@@ -495,9 +590,6 @@ msp_status direct_plan(Medium& M, cudaStream_t s) {
         for (int c = 0; c < P.cols; ++c) cols.push_back(make_int2(m, c));
         for (int q = 0; q < nch; ++q) chunks.push_back(make_int4(m, q * kCB, std::min(kCB, P.cols - q * kCB), q));
         max_ld = std::max(max_ld, g.ld);
-        const int G = std::max(1, (g.ld + 31) / 32);
-        fsm = std::max(fsm, (int)sizeof(float) * (g.ld * (g.ld + 1) + 4 * 16 * std::max(1, (g.ld + 15) / 16)));
-        csm = std::max(csm, (int)sizeof(float) * (g.ld * g.ld + 32 * G + 2 * g.ld * kCB));
     }
     // statistics slot of every column: its position in the mixed-precision item order
     std::vector<int> stat_idx(cols.size(), 0);
@@ -506,8 +598,20 @@ msp_status direct_plan(Medium& M, cudaStream_t s) {
     D.n_cols = (int)cols.size();
     D.n_chunks = (int)chunks.size();
     D.max_nxp = max_ld;
-    D.factor_smem_max = fsm;
-    D.chunk_smem_max = csm;
+    // CTAs of the sweeps: pairs of chunks (64 columns) where those fill the GPU twice, single
+    // chunks otherwise (a small medium then spreads over more SMs)
+    std::vector<int4> ctas;
+    for (size_t q = 0; q < chunks.size(); ++q) {
+        const bool two = q + 1 < chunks.size() && chunks[q + 1].x == chunks[q].x;
+        ctas.push_back(make_int4(chunks[q].x, chunks[q].y, chunks[q].z + (two ? chunks[q + 1].z : 0), chunks[q].w));
+        if (two) ++q;
+    }
+    D.wide = (int)ctas.size() >= 2 * num_sms();
+    if (!D.wide) ctas = chunks;
+    D.n_ctas = (int)ctas.size();
+    const int ts = std::max(1, (max_ld + 15) / 16);
+    D.factor_smem_max = (int)sizeof(float) * (max_ld * (max_ld + 1) + 2 * ts * 16 * ts);
+    D.chunk_smem_max = (int)sizeof(float) * solve_smem_floats(max_ld, D.wide ? 2 * kCB : kCB);
     D.w_elems = w; D.s_elems = sv; D.x_elems = x; D.r_elems = r; D.k_elems = k;
     MSP_TRY(upload(D.w_off, w_off, s));
     MSP_TRY(upload(D.s_off, s_off, s));
@@ -517,6 +621,7 @@ msp_status direct_plan(Medium& M, cudaStream_t s) {
     MSP_TRY(upload(D.col_base, col_base, s));
     MSP_TRY(upload(D.cols, cols, s));
     MSP_TRY(upload(D.chunks, chunks, s));
+    MSP_TRY(upload(D.ctas, ctas, s));
     MSP_TRY(upload(D.stat_idx, stat_idx, s));
     MSP_TRY(D.W.alloc(std::max<long long>(1, w), s));
     MSP_TRY(D.s.alloc(std::max<long long>(1, sv), s));
@@ -546,6 +651,7 @@ DirArgs direct_args(Medium& M, const LocalSolveCfg& cfg) {
     A.col_base = D.col_base.p;
     A.cols = D.cols.p;
     A.chunks = D.chunks.p;
+    A.ctas = D.ctas.p;
     A.stat_idx = D.stat_idx.p;
     A.W = D.W.p; A.D = D.D.p; A.R = D.R.p; A.K = D.K.p;
     A.s = D.s.p; A.X = D.X.p; A.b2 = D.b2.p; A.r2 = D.r2.p;
@@ -578,12 +684,23 @@ msp_status mark(Medium::Direct& D, int ph, bool begin, cudaStream_t s) {
     return MSP_OK;
 }
 
-template <int G>
+template <int G, int CPW>
 msp_status launch_solve_g(const DirArgs& A, int grid, int smem, cudaStream_t s) {
-    MSP_CUDA(cudaFuncSetAttribute(direct_solve_kernel<G>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    direct_solve_kernel<G><<<grid, kDirThreads, smem, s>>>(A);
+    MSP_CUDA(cudaFuncSetAttribute(direct_solve_kernel<G, CPW>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    direct_solve_kernel<G, CPW><<<grid, kDirThreads, smem, s>>>(A);
     count_launches(1);
     return MSP_OK;
+}
+
+template <int CPW>
+msp_status launch_solve(const DirArgs& A, int G, int grid, int smem, cudaStream_t s) {
+    switch (G) {
+        case 1: return launch_solve_g<1, CPW>(A, grid, smem, s);
+        case 2: return launch_solve_g<2, CPW>(A, grid, smem, s);
+        case 3: return launch_solve_g<3, CPW>(A, grid, smem, s);
+        case 4: return launch_solve_g<4, CPW>(A, grid, smem, s);
+        default: return launch_solve_g<5, CPW>(A, grid, smem, s);
+    }
 }
 
 }  // namespace
@@ -646,13 +763,8 @@ msp_status launch_local_solves_direct(Medium& M, const LocalSolveCfg& cfg, cudaS
     const int passes = std::max(1, std::min(cfg.max_ref, kDirMaxPasses));
     for (int p = 0; p < passes; ++p) {
         MSP_TRY(mark(D, kPhSolve, true, s));
-        switch (G) {
-            case 1: MSP_TRY(launch_solve_g<1>(A, D.n_chunks, D.chunk_smem_max, s)); break;
-            case 2: MSP_TRY(launch_solve_g<2>(A, D.n_chunks, D.chunk_smem_max, s)); break;
-            case 3: MSP_TRY(launch_solve_g<3>(A, D.n_chunks, D.chunk_smem_max, s)); break;
-            case 4: MSP_TRY(launch_solve_g<4>(A, D.n_chunks, D.chunk_smem_max, s)); break;
-            default: MSP_TRY(launch_solve_g<5>(A, D.n_chunks, D.chunk_smem_max, s)); break;
-        }
+        if (D.wide) MSP_TRY(launch_solve<8>(A, G, D.n_ctas, D.chunk_smem_max, s));
+        else MSP_TRY(launch_solve<4>(A, G, D.n_ctas, D.chunk_smem_max, s));
         MSP_TRY(mark(D, kPhSolve, false, s));
         MSP_TRY(mark(D, kPhResidual, true, s));
         direct_residual_kernel<<<D.n_chunks, kDirThreads, 0, s>>>(A, 0);

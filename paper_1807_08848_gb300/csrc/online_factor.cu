@@ -586,7 +586,7 @@ struct SweepLayout {
 };
 
 template <class T, int BT>
-__global__ void __launch_bounds__(512, BT >= 4 ? 2 : 1) sweep_kernel(SweepArgs<T> A) {
+__global__ void __launch_bounds__(512, BT >= 4 && sizeof(T) == 4 ? 2 : 1) sweep_kernel(SweepArgs<T> A) {
     extern __shared__ __align__(16) unsigned char sweep_smem[];
     T* xs = reinterpret_cast<T*>(sweep_smem);   // BT x sweep_kc
     unsigned int gen = atomicAdd(&A.bar[1], 0u);
