@@ -170,6 +170,13 @@ struct Medium {
         DevBuf<int4> ctas;                                      // the sweeps' CTAs: one chunk or two (wide) each
         bool wide = false;
         int n_ctas = 0;
+        // groups of patches whose launches run on streams of their own, and the second one's
+        struct Group {
+            int patch0, patches, col0, cols, chunk0, chunks, cta0, ctas;
+        };
+        std::vector<Group> groups;
+        cudaStream_t side = nullptr;
+        cudaEvent_t fork = nullptr, join = nullptr;
         DevBuf<int> stat_idx;                                   // global column -> statistics slot
         DevBuf<float> W, D, R, K;
         DevBuf<double> s, X, b2, r2;
@@ -183,6 +190,9 @@ struct Medium {
         int ev_used = 0;
         ~Direct() {
             for (cudaEvent_t e : ev) cudaEventDestroy(e);
+            if (fork) cudaEventDestroy(fork);
+            if (join) cudaEventDestroy(join);
+            if (side) cudaStreamDestroy(side);
         }
     } dir;
     // CUDA graph of the local-solve launches, replayed while the configuration is unchanged

@@ -68,6 +68,7 @@ struct DirArgs {
     double* snaps;
     int* stats;
     double tol;
+    int patch0, col0;          // first patch and column of the launch's group
 };
 
 struct Geo {
@@ -101,7 +102,7 @@ __host__ __device__ inline Geo geo(const PatchDev& P) {
 template <int TS>
 __global__ void __launch_bounds__(kDirThreads) direct_factor_kernel(DirArgs A) {
     extern __shared__ __align__(16) float fsm[];
-    const int m = blockIdx.x;
+    const int m = A.patch0 + blockIdx.x;
     const PatchDev P = A.patches[m];
     const Geo g = geo(P);
     if (g.nx < 1 || g.ny < 1) return;
@@ -260,7 +261,7 @@ __global__ void __launch_bounds__(kDirThreads) direct_factor_kernel(DirArgs A) {
 // ------------------------------------------------------------------ init
 // One CTA per column: the FP64 iterate is the ring data with a zero interior.
 __global__ void __launch_bounds__(kDirThreads) direct_init_kernel(DirArgs A) {
-    const int gcol = blockIdx.x;
+    const int gcol = A.col0 + blockIdx.x;
     const int2 mc = A.cols[gcol];
     const int m = mc.x, col = mc.y;
     const PatchDev P = A.patches[m];
@@ -290,42 +291,42 @@ __global__ void __launch_bounds__(kDirThreads) direct_init_kernel(DirArgs A) {
 }
 
 // ------------------------------------------------------------------ residual
-// One CTA per chunk: r = b - A x = -(A x) (x carries the ring data) in FP64, the
-// scaled residual g = S r in FP32 for the next solve, |r|^2 per column in a fixed
-// order (warp w takes columns w, w+8, w+16, w+24, lanes along the row).  first:
-// |b| = |r| of the initial iterate.  A column stays active while |r| > tol |b|.
-__global__ void __launch_bounds__(kDirThreads) direct_residual_kernel(DirArgs A, int first) {
+// r = b - A x = -(A x) (x carries the ring data) in FP64, the scaled residual g = S r in
+// FP32 for the next solve, |r|^2 per column in a fixed order: a warp per column, lanes
+// along the row, rows ascending.  first: |b| = |r| of the initial iterate.  A column stays
+// active while |r| > tol |b|.  A CTA takes 8 warps' columns of a chunk, 32 of them or 8
+// (blockIdx.y) when the chunks alone would leave SMs idle.
+// Bound: the FP64 pipe.  A difference across a face is formed once: the one to the left
+// is the left lane's to the right, negated, and the one below is the row below's upward,
+// kept in a register; with them a node costs 8 FP64 operations in place of 10.
+__device__ __forceinline__ void residual_done(const DirArgs& A, int gc, double t, int first) {
+    const double b2 = first ? t : A.b2[gc];
+    if (first) A.b2[gc] = t;
+    else A.passes[gc] += 1;
+    A.r2[gc] = t;
+    A.active[gc] = (b2 > 0.0 && t > A.tol * A.tol * b2) ? 1 : 0;
+}
+
+// The initial iterate: zero inside, so only nodes next to the ring have a nonzero
+// residual; the others are written as the zeros they are.
+__global__ void __launch_bounds__(kDirThreads) direct_residual_first_kernel(DirArgs A, int per) {
     const int4 ch = A.chunks[blockIdx.x];
     const int m = ch.x, c0 = ch.y, nc = ch.z, chunk = ch.w;
-    const int gbase = A.col_base[m] + c0;
-    __shared__ int s_act[kCB];
-    __shared__ int s_any;
-    if (threadIdx.x == 0) s_any = 0;
-    __syncthreads();
-    if (threadIdx.x < kCB) {
-        const int a = threadIdx.x < nc ? (first ? 1 : A.active[gbase + threadIdx.x]) : 0;
-        s_act[threadIdx.x] = a;
-        if (a) atomicOr(&s_any, 1);
-    }
-    __syncthreads();
-    if (!s_any) return;
     const PatchDev P = A.patches[m];
     const Geo g = geo(P);
     const int n = g.nx, N = A.N;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const double* sv = A.s + A.s_off[m];
     float* Rc = A.R + A.r_off[m] + (long long)chunk * g.ny * kCB * n;
-    double acc[4] = {0.0, 0.0, 0.0, 0.0};
-    for (int j = 0; j < g.ny; ++j) {
-        const long long gj = P.Y0 + 1 + j;
-        for (int q = 0; q < 4; ++q) {
-            const int c = warp + 8 * q;
-            if (c >= nc || !s_act[c]) continue;
+    for (int q = 0; q < per; ++q) {
+        const int c = warp + 8 * (per * blockIdx.y + q);
+        if (c >= nc) continue;
+        double acc = 0.0;
+        for (int j = 0; j < g.ny; ++j) {
+            const long long gj = P.Y0 + 1 + j;
             const double* x = A.X + A.x_off[m] + (long long)(c0 + c) * g.hd * g.wd + (j + 1) * g.wd + 1;
             float* rr = Rc + ((long long)j * kCB + c) * n;
-            // first pass: the interior of the iterate is zero, so only nodes next to the
-            // ring have a nonzero residual; the others are written as the zeros they are
-            const bool edge_only = first && j > 0 && j + 1 < g.ny;
+            const bool edge_only = j > 0 && j + 1 < g.ny;
             for (int k = lane; k < n; k += 32) {
                 if (edge_only && k > 0 && k + 1 < n) {
                     rr[k] = 0.f;
@@ -337,22 +338,77 @@ __global__ void __launch_bounds__(kDirThreads) direct_residual_kernel(DirArgs A,
                 const double xc = x[k];
                 const double r = ae * (x[k + 1] - xc) + aw * (x[k - 1] - xc) + an * (x[k + g.wd] - xc) +
                                  as * (x[k - g.wd] - xc);
-                acc[q] += r * r;
+                acc += r * r;
                 rr[k] = (float)(r * sv[j * n + k]);
             }
         }
+        const double t = warp_sum(acc);
+        if (lane == 0) residual_done(A, A.col_base[m] + c0 + c, t, 1);
     }
-    for (int q = 0; q < 4; ++q) {
-        const int c = warp + 8 * q;
-        const double t = warp_sum(acc[q]);
-        if (lane == 0 && c < nc && s_act[c]) {
-            const int gc = gbase + c;
-            double b2 = first ? t : A.b2[gc];
-            if (first) A.b2[gc] = t;
-            else A.passes[gc] += 1;
-            A.r2[gc] = t;
-            A.active[gc] = (b2 > 0.0 && t > A.tol * A.tol * b2) ? 1 : 0;
+}
+
+template <int G>
+__global__ void __launch_bounds__(kDirThreads) direct_residual_kernel(DirArgs A, int per) {
+    const int4 ch = A.chunks[blockIdx.x];
+    const int m = ch.x, c0 = ch.y, nc = ch.z, chunk = ch.w;
+    const int gbase = A.col_base[m] + c0;
+    const PatchDev P = A.patches[m];
+    const Geo g = geo(P);
+    const int n = g.nx, N = A.N, wd = g.wd;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const double* sv = A.s + A.s_off[m];
+    float* Rc = A.R + A.r_off[m] + (long long)chunk * g.ny * kCB * n;
+    const double* aEp = A.aE + (long long)(P.Y0 + 1) * N + P.X0 + 1;        // east face of node (0, 0)
+    const double* aNp = A.aN + (long long)(P.Y0 + 1) * (N + 1) + P.X0 + 1;  // north face
+    for (int q = 0; q < per; ++q) {
+        const int c = warp + 8 * (per * blockIdx.y + q);
+        if (c >= nc || !A.active[gbase + c]) continue;                      // warp-uniform
+        const double* x = A.X + A.x_off[m] + (long long)(c0 + c) * g.hd * wd + wd + 1;   // row 0
+        double xc[G], ds[G], an[G];                     // row j; difference and face below it
+#pragma unroll
+        for (int u = 0; u < G; ++u) {
+            const int k = lane + 32 * u;
+            xc[u] = k < n ? x[k] : 0.0;
+            ds[u] = k < n ? x[k - wd] - xc[u] : 0.0;
+            an[u] = k < n ? aNp[k - (N + 1)] : 0.0;
         }
+        double acc = 0.0;
+        for (int j = 0; j < g.ny; ++j) {
+            const double* xr = x + (long long)j * wd;
+            const double* ae_r = aEp + (long long)j * N;
+            const double* an_r = aNp + (long long)j * (N + 1);
+            float* rr = Rc + ((long long)j * kCB + c) * n;
+            double left = 0.0;                          // the last difference of the block of 32 before
+#pragma unroll
+            for (int u = 0; u < G; ++u) {
+                const int k = lane + 32 * u;
+                const bool in = k < n;
+                if (32 * u < n) {
+                    const double xe = in ? xr[k + 1] : 0.0, xn = in ? xr[k + wd] : 0.0;
+                    const double ae = in ? ae_r[k] : 0.0, aw = in ? ae_r[k - 1] : 0.0;
+                    const double anew = in ? an_r[k] : 0.0, s = in ? sv[j * n + k] : 0.0;
+                    const double de = xe - xc[u], dn = xn - xc[u];
+                    double dw = -__shfl_up_sync(0xffffffffu, de, 1);
+                    if (u == 0) {
+                        const double w0 = xr[-1] - xc[0];
+                        if (lane == 0) dw = w0;
+                    } else if (lane == 0) {
+                        dw = -left;
+                    }
+                    left = __shfl_sync(0xffffffffu, de, 31);
+                    if (in) {
+                        const double r = ae * de + aw * dw + anew * dn + an[u] * ds[u];
+                        acc += r * r;
+                        rr[k] = (float)(r * s);
+                    }
+                    ds[u] = -dn;
+                    an[u] = anew;
+                    xc[u] = xn;
+                }
+            }
+        }
+        const double t = warp_sum(acc);
+        if (lane == 0) residual_done(A, gbase + c, t, 0);
     }
 }
 
@@ -384,7 +440,7 @@ __host__ __device__ inline int solve_smem_floats(int ld, int cw) {
 }
 
 template <int G, int CPW>
-__global__ void __launch_bounds__(kDirThreads, G * CPW <= 24 ? 2 : 1) direct_solve_kernel(DirArgs A) {
+__global__ void __launch_bounds__(kDirThreads, 2) direct_solve_kernel(DirArgs A) {
     extern __shared__ __align__(16) float ssm[];
     constexpr int CW = 8 * CPW;                         // columns of the CTA
     const int4 ch = A.ctas[blockIdx.x];                 // patch, first column, columns, first chunk
@@ -461,6 +517,13 @@ __global__ void __launch_bounds__(kDirThreads, G * CPW <= 24 ? 2 : 1) direct_sol
         if (fwd) {
             if (!turn) load_r(j + 1);
         } else {
+            // the iterate's row into the L2: two 128-byte lines per 32 values
+#pragma unroll
+            for (int c = 0; c < CPW; ++c)
+                if (act >> c & 1u) {
+                    const double* xr = A.X + A.x_off[m] + (long long)(c0 + CPW * warp + c) * g.hd * g.wd + (j + 1) * g.wd + 1;
+                    if (16 * lane < n) asm volatile("prefetch.global.L2 [%0];" ::"l"(xr + 16 * lane));
+                }
 #pragma unroll
             for (int q = 0; q < G; ++q) {
                 const int i = lane + 32 * q;
@@ -543,7 +606,7 @@ __global__ void __launch_bounds__(kDirThreads, G * CPW <= 24 ? 2 : 1) direct_sol
 // ------------------------------------------------------------------ finish
 // One CTA per column: restriction to K_m and the column's statistics.
 __global__ void __launch_bounds__(kDirThreads) direct_finish_kernel(DirArgs A) {
-    const int gcol = blockIdx.x;
+    const int gcol = A.col0 + blockIdx.x;
     const int2 mc = A.cols[gcol];
     const int m = mc.x, col = mc.y;
     const PatchDev P = A.patches[m];
@@ -609,6 +672,28 @@ msp_status direct_plan(Medium& M, cudaStream_t s) {
     D.wide = (int)ctas.size() >= 2 * num_sms();
     if (!D.wide) ctas = chunks;
     D.n_ctas = (int)ctas.size();
+    // Two groups of patches with half of the columns each, on two streams: the residuals
+    // of one (FP64 pipe) run beside the sweeps of the other (FP32 pipe, load latency).
+    // One group where half of the sweeps' CTAs would not fill the GPU twice.
+    D.groups.assign(2, Medium::Direct::Group{});
+    Medium::Direct::Group& g0 = D.groups[0];
+    Medium::Direct::Group& g1 = D.groups[1];
+    int half = np;
+    if (D.n_ctas >= 4 * num_sms())
+        for (half = 0; half < np && 2 * col_base[half] < (int)cols.size(); ++half) {}
+    auto below = [half](const std::vector<int4>& v) {
+        return (int)(std::find_if(v.begin(), v.end(), [half](const int4& e) { return e.x >= half; }) - v.begin());
+    };
+    const int hc = below(chunks), ha = below(ctas), hcol = half < np ? col_base[half] : (int)cols.size();
+    g0 = {0, half, 0, hcol, 0, hc, 0, ha};
+    g1 = {half, np - half, hcol, (int)cols.size() - hcol, hc, (int)chunks.size() - hc, ha, (int)ctas.size() - ha};
+    if (g1.patches == 0) {
+        D.groups.pop_back();
+    } else if (!D.side) {
+        MSP_CUDA(cudaStreamCreateWithFlags(&D.side, cudaStreamNonBlocking));
+        MSP_CUDA(cudaEventCreateWithFlags(&D.fork, cudaEventDisableTiming));
+        MSP_CUDA(cudaEventCreateWithFlags(&D.join, cudaEventDisableTiming));
+    }
     const int ts = std::max(1, (max_ld + 15) / 16);
     D.factor_smem_max = (int)sizeof(float) * (max_ld * (max_ld + 1) + 2 * ts * 16 * ts);
     D.chunk_smem_max = (int)sizeof(float) * solve_smem_floats(max_ld, D.wide ? 2 * kCB : kCB);
@@ -720,42 +805,43 @@ static msp_status launch_factor(const DirArgs& A, int np, int smem, cudaStream_t
     return MSP_OK;
 }
 
-msp_status launch_local_solves_direct(Medium& M, const LocalSolveCfg& cfg, cudaStream_t s) {
-    if (!direct_fits(M)) {
-        set_error("direct local solver: a buffered patch is wider than 160 interior nodes");
-        return MSP_ERR_INVALID_ARG;
-    }
-    MSP_TRY(direct_plan(M, s));
-    Medium::Direct& D = M.dir;
-    DirArgs A = direct_args(M, cfg);
-    const int np = (int)M.patches.size();
-    D.ev_used = 0;
+// Factor (once per medium), residuals, sweeps and restriction of one group of patches.
+static msp_status launch_group(Medium::Direct& D, const Medium::Direct::Group& grp, DirArgs A, const LocalSolveCfg& cfg,
+                               cudaStream_t s) {
+    A.patch0 = grp.patch0;
+    A.col0 = grp.col0;
+    A.chunks += grp.chunk0;
+    A.ctas += grp.cta0;
     if (!D.factored) {
         MSP_TRY(mark(D, kPhFactor, true, s));
         // one sub-block size for the launch, from the widest padded row
         switch (std::max(1, (D.max_nxp + 15) / 16)) {
-            case 1: MSP_TRY(launch_factor<1>(A, np, D.factor_smem_max, s)); break;
-            case 2: MSP_TRY(launch_factor<2>(A, np, D.factor_smem_max, s)); break;
-            case 3: MSP_TRY(launch_factor<3>(A, np, D.factor_smem_max, s)); break;
-            case 4: MSP_TRY(launch_factor<4>(A, np, D.factor_smem_max, s)); break;
-            case 5: MSP_TRY(launch_factor<5>(A, np, D.factor_smem_max, s)); break;
-            case 6: MSP_TRY(launch_factor<6>(A, np, D.factor_smem_max, s)); break;
-            case 7: MSP_TRY(launch_factor<7>(A, np, D.factor_smem_max, s)); break;
-            case 8: MSP_TRY(launch_factor<8>(A, np, D.factor_smem_max, s)); break;
-            case 9: MSP_TRY(launch_factor<9>(A, np, D.factor_smem_max, s)); break;
-            default: MSP_TRY(launch_factor<10>(A, np, D.factor_smem_max, s)); break;
+            case 1: MSP_TRY(launch_factor<1>(A, grp.patches, D.factor_smem_max, s)); break;
+            case 2: MSP_TRY(launch_factor<2>(A, grp.patches, D.factor_smem_max, s)); break;
+            case 3: MSP_TRY(launch_factor<3>(A, grp.patches, D.factor_smem_max, s)); break;
+            case 4: MSP_TRY(launch_factor<4>(A, grp.patches, D.factor_smem_max, s)); break;
+            case 5: MSP_TRY(launch_factor<5>(A, grp.patches, D.factor_smem_max, s)); break;
+            case 6: MSP_TRY(launch_factor<6>(A, grp.patches, D.factor_smem_max, s)); break;
+            case 7: MSP_TRY(launch_factor<7>(A, grp.patches, D.factor_smem_max, s)); break;
+            case 8: MSP_TRY(launch_factor<8>(A, grp.patches, D.factor_smem_max, s)); break;
+            case 9: MSP_TRY(launch_factor<9>(A, grp.patches, D.factor_smem_max, s)); break;
+            default: MSP_TRY(launch_factor<10>(A, grp.patches, D.factor_smem_max, s)); break;
         }
         count_launches(1);
         MSP_TRY(mark(D, kPhFactor, false, s));
         MSP_CUDA(cudaGetLastError());
-        D.factored = true;
     }
+    if (grp.cols == 0) return MSP_OK;
     MSP_TRY(mark(D, kPhInit, true, s));
-    direct_init_kernel<<<D.n_cols, kDirThreads, 0, s>>>(A);
+    direct_init_kernel<<<grp.cols, kDirThreads, 0, s>>>(A);
     count_launches(1);
     MSP_TRY(mark(D, kPhInit, false, s));
     MSP_TRY(mark(D, kPhResidual, true, s));
-    direct_residual_kernel<<<D.n_chunks, kDirThreads, 0, s>>>(A, 1);
+    // columns per warp of the residual: 4 (a chunk per CTA), or 1 while that fills the GPU less
+    // than six CTAs per SM
+    const int per = grp.chunks >= 6 * num_sms() ? 4 : 1;
+    const dim3 rgrid(grp.chunks, 4 / per);
+    direct_residual_first_kernel<<<rgrid, kDirThreads, 0, s>>>(A, per);
     count_launches(1);
     MSP_TRY(mark(D, kPhResidual, false, s));
     MSP_CUDA(cudaGetLastError());
@@ -763,19 +849,53 @@ msp_status launch_local_solves_direct(Medium& M, const LocalSolveCfg& cfg, cudaS
     const int passes = std::max(1, std::min(cfg.max_ref, kDirMaxPasses));
     for (int p = 0; p < passes; ++p) {
         MSP_TRY(mark(D, kPhSolve, true, s));
-        if (D.wide) MSP_TRY(launch_solve<8>(A, G, D.n_ctas, D.chunk_smem_max, s));
-        else MSP_TRY(launch_solve<4>(A, G, D.n_ctas, D.chunk_smem_max, s));
+        if (D.wide) MSP_TRY(launch_solve<8>(A, G, grp.ctas, D.chunk_smem_max, s));
+        else MSP_TRY(launch_solve<4>(A, G, grp.ctas, D.chunk_smem_max, s));
         MSP_TRY(mark(D, kPhSolve, false, s));
         MSP_TRY(mark(D, kPhResidual, true, s));
-        direct_residual_kernel<<<D.n_chunks, kDirThreads, 0, s>>>(A, 0);
+        switch (G) {
+            case 1: direct_residual_kernel<1><<<rgrid, kDirThreads, 0, s>>>(A, per); break;
+            case 2: direct_residual_kernel<2><<<rgrid, kDirThreads, 0, s>>>(A, per); break;
+            case 3: direct_residual_kernel<3><<<rgrid, kDirThreads, 0, s>>>(A, per); break;
+            case 4: direct_residual_kernel<4><<<rgrid, kDirThreads, 0, s>>>(A, per); break;
+            default: direct_residual_kernel<5><<<rgrid, kDirThreads, 0, s>>>(A, per); break;
+        }
         count_launches(1);
         MSP_TRY(mark(D, kPhResidual, false, s));
         MSP_CUDA(cudaGetLastError());
     }
     MSP_TRY(mark(D, kPhFinish, true, s));
-    direct_finish_kernel<<<D.n_cols, kDirThreads, 0, s>>>(A);
+    direct_finish_kernel<<<grp.cols, kDirThreads, 0, s>>>(A);
     count_launches(1);
     MSP_TRY(mark(D, kPhFinish, false, s));
+    MSP_CUDA(cudaGetLastError());
+    return MSP_OK;
+}
+
+msp_status launch_local_solves_direct(Medium& M, const LocalSolveCfg& cfg, cudaStream_t s) {
+    if (!direct_fits(M)) {
+        set_error("direct local solver: a buffered patch is wider than 160 interior nodes");
+        return MSP_ERR_INVALID_ARG;
+    }
+    MSP_TRY(direct_plan(M, s));
+    Medium::Direct& D = M.dir;
+    const DirArgs A0 = direct_args(M, cfg);
+    D.ev_used = 0;
+    // phase timing reads one stream's events: the groups then run one after the other
+    const bool forked = D.groups.size() > 1 && !D.timing;
+    if (forked) {
+        MSP_CUDA(cudaEventRecord(D.fork, s));
+        MSP_CUDA(cudaStreamWaitEvent(D.side, D.fork, 0));
+    }
+    msp_status st = MSP_OK;
+    for (size_t q = 0; q < D.groups.size() && st == MSP_OK; ++q)
+        st = launch_group(D, D.groups[q], A0, cfg, forked && q > 0 ? D.side : s);
+    if (forked) {   // also after an error: the caller's stream waits for what was launched
+        MSP_CUDA(cudaEventRecord(D.join, D.side));
+        MSP_CUDA(cudaStreamWaitEvent(s, D.join, 0));
+    }
+    MSP_TRY(st);
+    D.factored = true;
     MSP_CUDA(cudaGetLastError());
     return MSP_OK;
 }
