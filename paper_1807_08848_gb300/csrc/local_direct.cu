@@ -321,27 +321,43 @@ __global__ void __launch_bounds__(kDirThreads) direct_residual_first_kernel(DirA
     for (int q = 0; q < per; ++q) {
         const int c = warp + 8 * (per * blockIdx.y + q);
         if (c >= nc) continue;
+        const double* x0 = A.X + A.x_off[m] + (long long)(c0 + c) * g.hd * g.wd + g.wd + 1;
+        auto residual = [&](int j, int k) {
+            const double* x = x0 + (long long)j * g.wd;
+            const long long gj = P.Y0 + 1 + j, gi = P.X0 + 1 + k;
+            const double ae = A.aE[gj * N + gi], aw = A.aE[gj * N + gi - 1];
+            const double an = A.aN[gj * (N + 1) + gi], as = A.aN[(gj - 1) * (N + 1) + gi];
+            const double xc = x[k];
+            const double r = ae * (x[k + 1] - xc) + aw * (x[k - 1] - xc) + an * (x[k + g.wd] - xc) +
+                             as * (x[k - g.wd] - xc);
+            Rc[((long long)j * kCB + c) * n + k] = (float)(r * sv[j * n + k]);
+            return r;
+        };
         double acc = 0.0;
-        for (int j = 0; j < g.ny; ++j) {
-            const long long gj = P.Y0 + 1 + j;
-            const double* x = A.X + A.x_off[m] + (long long)(c0 + c) * g.hd * g.wd + (j + 1) * g.wd + 1;
-            float* rr = Rc + ((long long)j * kCB + c) * n;
-            const bool edge_only = j > 0 && j + 1 < g.ny;
+        auto full_row = [&](int j) {
             for (int k = lane; k < n; k += 32) {
-                if (edge_only && k > 0 && k + 1 < n) {
-                    rr[k] = 0.f;
-                    continue;
-                }
-                const long long gi = P.X0 + 1 + k;
-                const double ae = A.aE[gj * N + gi], aw = A.aE[gj * N + gi - 1];
-                const double an = A.aN[gj * (N + 1) + gi], as = A.aN[(gj - 1) * (N + 1) + gi];
-                const double xc = x[k];
-                const double r = ae * (x[k + 1] - xc) + aw * (x[k - 1] - xc) + an * (x[k + g.wd] - xc) +
-                                 as * (x[k - g.wd] - xc);
+                const double r = residual(j, k);
                 acc += r * r;
-                rr[k] = (float)(r * sv[j * n + k]);
+            }
+        };
+        if (g.ny > 0) full_row(0);
+        // rows between: the lanes take 32 rows' first and last nodes at once; the squares are
+        // then added row by row in the lanes that hold those nodes
+        const int lr = (n - 1) & 31;
+        for (int j0 = 1; j0 + 1 < g.ny && n > 0; j0 += 32) {
+            const int jn = min(32, g.ny - 1 - j0);
+            const double rl = lane < jn ? residual(j0 + lane, 0) : 0.0;
+            const double rr = n > 1 && lane < jn ? residual(j0 + lane, n - 1) : 0.0;
+            for (int j = 0; j < jn; ++j) {
+                const double a = __shfl_sync(0xffffffffu, rl, j), b = __shfl_sync(0xffffffffu, rr, j);
+                if (lane == 0) acc += a * a;
+                if (n > 1 && lane == lr) acc += b * b;
+                float* row = Rc + ((long long)(j0 + j) * kCB + c) * n;
+                for (int k = lane; k < n; k += 32)
+                    if (k > 0 && k + 1 < n) row[k] = 0.f;
             }
         }
+        if (g.ny > 1) full_row(g.ny - 1);
         const double t = warp_sum(acc);
         if (lane == 0) residual_done(A, A.col_base[m] + c0 + c, t, 1);
     }

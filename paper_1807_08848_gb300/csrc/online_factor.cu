@@ -199,56 +199,108 @@ __global__ void __launch_bounds__(256) patch_post_kernel(const double* F, const 
 }
 
 // Cholesky of one <= 64 x 64 diagonal tile in shared memory; writes L (lower,
-// strict upper zeroed) in place.  One CTA of 256 threads on the factorisation's
-// critical path, in the LDL^T form so that each column costs one barrier: at step
-// k every thread (i, g) (row i = tid mod 64, g = tid / 64) updates
-// L[i][j] -= (L[i][k] / d_k) L[j][k] for j = k+1+g, k+5+g, ... up to i, with the
-// reciprocal 1 / d_k of the pivot taken in step k-1 by the thread that made the
-// last update of L[k][k] (while the others finish theirs).  At the end the columns
-// are scaled, L[i][j] / sqrt(d_j) below the diagonal and sqrt(d_j) on it.  A
-// non-positive pivot sets *fail (and continues with d = 1).  The inverse of the
-// factor is left to tile_inverse_kernel, off the critical path.
-template <class T>
-__device__ __forceinline__ T checked_pivot(T d, int* s_ok) {
-    if (!(d > T(0)) || !isfinite(d)) {
-        *s_ok = 0;
-        return T(1);
-    }
-    return d;
-}
-
+// strict upper zeroed) in place.  One CTA on the factorisation's critical path, in the
+// LDL^T form L[i][j] -= (L[i][k] / d_k) L[j][k] by panels of 4 columns, with the rest of the
+// panel before beside it (a warp's FP64 instructions take 64 clocks of its quarter of the
+// SM each, so the pivot chain must not share its quarter):
+//   A  warp 0 runs the panel's 4 x 4 corner, a lane per row, pivots passed by shuffles, while
+//      the warps of the other three quarters apply the panel before to the columns right
+//      of this panel (elements of that triangle dealt out evenly);
+//   B  the rows below the corner, a lane per row;
+//   C  the next panel's columns.
+// At the end the columns are scaled, L[i][j] / sqrt(d_j) below the diagonal and sqrt(d_j)
+// on it.  Every element takes its updates in ascending order of k, one FMA each.  A
+// non-positive pivot sets *fail (and continues with d = 1).  The inverse of the factor is
+// left to tile_inverse_kernel, off the critical path.  Bound: the pivot chain (reciprocal,
+// product, FMA: about 510 clocks a column).
+constexpr int kPotPanel = 4;
 template <class T>
 __global__ void __launch_bounds__(256) potrf_tile_kernel(T* A, int lda, int nb, int* fail) {
-    static_assert(kTile == 64, "thread layout assumes 64-wide tiles and 256 threads");
+    static_assert(kTile == 64, "two warps hold the rows of a tile");
+    constexpr int W = kPotPanel;
     __shared__ T L[kTile][kTile + 1];
-    __shared__ T s_inv[2];
+    __shared__ T Ts[2][W][kTile];            // multipliers L[i][k] / d_k of a panel, by panel parity
+    __shared__ T Vs[2][W][kTile];            // its values L[i][k]
+    __shared__ T s_inv[W];
     __shared__ T s_sq[kTile];
     __shared__ int s_ok;
-    const int tid = threadIdx.x;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     for (int e = tid; e < nb * nb; e += blockDim.x) {
         const int i = e % nb, j = e / nb;
         L[i][j] = (i >= j) ? A[i + (long long)j * lda] : T(0);
     }
+    if (tid == 0) s_ok = 1;
     __syncthreads();
-    if (tid == 0) {
-        s_ok = 1;
-        if (nb > 0) {
-            const T d = checked_pivot(L[0][0], &s_ok);
-            L[0][0] = d;
-            s_inv[0] = T(1) / d;
-        }
-    }
-    __syncthreads();
-    const int ri = tid & (kTile - 1), g = tid >> 6;
-    for (int k = 0; k < nb; ++k) {
-        if (ri > k && ri < nb) {
-            const T t = L[ri][k] * s_inv[k & 1];
-            for (int j = k + 1 + g; j <= ri; j += 4) L[ri][j] = fma(-t, L[j][k], L[ri][j]);
-            if (g == 0 && ri == k + 1) {   // L[k+1][k+1] is final: the next pivot
-                const T d = checked_pivot(L[ri][ri], &s_ok);
-                L[ri][ri] = d;
-                s_inv[(k + 1) & 1] = T(1) / d;
+    // one element's updates by a panel of wk columns
+    auto apply = [&](int q, int wk, int i, int j) {
+        T a = L[i][j];
+#pragma unroll
+        for (int k = 0; k < W; ++k)
+            if (k < wk) a = fma(-Ts[q][k][i], Vs[q][k][j], a);
+        L[i][j] = a;
+    };
+    for (int p = 0; p < nb; p += W) {
+        const int w = min(W, nb - p), par = (p / W) & 1;
+        if (warp == 0) {
+            T crn[W];
+#pragma unroll
+            for (int c = 0; c < W; ++c) crn[c] = (lane < w && c <= lane) ? L[p + lane][p + c] : T(0);
+#pragma unroll
+            for (int k = 0; k < W; ++k) {
+                if (k >= w) break;
+                T d = __shfl_sync(0xffffffffu, crn[k], k);
+                if (!(d > T(0)) || !isfinite(d)) {
+                    if (lane == 0) s_ok = 0;
+                    d = T(1);
+                }
+                const T inv = T(1) / d;
+                if (lane == k) crn[k] = d;
+                if (lane == 0) s_inv[k] = inv;
+                const T tc = crn[k] * inv;
+#pragma unroll
+                for (int j = k + 1; j < W; ++j) {
+                    const T ljk = __shfl_sync(0xffffffffu, crn[k], j);
+                    if (lane >= j && lane < w) crn[j] = fma(-tc, ljk, crn[j]);
+                }
             }
+#pragma unroll
+            for (int c = 0; c < W; ++c)
+                if (lane < w && c <= lane) L[p + lane][p + c] = crn[c];
+        } else if (p > 0 && (warp & 3) != 0) {
+            const int c0 = p + w, n = nb - c0, count = n * (n + 1) / 2;   // the panel before is a full one
+            for (int e = ((warp >> 2) * 3 + (warp & 3) - 1) * 32 + lane; e < count; e += 6 * 32) {
+                int r = (int)((sqrtf(8.f * e + 1.f) - 1.f) * 0.5f);
+                while ((r + 1) * (r + 2) / 2 <= e) ++r;
+                while (r * (r + 1) / 2 > e) --r;
+                apply(par ^ 1, W, c0 + r, c0 + e - r * (r + 1) / 2);
+            }
+        }
+        __syncthreads();
+        if (warp < 2) {
+            const int i = 32 * warp + lane;
+            if (i >= p + w && i < nb) {
+                T v[W];
+#pragma unroll
+                for (int c = 0; c < W; ++c) v[c] = c < w ? L[i][p + c] : T(0);
+#pragma unroll
+                for (int k = 0; k < W; ++k) {
+                    if (k >= w) break;
+                    const T tv = v[k] * s_inv[k];
+#pragma unroll
+                    for (int j = k + 1; j < W; ++j)
+                        if (j < w) v[j] = fma(-tv, L[p + j][p + k], v[j]);
+                    Ts[par][k][i] = tv;
+                    Vs[par][k][i] = v[k];
+                }
+#pragma unroll
+                for (int c = 0; c < W; ++c)
+                    if (c < w) L[i][p + c] = v[c];
+            }
+        }
+        __syncthreads();
+        {   // warp -> (column of the next panel, block of 32 rows)
+            const int j = p + w + (warp & 3), i = j + lane + 32 * (warp >> 2);
+            if (j < nb && i < nb) apply(par, w, i, j);
         }
         __syncthreads();
     }
@@ -303,42 +355,53 @@ __global__ void __launch_bounds__(256) tile_inverse_kernel(const T* D, int n, T*
 // Panel of the block Cholesky: P <- P L^{-T} for the m x nb panel P (ld ldp) under
 // the factored diagonal tile L (nb x nb lower, ld ldl): every row x solves
 // L x^T = p^T by column-oriented forward substitution, x_j = x_j / L[j][j], then
-// x_l -= L[l][j] x_j for l > j.  One warp per row, lane l holding x_l and x_{l+32}
-// in registers, x_j passed by one shuffle per column, so the chain of a column is
-// one product, one shuffle and one FMA; eight rows per CTA share L in shared memory.
-constexpr int kTrsmRows = 8;
+// x_l -= L[l][j] x_j for l > j.  Eight lanes per row, lane s holding x_s, x_{s+8}, ... in
+// registers and four rows per warp: a column costs one product for four rows and only the
+// FMAs right of it (a warp per row spends a product and two FMAs per column on one row,
+// most lanes idle; FP64-bound either way), x_j passed by one shuffle.  L is shared by the
+// CTA's rows.
+constexpr int kTrsmWarps = 4;            // 150 CTAs, a warp per quarter of an SM, for 2400 rows
+constexpr int kTrsmRows = 4 * kTrsmWarps;
 template <class T>
-__global__ void __launch_bounds__(32 * kTrsmRows) trsm_panel_kernel(const T* Lkk, int ldl, T* P, int ldp, int m,
-                                                                  int nb) {
-    __shared__ T L[kTile][kTile + 1];
+__global__ void __launch_bounds__(32 * kTrsmWarps) trsm_panel_kernel(const T* Lkk, int ldl, T* P, int ldp, int m, int nb) {
+    __shared__ T L[kTile][kTile + 1];        // L[j][l]: column j of the factor
     __shared__ T rd[kTile];
-    const int tid = threadIdx.x, lane = tid & 31;
+    constexpr int kPer = kTile / 8;
+    const int tid = threadIdx.x, lane = tid & 31, s = lane & 7;
     for (int e = tid; e < nb * nb; e += blockDim.x) {
         const int i = e % nb, j = e / nb;
-        L[i][j] = (i >= j) ? Lkk[i + (long long)j * ldl] : T(0);
+        if (i >= j) L[j][i] = Lkk[i + (long long)j * ldl];
     }
     __syncthreads();
     for (int i = tid; i < nb; i += blockDim.x) rd[i] = T(1) / L[i][i];
     __syncthreads();
-    const int row = blockIdx.x * kTrsmRows + (tid >> 5);
-    if (row >= m) return;   // warp-uniform; no barrier follows
-    T* pr = P + row;
-    const int l1 = lane + 32;
-    T x0 = lane < nb ? pr[(long long)lane * ldp] : T(0);
-    T x1 = l1 < nb ? pr[(long long)l1 * ldp] : T(0);
-    for (int j = 0; j < nb; ++j) {
-        T v = j < 32 ? x0 : x1;
-        if (lane == (j & 31)) {
-            v *= rd[j];
-            if (j < 32) x0 = v;
-            else x1 = v;
+    // lanes of one eighth of a warp hold four consecutive rows, so that a column's loads
+    // and stores touch whole sectors across the warp's quarters
+    const int row = blockIdx.x * kTrsmRows + (tid >> 5) * 4 + (lane >> 3);
+    const bool live = row < m;
+    T* pr = P + (live ? row : 0);
+    T x[kPer];
+#pragma unroll
+    for (int u = 0; u < kPer; ++u) x[u] = (live && s + 8 * u < nb) ? pr[(long long)(s + 8 * u) * ldp] : T(0);
+#pragma unroll
+    for (int uj = 0; uj < kPer; ++uj) {
+        for (int sj = 0; sj < 8; ++sj) {
+            const int j = 8 * uj + sj;
+            if (j >= nb) break;
+            const T v = x[uj] * rd[j];
+            if (s == sj) x[uj] = v;
+            const T xj = __shfl_sync(0xffffffffu, v, (lane & 24) + sj);
+#pragma unroll
+            for (int u = uj; u < kPer; ++u) {
+                const int l = s + 8 * u;
+                if (l > j && l < nb) x[u] = fma(-L[j][l], xj, x[u]);
+            }
         }
-        const T xj = __shfl_sync(0xffffffffu, v, j & 31);
-        if (lane > j && lane < nb) x0 = fma(-L[lane][j], xj, x0);
-        if (l1 > j && l1 < nb) x1 = fma(-L[l1][j], xj, x1);
     }
-    if (lane < nb) pr[(long long)lane * ldp] = x0;
-    if (l1 < nb) pr[(long long)l1 * ldp] = x1;
+    if (live)
+#pragma unroll
+        for (int u = 0; u < kPer; ++u)
+            if (s + 8 * u < nb) pr[(long long)(s + 8 * u) * ldp] = x[u];
 }
 
 template <class T>
@@ -771,17 +834,24 @@ msp_status factorize(Basis& B, const double* Hs64p, long long total, double shif
                     ts.nr = m;
                     ts.nb = nb;
                     steps.push_back(ts);
+                    if (kt > 0) steps.back().wait_ev = 3;   // this tile column's rows below the diagonal
                     steps.back().rec_ev = 0;          // panel kt final
-                    // trailing -= panel panel^T, with a lookahead of one tile: the next tile
-                    // column first, on the caller's stream (after the previous rest, which
-                    // also writes it), so that the next tile's factorisation and panel solve
-                    // run while the rest of the update runs on the side stream
+                    // trailing -= panel panel^T, with a lookahead of one tile: the next diagonal
+                    // tile first, on the caller's stream (after the previous rest, which also
+                    // writes it), so that its factorisation runs while the side stream updates
+                    // the rows below it, which the next panel solve waits for, and then the rest
                     const int nb1 = std::min(kTile, m);
-                    add_gemm(panel, n, panel, n, Dq + (r0 + nb) + (long long)(r0 + nb) * n, n, m, nb1, nb, T(-1), T(1),
+                    add_gemm(panel, n, panel, n, Dq + (r0 + nb) + (long long)(r0 + nb) * n, n, nb1, nb1, nb, T(-1), T(1),
                              false, true);
                     steps.back().wait_ev = 1;
                     steps.back().chain = true;
                     if (m > nb1) {
+                        add_gemm(panel + nb1, n, panel, n, Dq + (r0 + nb + nb1) + (long long)(r0 + nb) * n, n, m - nb1, nb1,
+                                 nb, T(-1), T(1), false, true);
+                        steps.back().stream = 1;
+                        steps.back().chain = true;
+                        steps.back().wait_ev = 0;
+                        steps.back().rec_ev = 3;
                         add_gemm(panel + nb1, n, panel + nb1, n, Dq + (r0 + nb + nb1) + (long long)(r0 + nb + nb1) * n, n,
                                  m - nb1, m - nb1, nb, T(-1), T(1), false, true, 1);
                         steps.back().stream = 1;
@@ -889,10 +959,10 @@ msp_status factorize(Basis& B, const double* Hs64p, long long total, double shif
         // before the stream, so that on every way out the stream is synchronised first
         OzakiWork ozw_side;
         // side stream of the trailing updates and its events (panel final, rest of a
-        // trailing update done, join), released on every way out
+        // trailing update done, join, next tile column done), released on every way out
         struct SideStream {
             cudaStream_t st = nullptr;
-            cudaEvent_t ev[3] = {nullptr, nullptr, nullptr};
+            cudaEvent_t ev[4] = {nullptr, nullptr, nullptr, nullptr};
             ~SideStream() {
                 if (st) cudaStreamSynchronize(st);
                 for (cudaEvent_t e : ev)
@@ -948,7 +1018,7 @@ msp_status factorize(Basis& B, const double* Hs64p, long long total, double shif
                 potrf_tile_kernel<T><<<1, 256, 0, s>>>(st.ptr, st.ld, st.nb, fail.p);
                 count_launches(1);
             } else if (st.kind == 6) {
-                trsm_panel_kernel<T><<<(st.nr + kTrsmRows - 1) / kTrsmRows, 32 * kTrsmRows, 0, s>>>(
+                trsm_panel_kernel<T><<<(st.nr + kTrsmRows - 1) / kTrsmRows, 32 * kTrsmWarps, 0, s>>>(
                     st.src, st.lds, st.ptr, st.ld, st.nr, st.nb);
                 count_launches(1);
             } else if (st.kind == 7) {

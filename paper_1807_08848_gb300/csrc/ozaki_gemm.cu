@@ -183,19 +183,35 @@ __device__ __forceinline__ double op_elem(const OpView& v, int r, int k) {
     return v.base[(long long)r * v.sr + (long long)k * v.sk];
 }
 
+// The products of a launch: tables in device memory, or one product by value (the
+// trailing updates of the online factorisation are single products on its critical
+// path, where copying two tables costs as much as a kernel).
+struct OzTables {
+    const GemmDesc* descs;
+    const OzEntry* ents;
+    __device__ const GemmDesc& desc(int z) const { return descs[z]; }
+    __device__ const OzEntry& entry(int z) const { return ents[z]; }
+};
+struct OzSingle {
+    GemmDesc d;
+    OzEntry e;
+    __device__ const GemmDesc& desc(int) const { return d; }
+    __device__ const OzEntry& entry(int) const { return e; }
+};
+
 // Per row: the scale 2^e with 2^(e-1) <= max|x| < 2^e (1 for an all-zero row),
 // stored as the exponent e.  The magnitude of an FP64 value orders like its bit
 // pattern with the sign cleared, so the maximum is an integer maximum (no FP64
 // arithmetic: the FP64 pipe is the narrow one on this part).  One warp per row.
-template <bool IS_B>
-__global__ void __launch_bounds__(256) oz_scale_kernel(const GemmDesc* descs, const OzEntry* ents, bool tA, bool tB,
-                                                       int* scale_exp, int max_rows) {
-    const int z = blockIdx.y;
-    const GemmDesc D = descs[z];
-    const OpView v = IS_B ? view_b(D, tB) : view_a(D, tA);
+// The blocks of op(A)'s rows first, then those of op(B).
+template <class Batch>
+__global__ void __launch_bounds__(256) oz_scale_kernel(const __grid_constant__ Batch W, bool tA, bool tB, int* scale_exp, int blocks_a) {
+    const bool is_b = (int)blockIdx.x >= blocks_a;
+    const GemmDesc D = W.desc(blockIdx.y);
+    const OpView v = is_b ? view_b(D, tB) : view_a(D, tA);
     const int lane = threadIdx.x & 31;
-    const int r = blockIdx.x * 8 + (threadIdx.x >> 5);
-    if (r >= v.R || r >= max_rows) return;
+    const int r = (is_b ? (int)blockIdx.x - blocks_a : (int)blockIdx.x) * 8 + (threadIdx.x >> 5);
+    if (r >= v.R) return;
     unsigned long long mx = 0;
     for (int k = lane; k < v.K; k += 32) {
         const unsigned long long b = (unsigned long long)__double_as_longlong(op_elem(v, r, k)) & 0x7FFFFFFFFFFFFFFFull;
@@ -213,7 +229,8 @@ __global__ void __launch_bounds__(256) oz_scale_kernel(const GemmDesc* descs, co
             const int be = (int)(mx >> 52);
             e = be > 0 ? be - 1023 + 1 : -1022;   // subnormals lie below 2^-1022
         }
-        scale_exp[(IS_B ? ents[z].b_sc : ents[z].a_sc) + r] = e;
+        const OzEntry E = W.entry(blockIdx.y);
+        scale_exp[(is_b ? E.b_sc : E.a_sc) + r] = e;
     }
 }
 
@@ -223,11 +240,8 @@ __global__ void __launch_bounds__(256) oz_scale_kernel(const GemmDesc* descs, co
 // |a| / 2^e in (0, 1); slice t is bits 55-7t .. 49-7t of F with the sign of a --
 // the digits of the truncated base-128 expansion, found with integer operations.
 template <bool IS_B>
-__global__ void __launch_bounds__(256) oz_slice_kernel(const GemmDesc* descs, const OzEntry* ents, bool tA, bool tB,
-                                                       const int* scale_exp, __nv_bfloat16* out) {
-    const int z = blockIdx.y;
-    const GemmDesc D = descs[z];
-    const OzEntry E = ents[z];
+__device__ __forceinline__ void oz_slice(const GemmDesc& D, const OzEntry& E, bool tA, bool tB, const int* scale_exp,
+                                         __nv_bfloat16* out, unsigned block, unsigned blocks) {
     const OpView v = IS_B ? view_b(D, tB) : view_a(D, tA);
     const int RT = IS_B ? kTN : kTM;
     const int tiles = IS_B ? E.rtb : E.rta;
@@ -237,7 +251,7 @@ __global__ void __launch_bounds__(256) oz_slice_kernel(const GemmDesc* descs, co
     // per_slice < 2^31 (checked on the host): the tiled index fits 32 bits
     const unsigned slabs_u = (unsigned)E.slabs;
     const unsigned blk = (unsigned)(RT * kSlabK);   // one (tile, slab) block of one slice
-    for (unsigned e = blockIdx.x * blockDim.x + threadIdx.x; e < (unsigned)per_slice; e += gridDim.x * blockDim.x) {
+    for (unsigned e = block * blockDim.x + threadIdx.x; e < (unsigned)per_slice; e += blocks * blockDim.x) {
         // e = [tile][slab][row group][k core][row][k]
         const int kk = (int)(e & 7);
         const int rr = (int)((e >> 3) & 7);
@@ -268,24 +282,35 @@ __global__ void __launch_bounds__(256) oz_slice_kernel(const GemmDesc* descs, co
     }
 }
 
+// the blocks of op(A) first, then those of op(B)
+template <class Batch>
+__global__ void __launch_bounds__(256) oz_slice_kernel(const __grid_constant__ Batch W, bool tA, bool tB, const int* scale_exp,
+                                                       __nv_bfloat16* out, unsigned blocks_a) {
+    const GemmDesc D = W.desc(blockIdx.y);
+    const OzEntry E = W.entry(blockIdx.y);
+    if (blockIdx.x < blocks_a) oz_slice<false>(D, E, tA, tB, scale_exp, out, blockIdx.x, blocks_a);
+    else oz_slice<true>(D, E, tA, tB, scale_exp, out, blockIdx.x - blocks_a, gridDim.x - blocks_a);
+}
+
 // ------------------------------------------------------------------ MMA
+template <class Batch>
 struct OzArgs {
-    const GemmDesc* descs;
-    const OzEntry* ents;
+    Batch batch;
     const __nv_bfloat16* slices;
     long long n_slices;        // elements of the slice buffer (bounds of every bulk copy)
     const int* scale_exp;      // power-of-two scale exponents of the rows / columns
     int* err;
 };
 
-__global__ void __launch_bounds__(kOzThreads, kCtasPerSm) oz_mma_kernel(OzArgs A) {
+template <class Batch>
+__global__ void __launch_bounds__(kOzThreads, kCtasPerSm) oz_mma_kernel(const __grid_constant__ OzArgs<Batch> A) {
     extern __shared__ __align__(1024) unsigned char oz_smem[];
     __shared__ __align__(8) unsigned long long full[kStages], empty[kStages], accb[kAccBufs], accfree[kAccBufs];
     __shared__ unsigned s_tmem;
     __shared__ int s_fail;
     const int z = blockIdx.z;
-    const GemmDesc D = A.descs[z];
-    const OzEntry E = A.ents[z];
+    const GemmDesc D = A.batch.desc(z);
+    const OzEntry E = A.batch.entry(z);
     const int tm = blockIdx.x % E.rta, tn = blockIdx.x / E.rta;
     if (blockIdx.x >= E.rta * E.rtb) return;                       // whole CTA: uniform
     if (D.lower && tn * kTN > tm * kTM + kTM - 1) return;          // tile above the diagonal
@@ -553,46 +578,44 @@ msp_status ozaki_gemm_batched(const std::vector<GemmDesc>& h, const GemmDesc* d_
         max_b_elems = std::max(max_b_elems, b_el / kSlices);
     }
     const size_t ent_words = sizeof(OzEntry) / sizeof(long long) * (size_t)batch;
-    const bool grow = (long long)w.slices.n < sl || (long long)w.scales.n < sc || w.ents.n < ent_words;
+    const bool one = batch == 1;
+    const bool grow = (long long)w.slices.n < sl || (long long)w.scales.n < sc || (!one && w.ents.n < ent_words);
     // products of earlier calls may still be queued on the stream and read these
     // buffers: they finish before a buffer is given up for a larger one
     if (grow) MSP_CUDA(cudaStreamSynchronize(s));
     if ((long long)w.slices.n < sl) MSP_TRY(w.slices.alloc((size_t)sl, s));
     if ((long long)w.scales.n < sc) MSP_TRY(w.scales.alloc((size_t)sc, s));
-    if (w.ents.n < ent_words) MSP_TRY(w.ents.alloc(ent_words, s));
+    if (!one && w.ents.n < ent_words) MSP_TRY(w.ents.alloc(ent_words, s));
     if (!w.err.p) {
         MSP_TRY(w.err.alloc(1, s));
         MSP_CUDA(cudaMemsetAsync(w.err.p, 0, sizeof(int), s));
     }
-    MSP_CUDA(cudaMemcpyAsync(w.ents.p, ents.data(), sizeof(OzEntry) * batch, cudaMemcpyHostToDevice, s));
+    if (!one) MSP_CUDA(cudaMemcpyAsync(w.ents.p, ents.data(), sizeof(OzEntry) * batch, cudaMemcpyHostToDevice, s));
     const OzEntry* d_ents = reinterpret_cast<const OzEntry*>(w.ents.p);
     __nv_bfloat16* slices = reinterpret_cast<__nv_bfloat16*>(w.slices.p);
-    for (int z0 = 0; z0 < batch; z0 += 65535) {
-        const int nb = std::min(65535, batch - z0);
-        oz_scale_kernel<false><<<dim3((max_rows_a + 7) / 8, nb), 256, 0, s>>>(d_dev + z0, d_ents + z0, transA, transB,
-                                                                              w.scales.p, max_rows_a);
-        oz_scale_kernel<true><<<dim3((max_rows_b + 7) / 8, nb), 256, 0, s>>>(d_dev + z0, d_ents + z0, transA, transB,
-                                                                             w.scales.p, max_rows_b);
-        const int ga = (int)std::min<long long>((max_a_elems + 255) / 256, 4096);
-        const int gb = (int)std::min<long long>((max_b_elems + 255) / 256, 4096);
-        oz_slice_kernel<false><<<dim3(std::max(ga, 1), nb), 256, 0, s>>>(d_dev + z0, d_ents + z0, transA, transB,
-                                                                         w.scales.p, slices);
-        oz_slice_kernel<true><<<dim3(std::max(gb, 1), nb), 256, 0, s>>>(d_dev + z0, d_ents + z0, transA, transB,
-                                                                        w.scales.p, slices);
-        count_launches(4);
-        OzArgs a{};
-        a.descs = d_dev + z0;
-        a.ents = d_ents + z0;
+    const int ra = (max_rows_a + 7) / 8, rb = (max_rows_b + 7) / 8;
+    const int ga = std::max(1, (int)std::min<long long>((max_a_elems + 255) / 256, 4096));
+    const int gb = std::max(1, (int)std::min<long long>((max_b_elems + 255) / 256, 4096));
+    auto launch = [&](auto tables, int nb) -> msp_status {
+        using Batch = decltype(tables);
+        const int smem = kStages * (int)kStageBytes;
+        MSP_CUDA(cudaFuncSetAttribute(oz_mma_kernel<Batch>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+        oz_scale_kernel<Batch><<<dim3(ra + rb, nb), 256, 0, s>>>(tables, transA, transB, w.scales.p, ra);
+        oz_slice_kernel<Batch><<<dim3(ga + gb, nb), 256, 0, s>>>(tables, transA, transB, w.scales.p, slices, (unsigned)ga);
+        OzArgs<Batch> a{};
+        a.batch = tables;
         a.slices = slices;
         a.n_slices = (long long)w.slices.n;
         a.scale_exp = w.scales.p;
         a.err = w.err.p;
-        const int smem = kStages * (int)kStageBytes;
-        MSP_CUDA(cudaFuncSetAttribute(oz_mma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-        oz_mma_kernel<<<dim3(max_tiles, 1, nb), kOzThreads, smem, s>>>(a);
-        count_launches(1);
+        oz_mma_kernel<Batch><<<dim3(max_tiles, 1, nb), kOzThreads, smem, s>>>(a);
+        count_launches(3);
         MSP_CUDA(cudaGetLastError());
-    }
+        return MSP_OK;
+    };
+    if (one) return launch(OzSingle{h[0], ents[0]}, 1);
+    for (int z0 = 0; z0 < batch; z0 += 65535)
+        MSP_TRY(launch(OzTables{d_dev + z0, d_ents + z0}, std::min(65535, batch - z0)));
     return MSP_OK;
 }
 
