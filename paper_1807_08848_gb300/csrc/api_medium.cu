@@ -4,6 +4,7 @@
 #include <algorithm>
 #include <atomic>
 #include <cstring>
+#include <mutex>
 #include <numeric>
 
 
@@ -53,6 +54,66 @@ int num_sms() {
 }
 
 void wait_for_device() { cudaDeviceSynchronize(); }
+
+cudaError_t pool_alloc(void** p, size_t bytes, cudaStream_t s) {
+    struct DevicePool {
+        cudaMemPool_t pool = nullptr;
+        size_t total = 0;
+    };
+    static std::mutex mu;
+    static std::vector<DevicePool> pools;   // per device; never destroyed (the driver may be gone by then)
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    DevicePool d;
+    {
+        std::lock_guard<std::mutex> lock(mu);
+        if ((int)pools.size() <= dev) pools.resize(dev + 1);
+        if (!pools[dev].pool) {
+            size_t free_b = 0, total_b = 0;
+            e = cudaMemGetInfo(&free_b, &total_b);
+            if (e != cudaSuccess) return e;
+            cudaMemPoolProps props{};
+            props.allocType = cudaMemAllocationTypePinned;
+            props.handleTypes = cudaMemHandleTypeNone;
+            props.location.type = cudaMemLocationTypeDevice;
+            props.location.id = dev;
+            cudaMemPool_t pool = nullptr;
+            e = cudaMemPoolCreate(&pool, &props);
+            if (e != cudaSuccess) return e;
+            uint64_t keep = (uint64_t)total_b / 8;
+            e = cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
+            if (e != cudaSuccess) {
+                cudaMemPoolDestroy(pool);
+                return e;
+            }
+            pools[dev].pool = pool;
+            pools[dev].total = total_b;
+        }
+        d = pools[dev];
+    }
+    if (bytes > d.total) return cudaErrorMemoryAllocation;
+    for (int attempt = 0; attempt < 2; ++attempt) {
+        *p = nullptr;
+        e = cudaMallocFromPoolAsync(p, bytes, d.pool, s);
+        if (e == cudaSuccess) {
+            // a stream-ordered allocation may also report its failure through the last-error
+            // state instead of its return value
+            const cudaError_t late = cudaGetLastError();
+            if (late != cudaSuccess) {
+                if (*p) cudaFreeAsync(*p, s);
+                *p = nullptr;
+                e = late;
+            }
+        } else {
+            (void)cudaGetLastError();
+        }
+        if (e != cudaErrorMemoryAllocation || attempt == 1) break;
+        cudaStreamSynchronize(s);           // pending frees complete, then the pool gives all it holds back
+        cudaMemPoolTrimTo(d.pool, 0);
+    }
+    return e;
+}
 
 static msp_status need_device() {
     int n = 0;

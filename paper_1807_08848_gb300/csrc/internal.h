@@ -38,6 +38,13 @@ msp_status cuda_fail(cudaError_t e, const char* what, const char* file, int line
 // without iteration counts, a snapshot copy) may still be running.
 void wait_for_device();
 
+// Stream-ordered allocation from the library's pool of the current device (freed with
+// cudaFree).  The default pool gives its free memory back at every synchronisation, and
+// mapping it again took a third of a pass that builds a new medium; this pool keeps up to
+// an eighth of the device's memory between calls, gives the rest back, and is emptied
+// before a request is refused.
+cudaError_t pool_alloc(void** p, size_t bytes, cudaStream_t s);
+
 // Stream-ordered device buffer owned by a handle.
 template <class T>
 struct DevBuf {
@@ -45,24 +52,12 @@ struct DevBuf {
     size_t n = 0;
     // A request beyond the device's whole memory is refused before the call (free
     // memory is no test: the stream-ordered pool may serve a request from memory it
-    // holds); a stream-ordered allocation may also report its failure through the
-    // last-error state instead of its return value, so that is read (and cleared)
-    // right after.
+    // holds).
     msp_status alloc(size_t count, cudaStream_t s) {
         free_now();
         if (count == 0) return MSP_OK;
         const size_t bytes = count * sizeof(T);
-        size_t free_b = 0, total_b = 0;
-        cudaError_t e = cudaMemGetInfo(&free_b, &total_b);
-        if (e == cudaSuccess && bytes > total_b) e = cudaErrorMemoryAllocation;
-        if (e == cudaSuccess) e = cudaMallocAsync((void**)&p, bytes, s);
-        if (e == cudaSuccess) {
-            const cudaError_t late = cudaGetLastError();
-            if (late != cudaSuccess) {
-                if (p) cudaFreeAsync(p, s);
-                e = late;
-            }
-        }
+        const cudaError_t e = pool_alloc((void**)&p, bytes, s);
         if (e != cudaSuccess) {
             p = nullptr;
             set_error(std::string("device allocation of ") + std::to_string(bytes) + " bytes failed: " +

@@ -990,8 +990,29 @@ msp_status online_solve_map(const Basis& Bs, const double* phi, int batch, doubl
     const int N = Bs.N, n4 = 4 * N, Np = Bs.Np, np = (int)Bs.patches.size();
     const long long nn = (long long)(N + 1) * (N + 1);
     MapWork own{};
+    DevBuf<unsigned char> block;   // the call's own buffers, one stream-ordered allocation
     if (!work) {
-        MSP_TRY(map_work_alloc(Bs, std::min(batch, kMaxBatch), own));
+        const size_t B = (size_t)std::max(1, std::min(batch, kMaxBatch));
+        const size_t sizes[6] = {sizeof(float) * n4 * B,
+                                 sizeof(float) * (size_t)std::max(Np, 1) * B,
+                                 sizeof(double) * (size_t)std::max(Bs.n_slots, 1) * B,
+                                 sizeof(float) * (size_t)tc_b_floats((int)B, n4),
+                                 sizeof(float) * (size_t)tc_b_floats((int)B, n4),
+                                 sizeof(int)};
+        size_t at[6], total = 0;
+        for (int i = 0; i < 6; ++i) {
+            at[i] = total;
+            total += (sizes[i] + 255) / 256 * 256;
+        }
+        MSP_TRY(block.alloc(total, s));
+        own.phi32 = reinterpret_cast<float*>(block.p + at[0]);
+        own.c32 = reinterpret_cast<float*>(block.p + at[1]);
+        own.e = reinterpret_cast<double*>(block.p + at[2]);
+        own.b_hi = reinterpret_cast<float*>(block.p + at[3]);
+        own.b_lo = reinterpret_cast<float*>(block.p + at[4]);
+        own.err = reinterpret_cast<int*>(block.p + at[5]);
+        own.cap = (int)B;
+        MSP_CUDA(cudaMemsetAsync(own.err, 0, sizeof(int), s));
         work = &own;
     }
     msp_status st = MSP_OK;
@@ -1013,7 +1034,8 @@ msp_status online_solve_map(const Basis& Bs, const double* phi, int batch, doubl
             ta.n_slabs = tc_slabs(n4);
             ta.c = work->c32;
             ta.err = work->err;
-            MSP_TRY(tc_map_gemm(ta, s));
+            st = tc_map_gemm(ta, s);
+            if (st != MSP_OK) break;
         } else {
             const int tiles = ((Np + 63) / 64) * ((B + 63) / 64);
             map_gemm_kernel<<<tiles, 256, 0, s>>>(Bs.G32.p, work->phi32, work->c32, Np, n4, B);
@@ -1035,8 +1057,7 @@ msp_status online_solve_map(const Basis& Bs, const double* phi, int batch, doubl
     }
     if (work == &own) {
         if (st == MSP_OK) st = map_work_check(own, s);
-        cudaStreamSynchronize(s);
-        map_work_free(own);
+        cudaStreamSynchronize(s);   // the work block is released on return
     }
     return st;
 }
