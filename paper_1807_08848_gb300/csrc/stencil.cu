@@ -5,11 +5,12 @@
 // read from and written to HBM once, the face coefficients of a patch are staged
 // once per CTA and shared by all its samples.
 //
-// One CTA per (patch, chunk of samples).  The patch's faces go to shared memory
-// with ordinary loads; the sample tiles arrive by one bulk asynchronous copy each
-// (cp.async.bulk, the TMA engine), double-buffered and completed on an mbarrier,
-// so the next tile is in flight while the current one is computed.  Every
-// mbarrier wait is bounded: on timeout the CTA raises *err and leaves.
+// The sample tiles arrive by one bulk asynchronous copy each (cp.async.bulk, the TMA
+// engine), completed on mbarriers, several ahead of the one that is computed.  FP32: one
+// persistent CTA per resident slot takes a contiguous range of (patch, sample) tiles, every
+// thread the same strips of nodes in each with their faces in registers.  FP64 (twice the
+// bytes): one CTA per (patch, chunk of samples), double-buffered, the faces read through
+// the L1.  Every mbarrier wait is bounded: on timeout the CTA raises *err and leaves.
 #include "internal.h"
 
 namespace msp {
@@ -61,6 +62,120 @@ __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, unsigned by
                  : "memory");
 }
 
+// FP32, persistent.  Thread t takes strip t of every tile: four consecutive nodes (a quad)
+// of R consecutive rows, and keeps the strip's faces in registers until its CTA moves on
+// to the next patch; a node then costs the loads of its own quad (the rows above and
+// below are the strip's neighbours) and its horizontal neighbours from shared memory.
+// Bound: HBM (each tile read and written once); with the faces in shared memory, two more
+// rows per quad and two barriers per tile the 256 x 96 tiles of 97 x 100 took 513 us
+// against 265 us of copying.
+template <int R>
+__global__ void __launch_bounds__(512) stencil_stream_kernel(StencilArgs A, int nb_buf) {
+    constexpr int kMaxBuf = 8;
+    extern __shared__ __align__(128) unsigned char st_smem[];
+    __shared__ __align__(8) unsigned long long bar[kMaxBuf];
+    __shared__ int s_fail;
+    float* xb = reinterpret_cast<float*>(st_smem);
+    const int H = A.H, P = A.P, N = A.N;
+    const long long tile = (long long)H * P, total = (long long)A.n_patches * A.S;
+    const long long t0 = total * blockIdx.x / gridDim.x, t1 = total * (blockIdx.x + 1) / gridDim.x;
+    const unsigned bytes = (unsigned)(tile * sizeof(float));
+    const float* X = static_cast<const float*>(A.x);
+    float* Y = static_cast<float*>(A.y);
+    const float* aE = static_cast<const float*>(A.aE);
+    const float* aN = static_cast<const float*>(A.aN);
+    auto issue = [&](long long t) {
+        const int b = (int)((t - t0) % nb_buf);
+        mbar_expect_tx(&bar[b], bytes);
+        bulk_g2s(xb + b * tile, X + t * tile, bytes, &bar[b]);
+    };
+    if (threadIdx.x == 0) {
+        for (int b = 0; b < nb_buf; ++b) mbar_init(&bar[b], 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        s_fail = 0;
+        for (long long t = t0; t < t1 && t < t0 + nb_buf; ++t) issue(t);
+    }
+    __syncthreads();
+    const int quads = P / 4;
+    const int c0 = (int)(threadIdx.x % quads) * 4, r0 = (int)(threadIdx.x / quads) * R;
+    float ce[R][4], cn[R + 1][4], cw[R];   // east faces, north faces of rows r0 - 1 .. r0 + R - 1, west face
+    unsigned rows_in = 0;                  // rows of the strip with interior nodes in this quad
+    unsigned cols_in = 0;                  // interior columns of the quad
+    int m = -1;
+    for (long long t = t0; t < t1; ++t) {
+        if ((int)(t / A.S) != m) {
+            m = (int)(t / A.S);
+            const PatchDev Pd = A.patches[m];
+            const int W = Pd.X1 - Pd.X0 + 1, Hm = Pd.Y1 - Pd.Y0 + 1;
+            rows_in = cols_in = 0;
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                if (c0 + k >= 1 && c0 + k < W - 1) cols_in |= 1u << k;
+#pragma unroll
+            for (int u = 0; u < R + 1; ++u) {
+                const int r = r0 + u - 1;
+                const float* gN = aN + (long long)(Pd.Y0 + r) * (N + 1) + Pd.X0;
+#pragma unroll
+                for (int k = 0; k < 4; ++k) cn[u][k] = (r >= 0 && r < Hm - 1 && c0 + k < W) ? gN[c0 + k] : 0.f;
+            }
+#pragma unroll
+            for (int u = 0; u < R; ++u) {
+                const int r = r0 + u;
+                const float* gE = aE + (long long)(Pd.Y0 + r) * N + Pd.X0;
+#pragma unroll
+                for (int k = 0; k < 4; ++k) ce[u][k] = (r < Hm && c0 + k < W - 1) ? gE[c0 + k] : 0.f;
+                cw[u] = (r < Hm && c0 > 0 && c0 - 1 < W - 1) ? gE[c0 - 1] : 0.f;
+                if (r >= 1 && r < Hm - 1 && cols_in) rows_in |= 1u << u;
+            }
+        }
+        const long long it = t - t0;
+        const int buf = (int)(it % nb_buf);
+        if (!mbar_wait(&bar[buf], (unsigned)((it / nb_buf) & 1))) s_fail = 1;
+        const float* x = xb + buf * tile;
+        float* yt = Y + t * tile;
+        if (r0 < H) {
+            float4 xd, xc, xu;
+            const int e = r0 * P + c0;
+            xd = r0 > 0 ? *reinterpret_cast<const float4*>(x + e - P) : make_float4(0.f, 0.f, 0.f, 0.f);
+            xc = *reinterpret_cast<const float4*>(x + e);
+#pragma unroll
+            for (int u = 0; u < R; ++u) {
+                if (r0 + u >= H) break;
+                const int eu = e + u * P;
+                xu = r0 + u + 1 < H ? *reinterpret_cast<const float4*>(x + eu + P) : make_float4(0.f, 0.f, 0.f, 0.f);
+                float out[4] = {0.f, 0.f, 0.f, 0.f};
+                if (rows_in >> u & 1u) {
+                    const float xl = c0 > 0 ? x[eu - 1] : 0.f, xr = c0 + 4 < P ? x[eu + 4] : 0.f;
+                    const float c[4] = {xc.x, xc.y, xc.z, xc.w}, up[4] = {xu.x, xu.y, xu.z, xu.w},
+                                dn[4] = {xd.x, xd.y, xd.z, xd.w};
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        const float left = k == 0 ? xl : c[k - 1], right = k == 3 ? xr : c[k + 1];
+                        const float fw = k == 0 ? cw[u] : ce[u][k - 1];
+                        const float v = ce[u][k] * (c[k] - right) + fw * (c[k] - left) + cn[u + 1][k] * (c[k] - up[k]) +
+                                        cn[u][k] * (c[k] - dn[k]);
+                        out[k] = (cols_in >> k & 1u) ? v : 0.f;
+                    }
+                }
+                *reinterpret_cast<float4*>(yt + eu) = make_float4(out[0], out[1], out[2], out[3]);
+                xd = xc;
+                xc = xu;
+            }
+        }
+        __syncthreads();   // every thread has waited for the tile and read it
+        if (s_fail) {
+            if (threadIdx.x == 0) {
+                atomicExch(A.err, 1);
+                // bounded waits for the copies issued into the other buffers before leaving
+                for (long long q = t + 1; q < t1 && q < t + nb_buf; ++q)
+                    mbar_wait(&bar[(q - t0) % nb_buf], (unsigned)(((q - t0) / nb_buf) & 1));
+            }
+            return;
+        }
+        if (threadIdx.x == 0 && t + nb_buf < t1) issue(t + nb_buf);
+    }
+}
+
 template <class T>
 struct Vec4;
 template <>
@@ -87,14 +202,12 @@ struct Vec4<double> {
     }
 };
 
-// FP32: the patch's faces and three sample tiles in shared memory (two copies in
-// flight while one tile is computed).  FP64 (twice the bytes): two sample tiles,
-// the faces read through L1.  Each thread computes four consecutive nodes of a
-// row from vector loads of shared memory and writes them with one vector store.
+// FP64, and FP32 tiles too wide for 512 strips: two sample tiles in shared memory, the
+// faces read through L1.  Each thread computes four consecutive nodes of a row from
+// vector loads of shared memory and writes them with one vector store.
 template <class T>
 __global__ void __launch_bounds__(512) stencil_apply_kernel(StencilArgs A) {
-    constexpr bool kFacesInSmem = sizeof(T) == 4;
-    constexpr int NB = kFacesInSmem ? 3 : 2;   // sample-tile buffers
+    constexpr int NB = 2;   // sample-tile buffers
     extern __shared__ __align__(128) unsigned char st_smem[];
     __shared__ __align__(8) unsigned long long bar[NB];
     __shared__ int s_fail;
@@ -107,9 +220,7 @@ __global__ void __launch_bounds__(512) stencil_apply_kernel(StencilArgs A) {
     const int W = Pd.X1 - Pd.X0 + 1, Hm = Pd.Y1 - Pd.Y0 + 1;
     const int H = A.H, P = A.P, N = A.N;
     const long long tile = (long long)H * P;
-    T* cE = reinterpret_cast<T*>(st_smem);   // east face of node (r, c): between c and c + 1
-    T* cN = cE + tile;                       // north face of node (r, c): between r and r + 1
-    T* xb = kFacesInSmem ? cN + tile : reinterpret_cast<T*>(st_smem);
+    T* xb = reinterpret_cast<T*>(st_smem);
     const T* aE = static_cast<const T*>(A.aE);
     const T* aN = static_cast<const T*>(A.aN);
     const T* X = static_cast<const T*>(A.x);
@@ -123,14 +234,6 @@ __global__ void __launch_bounds__(512) stencil_apply_kernel(StencilArgs A) {
         for (int b = 0; b < NB - 1 && s0 + b < s1; ++b) {
             mbar_expect_tx(&bar[b], bytes);
             bulk_g2s(xb + b * tile, X + base + (long long)(s0 + b) * tile, bytes, &bar[b]);
-        }
-    }
-    if constexpr (kFacesInSmem) {
-        for (long long e = threadIdx.x; e < tile; e += blockDim.x) {
-            const int r = (int)(e / P), c = (int)(e % P);
-            const int j = Pd.Y0 + r, i = Pd.X0 + c;
-            cE[e] = (r < Hm && c < W - 1) ? aE[(long long)j * N + i] : T(0);
-            cN[e] = (r < Hm - 1 && c < W) ? aN[(long long)j * (N + 1) + i] : T(0);
         }
     }
     __syncthreads();
@@ -167,24 +270,16 @@ __global__ void __launch_bounds__(512) stencil_apply_kernel(StencilArgs A) {
                 xd.load(x + e0 - P);
                 const T xl = c0 > 0 ? x[e0 - 1] : T(0);
                 const T xr = c0 + 4 < P ? x[e0 + 4] : T(0);
-                T cw;
-                if constexpr (kFacesInSmem) {
-                    ce.load(cE + e0);
-                    cn.load(cN + e0);
-                    cs.load(cN + e0 - P);
-                    cw = c0 > 0 ? cE[e0 - 1] : T(0);
-                } else {
-                    const T* gE = aE + (long long)(Pd.Y0 + r) * N + Pd.X0;
-                    const T* gN = aN + (long long)(Pd.Y0 + r) * (N + 1) + Pd.X0;
+                const T* gE = aE + (long long)(Pd.Y0 + r) * N + Pd.X0;
+                const T* gN = aN + (long long)(Pd.Y0 + r) * (N + 1) + Pd.X0;
 #pragma unroll
-                    for (int t = 0; t < 4; ++t) {
-                        const int c = c0 + t;
-                        ce.v[t] = (c < W - 1) ? __ldg(gE + c) : T(0);
-                        cn.v[t] = (c < W) ? __ldg(gN + c) : T(0);
-                        cs.v[t] = (c < W) ? __ldg(gN - (N + 1) + c) : T(0);
-                    }
-                    cw = c0 > 0 ? __ldg(gE + c0 - 1) : T(0);
+                for (int t = 0; t < 4; ++t) {
+                    const int c = c0 + t;
+                    ce.v[t] = (c < W - 1) ? __ldg(gE + c) : T(0);
+                    cn.v[t] = (c < W) ? __ldg(gN + c) : T(0);
+                    cs.v[t] = (c < W) ? __ldg(gN - (N + 1) + c) : T(0);
                 }
+                const T cw = c0 > 0 ? __ldg(gE + c0 - 1) : T(0);
 #pragma unroll
                 for (int t = 0; t < 4; ++t) {
                     const int c = c0 + t;
@@ -192,7 +287,7 @@ __global__ void __launch_bounds__(512) stencil_apply_kernel(StencilArgs A) {
                     const T right = t == 3 ? xr : xc.v[t + 1];
                     const T fw = t == 0 ? cw : ce.v[t - 1];
                     const T v = ce.v[t] * (xc.v[t] - right) + fw * (xc.v[t] - left) + cn.v[t] * (xc.v[t] - xu.v[t]) +
-                                cs.v[t] * (xc.v[t] - xd.v[t]);
+                                     cs.v[t] * (xc.v[t] - xd.v[t]);
                     out.v[t] = (c >= 1 && c < W - 1) ? v : T(0);
                 }
             }
@@ -200,6 +295,26 @@ __global__ void __launch_bounds__(512) stencil_apply_kernel(StencilArgs A) {
         }
         __syncthreads();
     }
+}
+
+template <class T>
+msp_status launch_apply(const StencilArgs& A, int grid, size_t smem, cudaStream_t s) {
+    MSP_CUDA(cudaFuncSetAttribute(stencil_apply_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    stencil_apply_kernel<T><<<grid, 512, smem, s>>>(A);
+    return MSP_OK;
+}
+
+template <int R>
+msp_status launch_stream(const StencilArgs& A, size_t tile_bytes, cudaStream_t s) {
+    // as many tile buffers as fit, at most eight
+    const int nb = (int)std::min<size_t>(8, (227 * 1024 - 256) / tile_bytes);
+    const size_t smem = nb * tile_bytes;
+    MSP_CUDA(cudaFuncSetAttribute(stencil_stream_kernel<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    int occ = 0;
+    MSP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, stencil_stream_kernel<R>, 512, smem));
+    const long long grid = std::min((long long)A.n_patches * A.S, (long long)num_sms() * std::max(1, occ));
+    stencil_stream_kernel<R><<<(int)grid, 512, smem, s>>>(A, nb);
+    return MSP_OK;
 }
 
 }  // namespace
@@ -256,11 +371,20 @@ msp_status apply_operator(const Medium& M, int S, int precision, const void* x, 
         MSP_CUDA(cudaEventRecord(e0, s));
     }
     if (f32) {
-        MSP_CUDA(cudaFuncSetAttribute(stencil_apply_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        stencil_apply_kernel<float><<<grid, 512, smem, s>>>(A);
+        // rows per strip: the fewest with which 512 threads cover a tile (at most 11.6k
+        // nodes, by the shared-memory bound above: 6 do unless the tile is very wide)
+        const size_t bytes = (size_t)rows * pitch * esz;
+        auto covers = [&](int r) { return (pitch / 4) * ((rows + r - 1) / r) <= 512; };
+        if (covers(1)) MSP_TRY(launch_stream<1>(A, bytes, s));
+        else if (covers(2)) MSP_TRY(launch_stream<2>(A, bytes, s));
+        else if (covers(3)) MSP_TRY(launch_stream<3>(A, bytes, s));
+        else if (covers(4)) MSP_TRY(launch_stream<4>(A, bytes, s));
+        else if (covers(5)) MSP_TRY(launch_stream<5>(A, bytes, s));
+        else if (covers(6)) MSP_TRY(launch_stream<6>(A, bytes, s));
+        else if (covers(8)) MSP_TRY(launch_stream<8>(A, bytes, s));
+        else MSP_TRY(launch_apply<float>(A, grid, 2 * bytes, s));
     } else {
-        MSP_CUDA(cudaFuncSetAttribute(stencil_apply_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        stencil_apply_kernel<double><<<grid, 512, smem, s>>>(A);
+        MSP_TRY(launch_apply<double>(A, grid, smem, s));
     }
     count_launches(1);
     MSP_CUDA(cudaGetLastError());
