@@ -18,7 +18,7 @@
 // factor kernel keeps W_i = S_i^{-1} for every node (one CTA per patch, the
 // n_v x n_v block in registers over a 16 x 16 thread grid).
 //
-// The solve kernel takes one CTA per (patch, 32 samples), one sample per lane,
+// The solve kernel takes one CTA per (patch, 16 samples), one sample per lane,
 // and refines in FP64: r = b - A f (FP64, sweeping a three-node window of f
 // through shared memory), forward y_i = W_i (r_i - L_i y_{i-1}), backward
 // x_i = y_i - W_i U_i x_{i+1}, f += x.  With the FP64 factor one pass solves
@@ -34,8 +34,9 @@ namespace msp {
 namespace {
 
 constexpr int kKdThreads = 256;
-constexpr int kKdG = 32;        // samples per CTA of the solve, one per lane
-constexpr int kKdLd = 33;       // padded row stride of the [velocity][sample] tiles
+constexpr int kKdG = 16;        // samples per CTA of the solve, one per lane of a half-warp
+constexpr int kKdHalves = kKdThreads / kKdG;   // half-warps of a CTA
+constexpr int kKdLd = 17;       // padded row stride of the [velocity][sample] tiles
 constexpr int kKdMaxNv = 128;
 constexpr int kKdMaxPasses = 16;   // corrections per solve at most
 
@@ -180,15 +181,19 @@ __device__ __forceinline__ double kd_datum(const KdArgs& A, int m, int s, int l,
     return (t & 1) ? z.y : z.x;
 }
 
-// One CTA per (patch, 32 samples); warp w owns the velocity rows w + 8 j (j < RJ),
-// lane = sample.  y (in T) shares the f layout: [node][velocity][sample]; it holds
-// the residual after the residual sweep and y_i after the forward sweep.
+// One CTA per (patch, kKdG samples); half-warp h owns the velocity rows h + 16 j (j < RJ),
+// lane of the half = sample, so that an FP64 instruction (as long for 16 lanes as for 32)
+// carries two rows and a patch spreads over twice as many CTAs: with 32 samples each the
+// 192 CTAs of 64 patches x 96 samples gave 40 of 152 SMs two and the others one (8193
+// nodes, 64 velocities: offline + online 127.4 ms, now 114.2).  y (in T) shares the f
+// layout: [node][velocity][sample]; it holds the residual after the residual sweep and y_i
+// after the forward sweep.
 template <class T, int RJ>
 __global__ void __launch_bounds__(kKdThreads) kd_solve_kernel(KdArgs A, const T* W, T* y) {
     extern __shared__ __align__(16) unsigned char kd_dyn[];
     __shared__ double red[32];
     __shared__ double c_v[kKdMaxNv], c_a[kKdMaxNv], c_d[kKdMaxNv];
-    const int nv = A.n_v, m = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int nv = A.n_v, m = blockIdx.x, lane = threadIdx.x & (kKdG - 1), half = threadIdx.x / kKdG;
     const KPatchDev P = A.patches[m];
     const int nn = P.X1 - P.X0 + 1;
     const int s = blockIdx.y * kKdG + lane;
@@ -217,7 +222,7 @@ __global__ void __launch_bounds__(kKdThreads) kd_solve_kernel(KdArgs A, const T*
             for (int i = 0; i < nn; ++i) {
 #pragma unroll
                 for (int j = 0; j < RJ; ++j) {
-                    const int l = warp + 8 * j;
+                    const int l = half + kKdHalves * j;
                     if (l >= nv || !live) continue;
                     const double r = kd_identity(i, nn, c_v[l]) ? kd_datum(A, m, s, l, c_v[l]) : 0.0;
                     rmax = fmax(rmax, fabs(r));
@@ -230,7 +235,7 @@ __global__ void __launch_bounds__(kKdThreads) kd_solve_kernel(KdArgs A, const T*
                 double* dst = Fw + (node % 3) * nv * kKdLd;
 #pragma unroll
                 for (int j = 0; j < RJ; ++j) {
-                    const int l = warp + 8 * j;
+                    const int l = half + kKdHalves * j;
                     if (l < nv) dst[l * kKdLd + lane] = live ? A.f[fidx(node, l)] : 0.0;
                 }
             };
@@ -243,7 +248,7 @@ __global__ void __launch_bounds__(kKdThreads) kd_solve_kernel(KdArgs A, const T*
                 const double* Fn = Fw + ((i + 1) % 3) * nv * kKdLd;   // node i+1 (unused at i = nn-1)
 #pragma unroll
                 for (int j = 0; j < RJ; ++j) {
-                    const int l = warp + 8 * j;
+                    const int l = half + kKdHalves * j;
                     if (l >= nv) continue;
                     const double vl = c_v[l], fi = Fi[l * kKdLd + lane];
                     double r, scale;
@@ -286,7 +291,7 @@ __global__ void __launch_bounds__(kKdThreads) kd_solve_kernel(KdArgs A, const T*
         for (int i = 0; i < nn; ++i) {
 #pragma unroll
             for (int j = 0; j < RJ; ++j) {
-                const int l = warp + 8 * j;
+                const int l = half + kKdHalves * j;
                 if (l >= nv) continue;
                 T z = live ? y[fidx(i, l)] : T(0);
                 if (i > 0 && c_v[l] > 0.0) z += (T)c_a[l] * yprev[j];
@@ -301,13 +306,13 @@ __global__ void __launch_bounds__(kKdThreads) kd_solve_kernel(KdArgs A, const T*
                 const T zk = Z[k * kKdLd + lane];
 #pragma unroll
                 for (int j = 0; j < RJ; ++j) {
-                    const int l = warp + 8 * j;
+                    const int l = half + kKdHalves * j;
                     if (l < nv) acc[j] += __ldg(Wi + (long long)l * nv + k) * zk;
                 }
             }
 #pragma unroll
             for (int j = 0; j < RJ; ++j) {
-                const int l = warp + 8 * j;
+                const int l = half + kKdHalves * j;
                 if (l >= nv) continue;
                 yprev[j] = acc[j];
                 if (live) y[fidx(i, l)] = acc[j];
@@ -325,7 +330,7 @@ __global__ void __launch_bounds__(kKdThreads) kd_solve_kernel(KdArgs A, const T*
             if (i < nn - 1) {
 #pragma unroll
                 for (int j = 0; j < RJ; ++j) {
-                    const int l = warp + 8 * j;
+                    const int l = half + kKdHalves * j;
                     if (l < nneg) Z[l * kKdLd + lane] = (T)c_a[l] * xnext[j];
                 }
                 __syncthreads();
@@ -334,7 +339,7 @@ __global__ void __launch_bounds__(kKdThreads) kd_solve_kernel(KdArgs A, const T*
                     const T zk = Z[k * kKdLd + lane];
 #pragma unroll
                     for (int j = 0; j < RJ; ++j) {
-                        const int l = warp + 8 * j;
+                        const int l = half + kKdHalves * j;
                         if (l < nv) x[j] += __ldg(Wi + (long long)l * nv + k) * zk;
                     }
                 }
@@ -342,7 +347,7 @@ __global__ void __launch_bounds__(kKdThreads) kd_solve_kernel(KdArgs A, const T*
             }
 #pragma unroll
             for (int j = 0; j < RJ; ++j) {
-                const int l = warp + 8 * j;
+                const int l = half + kKdHalves * j;
                 if (l >= nv) continue;
                 if (live) {
                     const long long q = fidx(i, l);
@@ -361,11 +366,11 @@ __global__ void __launch_bounds__(kKdThreads) kd_solve_kernel(KdArgs A, const T*
         for (int i = 0; i < nk_nodes; ++i) {
 #pragma unroll
             for (int j = 0; j < RJ; ++j) {
-                const int l = warp + 8 * j;
+                const int l = half + kKdHalves * j;
                 if (l < nv) out[(long long)i * nv + l] = A.f[fidx(i0 + i, l)];
             }
         }
-        if (warp == 0) {
+        if (half == 0) {
             A.stats[2 * ((long long)m * A.S + s) + 0] = pass;
             A.stats[2 * ((long long)m * A.S + s) + 1] = converged ? 0 : 1;
         }
@@ -403,11 +408,10 @@ msp_status launch_solve(const KdArgs& A, int M, const T* W, T* y, cudaStream_t s
 template <class T>
 msp_status solve(const KdArgs& A, int M, const T* W, T* y, cudaStream_t s) {
     const int nv = A.n_v;
-    if (nv <= 8) return launch_solve<T, 1>(A, M, W, y, s);
-    if (nv <= 16) return launch_solve<T, 2>(A, M, W, y, s);
-    if (nv <= 32) return launch_solve<T, 4>(A, M, W, y, s);
-    if (nv <= 64) return launch_solve<T, 8>(A, M, W, y, s);
-    return launch_solve<T, 16>(A, M, W, y, s);
+    if (nv <= 16) return launch_solve<T, 1>(A, M, W, y, s);
+    if (nv <= 32) return launch_solve<T, 2>(A, M, W, y, s);
+    if (nv <= 64) return launch_solve<T, 4>(A, M, W, y, s);
+    return launch_solve<T, 8>(A, M, W, y, s);
 }
 
 }  // namespace
