@@ -15,8 +15,7 @@
 // nonsingular M-matrix (weakly row-diagonally dominant since the gain row sums
 // equal the loss rates, strictly at the identity rows), so neither the block
 // elimination nor the Gauss-Jordan inversion of each S_i needs pivoting.  The
-// factor kernel keeps W_i = S_i^{-1} for every node (one CTA per patch, the
-// n_v x n_v block in registers over a 16 x 16 thread grid).
+// factor keeps W_i = S_i^{-1} for every node, formed in halves of the velocities.
 //
 // The solve kernel takes one CTA per (patch, 16 samples), one sample per lane,
 // and refines in FP64: r = b - A f (FP64, sweeping a three-node window of f
@@ -58,103 +57,283 @@ __device__ __forceinline__ bool kd_identity(int i, int nn, double vl) {
     return (i == 0 && vl > 0.0) || (i == nn - 1 && vl < 0.0);
 }
 
-// One CTA per patch.  Thread (ty, tx) of the 16 x 16 grid owns the entries
-// (ty + 16 a, tx + 16 b), a, b < RA, of the n_v x n_v block (n_v <= 16 RA).
+// The factor in halves.  With the h = n_v/2 negative velocities first, S_i = [A B; C D],
+// and of the interior nodes' blocks only C depends on the node:
+//
+//   C_i = C_0 - a_+ (W_{i-1})_{+-} a_-,   X_i = D^{-1} C_i = X_0 + F P_{i-1} a_-,
+//   E_i = A - B X_i,   P_i = X_i E_i^{-1},   F = D^{-1} a_+,   G = B D^{-1},
+//   W_i = [ E^{-1}, -E^{-1} G ; -P, D^{-1} + P G ]
+//
+// (end nodes: C = 0, D = I at the first, A = I, B = 0 at the last).  E is a Schur
+// complement of an M-matrix, so it needs no pivoting either.  A node's serial part is one
+// h x h inverse and three h x h products instead of an n_v x n_v inverse, 4 h^3 for 8 h^3
+// multiply-adds and h barriers for 2 h; the + columns of W, 2 h^3, are independent of each
+// other over all nodes and run on the whole GPU.
+struct KdHalf {   // offsets (in h*h) of the node-independent blocks
+    static constexpr int kA = 0, kB = 1, kDinv = 2, kG = 3, kX0 = 4, kF = 5, kCount = 6;
+};
+constexpr int kKdMaxHalf = kKdMaxNv / 2;
+
+// The blocks that no node changes, by one CTA: D inverted by Gauss-Jordan in shared memory
+// (one thread takes each pivot's reciprocal), then G, X_0 and F.
+template <class T>
+__global__ void __launch_bounds__(1024) kd_blocks_kernel(KdArgs A, T* __restrict__ out) {
+    extern __shared__ __align__(16) unsigned char kd_dyn[];
+    double* D = reinterpret_cast<double*>(kd_dyn);   // h x h
+    __shared__ double col[kKdMaxHalf], row[kKdMaxHalf], rcp;
+    const int nv = A.n_v, h = nv / 2, hh = h * h;
+    const double dx = 1.0 / A.N, ie = 1.0 / A.eps;
+    auto entry = [&](int r, int c) {   // interior row r, without the neighbours' term
+        double s = -ie * A.Kw[(long long)r * nv + c];
+        if (r == c) s += fabs(A.v[r]) / dx + ie * A.sigma[r];
+        return s;
+    };
+    for (int e = threadIdx.x; e < hh; e += blockDim.x) {
+        const int r = e / h, c = e % h;
+        D[e] = entry(h + r, h + c);
+        out[KdHalf::kA * hh + e] = (T)entry(r, c);
+        out[KdHalf::kB * hh + e] = (T)entry(r, h + c);
+    }
+    __syncthreads();
+    for (int k = 0; k < h; ++k) {
+        if (threadIdx.x < h) {
+            col[threadIdx.x] = D[threadIdx.x * h + k];
+            row[threadIdx.x] = D[k * h + threadIdx.x];
+        }
+        if (threadIdx.x == 0) rcp = 1.0 / D[k * h + k];
+        __syncthreads();
+        for (int e = threadIdx.x; e < hh; e += blockDim.x) {
+            const int r = e / h, c = e % h;
+            const double cr = col[r] * rcp;
+            double x = D[e];
+            if (r != k) x = (c != k) ? fma(-cr, row[c], x) : -cr;
+            else x = (c != k) ? row[c] * rcp : rcp;
+            D[e] = x;
+        }
+        __syncthreads();
+    }
+    for (int e = threadIdx.x; e < hh; e += blockDim.x) {
+        const int r = e / h, c = e % h;
+        double g = 0.0, x = 0.0;
+        for (int k = 0; k < h; ++k) {
+            g = fma(entry(r, h + k), D[k * h + c], g);
+            x = fma(D[r * h + k], entry(h + k, c), x);
+        }
+        out[KdHalf::kDinv * hh + e] = (T)D[e];
+        out[KdHalf::kG * hh + e] = (T)g;
+        out[KdHalf::kX0 * hh + e] = (T)x;
+        out[KdHalf::kF * hh + e] = (T)(D[e] * (fabs(A.v[h + c]) / dx));
+    }
+}
+
+// acc[a][b] += sum_k L[ty + 16 a][k] R[k][tx + 16 b] of h x h blocks in shared memory with
+// row stride ld (entries beyond h are left alone).
 template <class T, int RA>
-__global__ void __launch_bounds__(kKdThreads) kd_factor_kernel(KdArgs A, T* W) {
-    __shared__ T colk[2][kKdMaxNv];
-    __shared__ T rowk[2][kKdMaxNv];
-    const int m = blockIdx.x, nv = A.n_v;
+__device__ __forceinline__ void kd_product(T (&acc)[RA][RA], const T* L, const T* R, int h, int ld, int tx, int ty) {
+    for (int k = 0; k < h; ++k) {
+        T l[RA], r[RA];
+#pragma unroll
+        for (int a = 0; a < RA; ++a) {
+            l[a] = (ty + 16 * a < h) ? L[(ty + 16 * a) * ld + k] : T(0);
+            r[a] = (tx + 16 * a < h) ? R[k * ld + tx + 16 * a] : T(0);
+        }
+#pragma unroll
+        for (int a = 0; a < RA; ++a)
+#pragma unroll
+            for (int b = 0; b < RA; ++b) acc[a][b] += l[a] * r[b];
+    }
+}
+
+// The serial part, one CTA per patch: E_i, its inverse and P_i of every node, written to the
+// - columns of W.  Thread (ty, tx) of the 16 x 16 grid owns the entries (ty + 16 a,
+// tx + 16 b), a, b < RA, of each h x h block (h <= 16 RA).  Bound by FP64 issue: a warp's
+// instruction holds its quarter of the SM for 64 clocks, a division for about 380, so only
+// the thread that finishes the next pivot divides and publishes the reciprocal.  8193
+// nodes, 64 velocities, 64 patches: the factor as one n_v x n_v inverse per node took
+// 42 ms of a pass of 114.2; with the halves the pass takes 85.4.
+template <class T, int RA>
+__global__ void __launch_bounds__(kKdThreads) kd_chain_kernel(KdArgs A, const T* __restrict__ blocks, T* W) {
+    extern __shared__ __align__(16) unsigned char kd_dyn[];
+    __shared__ T colk[2][kKdMaxHalf], rowk[2][kKdMaxHalf], rcp[2];
+    const int m = blockIdx.x, nv = A.n_v, h = nv / 2, hh = h * h, ld = h + 1;
+    T* sB = reinterpret_cast<T*>(kd_dyn);
+    T* sF = sB + h * ld;
+    T* sX = sF + h * ld;   // X_i
+    T* sE = sX + h * ld;   // E_i^{-1}, then P_i a_-
     const KPatchDev P = A.patches[m];
     const int nn = P.X1 - P.X0 + 1;
     const long long n2 = (long long)nv * nv;
-    const double dx = 1.0 / A.N, ie = 1.0 / A.eps;
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-    T x[RA][RA];
     T* Wm = W + A.node_off[m] * n2;
+    for (int e = threadIdx.x; e < hh; e += kKdThreads) {
+        const int q = (e / h) * ld + e % h;
+        sB[q] = blocks[KdHalf::kB * hh + e];
+        sF[q] = blocks[KdHalf::kF * hh + e];
+        sX[q] = T(0);   // C = 0 at the first node
+    }
+    T a0[RA][RA], x0[RA][RA], am[RA];
 #pragma unroll
-    for (int a = 0; a < RA; ++a)
+    for (int a = 0; a < RA; ++a) {
+        am[a] = (tx + 16 * a < h) ? (T)(fabs(A.v[tx + 16 * a]) * (double)A.N) : T(0);
 #pragma unroll
-        for (int b = 0; b < RA; ++b) x[a][b] = T(0);
-    int par = 0;
-    for (int i = 0; i < nn; ++i) {
-        // S_i over W_{i-1}: each entry depends only on the previous value at the same place
-#pragma unroll
-        for (int a = 0; a < RA; ++a) {
-            const int r = ty + 16 * a;
-            if (r >= nv) continue;
-            const double vr = A.v[r], ar = fabs(vr) / dx;
-            const bool ident = kd_identity(i, nn, vr);
-#pragma unroll
-            for (int b = 0; b < RA; ++b) {
-                const int c = tx + 16 * b;
-                if (c >= nv) continue;
-                double s;
-                if (ident) {
-                    s = (r == c) ? 1.0 : 0.0;
-                } else {
-                    s = -ie * A.Kw[(long long)r * nv + c];
-                    if (r == c) s += ar + ie * A.sigma[r];
-                    const double vc = A.v[c];
-                    if (i > 0 && vr > 0.0 && vc < 0.0) s -= ar * (double)x[a][b] * (fabs(vc) / dx);
-                }
-                x[a][b] = (T)s;
-            }
+        for (int b = 0; b < RA; ++b) {
+            const bool in = ty + 16 * a < h && tx + 16 * b < h;
+            const int e = (ty + 16 * a) * h + tx + 16 * b;
+            a0[a][b] = in ? blocks[KdHalf::kA * hh + e] : T(0);
+            x0[a][b] = in ? blocks[KdHalf::kX0 * hh + e] : T(0);
         }
-        // Gauss-Jordan inversion in place, no pivoting; column and row k are
-        // published through alternating buffers, one barrier per step
-        for (int k = 0; k < nv; ++k) {
-            const int kq = k >> 4;   // register block of row / column k (selected by predicates)
-            if (tx == (k & 15)) {
+    }
+    __syncthreads();
+    // publishes column k, row k and 1 / pivot of the block in x
+    auto publish = [&](const T (&x)[RA][RA], int k, int par) {
+        const int kq = k >> 4;
+        if (tx == (k & 15)) {
+#pragma unroll
+            for (int a = 0; a < RA; ++a)
+#pragma unroll
+                for (int b = 0; b < RA; ++b)
+                    if (b == kq && ty + 16 * a < h) colk[par][ty + 16 * a] = x[a][b];
+        }
+        if (ty == (k & 15)) {
+#pragma unroll
+            for (int a = 0; a < RA; ++a)
+#pragma unroll
+                for (int b = 0; b < RA; ++b)
+                    if (a == kq && tx + 16 * b < h) {
+                        rowk[par][tx + 16 * b] = x[a][b];
+                        if (b == kq && tx == (k & 15)) rcp[par] = T(1) / x[a][b];
+                    }
+        }
+    };
+    for (int i = 0; i < nn; ++i) {
+        T x[RA][RA];
+#pragma unroll
+        for (int a = 0; a < RA; ++a)
+#pragma unroll
+            for (int b = 0; b < RA; ++b) x[a][b] = T(0);
+        if (i == nn - 1) {
+#pragma unroll
+            for (int a = 0; a < RA; ++a)
+#pragma unroll
+                for (int b = 0; b < RA; ++b) x[a][b] = (ty + 16 * a == tx + 16 * b) ? T(1) : T(0);
+        } else {
+            if (i > 0) kd_product<T, RA>(x, sB, sX, h, ld, tx, ty);
+#pragma unroll
+            for (int a = 0; a < RA; ++a)
+#pragma unroll
+                for (int b = 0; b < RA; ++b) x[a][b] = a0[a][b] - x[a][b];
+            publish(x, 0, 0);
+            for (int k = 0; k < h; ++k) {
+                const int par = k & 1;
+                __syncthreads();
+                const T p = rcp[par];
 #pragma unroll
                 for (int a = 0; a < RA; ++a) {
                     const int r = ty + 16 * a;
-#pragma unroll
-                    for (int b = 0; b < RA; ++b)
-                        if (b == kq && r < nv) colk[par][r] = x[a][b];
-                }
-            }
-            if (ty == (k & 15)) {
-#pragma unroll
-                for (int a = 0; a < RA; ++a) {
-                    if (a != kq) continue;
+                    if (r >= h) continue;
+                    const T cr = colk[par][r] * p;
 #pragma unroll
                     for (int b = 0; b < RA; ++b) {
                         const int c = tx + 16 * b;
-                        if (c < nv) rowk[par][c] = x[a][b];
+                        if (c >= h) continue;
+                        if (r == k) x[a][b] = (c == k) ? p : rowk[par][c] * p;
+                        else x[a][b] = (c == k) ? -cr : x[a][b] - cr * rowk[par][c];
                     }
                 }
+                if (k + 1 < h) publish(x, k + 1, par ^ 1);
             }
-            __syncthreads();
-            const T p = T(1) / rowk[par][k];
-#pragma unroll
-            for (int a = 0; a < RA; ++a) {
-                const int r = ty + 16 * a;
-                if (r >= nv) continue;
-                const T cr = colk[par][r] * p;
-#pragma unroll
-                for (int b = 0; b < RA; ++b) {
-                    const int c = tx + 16 * b;
-                    if (c >= nv) continue;
-                    if (r != k) {
-                        x[a][b] = (c != k) ? x[a][b] - cr * rowk[par][c] : -cr;
-                    } else {
-                        x[a][b] = (c != k) ? rowk[par][c] * p : p;
-                    }
-                }
-            }
-            par ^= 1;
         }
         T* Wi = Wm + (long long)i * n2;
 #pragma unroll
-        for (int a = 0; a < RA; ++a) {
-            const int r = ty + 16 * a;
-            if (r >= nv) continue;
+        for (int a = 0; a < RA; ++a)
 #pragma unroll
             for (int b = 0; b < RA; ++b) {
-                const int c = tx + 16 * b;
-                if (c < nv) Wi[(long long)r * nv + c] = x[a][b];
+                const int r = ty + 16 * a, c = tx + 16 * b;
+                if (r < h && c < h) {
+                    sE[r * ld + c] = x[a][b];
+                    Wi[(long long)r * nv + c] = x[a][b];
+                }
             }
+        __syncthreads();
+        T pr[RA][RA];
+#pragma unroll
+        for (int a = 0; a < RA; ++a)
+#pragma unroll
+            for (int b = 0; b < RA; ++b) pr[a][b] = T(0);
+        if (i > 0) kd_product<T, RA>(pr, sX, sE, h, ld, tx, ty);
+        __syncthreads();   // every thread is done with E^{-1} and X_i
+#pragma unroll
+        for (int a = 0; a < RA; ++a)
+#pragma unroll
+            for (int b = 0; b < RA; ++b) {
+                const int r = ty + 16 * a, c = tx + 16 * b;
+                if (r < h && c < h) {
+                    Wi[(long long)(h + r) * nv + c] = -pr[a][b];
+                    sE[r * ld + c] = pr[a][b] * am[b];
+                }
+            }
+        if (i == nn - 1) break;
+        __syncthreads();
+        T xn[RA][RA];
+#pragma unroll
+        for (int a = 0; a < RA; ++a)
+#pragma unroll
+            for (int b = 0; b < RA; ++b) xn[a][b] = x0[a][b];
+        if (i > 0) kd_product<T, RA>(xn, sF, sE, h, ld, tx, ty);
+#pragma unroll
+        for (int a = 0; a < RA; ++a)
+#pragma unroll
+            for (int b = 0; b < RA; ++b) {
+                const int r = ty + 16 * a, c = tx + 16 * b;
+                if (r < h && c < h) sX[r * ld + c] = xn[a][b];
+            }
+        __syncthreads();
+    }
+}
+
+// The + columns of W of every node, from its - columns: CTA (x, m) takes the nodes x,
+// x + gridDim.x, ... of patch m with G in shared memory; the - columns pass through it too.
+template <class T, int RA>
+__global__ void __launch_bounds__(kKdThreads) kd_columns_kernel(KdArgs A, const T* __restrict__ blocks, T* W) {
+    extern __shared__ __align__(16) unsigned char kd_dyn[];
+    const int m = blockIdx.y, nv = A.n_v, h = nv / 2, hh = h * h, ld = h + 1;
+    T* sG = reinterpret_cast<T*>(kd_dyn);
+    T* sL = sG + h * ld;   // 2 h rows: E^{-1} over -P
+    const KPatchDev P = A.patches[m];
+    const int nn = P.X1 - P.X0 + 1;
+    const long long n2 = (long long)nv * nv;
+    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+    T* Wm = W + A.node_off[m] * n2;
+    int held = -1;   // 0: B (the first node, where D = I), 1: G
+    for (int i = blockIdx.x; i < nn; i += gridDim.x) {
+        T* Wi = Wm + (long long)i * n2;
+        const int want = i > 0;
+        __syncthreads();   // the previous node's products are done
+        if (held != want)
+            for (int e = threadIdx.x; e < hh; e += kKdThreads)
+                sG[(e / h) * ld + e % h] = blocks[(want ? KdHalf::kG : KdHalf::kB) * hh + e];
+        held = want;
+        for (int e = threadIdx.x; e < 2 * hh; e += kKdThreads) sL[(e / h) * ld + e % h] = Wi[(long long)(e / h) * nv + e % h];
+        __syncthreads();
+#pragma unroll
+        for (int half = 0; half < 2; ++half) {
+            T acc[RA][RA];
+#pragma unroll
+            for (int a = 0; a < RA; ++a)
+#pragma unroll
+                for (int b = 0; b < RA; ++b) acc[a][b] = T(0);
+            const bool zero = half == 0 ? i == nn - 1 : (i == 0 || i == nn - 1);
+            if (!zero) kd_product<T, RA>(acc, sL + half * h * ld, sG, h, ld, tx, ty);
+#pragma unroll
+            for (int a = 0; a < RA; ++a)
+#pragma unroll
+                for (int b = 0; b < RA; ++b) {
+                    const int r = ty + 16 * a, c = tx + 16 * b;
+                    if (r >= h || c >= h) continue;
+                    T w = -acc[a][b];
+                    if (half) w += i > 0 ? blocks[KdHalf::kDinv * hh + r * h + c] : (r == c ? T(1) : T(0));
+                    Wi[(long long)(half * h + r) * nv + h + c] = w;
+                }
         }
     }
 }
@@ -378,20 +557,32 @@ __global__ void __launch_bounds__(kKdThreads) kd_solve_kernel(KdArgs A, const T*
 }
 
 template <class T, int RA>
-msp_status launch_factor(const KdArgs& A, int M, T* W, cudaStream_t s) {
-    kd_factor_kernel<T, RA><<<M, kKdThreads, 0, s>>>(A, W);
-    count_launches(1);
+msp_status launch_factor(const KdArgs& A, int M, int max_nn, T* blocks, T* W, cudaStream_t s) {
+    const int h = A.n_v / 2;
+    const size_t tile = sizeof(T) * h * (h + 1);
+    MSP_CUDA(cudaFuncSetAttribute(kd_chain_kernel<T, RA>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(4 * tile)));
+    MSP_CUDA(cudaFuncSetAttribute(kd_columns_kernel<T, RA>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(3 * tile)));
+    kd_blocks_kernel<T><<<1, 1024, sizeof(double) * h * h, s>>>(A, blocks);
     MSP_CUDA(cudaGetLastError());
+    kd_chain_kernel<T, RA><<<M, kKdThreads, 4 * tile, s>>>(A, blocks, W);
+    MSP_CUDA(cudaGetLastError());
+    // about eight CTAs per SM over all patches
+    const int per = std::max(1, std::min(max_nn, (8 * 152 + M - 1) / M));
+    kd_columns_kernel<T, RA><<<dim3(per, M), kKdThreads, 3 * tile, s>>>(A, blocks, W);
+    MSP_CUDA(cudaGetLastError());
+    count_launches(3);
     return MSP_OK;
 }
 
 template <class T>
-msp_status factor(const KdArgs& A, int M, T* W, cudaStream_t s) {
-    const int nv = A.n_v;
-    if (nv <= 16) return launch_factor<T, 1>(A, M, W, s);
-    if (nv <= 32) return launch_factor<T, 2>(A, M, W, s);
-    if (nv <= 64) return launch_factor<T, 4>(A, M, W, s);
-    return launch_factor<T, 8>(A, M, W, s);
+msp_status factor(const KMedium& K, const KdArgs& A, DevBuf<T>& blocks, T* W, cudaStream_t s) {
+    const int h = A.n_v / 2;
+    int max_nn = 1;
+    for (auto& P : K.patches) max_nn = std::max(max_nn, P.nn);
+    MSP_TRY(blocks.alloc((size_t)KdHalf::kCount * h * h, s));
+    if (h <= 16) return launch_factor<T, 1>(A, K.M, max_nn, blocks.p, W, s);
+    if (h <= 32) return launch_factor<T, 2>(A, K.M, max_nn, blocks.p, W, s);
+    return launch_factor<T, 4>(A, K.M, max_nn, blocks.p, W, s);
 }
 
 template <class T, int RJ>
@@ -445,7 +636,7 @@ msp_status kinetic_direct_sample(KMedium& K, uint64_t seed, bool mixed, double t
     if (mixed) {
         if (!D.factored32) {
             MSP_TRY(D.W32.alloc((size_t)D.n_nodes * n2, s));
-            MSP_TRY(factor<float>(A, K.M, D.W32.p, s));
+            MSP_TRY(factor<float>(K, A, D.blocks32, D.W32.p, s));
             D.factored32 = true;
         }
         if (D.y32.n < nf) MSP_TRY(D.y32.alloc(nf, s));
@@ -453,7 +644,7 @@ msp_status kinetic_direct_sample(KMedium& K, uint64_t seed, bool mixed, double t
     }
     if (!D.factored64) {
         MSP_TRY(D.W64.alloc((size_t)D.n_nodes * n2, s));
-        MSP_TRY(factor<double>(A, K.M, D.W64.p, s));
+        MSP_TRY(factor<double>(K, A, D.blocks64, D.W64.p, s));
         D.factored64 = true;
     }
     if (D.y64.n < nf) MSP_TRY(D.y64.alloc(nf, s));

@@ -21,6 +21,8 @@ struct KDirect {
     long long n_nodes = 0;
     DevBuf<double> W64;
     DevBuf<float> W32;
+    DevBuf<double> blocks64;   // the factor's node-independent half blocks
+    DevBuf<float> blocks32;
     bool factored64 = false, factored32 = false;
     DevBuf<double> f;
     DevBuf<double> y64;
