@@ -20,7 +20,6 @@ namespace {
 
 constexpr int kPan = 16;            // columns per Cholesky panel
 constexpr int kCholThreads = 512;
-constexpr int kInvWarps = 16;       // columns of the inverse per CTA
 
 // Doubles of the panels p = rank, rank + nc, ... of an order-c block: rows 16 p .. c of
 // 16 columns each
@@ -161,60 +160,99 @@ __global__ void __launch_bounds__(kCholThreads) patch_chol_kernel(const PatchBlo
     cl.sync();                       // no CTA leaves while another may write its flag
 }
 
+// Sums over the warp of four values per lane: the lanes with (lane >> 3 & 3) == c get
+// column c's.  Each value is added over the lanes in the tree of warp_sum (16, 8, ... 1),
+// but with the first two levels shared, 6 additions and shuffles instead of 20.
+__device__ __forceinline__ double warp_sum4(const double (&a)[4], int lane) {
+    const bool hi = lane & 16, odd = lane & 8;
+    double u = (hi ? a[2] : a[0]) + __shfl_xor_sync(0xffffffffu, hi ? a[0] : a[2], 16);
+    double w = (hi ? a[3] : a[1]) + __shfl_xor_sync(0xffffffffu, hi ? a[1] : a[3], 16);
+    double v = (odd ? w : u) + __shfl_xor_sync(0xffffffffu, odd ? u : w, 8);
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+
 // F = L^T and Fi = L^{-T}.  X = L^{-1} column by column: X(i, j) = (delta_ij - sum_{q < i}
-// l_iq X(q, j)) / l_ii, one warp per column j with lanes along q (q = j + lane + 32 u) and
-// the warp's partial sums combined by shuffles, sixteen columns per CTA sharing the
-// rows of L they stage in shared memory, tr rows at a time.  X(i, j) is stored at
-// Fi(j, i); the CTA of the first columns also writes F.  Columns are independent, so a
-// patch takes c / 16 CTAs.
-__global__ void __launch_bounds__(32 * kInvWarps) patch_inverse_kernel(const PatchBlock* blocks, const double* L,
-                                                                       double* F, double* Fi, const int* status,
-                                                                       int tr) {
+// l_iq X(q, j)) / l_ii, CPW columns per warp with lanes along q (q = j + lane + 32 u) and
+// the partial sums combined by shuffles.  The columns of a CTA share the rows of L they
+// stage in shared memory, tr rows at a time, and the reciprocals of their diagonal, one
+// division per row and CTA (it takes as long as six FMAs).  X(i, j) is stored at Fi(j, i);
+// the CTA of the first columns also writes F.  Columns are independent, so a patch takes
+// c / kCols CTAs, and a column's sums do not depend on CPW.
+// Bound by FP64 issue: 1024 patches of up to 290 columns took 9.5 ms a call with a division
+// per row and column and one column per warp; a 513^2 extraction went from 115.8 to 104.4 ms
+// with both changes, a 2049^2 step from 1121 to 1100.
+template <int CPW>
+struct InvShape {
+    static constexpr int kWarps = CPW == 1 ? 16 : 8;
+    static constexpr int kCols = CPW * kWarps;
+};
+
+template <int CPW>
+__global__ void __launch_bounds__(32 * InvShape<CPW>::kWarps) patch_inverse_kernel(const PatchBlock* blocks, const double* L,
+                                                                                   double* F, double* Fi,
+                                                                                   const int* status, int tr) {
+    constexpr int kWarps = InvShape<CPW>::kWarps, kCols = InvShape<CPW>::kCols;
+    static_assert(CPW == 1 || CPW == 4, "");
     extern __shared__ __align__(16) double ism[];
     const PatchBlock P = blocks[blockIdx.y];
-    const int c = P.c, j0 = blockIdx.x * kInvWarps;
+    const int c = P.c, j0 = blockIdx.x * kCols;
     if (j0 >= c || (status && status[P.idx] < 0)) return;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int j = j0 + warp;
+    const int jb = j0 + CPW * warp;                    // the warp's first column
+    const int mine = CPW == 1 ? 0 : (lane >> 3) & 3;   // the column whose sum this lane gets
+    const bool writes = CPW == 1 ? lane == 0 : (lane & 7) == 0;
+    const int jm = jb + mine;
     const double* l = L + P.off;
     double* f = F + P.off;
     double* fi = Fi + P.off;
     double* Ls = ism;                                  // tr x c: rows of L
-    double* out = Ls + (size_t)tr * c;                 // tr x kInvWarps
-    double* x = out + tr * kInvWarps + (size_t)warp * c;   // X(:, j)
+    double* out = Ls + (size_t)tr * c;                 // tr x kCols
+    double* rl = out + tr * kCols;                     // 1 / l_ii of the rows
+    double* x = rl + tr + (size_t)CPW * warp * c;      // X(:, jb ..)
     for (int i0 = 0; i0 < c; i0 += tr) {
         const int rows = min(tr, c - i0);
         const bool live = i0 + rows > j0;              // rows above the CTA's columns hold zeros
         if (live || blockIdx.x == 0) {
+            if (tid < rows) rl[tid] = 1.0 / l[(size_t)(i0 + tid) * (c + 1)];
             for (int e = tid; e < tr * (i0 + rows); e += blockDim.x) {
                 const int r = e % tr, q = e / tr;
                 if (r < rows) Ls[(size_t)r * c + q] = q <= i0 + r ? l[i0 + r + (size_t)q * c] : 0.0;
             }
             __syncthreads();
         }
-        if (live && j < c) {
+        if (live && jb < c) {
             for (int r = 0; r < rows; ++r) {
                 const int i = i0 + r;
                 double v = 0.0;
-                if (i >= j) {
+                if (i >= jb) {
                     const double* li = Ls + (size_t)r * c;
-                    const double rli = 1.0 / li[i];
-                    double a = 0.0;
-                    for (int q = j + lane; q < i; q += 32) a += li[q] * x[q];
-                    a = warp_sum(a);
-                    v = ((i == j ? 1.0 : 0.0) - a) * rli;
-                    if (lane == 0) x[i] = v;
+                    double a[CPW];
+#pragma unroll
+                    for (int k = 0; k < CPW; ++k) a[k] = 0.0;
+                    for (int q = jb + lane; q < i; q += 32)
+#pragma unroll
+                        for (int k = 0; k < CPW; ++k)
+                            if (q + k < i) a[k] += li[q + k] * x[(size_t)k * c + q + k];
+                    double s;
+                    if constexpr (CPW == 1) s = warp_sum(a[0]);
+                    else s = warp_sum4(a, lane);
+                    if (i >= jm) {
+                        v = ((i == jm ? 1.0 : 0.0) - s) * rl[r];
+                        if (writes) x[(size_t)mine * c + i] = v;
+                    }
                     __syncwarp();
                 }
-                if (lane == 0) out[r * kInvWarps + warp] = v;
+                if (writes) out[r * kCols + CPW * warp + mine] = v;
             }
         }
         if (blockIdx.x == 0 && F)
-            for (int r = warp; r < rows; r += kInvWarps)
+            for (int r = warp; r < rows; r += kWarps)
                 for (int q = lane; q < c; q += 32) f[q + (size_t)(i0 + r) * c] = q <= i0 + r ? Ls[(size_t)r * c + q] : 0.0;
         __syncthreads();
-        for (int e = tid; e < rows * kInvWarps; e += blockDim.x) {
-            const int r = e / kInvWarps, w = e % kInvWarps;
+        for (int e = tid; e < rows * kCols; e += blockDim.x) {
+            const int r = e / kCols, w = e % kCols;
             if (j0 + w < c) fi[j0 + w + (size_t)(i0 + r) * c] = live ? out[e] : 0.0;
         }
         __syncthreads();
@@ -791,25 +829,37 @@ PatchClasses classify_patches(const std::vector<int>& cols, const std::vector<lo
     return C;
 }
 
-static msp_status launch_inverse(const PatchClasses& C, const PatchBlock* blocks, const double* L, double* F, double* Fi,
-                                 const int* status, cudaStream_t s) {
+template <int CPW>
+static msp_status launch_inverse(const PatchClasses& C, int c, const PatchBlock* blocks, const double* L, double* F,
+                                 double* Fi, const int* status, cudaStream_t s) {
+    constexpr int kWarps = InvShape<CPW>::kWarps, kCols = InvShape<CPW>::kCols;
     size_t room = 0;
     MSP_TRY(smem_room(&room));
-    const int c = std::max(C.max_c[0], C.max_c[1]);
-    if (c > 0) {
-        int tr = 16;
-        auto bytes = [&](int t) { return sizeof(double) * ((size_t)t * c + (size_t)t * kInvWarps + (size_t)kInvWarps * c); };
-        while (tr > 1 && bytes(tr) > room) tr /= 2;
-        MSP_CUDA(cudaFuncSetAttribute(patch_inverse_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes(tr)));
-        for (size_t b0 = 0; b0 < C.blocks.size(); b0 += 65535) {
-            const unsigned nb = (unsigned)std::min<size_t>(65535, C.blocks.size() - b0);
-            patch_inverse_kernel<<<dim3((c + kInvWarps - 1) / kInvWarps, nb), 32 * kInvWarps, bytes(tr), s>>>(
-                blocks + b0, L, F, Fi, status, tr);
-            count_launches(1);
-        }
-        MSP_CUDA(cudaGetLastError());
+    int tr = 16;
+    auto bytes = [&](int t) { return sizeof(double) * ((size_t)t * (c + kCols + 1) + (size_t)kCols * c); };
+    while (tr > 1 && bytes(tr) > room) tr /= 2;
+    MSP_CUDA(cudaFuncSetAttribute(patch_inverse_kernel<CPW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes(tr)));
+    for (size_t b0 = 0; b0 < C.blocks.size(); b0 += 65535) {
+        const unsigned nb = (unsigned)std::min<size_t>(65535, C.blocks.size() - b0);
+        patch_inverse_kernel<CPW><<<dim3((c + kCols - 1) / kCols, nb), 32 * kWarps, bytes(tr), s>>>(blocks + b0, L, F, Fi,
+                                                                                                  status, tr);
+        count_launches(1);
     }
+    MSP_CUDA(cudaGetLastError());
     return MSP_OK;
+}
+
+static msp_status launch_inverse(const PatchClasses& C, const PatchBlock* blocks, const double* L, double* F, double* Fi,
+                                 const int* status, cudaStream_t s) {
+    const int c = std::max(C.max_c[0], C.max_c[1]);
+    if (c <= 0) return MSP_OK;
+    long long columns = 0;
+    for (const PatchBlock& b : C.blocks) columns += b.c;
+    // Four columns a warp need about 26 FP64 instructions a row where one needs 11.5, so they
+    // win from about two columns per quarter of an SM on; beyond 512 columns their 32 vectors
+    // would leave shared memory no room for the rows.
+    const bool four = columns >= 2LL * 4 * num_sms() && c <= 512;
+    return four ? launch_inverse<4>(C, c, blocks, L, F, Fi, status, s) : launch_inverse<1>(C, c, blocks, L, F, Fi, status, s);
 }
 
 msp_status patch_triangular_inverse(const PatchClasses& C, const PatchBlock* blocks, const double* L, double* Fi,

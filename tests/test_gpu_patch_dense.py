@@ -42,3 +42,21 @@ def test_bases_at_layout_edges(side, buffer, samples):
             gap = s[j - 1] - s[j]
             if gap > 1e-3 * s[0]:
                 assert np.linalg.norm(U[:, :j] - Q[:, :j] @ (Q[:, :j].T @ U[:, :j]), 2) <= 1e-11 * s[0] / gap + 1e-10
+
+
+@pytest.mark.parametrize("side,samples", [(4, 2), (4, 3), (4, 4), (12, 3), (12, 18), (12, 20)])
+def test_many_patches(side, samples):
+    """81 patches: from 1216 columns on (at 152 SMs) a warp of the triangular inverse takes
+    four columns, here with one to three of them beyond the block's order."""
+    N = 9 * side
+    med = msp.Medium(synth.lognormal(N, 4.0 / N, 16, 3), synth.uniform_patches(N, 9, 9, 2, samples))
+    med.sample(12, "fp64", tol=1e-12, max_iter=20000)
+    basis = med.extract(1e-6, "fp64")
+    for m in range(0, 81, 8):
+        R = med.snapshots(m).cpu().numpy()
+        s = np.linalg.svd(R, compute_uv=False)
+        got, Q = basis.sigma(m), basis.Q(m).cpu().numpy()
+        res = s >= 1e-7 * s[0]
+        assert np.max(np.abs(got[: len(s)] - s)[res]) <= 1e-10 * s[0], m
+        assert np.max(np.abs(Q.T @ Q - np.eye(Q.shape[1]))) <= 1e-10, m
+        assert np.linalg.norm(R - Q @ (Q.T @ R), 2) <= 1.01e-6 * s[0] + 1e-10 * s[0], m
