@@ -58,8 +58,13 @@ struct OnArgs {
 // chain of FMAs in the order of the terms, so no result depends on the tiling or the batch.
 // These products are bound by the FP64 pipe in batches and by the chain's latency for one
 // data set; as one CTA per patch they kept 64 of 152 SMs busy at 513^2 and read the operator
-// once per data set.
+// once per data set.  32 data sets at 513^2: edge values 1.06 -> 0.24 ms, right-hand side
+// 1.59 -> 0.55 a call.
+// The next slab is read into registers while this one is multiplied (one data set at 2049^2:
+// a solve of 8.33 ms became 7.88).
 constexpr int kOpRows = 64, kOpK = 32, kOpBatch = 8;
+template <int BT>
+constexpr int kOpX = (kOpK * 4 * BT + 255) / 256;   // vector entries a thread stages per slab
 
 __host__ __device__ inline int op_bt(int B) { return B <= 4 ? 1 : kOpBatch; }
 inline unsigned op_groups(int B) { return (unsigned)((B + 4 * op_bt(B) - 1) / (4 * op_bt(B))); }
@@ -81,17 +86,35 @@ __global__ void __launch_bounds__(256) edge_apply_kernel(OnArgs A, const double*
     double acc[BT];
 #pragma unroll
     for (int t = 0; t < BT; ++t) acc[t] = 0.0;
+    double pe[kOpRows * kOpK / 256], px[kOpX<BT>];
+    auto fetch = [&](int j0) {
+        const int jn = min(kOpK, k - j0);
+#pragma unroll
+        for (int u = 0; u < kOpRows * kOpK / 256; ++u) {
+            const int q = threadIdx.x + 256 * u, r = q / kOpK, j = q % kOpK;
+            pe[u] = (j < jn && s0 + r < ns) ? Em[(long long)(s0 + r) * k + j0 + j] : 0.0;
+        }
+#pragma unroll
+        for (int u = 0; u < kOpX<BT>; ++u) {
+            const int q = threadIdx.x + 256 * u, j = q / (4 * BT), b = q % (4 * BT);
+            px[u] = (j < jn && b0 + b < B) ? xm[(long long)(j0 + j) * B + b0 + b] : 0.0;
+        }
+    };
+    fetch(0);
     for (int j0 = 0; j0 < k; j0 += kOpK) {
         const int jn = min(kOpK, k - j0);
-        for (int q = threadIdx.x; q < kOpRows * kOpK; q += 256) {
-            const int r = q / kOpK, j = q % kOpK;
-            if (j < jn && s0 + r < ns) Es[r][j] = Em[(long long)(s0 + r) * k + j0 + j];
+#pragma unroll
+        for (int u = 0; u < kOpRows * kOpK / 256; ++u) {
+            const int q = threadIdx.x + 256 * u;
+            Es[q / kOpK][q % kOpK] = pe[u];
         }
-        for (int q = threadIdx.x; q < kOpK * 4 * BT; q += 256) {
-            const int j = q / (4 * BT), b = q % (4 * BT);
-            if (j < jn && b0 + b < B) xs[j][b] = xm[(long long)(j0 + j) * B + b0 + b];
+#pragma unroll
+        for (int u = 0; u < kOpX<BT>; ++u) {
+            const int q = threadIdx.x + 256 * u;
+            if (q < kOpK * 4 * BT) xs[q / (4 * BT)][q % (4 * BT)] = px[u];
         }
         __syncthreads();
+        if (j0 + kOpK < k) fetch(j0 + kOpK);
         if (live)
             for (int j = 0; j < jn; ++j) {
                 const double v = Es[row][j];
@@ -263,17 +286,35 @@ __global__ void __launch_bounds__(256) normal_rhs_kernel(OnArgs A, const double*
     double acc[BT];
 #pragma unroll
     for (int u = 0; u < BT; ++u) acc[u] = 0.0;
+    double pe[kOpRows * kOpK / 256], pt[kOpX<BT>];
+    auto fetch = [&](int s0) {
+        const int sn = min(kOpK, ns - s0);
+#pragma unroll
+        for (int u = 0; u < kOpRows * kOpK / 256; ++u) {
+            const int q = threadIdx.x + 256 * u, s = q / kOpRows, c = q % kOpRows;
+            pe[u] = (s < sn && j0 + c < k) ? Em[(long long)(s0 + s) * k + j0 + c] : 0.0;
+        }
+#pragma unroll
+        for (int u = 0; u < kOpX<BT>; ++u) {
+            const int q = threadIdx.x + 256 * u, s = q / (4 * BT), b = q % (4 * BT);
+            pt[u] = (s < sn && b0 + b < B) ? tm[(long long)(s0 + s) * B + b0 + b] : 0.0;
+        }
+    };
+    fetch(0);
     for (int s0 = 0; s0 < ns; s0 += kOpK) {
         const int sn = min(kOpK, ns - s0);
-        for (int q = threadIdx.x; q < kOpRows * kOpK; q += 256) {
-            const int s = q / kOpRows, c = q % kOpRows;
-            if (s < sn && j0 + c < k) Es[s][c] = Em[(long long)(s0 + s) * k + j0 + c];
+#pragma unroll
+        for (int u = 0; u < kOpRows * kOpK / 256; ++u) {
+            const int q = threadIdx.x + 256 * u;
+            Es[q / kOpRows][q % kOpRows] = pe[u];
         }
-        for (int q = threadIdx.x; q < kOpK * 4 * BT; q += 256) {
-            const int s = q / (4 * BT), b = q % (4 * BT);
-            if (s < sn && b0 + b < B) ts[s][b] = tm[(long long)(s0 + s) * B + b0 + b];
+#pragma unroll
+        for (int u = 0; u < kOpX<BT>; ++u) {
+            const int q = threadIdx.x + 256 * u;
+            if (q < kOpK * 4 * BT) ts[q / (4 * BT)][q % (4 * BT)] = pt[u];
         }
         __syncthreads();
+        if (s0 + kOpK < ns) fetch(s0 + kOpK);
         if (live)
             for (int s = 0; s < sn; ++s) {
                 const double v = Es[s][row];
@@ -374,7 +415,8 @@ __global__ void update_p_kernel(OnArgs A, double* p, const double* z, const doub
 // FP64.  A thread takes one node and BT data sets, so that a column of Q is read once,
 // coalesced, for all of them, and u is written along the rows; blockIdx (data-set group,
 // node tile, patch).  FP64: bound by the FP64 pipe in batches (n_k k B FMA), by the reading
-// of Q for one data set; FP32: by Q.
+// of Q for one data set; FP32: by Q.  32 data sets at 513^2: FP64 8.8 -> 1.4 ms, FP32
+// 4.2 -> 0.26; one at 2049^2: 1.19 -> 0.68.
 template <class TQ, class TC, int BT>
 __global__ void __launch_bounds__(256) recon_interior_kernel(OnArgs A, const PatchDev* patches, const long long* q_off,
                                                              const TQ* Q, const TC* c, double* u, int N) {
