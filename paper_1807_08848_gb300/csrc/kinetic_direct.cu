@@ -150,7 +150,7 @@ __device__ __forceinline__ void kd_product(T (&acc)[RA][RA], const T* L, const T
 // instruction holds its quarter of the SM for 64 clocks, a division for about 380, so only
 // the thread that finishes the next pivot divides and publishes the reciprocal.  8193
 // nodes, 64 velocities, 64 patches: the factor as one n_v x n_v inverse per node took
-// 42 ms of a pass of 114.2; with the halves the pass takes 85.4.
+// 42 ms of a pass of 114.2; with the halves it takes 13.2, the pass 85.4.
 template <class T, int RA>
 __global__ void __launch_bounds__(kKdThreads) kd_chain_kernel(KdArgs A, const T* __restrict__ blocks, T* W) {
     extern __shared__ __align__(16) unsigned char kd_dyn[];

@@ -68,7 +68,7 @@ __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, unsigned by
 // below are the strip's neighbours) and its horizontal neighbours from shared memory.
 // Bound: HBM (each tile read and written once); with the faces in shared memory, two more
 // rows per quad and two barriers per tile the 256 x 96 tiles of 97 x 100 took 513 us
-// against 265 us of copying.
+// against 265 us of copying; now 317 us, 5.65 TB/s.
 template <int R>
 __global__ void __launch_bounds__(512) stencil_stream_kernel(StencilArgs A, int nb_buf) {
     constexpr int kMaxBuf = 8;
