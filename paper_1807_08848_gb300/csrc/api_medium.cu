@@ -61,7 +61,7 @@ cudaError_t pool_alloc(void** p, size_t bytes, cudaStream_t s) {
         size_t total = 0;
     };
     static std::mutex mu;
-    static std::vector<DevicePool> pools;   // per device; never destroyed (the driver may be gone by then)
+    static std::vector<DevicePool> pools;   // per device; never destroyed (at exit the CUDA driver may be gone)
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
