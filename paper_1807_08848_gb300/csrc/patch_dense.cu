@@ -41,7 +41,11 @@ __global__ void __launch_bounds__(kCholThreads) patch_chol_kernel(const PatchBlo
                                                                   int in_smem) {
     extern __shared__ __align__(16) double csm[];
     __shared__ double s_trace;
-    __shared__ int s_bad;            // set by the owner of a panel with a bad pivot, in every CTA
+    // Set by the owner of a panel with a bad pivot, in every CTA, by panel parity: a thread reads
+    // panel p's flag after the barrier that ends the panel, while the owner of panel p + 1 may
+    // already store its own; the next store to the same word, panel p + 2's, comes only after a
+    // barrier that waits for every reader.
+    __shared__ int s_bad[2];
     __shared__ int s_ok;
     cg::cluster_group cl = cg::this_cluster();
     const int nc = (int)cl.num_blocks(), rank = (int)cl.block_rank();
@@ -56,14 +60,14 @@ __global__ void __launch_bounds__(kCholThreads) patch_chol_kernel(const PatchBlo
     auto panel = [&](int p, size_t at) { return in_smem ? own + at - (size_t)p * kPan : l + (size_t)p * kPan * c; };
     auto ldp = [&](int p) { return in_smem ? (size_t)(c - p * kPan) : (size_t)c; };
     for (int i = tid; i < c; i += blockDim.x) buf[i] = g[i + (size_t)i * c];
-    if (tid == 0) s_bad = 0;
+    if (tid < 2) s_bad[tid] = 0;
     __syncthreads();
     if (tid == 0) {
         double t = 0.0;
         for (int i = 0; i < c; ++i) t += buf[i];
         s_trace = t;
     }
-    cl.sync();                       // every CTA runs, and its flag is clear, before one may set it
+    cl.sync();                       // every CTA runs, and its flags are clear, before one may set them
     const double trace = s_trace;
     double shift = 0.0;
     if (shifted) shift = shift_scale[P.idx] * trace;
@@ -114,13 +118,13 @@ __global__ void __launch_bounds__(kCholThreads) patch_chol_kernel(const PatchBlo
                         for (int jj = warp; jj < w; jj += nw)
                             for (int i = k0 + jj + lane; i < c; i += 32) __stcg(l + i + (size_t)(k0 + jj) * c, pp[(size_t)jj * ld + i]);
                 } else if (tid < nc) {
-                    *cl.map_shared_rank(&s_bad, tid) = 1;
+                    cl.map_shared_rank(s_bad, tid)[p & 1] = 1;
                 }
                 at_next += (size_t)kPan * (c - k0);
                 __threadfence();
             }
             cl.sync();
-            if (s_bad) { ok = false; break; }
+            if (s_bad[p & 1]) { ok = false; break; }
             const int r0 = k0 + w;
             if (r0 >= c) break;
             for (int k = warp; k < w; k += nw)
@@ -153,12 +157,12 @@ __global__ void __launch_bounds__(kCholThreads) patch_chol_kernel(const PatchBlo
         if (!ok) {
             shift = (shift == 0.0) ? 1e-14 * trace : shift * 100.0;
             cl.sync();               // every CTA has read its flag
-            if (tid == 0) s_bad = 0;
+            if (tid < 2) s_bad[tid] = 0;
             cl.sync();
         }
     }
     if (rank == 0 && tid == 0) status[P.idx] = ok ? tries : -1;
-    cl.sync();                       // no CTA leaves while another may write its flag
+    cl.sync();                       // no CTA leaves while another may write its flags
 }
 
 // Sums over the warp of four values per lane: the lanes with (lane >> 3 & 3) == c get
