@@ -291,12 +291,13 @@ __global__ void __launch_bounds__(kKdThreads) kd_chain_kernel(KdArgs A, const T*
     }
 }
 
-// The + columns of W of every node, from its - columns: CTA (x, m) takes the nodes x,
-// x + gridDim.x, ... of patch m with G in shared memory; the - columns pass through it too.
+// The + columns of W of every node, from its - columns: CTA x of a patch's `per` takes the
+// nodes x, x + per, ... of the patch with G in shared memory; the - columns pass through it
+// too.  blockIdx.x numbers the CTAs patch by patch: a second grid dimension ends at 65535.
 template <class T, int RA>
-__global__ void __launch_bounds__(kKdThreads) kd_columns_kernel(KdArgs A, const T* __restrict__ blocks, T* W) {
+__global__ void __launch_bounds__(kKdThreads) kd_columns_kernel(KdArgs A, const T* __restrict__ blocks, T* W, int per) {
     extern __shared__ __align__(16) unsigned char kd_dyn[];
-    const int m = blockIdx.y, nv = A.n_v, h = nv / 2, hh = h * h, ld = h + 1;
+    const int m = blockIdx.x / per, nv = A.n_v, h = nv / 2, hh = h * h, ld = h + 1;
     T* sG = reinterpret_cast<T*>(kd_dyn);
     T* sL = sG + h * ld;   // 2 h rows: E^{-1} over -P
     const KPatchDev P = A.patches[m];
@@ -305,7 +306,7 @@ __global__ void __launch_bounds__(kKdThreads) kd_columns_kernel(KdArgs A, const 
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
     T* Wm = W + A.node_off[m] * n2;
     int held = -1;   // 0: B (the first node, where D = I), 1: G
-    for (int i = blockIdx.x; i < nn; i += gridDim.x) {
+    for (int i = blockIdx.x - m * per; i < nn; i += per) {
         T* Wi = Wm + (long long)i * n2;
         const int want = i > 0;
         __syncthreads();   // the previous node's products are done
@@ -368,14 +369,15 @@ __device__ __forceinline__ double kd_datum(const KdArgs& A, int m, int s, int l,
 // layout: [node][velocity][sample]; it holds the residual after the residual sweep and y_i
 // after the forward sweep.
 template <class T, int RJ>
-__global__ void __launch_bounds__(kKdThreads) kd_solve_kernel(KdArgs A, const T* W, T* y) {
+__global__ void __launch_bounds__(kKdThreads) kd_solve_kernel(KdArgs A, int M, const T* W, T* y) {
     extern __shared__ __align__(16) unsigned char kd_dyn[];
     __shared__ double red[32];
     __shared__ double c_v[kKdMaxNv], c_a[kKdMaxNv], c_d[kKdMaxNv];
-    const int nv = A.n_v, m = blockIdx.x, lane = threadIdx.x & (kKdG - 1), half = threadIdx.x / kKdG;
+    const int nv = A.n_v, chunk = blockIdx.x / M, m = blockIdx.x - chunk * M;   // patch fastest
+    const int lane = threadIdx.x & (kKdG - 1), half = threadIdx.x / kKdG;
     const KPatchDev P = A.patches[m];
     const int nn = P.X1 - P.X0 + 1;
-    const int s = blockIdx.y * kKdG + lane;
+    const int s = chunk * kKdG + lane;
     const bool live = s < A.S;
     const long long n2 = (long long)nv * nv, S = A.S;
     const long long base = A.node_off[m];
@@ -567,8 +569,8 @@ msp_status launch_factor(const KdArgs& A, int M, int max_nn, T* blocks, T* W, cu
     kd_chain_kernel<T, RA><<<M, kKdThreads, 4 * tile, s>>>(A, blocks, W);
     MSP_CUDA(cudaGetLastError());
     // about eight CTAs per SM over all patches
-    const int per = std::max(1, std::min(max_nn, (8 * 152 + M - 1) / M));
-    kd_columns_kernel<T, RA><<<dim3(per, M), kKdThreads, 3 * tile, s>>>(A, blocks, W);
+    const int per = std::max(1, std::min(max_nn, (8 * num_sms() + M - 1) / M));
+    kd_columns_kernel<T, RA><<<M * per, kKdThreads, 3 * tile, s>>>(A, blocks, W, per);
     MSP_CUDA(cudaGetLastError());
     count_launches(3);
     return MSP_OK;
@@ -589,8 +591,8 @@ template <class T, int RJ>
 msp_status launch_solve(const KdArgs& A, int M, const T* W, T* y, cudaStream_t s) {
     const size_t smem = sizeof(double) * 3 * A.n_v * kKdLd + sizeof(T) * A.n_v * kKdLd;
     MSP_CUDA(cudaFuncSetAttribute(kd_solve_kernel<T, RJ>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    dim3 grid(M, (A.S + kKdG - 1) / kKdG);
-    kd_solve_kernel<T, RJ><<<grid, kKdThreads, smem, s>>>(A, W, y);
+    // M x chunks CTAs: the iterate alone, 32 bytes or more a (patch, sample), keeps them below 2^31
+    kd_solve_kernel<T, RJ><<<M * ((A.S + kKdG - 1) / kKdG), kKdThreads, smem, s>>>(A, M, W, y);
     count_launches(1);
     MSP_CUDA(cudaGetLastError());
     return MSP_OK;
