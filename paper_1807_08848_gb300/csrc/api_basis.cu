@@ -26,8 +26,7 @@ extern "C" msp_status msp_extract_basis(msp_medium m, double tau, int precision,
 
 extern "C" void msp_basis_destroy(msp_basis b) {
     if (!b) return;
-    wait_for_device();
-    delete b;
+    destroy_handle(b, b->B.device, "msp_basis_destroy");
 }
 
 extern "C" msp_status msp_basis_info(msp_basis b, int patch, int* k, double* sigma_host) {

@@ -53,8 +53,6 @@ int num_sms() {
     return n;
 }
 
-void wait_for_device() { cudaDeviceSynchronize(); }
-
 cudaError_t pool_alloc(void** p, size_t bytes, cudaStream_t s) {
     struct DevicePool {
         cudaMemPool_t pool = nullptr;
@@ -308,11 +306,7 @@ extern "C" msp_status msp_build_medium_full(const msp_medium_desc* d, const msp_
 
 extern "C" void msp_medium_destroy(msp_medium m) {
     if (!m) return;
-    wait_for_device();
-    for (auto& g : m->M.graph)
-        if (g) cudaGraphExecDestroy(g);
-    if (m->M.capture_stream) cudaStreamDestroy(m->M.capture_stream);
-    delete m;
+    destroy_handle(m, m->M.device, "msp_medium_destroy");
 }
 
 extern "C" msp_status msp_medium_counts(msp_medium m, int* n_patches, int64_t* snapshot_elems, int* n_cells) {

@@ -10,6 +10,7 @@
 
 #include "../../include/msp.h"
 #include "dense.cuh"
+#include "handle.h"
 
 namespace msp {
 
@@ -32,11 +33,15 @@ msp_status cuda_fail(cudaError_t e, const char* what, const char* file, int line
 #define MSP_TRY(call)                                                               \
     do { msp_status s_ = (call); if (s_ != MSP_OK) return s_; } while (0)
 
-// Waits for every kernel of the current device: called before a handle's buffers
-// go back to the pool.  cudaFree of a stream-ordered allocation takes its accesses
-// to be complete and waits for nothing, while a call that only enqueues (a solve
-// without iteration counts, a snapshot copy) may still be running.
-void wait_for_device();
+// release_handle (handle.h) for a *_destroy entry point; a handle that has to stay is reported
+// in msp_last_error.
+template <class Handle>
+void destroy_handle(Handle* h, int device, const char* who) {
+    const cudaError_t e = release_handle(h, device);
+    if (e != cudaSuccess)
+        set_error(std::string(who) + ": the device could not be waited for, the handle's memory stays allocated: " +
+                  cudaGetErrorString(e));
+}
 
 // Stream-ordered allocation from the library's pool of the current device (freed with
 // cudaFree).  The default pool gives its free memory back at every synchronisation, and
@@ -196,6 +201,11 @@ struct Medium {
     cudaStream_t capture_stream = nullptr;
     double graph_key[2][6] = {};
     long long graph_launches[2] = {0, 0};   // kernel launches one replay of the graph makes
+    ~Medium() {
+        for (cudaGraphExec_t g : graph)
+            if (g) cudaGraphExecDestroy(g);
+        if (capture_stream) cudaStreamDestroy(capture_stream);
+    }
 };
 
 // Ring node t of node box (X0,X1,Y0,Y1): counter-clockwise from (X0,Y0).

@@ -44,6 +44,7 @@ struct KBasis {
     DevBuf<long long> d_l_off, d_c_blk_off;
     int k_max = 0;
     int max_sweeps = 0, max_tries = 0;
+    int device = 0;
 };
 
 }  // namespace msp
@@ -434,8 +435,11 @@ extern "C" msp_status msp_kinetic_build_hg(int n_cells, double eps, double g, in
         set_error("msp_kinetic_build: no usable CUDA device");
         return MSP_ERR_CUDA;
     }
+    int device = 0;
+    MSP_CUDA(cudaGetDevice(&device));
     auto* h = new msp_kmedium_s();
     KMedium& K = h->K;
+    K.device = device;
     K.N = n_cells; K.eps = eps; K.g = g; K.n_v = n_v; K.M = n_patches; K.buffer = buffer; K.S = samples;
     K.solver = (g == 0.0) ? MSP_KINETIC_SOURCE_ITERATION : MSP_KINETIC_DIRECT;
     gauss_legendre(n_v, K.v, K.w);
@@ -481,8 +485,7 @@ extern "C" msp_status msp_kinetic_build_hg(int n_cells, double eps, double g, in
 
 extern "C" void msp_kinetic_destroy(msp_kmedium k) {
     if (!k) return;
-    wait_for_device();
-    delete k;
+    destroy_handle(k, k->K.device, "msp_kinetic_destroy");
 }
 
 extern "C" msp_status msp_kinetic_velocities(msp_kmedium k, double* v_host, double* w_host) {
@@ -581,6 +584,7 @@ extern "C" msp_status msp_kinetic_extract(msp_kmedium km, double tau, void* stre
     auto* h = new msp_kbasis_s();
     KBasis& B = h->B;
     B.N = K.N; B.n_v = K.n_v; B.M = K.M; B.v = K.v; B.patches = K.patches;
+    B.device = K.device;
     std::vector<long long> soff(K.M);
     std::vector<int> rows(K.M), cols(K.M);
     for (int m = 0; m < K.M; ++m) {
@@ -632,8 +636,7 @@ extern "C" msp_status msp_kinetic_extract(msp_kmedium km, double tau, void* stre
 
 extern "C" void msp_kinetic_basis_destroy(msp_kbasis b) {
     if (!b) return;
-    wait_for_device();
-    delete b;
+    destroy_handle(b, b->B.device, "msp_kinetic_basis_destroy");
 }
 
 extern "C" msp_status msp_kinetic_basis_info(msp_kbasis b, int patch, int* k, double* sigma_host) {

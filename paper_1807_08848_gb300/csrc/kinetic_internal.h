@@ -42,6 +42,7 @@ struct KMedium {
     long long snap_elems = 0;
     DevBuf<int> stats;    // per (patch, sample): iterations, flag
     bool sampled = false;
+    int device = 0;
     KDirect D;
 };
 
