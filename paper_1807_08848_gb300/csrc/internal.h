@@ -57,8 +57,11 @@ struct DevBuf {
     size_t n = 0;
     // A request beyond the device's whole memory is refused before the call (free
     // memory is no test: the stream-ordered pool may serve a request from memory it
-    // holds).
+    // holds).  A buffer that is replaced (a work space growing between calls) may still be in
+    // use by an earlier call that only enqueued, on this stream or another: the device is waited
+    // for before it goes back to the pool.  A caller that knows its users are done frees it first.
     msp_status alloc(size_t count, cudaStream_t s) {
+        if (p) MSP_CUDA(cudaDeviceSynchronize());
         free_now();
         if (count == 0) return MSP_OK;
         const size_t bytes = count * sizeof(T);

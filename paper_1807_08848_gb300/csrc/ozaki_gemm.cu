@@ -581,11 +581,18 @@ msp_status ozaki_gemm_batched(const std::vector<GemmDesc>& h, const GemmDesc* d_
     const bool one = batch == 1;
     const bool grow = (long long)w.slices.n < sl || (long long)w.scales.n < sc || (!one && w.ents.n < ent_words);
     // products of earlier calls may still be queued on the stream and read these
-    // buffers: they finish before a buffer is given up for a larger one
+    // buffers: they finish before a buffer is given up for a larger one.  A work space is used on
+    // one stream, so that one is waited for and not the device (the factorisation's other stream
+    // goes on).
     if (grow) MSP_CUDA(cudaStreamSynchronize(s));
-    if ((long long)w.slices.n < sl) MSP_TRY(w.slices.alloc((size_t)sl, s));
-    if ((long long)w.scales.n < sc) MSP_TRY(w.scales.alloc((size_t)sc, s));
-    if (!one && w.ents.n < ent_words) MSP_TRY(w.ents.alloc(ent_words, s));
+    auto renew = [s](auto& buf, size_t n) -> msp_status {
+        if (buf.n >= n) return MSP_OK;
+        buf.free_now();
+        return buf.alloc(n, s);
+    };
+    MSP_TRY(renew(w.slices, (size_t)sl));
+    MSP_TRY(renew(w.scales, (size_t)sc));
+    if (!one) MSP_TRY(renew(w.ents, ent_words));
     if (!w.err.p) {
         MSP_TRY(w.err.alloc(1, s));
         MSP_CUDA(cudaMemsetAsync(w.err.p, 0, sizeof(int), s));
