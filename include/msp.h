@@ -43,6 +43,11 @@
  *  - Handles (msp_medium, msp_basis, msp_kmedium, msp_kbasis, msp_server) are
  *    opaque and own device memory allocated by the library (stream-ordered);
  *    free them with the matching *_destroy.
+ *  - The library allocates from a memory pool of its own, one per device, that
+ *    keeps up to an eighth of the device's memory between calls so that the
+ *    next call does not map it again.  It is emptied before a request of the
+ *    library is refused; other allocators of the process (PyTorch's, cudaMalloc)
+ *    cannot use what it keeps until msp_trim_memory gives it back.
  *  - Fine grid: N cells per side, n = N+1 nodes, h = 1/N, node (i, j) at
  *    (ih, jh), grids row-major with i fastest.  Face coefficients:
  *    aE[j][i] = a((i+1/2)h, jh), (N+1) x N;  aN[j][i] = a(ih, (j+1/2)h),
@@ -161,6 +166,12 @@ int64_t msp_kernel_launches(void);
  * every launch.  polls = 0 restores the default (2^24 polls, tens of seconds);
  * INVALID_ARG if polls < 0.  Small values are for tests of the timeout path. */
 msp_status msp_set_wait_limit(int64_t polls);
+
+/* Gives memory of the current device that the library's pool keeps back to the
+ * device, down to keep_bytes (0: all of it).  Memory of live handles stays.
+ * Synchronises the device.  The pool fills again with the next calls.
+ * INVALID_ARG if keep_bytes < 0, CUDA without a usable device. */
+msp_status msp_trim_memory(int64_t keep_bytes);
 
 /* Engine of the FP64 matrix products inside msp_extract_basis (the Gram and
  * triangular products of Cholesky-QR, the projection onto the singular vectors)

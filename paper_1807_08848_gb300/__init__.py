@@ -21,7 +21,7 @@ from . import _native as N
 from ._native import MspError, MSP_FP64, MSP_MIXED
 
 __all__ = ["Medium", "Basis", "Server", "KineticMedium", "KineticBasis", "MspError", "MSP_FP64", "MSP_MIXED", "load_library",
-           "precision_code", "set_wait_limit", "set_gemm_engine", "set_extract_timing", "set_svd_mode"]
+           "precision_code", "set_wait_limit", "trim_memory", "set_gemm_engine", "set_extract_timing", "set_svd_mode"]
 
 
 def load_library():
@@ -32,6 +32,13 @@ def set_wait_limit(polls: int = 0):
     """Poll bound of the device-side grid barriers (msp_set_wait_limit); 0 restores
     the default."""
     N.check(N.load().msp_set_wait_limit(int(polls)))
+
+
+def trim_memory(keep_bytes: int = 0):
+    """Give the device memory that the library's pool keeps between calls (up to an
+    eighth of the device) back, down to keep_bytes: other allocators of the process,
+    PyTorch's among them, can then use it.  Live handles keep theirs (msp_trim_memory)."""
+    N.check(N.load().msp_trim_memory(int(keep_bytes)))
 
 
 def set_extract_timing(enable: bool = True):

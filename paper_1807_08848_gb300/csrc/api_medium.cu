@@ -53,43 +53,54 @@ int num_sms() {
     return n;
 }
 
-cudaError_t pool_alloc(void** p, size_t bytes, cudaStream_t s) {
-    struct DevicePool {
-        cudaMemPool_t pool = nullptr;
-        size_t total = 0;
-    };
+namespace {
+
+struct DevicePool {
+    cudaMemPool_t pool = nullptr;
+    size_t total = 0;
+};
+
+// The current device's pool, created on its first allocation; create = false: as it is
+// (pool null before that).
+cudaError_t device_pool(bool create, DevicePool* out) {
     static std::mutex mu;
     static std::vector<DevicePool> pools;   // per device; never destroyed (at exit the CUDA driver may be gone)
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
-    DevicePool d;
-    {
-        std::lock_guard<std::mutex> lock(mu);
-        if ((int)pools.size() <= dev) pools.resize(dev + 1);
-        if (!pools[dev].pool) {
-            size_t free_b = 0, total_b = 0;
-            e = cudaMemGetInfo(&free_b, &total_b);
-            if (e != cudaSuccess) return e;
-            cudaMemPoolProps props{};
-            props.allocType = cudaMemAllocationTypePinned;
-            props.handleTypes = cudaMemHandleTypeNone;
-            props.location.type = cudaMemLocationTypeDevice;
-            props.location.id = dev;
-            cudaMemPool_t pool = nullptr;
-            e = cudaMemPoolCreate(&pool, &props);
-            if (e != cudaSuccess) return e;
-            uint64_t keep = (uint64_t)total_b / 8;
-            e = cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
-            if (e != cudaSuccess) {
-                cudaMemPoolDestroy(pool);
-                return e;
-            }
-            pools[dev].pool = pool;
-            pools[dev].total = total_b;
+    std::lock_guard<std::mutex> lock(mu);
+    if ((int)pools.size() <= dev) pools.resize(dev + 1);
+    if (!pools[dev].pool && create) {
+        size_t free_b = 0, total_b = 0;
+        e = cudaMemGetInfo(&free_b, &total_b);
+        if (e != cudaSuccess) return e;
+        cudaMemPoolProps props{};
+        props.allocType = cudaMemAllocationTypePinned;
+        props.handleTypes = cudaMemHandleTypeNone;
+        props.location.type = cudaMemLocationTypeDevice;
+        props.location.id = dev;
+        cudaMemPool_t pool = nullptr;
+        e = cudaMemPoolCreate(&pool, &props);
+        if (e != cudaSuccess) return e;
+        uint64_t keep = (uint64_t)total_b / 8;
+        e = cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
+        if (e != cudaSuccess) {
+            cudaMemPoolDestroy(pool);
+            return e;
         }
-        d = pools[dev];
+        pools[dev].pool = pool;
+        pools[dev].total = total_b;
     }
+    *out = pools[dev];
+    return cudaSuccess;
+}
+
+}  // namespace
+
+cudaError_t pool_alloc(void** p, size_t bytes, cudaStream_t s) {
+    DevicePool d;
+    cudaError_t e = device_pool(true, &d);
+    if (e != cudaSuccess) return e;
     if (bytes > d.total) return cudaErrorMemoryAllocation;
     for (int attempt = 0; attempt < 2; ++attempt) {
         *p = nullptr;
@@ -149,6 +160,18 @@ extern "C" msp_status msp_set_gemm_engine(int engine) {
 extern "C" msp_status msp_set_extract_timing(int enable) {
     clear_error();
     g_extract_timing.store(enable != 0 ? 1 : 0, std::memory_order_relaxed);
+    return MSP_OK;
+}
+
+extern "C" msp_status msp_trim_memory(int64_t keep_bytes) {
+    clear_error();
+    MSP_CHECK_ARG(keep_bytes >= 0, "msp_trim_memory: keep_bytes must be >= 0");
+    MSP_TRY(need_device());
+    DevicePool d;
+    MSP_CUDA(device_pool(false, &d));
+    if (!d.pool) return MSP_OK;
+    MSP_CUDA(cudaDeviceSynchronize());   // pending frees complete
+    MSP_CUDA(cudaMemPoolTrimTo(d.pool, (size_t)keep_bytes));
     return MSP_OK;
 }
 

@@ -47,7 +47,7 @@ void destroy_handle(Handle* h, int device, const char* who) {
 // cudaFree).  The default pool gives its free memory back at every synchronisation, and
 // mapping it again took a third of a pass that builds a new medium; this pool keeps up to
 // an eighth of the device's memory between calls, gives the rest back, and is emptied
-// before a request is refused.
+// before a request is refused and by msp_trim_memory.
 cudaError_t pool_alloc(void** p, size_t bytes, cudaStream_t s);
 
 // Stream-ordered device buffer owned by a handle.
