@@ -4,6 +4,7 @@
 #include <algorithm>
 #include <atomic>
 #include <cstring>
+#include <map>
 #include <mutex>
 #include <numeric>
 
@@ -51,6 +52,23 @@ int num_sms() {
     if (cudaGetDevice(&dev) != cudaSuccess) return 1;
     if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0) return 1;
     return n;
+}
+
+msp_status allow_smem_of(const void* kernel, size_t bytes) {
+    static std::mutex mu;
+    static std::map<std::pair<int, const void*>, size_t> limits;   // per device and kernel
+    int dev = 0;
+    MSP_CUDA(cudaGetDevice(&dev));
+    std::lock_guard<std::mutex> lock(mu);
+    const auto it = limits.find({dev, kernel});
+    if (it != limits.end() && bytes <= it->second) return MSP_OK;
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    if (e != cudaSuccess) {
+        (void)cudaGetLastError();
+        return cuda_fail(e, "dynamic shared memory limit", __FILE__, __LINE__);
+    }
+    limits[{dev, kernel}] = bytes;
+    return MSP_OK;
 }
 
 namespace {

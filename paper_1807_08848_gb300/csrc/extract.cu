@@ -566,7 +566,7 @@ msp_status svd_bases(const double* snaps, long long snap_elems, const std::vecto
             while (2LL * (c32 + 1) * (c32 + 2) * (long long)sizeof(float) <= dyn_max) ++c32;
             c32 = std::min(c32, maxc);
             const size_t sm32 = 2 * (size_t)c32 * (c32 + 1) * sizeof(float);
-            MSP_CUDA(cudaFuncSetAttribute(jacobi_svd32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm32));
+            MSP_TRY(allow_smem(jacobi_svd32_kernel, sm32));
             // FP32 scratch of the blocks too large for shared memory (2 c^2 floats
             // each): the second Cholesky-QR output buffer, free now, when it holds
             // them all (sum of c^2 <= sum of n c doubles)
@@ -630,7 +630,7 @@ msp_status svd_bases(const double* snaps, long long snap_elems, const std::vecto
         while ((long long)(c64 + 1) * (c64 + 2) * (long long)sizeof(double) <= dyn_max) ++c64;
         c64 = std::min(c64, maxc);
         const size_t sm64 = (size_t)c64 * (c64 + 1) * sizeof(double);
-        MSP_CUDA(cudaFuncSetAttribute(jacobi_svd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm64));
+        MSP_TRY(allow_smem(jacobi_svd_kernel, sm64));
         if (!rest.empty()) {
             jacobi_svd_kernel<<<(int)rest.size(), 512, sm64, s>>>(d_rest.p, W.p, V.p, 40, maxc * 1.12e-16, small_rel, c64,
                                                                   sweeps.p);

@@ -43,6 +43,15 @@ void destroy_handle(Handle* h, int device, const char* who) {
                   cudaGetErrorString(e));
 }
 
+// Lets launches of `kernel` ask for `bytes` of dynamic shared memory on the current device.
+// The limit is the process's, not the launch's: it is only ever raised, so that no call
+// takes it from another thread's launch between that thread's call and its launch.
+msp_status allow_smem_of(const void* kernel, size_t bytes);
+template <class... Args>
+msp_status allow_smem(void (*kernel)(Args...), size_t bytes) {
+    return allow_smem_of(reinterpret_cast<const void*>(kernel), bytes);
+}
+
 // Stream-ordered allocation from the library's pool of the current device (freed with
 // cudaFree).  The default pool gives its free memory back at every synchronisation, and
 // mapping it again took a third of a pass that builds a new medium; this pool keeps up to

@@ -542,10 +542,10 @@ extern "C" msp_status msp_kinetic_sample(msp_kmedium k, uint64_t seed, int preci
     const size_t smem = per * G;
     dim3 grid(K.M, (K.S + G - 1) / G);
     if (mixed) {
-        MSP_CUDA(cudaFuncSetAttribute(kinetic_si_mixed_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        MSP_TRY(allow_smem(kinetic_si_mixed_kernel, smem));
         kinetic_si_mixed_kernel<<<grid, G * K.n_v, smem, s>>>(A);
     } else {
-        MSP_CUDA(cudaFuncSetAttribute(kinetic_si_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        MSP_TRY(allow_smem(kinetic_si_kernel, smem));
         kinetic_si_kernel<<<grid, G * K.n_v, smem, s>>>(A);
     }
     count_launches(1);

@@ -562,8 +562,8 @@ template <class T, int RA>
 msp_status launch_factor(const KdArgs& A, int M, int max_nn, T* blocks, T* W, cudaStream_t s) {
     const int h = A.n_v / 2;
     const size_t tile = sizeof(T) * h * (h + 1);
-    MSP_CUDA(cudaFuncSetAttribute(kd_chain_kernel<T, RA>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(4 * tile)));
-    MSP_CUDA(cudaFuncSetAttribute(kd_columns_kernel<T, RA>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(3 * tile)));
+    MSP_TRY(allow_smem(kd_chain_kernel<T, RA>, 4 * tile));
+    MSP_TRY(allow_smem(kd_columns_kernel<T, RA>, 3 * tile));
     kd_blocks_kernel<T><<<1, 1024, sizeof(double) * h * h, s>>>(A, blocks);
     MSP_CUDA(cudaGetLastError());
     kd_chain_kernel<T, RA><<<M, kKdThreads, 4 * tile, s>>>(A, blocks, W);
@@ -590,7 +590,7 @@ msp_status factor(const KMedium& K, const KdArgs& A, DevBuf<T>& blocks, T* W, cu
 template <class T, int RJ>
 msp_status launch_solve(const KdArgs& A, int M, const T* W, T* y, cudaStream_t s) {
     const size_t smem = sizeof(double) * 3 * A.n_v * kKdLd + sizeof(T) * A.n_v * kKdLd;
-    MSP_CUDA(cudaFuncSetAttribute(kd_solve_kernel<T, RJ>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    MSP_TRY(allow_smem(kd_solve_kernel<T, RJ>, smem));
     // M x chunks CTAs: the iterate alone, 32 bytes or more a (patch, sample), keeps them below 2^31
     kd_solve_kernel<T, RJ><<<M * ((A.S + kKdG - 1) / kKdG), kKdThreads, smem, s>>>(A, M, W, y);
     count_launches(1);

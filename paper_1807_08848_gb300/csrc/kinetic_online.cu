@@ -433,7 +433,7 @@ msp_status kinetic_factor(const KOnArgs& A, const std::vector<int>& k, const std
     MSP_TRY(fail.alloc(1, s));
     if (A.k_max <= kKfMaxK) {
         const size_t smem = sizeof(double) * std::max<size_t>((size_t)A.k_max * (A.k_max | 1), kKfChunk + A.k_max);
-        MSP_CUDA(cudaFuncSetAttribute(kinetic_chain_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        MSP_TRY(allow_smem(kinetic_chain_kernel, smem));
         cudaLaunchConfig_t cfg{};
         cfg.gridDim = dim3(kPatchCluster);
         cfg.blockDim = dim3(kKfThreads);

@@ -789,7 +789,7 @@ msp_status mark(Medium::Direct& D, int ph, bool begin, cudaStream_t s) {
 
 template <int G, int CPW>
 msp_status launch_solve_g(const DirArgs& A, int grid, int smem, cudaStream_t s) {
-    MSP_CUDA(cudaFuncSetAttribute(direct_solve_kernel<G, CPW>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    MSP_TRY(allow_smem(direct_solve_kernel<G, CPW>, smem));
     direct_solve_kernel<G, CPW><<<grid, kDirThreads, smem, s>>>(A);
     count_launches(1);
     return MSP_OK;
@@ -818,7 +818,7 @@ bool direct_fits(const Medium& M) {
 
 template <int TS>
 static msp_status launch_factor(const DirArgs& A, int np, int smem, cudaStream_t s) {
-    MSP_CUDA(cudaFuncSetAttribute(direct_factor_kernel<TS>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    MSP_TRY(allow_smem(direct_factor_kernel<TS>, smem));
     direct_factor_kernel<TS><<<np, kDirThreads, smem, s>>>(A);
     return MSP_OK;
 }

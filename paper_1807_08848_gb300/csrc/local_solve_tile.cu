@@ -457,8 +457,7 @@ int rows_instance(int rps) {
 
 template <class T, int RPS, bool FUSED = false>
 msp_status launch_rps(const TileArgs& A, int grid, size_t smem, cudaStream_t s) {
-    MSP_CUDA(cudaFuncSetAttribute(local_solve_tile<T, RPS, false, FUSED>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)smem));
+    MSP_TRY(allow_smem(local_solve_tile<T, RPS, false, FUSED>, smem));
     local_solve_tile<T, RPS, false, FUSED><<<grid, kTileThreads, smem, s>>>(A);
     count_launches(1);
     MSP_CUDA(cudaGetLastError());
@@ -684,8 +683,7 @@ extern "C" msp_status msp_sample_patch_static(const double* aE_dev, const double
     const int grid = (int)std::max<long long>(1, std::min<long long>({(long long)samples, slots, (long long)num_sms()}));
 #define MSP_STATIC_LAUNCH(T, RR)                                                                                   \
     do {                                                                                                           \
-        MSP_CUDA(cudaFuncSetAttribute(local_solve_tile<T, RR, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,   \
-                                      (int)smem));                                                                 \
+        MSP_TRY(allow_smem(local_solve_tile<T, RR, true>, smem));                                                  \
         local_solve_tile<T, RR, true><<<grid, kTileThreads, smem, s>>>(A);                                          \
     } while (0)
     if (mixed) {

@@ -758,9 +758,7 @@ static msp_status online_batch(Basis& Bs, const double* phi, int B, double tol, 
         max_k = std::max(max_k, Bs.k[m]);
     }
     const size_t smem = sizeof(double) * ((size_t)max_ns * B + (size_t)max_k * B);
-    if (smem > 48 * 1024) {
-        MSP_CUDA(cudaFuncSetAttribute(normal_precond_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    }
+    MSP_TRY(allow_smem(normal_precond_kernel, smem));
     if (Bs.w_s.n < (size_t)nc) MSP_TRY(Bs.w_s.alloc((size_t)std::max(Bs.Np, 1) * kMaxBatch, s));
     // z = M^{-1} P~^T r and the partial sums (s.z, s.s): block-row factor when built,
     // patch-block (additive Schwarz) inverses otherwise

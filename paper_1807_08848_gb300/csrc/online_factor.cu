@@ -1313,7 +1313,7 @@ msp_status launch_sweeps_bt(SweepArgs<T> A, int max_n, cudaStream_t s) {
         std::lock_guard<std::mutex> lock(mu);
         if ((int)grids.size() <= dev) grids.resize(dev + 1, 0);
         if (grids[dev] == 0) {
-            MSP_CUDA(cudaFuncSetAttribute(sweep_kernel<T, BT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+            MSP_TRY(allow_smem(sweep_kernel<T, BT>, smem));
             int occ = 0;
             MSP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, sweep_kernel<T, BT>, 512, smem));
             if (occ < 1) {

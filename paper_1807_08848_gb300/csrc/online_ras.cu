@@ -721,7 +721,7 @@ msp_status ras_setup(Basis& Bs, const Medium& F, bool coarse, cudaStream_t s) {
         ras_aug_init_kernel<<<ew_grid(2LL * M * M), 256, 0, s>>>(R->aug.p, M);
         const RasArgs A = ras_args(Bs, *R, 1);
         const size_t smem = sizeof(double) * ((size_t)R->max_ring + R->max_patch_ents);
-        MSP_CUDA(cudaFuncSetAttribute(ras_coarse_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        MSP_TRY(allow_smem(ras_coarse_kernel, smem));
         ras_coarse_kernel<<<M, 256, smem, s>>>(A, R->z.p, d_nb_ptr.p, d_nb_patch.p, d_nb.p, R->aug.p);
         count_launches(3);
         DevBuf<double> col;
@@ -783,7 +783,7 @@ static msp_status ras_batch(Basis& Bs, RasOnline& R, const double* phi, int B, d
     const long long nb = (long long)Np * B;
     const RasArgs A = ras_args(Bs, R, B);
     const size_t smem = sizeof(double) * ((size_t)R.max_ring * B + (size_t)std::max(kRasThreads, R.max_k));
-    MSP_CUDA(cudaFuncSetAttribute(ras_bm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    MSP_TRY(allow_smem(ras_bm_kernel, smem));
     const int ring_grid = std::max(1, std::min((R.n_ring_tot + 31) / 32, num_sms() * 16));
     auto apply = [&](const double* x, const double* a, double* out, int mode) {
         ras_ring_kernel<<<ring_grid, kRasThreads, 0, s>>>(A, R.n_ring_tot, x, phi, n4, R.gv.p, mode);

@@ -606,7 +606,7 @@ msp_status ozaki_gemm_batched(const std::vector<GemmDesc>& h, const GemmDesc* d_
     auto launch = [&](auto tables, int nb) -> msp_status {
         using Batch = decltype(tables);
         const int smem = kStages * (int)kStageBytes;
-        MSP_CUDA(cudaFuncSetAttribute(oz_mma_kernel<Batch>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+        MSP_TRY(allow_smem(oz_mma_kernel<Batch>, smem));
         oz_scale_kernel<Batch><<<dim3(ra + rb, nb), 256, 0, s>>>(tables, transA, transB, w.scales.p, ra);
         oz_slice_kernel<Batch><<<dim3(ga + gb, nb), 256, 0, s>>>(tables, transA, transB, w.scales.p, slices, (unsigned)ga);
         OzArgs<Batch> a{};

@@ -782,7 +782,7 @@ __global__ void __launch_bounds__(kJacThreads, 3) patch_jacobi_kernel(JacArgs A)
 template <class... KArgs, class... Args>
 msp_status launch_cluster(void (*kernel)(KArgs...), int patches, int nc, int threads, size_t smem, cudaStream_t s,
                           Args... args) {
-    MSP_CUDA(cudaFuncSetAttribute((const void*)kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    MSP_TRY(allow_smem(kernel, smem));
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)(patches * nc));
     cfg.blockDim = dim3((unsigned)threads);
@@ -845,7 +845,7 @@ static msp_status launch_inverse(const PatchClasses& C, int c, const PatchBlock*
     int tr = 16;
     auto bytes = [&](int t) { return sizeof(double) * ((size_t)t * (c + kCols + 1) + (size_t)kCols * c); };
     while (tr > 1 && bytes(tr) > room) tr /= 2;
-    MSP_CUDA(cudaFuncSetAttribute(patch_inverse_kernel<CPW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes(tr)));
+    MSP_TRY(allow_smem(patch_inverse_kernel<CPW>, bytes(tr)));
     for (size_t b0 = 0; b0 < C.blocks.size(); b0 += 65535) {
         const unsigned nb = (unsigned)std::min<size_t>(65535, C.blocks.size() - b0);
         patch_inverse_kernel<CPW><<<dim3((c + kCols - 1) / kCols, nb), 32 * kWarps, bytes(tr), s>>>(blocks + b0, L, F, Fi,
@@ -906,7 +906,7 @@ msp_status patch_qrcp(const PatchClasses& C, const PatchBlock* blocks, const dou
     const int c = std::max(C.max_c[0], C.max_c[1]);
     if (c > 0) {
         const size_t bytes = sizeof(double) * (size_t)kFormWarps * c;
-        MSP_CUDA(cudaFuncSetAttribute(patch_form_q_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+        MSP_TRY(allow_smem(patch_form_q_kernel, bytes));
         for (size_t b0 = 0; b0 < C.blocks.size(); b0 += 65535) {
             const unsigned nb = (unsigned)std::min<size_t>(65535, C.blocks.size() - b0);
             patch_form_q_kernel<<<dim3((c + kFormWarps - 1) / kFormWarps, nb), 32 * kFormWarps, bytes, s>>>(blocks + b0, R, Q);
@@ -993,7 +993,7 @@ msp_status patch_jacobi(const std::vector<PatchBlock>& all, double* W, double* V
     // more than 8 CTAs in a cluster are an option of the device: ask whether one can be resident
     int max_nc = kPatchCluster;
     MSP_CUDA(cudaFuncSetAttribute(patch_jacobi_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-    MSP_CUDA(cudaFuncSetAttribute(patch_jacobi_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)room));
+    MSP_TRY(allow_smem(patch_jacobi_kernel, room));
     for (int q = 0; q < kJacSizes && kJacNc[q] > max_nc; ++q) {
         cudaLaunchConfig_t cfg{};
         cfg.gridDim = dim3((unsigned)kJacNc[q]);

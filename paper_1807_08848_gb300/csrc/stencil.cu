@@ -299,7 +299,7 @@ __global__ void __launch_bounds__(512) stencil_apply_kernel(StencilArgs A) {
 
 template <class T>
 msp_status launch_apply(const StencilArgs& A, int grid, size_t smem, cudaStream_t s) {
-    MSP_CUDA(cudaFuncSetAttribute(stencil_apply_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    MSP_TRY(allow_smem(stencil_apply_kernel<T>, smem));
     stencil_apply_kernel<T><<<grid, 512, smem, s>>>(A);
     return MSP_OK;
 }
@@ -309,7 +309,7 @@ msp_status launch_stream(const StencilArgs& A, size_t tile_bytes, cudaStream_t s
     // as many tile buffers as fit, at most eight
     const int nb = (int)std::min<size_t>(8, (227 * 1024 - 256) / tile_bytes);
     const size_t smem = nb * tile_bytes;
-    MSP_CUDA(cudaFuncSetAttribute(stencil_stream_kernel<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    MSP_TRY(allow_smem(stencil_stream_kernel<R>, smem));
     int occ = 0;
     MSP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, stencil_stream_kernel<R>, 512, smem));
     const long long grid = std::min((long long)A.n_patches * A.S, (long long)num_sms() * std::max(1, occ));

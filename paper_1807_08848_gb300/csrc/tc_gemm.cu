@@ -322,11 +322,7 @@ void tc_tile_split(const float* X, long long ld_r, long long ld_k, int rows, int
 
 msp_status tc_map_gemm(const TcMapArgs& args, cudaStream_t s) {
     const size_t smem = (size_t)kStages * kStageBytes;
-    static bool attr = false;
-    if (!attr) {
-        MSP_CUDA(cudaFuncSetAttribute(tc_map_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        attr = true;
-    }
+    MSP_TRY(allow_smem(tc_map_gemm_kernel, smem));
     dim3 grid(tc_row_tiles(args.M), tc_n_tiles(args.B));
     tc_map_gemm_kernel<<<grid, 128, smem, s>>>(args);
     count_launches(1);
