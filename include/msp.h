@@ -205,7 +205,7 @@ msp_status msp_set_gemm_engine(int engine);
  *     T P = Q R in FP64 first (Drmac and Veselic 2008), then FP64 sweeps on the
  *     columns of R^T with V started at Q: the rows of R decay with the pivots,
  *     so the sweeps start from graded, nearly orthogonal columns (measured at
- *     2049^2: 46 ms of QR and 229 ms of sweeps, at most 10 and 6.3 on average,
+ *     2049^2: 37 ms of QR and 229 ms of sweeps, at most 10 and 6.3 on average,
  *     against 370 ms and 20 / 8.1 sweeps from V = I).
  * Both end at the same FP64 stopping test; process-wide, read by every
  * extraction.  INVALID_ARG on an unknown mode. */

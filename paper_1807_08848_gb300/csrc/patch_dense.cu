@@ -456,6 +456,148 @@ __global__ void __launch_bounds__(32 * kFormWarps) patch_form_q_kernel(const Pat
     for (int i = lane; i < c; i += 32) Q[P.off + (size_t)k * c + i] = q[i];
 }
 
+// The same factorisation by one CTA per patch, with Q: the columns live in shared memory (or in
+// W, orders above smem_c, which R^T overwrites at the end either way), are swapped into
+// place, and the reflectors are applied to Q where they lie.  Every element takes the
+// operations of the two kernels above in their order.  Bound by FP64 issue: what a patch has
+// less of than on a cluster is SMs, so this form is for batches that keep them all busy; both
+// sides' times stand at the rule in patch_qrcp.
+constexpr int kQrMaxCols = 1024;    // the extraction's largest order
+__global__ void __launch_bounds__(kQrThreads) patch_qr_one_kernel(const PatchBlock* blocks, const double* Tm, double* W,
+                                                                  double* Q, int smem_c) {
+    extern __shared__ __align__(16) double osm[];
+    __shared__ double s_nrm[kQrMaxCols];
+    __shared__ double s_tau[kQrMaxCols];
+    __shared__ int s_piv;
+    const PatchBlock S = blocks[blockIdx.x];
+    const int c = S.c;
+    if (c < 1 || c > kQrMaxCols) return;
+    const bool in_smem = c <= smem_c;
+    const int lda = in_smem ? c + 1 : c;
+    double* a = in_smem ? osm : W + S.off;
+    double* q = Q + S.off;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    for (long long e = threadIdx.x; e < (long long)c * c; e += blockDim.x) {
+        const int i = (int)(e % c), j = (int)(e / c);
+        a[i + (long long)j * lda] = Tm[S.off + e];
+    }
+    __syncthreads();
+    for (int j = 0; j < c; ++j) {
+        // squared norms of columns j.. over rows j..
+        for (int col = j + warp; col < c; col += nw) {
+            const double* ac = a + (long long)col * lda;
+            double t = 0.0;
+            for (int i = j + lane; i < c; i += 32) t = fma(ac[i], ac[i], t);
+            t = warp_sum(t);
+            if (lane == 0) s_nrm[col] = t;
+        }
+        __syncthreads();
+        if (warp == 0) {
+            double best = -1.0;
+            int bi = j;
+            for (int col = j + lane; col < c; col += 32)
+                if (s_nrm[col] > best) { best = s_nrm[col]; bi = col; }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                const double ob = __shfl_xor_sync(0xffffffffu, best, o);
+                const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
+                if (ob > best || (ob == best && oi < bi)) { best = ob; bi = oi; }
+            }
+            if (lane == 0) s_piv = bi;
+        }
+        __syncthreads();
+        const int p = s_piv;
+        if (p != j) {
+            for (int i = threadIdx.x; i < c; i += blockDim.x) {
+                const double x = a[i + (long long)j * lda];
+                a[i + (long long)j * lda] = a[i + (long long)p * lda];
+                a[i + (long long)p * lda] = x;
+            }
+        }
+        __syncthreads();
+        // reflector of column j: beta = -sign(alpha) |x|, tau = (beta - alpha) / beta,
+        // v = x(1:) / (alpha - beta) below the diagonal, R(j, j) = beta; the squared
+        // norm below the diagonal is summed afresh (a difference of the column norm
+        // and alpha^2 could cancel, and tau must match v for H_j to be orthogonal)
+        double* aj = a + (long long)j * lda;
+        if (warp == 0) {
+            double t = 0.0;
+            for (int i = j + 1 + lane; i < c; i += 32) t = fma(aj[i], aj[i], t);
+            t = warp_sum(t);
+            if (lane == 0) s_nrm[j] = t;
+        }
+        __syncthreads();
+        const double alpha = aj[j];
+        const double xn2 = s_nrm[j];
+        double tau = 0.0, scal = 0.0, beta = alpha;
+        if (xn2 > 0.0) {
+            beta = -copysign(sqrt(alpha * alpha + xn2), alpha);
+            tau = (beta - alpha) / beta;
+            scal = 1.0 / (alpha - beta);
+        }
+        __syncthreads();
+        if (tau != 0.0) {
+            for (int i = j + 1 + threadIdx.x; i < c; i += blockDim.x) aj[i] *= scal;
+        }
+        if (threadIdx.x == 0) {
+            aj[j] = beta;
+            s_tau[j] = tau;
+        }
+        __syncthreads();
+        if (tau != 0.0) {
+            // A(j:, col) -= tau v (v^T A(j:, col)) for the trailing columns, a warp each
+            for (int col = j + 1 + warp; col < c; col += nw) {
+                double* ac = a + (long long)col * lda;
+                double t = (lane == 0) ? ac[j] : 0.0;
+                for (int i = j + 1 + lane; i < c; i += 32) t = fma(aj[i], ac[i], t);
+                t = warp_sum(t) * tau;
+                if (lane == 0) ac[j] -= t;
+                for (int i = j + 1 + lane; i < c; i += 32) ac[i] = fma(-t, aj[i], ac[i]);
+            }
+        }
+        __syncthreads();
+    }
+    // Q = H_0 ... H_{c-1}: from the identity, H_j applied to rows j.. of columns j..
+    for (long long e = threadIdx.x; e < (long long)c * c; e += blockDim.x) {
+        const int i = (int)(e % c), j = (int)(e / c);
+        q[e] = (i == j) ? 1.0 : 0.0;
+    }
+    __syncthreads();
+    for (int j = c - 1; j >= 0; --j) {
+        const double tau = s_tau[j];
+        if (tau != 0.0) {
+            const double* aj = a + (long long)j * lda;
+            for (int col = j + warp; col < c; col += nw) {
+                double* qc = q + (long long)col * c;
+                double t = (lane == 0) ? qc[j] : 0.0;
+                for (int i = j + 1 + lane; i < c; i += 32) t = fma(aj[i], qc[i], t);
+                t = warp_sum(t) * tau;
+                if (lane == 0) qc[j] -= t;
+                for (int i = j + 1 + lane; i < c; i += 32) qc[i] = fma(-t, aj[i], qc[i]);
+            }
+        }
+        __syncthreads();
+    }
+    // W = R^T (lower triangular); in the global case R is read before W is written
+    // over it, column by column of W = row by row of R, through registers
+    if (in_smem) {
+        for (long long e = threadIdx.x; e < (long long)c * c; e += blockDim.x) {
+            const int i = (int)(e % c), j = (int)(e / c);
+            W[S.off + e] = (i >= j) ? a[j + (long long)i * lda] : 0.0;
+        }
+    } else {
+        // transpose in place: swap (i, j) and (j, i) for i > j, zero the upper part
+        for (long long e = threadIdx.x; e < (long long)c * c; e += blockDim.x) {
+            const int i = (int)(e % c), j = (int)(e / c);
+            if (i > j) {
+                const double r = a[j + (long long)i * lda];   // R(j, i), upper part
+                a[i + (long long)j * lda] = r;                // W(i, j)
+                a[j + (long long)i * lda] = 0.0;
+            }
+        }
+    }
+}
+
 // ------------------------------------------------------------------ Jacobi
 constexpr int kJacThreads = 256;
 constexpr int kJacLanes = 8;                           // threads per column pair
@@ -894,24 +1036,47 @@ msp_status patch_qrcp(const PatchClasses& C, const PatchBlock* blocks, const dou
                       double* cols, cudaStream_t s) {
     size_t room = 0;
     MSP_TRY(smem_room(&room));
-    const int count[2] = {C.n_big, (int)C.blocks.size() - C.n_big};
-    for (int cls = 0; cls < 2; ++cls) {
-        if (!count[cls] || C.max_c[cls] <= 0) continue;
-        const int nc = cls == 0 ? kPatchCluster : 1, c = C.max_c[cls];
-        const size_t own = sizeof(double) * ((size_t)(c + nc - 1) / nc) * (c | 1), head = qr_head(c, nc);
+    double total = 0.0;
+    for (const PatchBlock& b : C.blocks) total += (double)b.c * b.c * b.c;
+    const double share = total / num_sms();
+    // Clusters for the patches classified for them where the largest one alone would keep its SM
+    // for more than three times the batch's share of an SM, and above 80 columns (a cluster's
+    // step is two cluster barriers, longer than a smaller patch's step on one SM); else every
+    // patch on one CTA.  QR and Q, clusters against one CTA each: 64 patches of 128 to 289
+    // columns (9 times the share) 7.7 ms against 25.9; 256 of 128 to 289 (3.6) 18.3 against 26.0;
+    // 256 of 60 to 181 (4.5) 6.4 against 8.2.  The other way: 1024 of 128 to 289 (1.2) 45.8
+    // against 36.5; 576 of 100 to 177 (1.1) 16.6 against 11.4; 256 of 128 to 165 (1.1) 17.8
+    // against 8.8; 100 of 128 to 165 (2.7) 7.5 against 6.7; 400 of 20 to 69 (4.0) 2.2 against 1.2.
+    const int c0 = C.n_big > 0 ? C.max_c[0] : 0;
+    const int n_cluster = c0 > 80 && (double)c0 * c0 * c0 > 3.0 * share ? C.n_big : 0;
+    const int n_one = (int)C.blocks.size() - n_cluster;
+    if (n_cluster > 0) {
+        const size_t own = sizeof(double) * ((size_t)(c0 + kPatchCluster - 1) / kPatchCluster) * (c0 | 1),
+                     head = qr_head(c0, kPatchCluster);
         const int in_smem = head + own <= room ? 1 : 0;
-        MSP_TRY(launch_cluster(patch_qrcp_kernel, count[cls], nc, kQrThreads, in_smem ? head + own : head, s,
-                               blocks + (cls == 0 ? 0 : C.n_big), T, W, R, cols, in_smem));
-    }
-    const int c = std::max(C.max_c[0], C.max_c[1]);
-    if (c > 0) {
-        const size_t bytes = sizeof(double) * (size_t)kFormWarps * c;
+        MSP_TRY(launch_cluster(patch_qrcp_kernel, n_cluster, kPatchCluster, kQrThreads, in_smem ? head + own : head, s,
+                               blocks, T, W, R, cols, in_smem));
+        const size_t bytes = sizeof(double) * (size_t)kFormWarps * c0;
         MSP_TRY(allow_smem(patch_form_q_kernel, bytes));
-        for (size_t b0 = 0; b0 < C.blocks.size(); b0 += 65535) {
-            const unsigned nb = (unsigned)std::min<size_t>(65535, C.blocks.size() - b0);
-            patch_form_q_kernel<<<dim3((c + kFormWarps - 1) / kFormWarps, nb), 32 * kFormWarps, bytes, s>>>(blocks + b0, R, Q);
+        for (int b0 = 0; b0 < n_cluster; b0 += 65535) {
+            const unsigned nb = (unsigned)std::min(65535, n_cluster - b0);
+            patch_form_q_kernel<<<dim3((c0 + kFormWarps - 1) / kFormWarps, nb), 32 * kFormWarps, bytes, s>>>(blocks + b0, R, Q);
             count_launches(1);
         }
+        MSP_CUDA(cudaGetLastError());
+    }
+    if (n_one > 0) {
+        const int c = std::max(n_cluster > 0 ? 0 : C.max_c[0], C.max_c[1]);
+        cudaFuncAttributes fa{};
+        MSP_CUDA(cudaFuncGetAttributes(&fa, patch_qr_one_kernel));
+        room += 3072;                                        // all but the 1 KB a block reserves
+        room -= fa.sharedSizeBytes;
+        int cq = 0;                                          // largest order held in shared memory
+        while (cq < c && (size_t)(cq + 1) * (cq + 2) * sizeof(double) <= room) ++cq;
+        const size_t bytes = (size_t)cq * (cq + 1) * sizeof(double);
+        MSP_TRY(allow_smem(patch_qr_one_kernel, bytes));
+        patch_qr_one_kernel<<<n_one, kQrThreads, bytes, s>>>(blocks + n_cluster, T, W, Q, cq);
+        count_launches(1);
         MSP_CUDA(cudaGetLastError());
     }
     return MSP_OK;

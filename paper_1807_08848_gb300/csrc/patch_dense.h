@@ -38,7 +38,8 @@ msp_status patch_triangular_inverse(const PatchClasses& C, const PatchBlock* blo
 // preconditioner of the Jacobi sweeps in the manner of Drmac and Veselic (2008): the
 // sweeps run on the columns of R^T, whose rows decay with the pivots, with V started at Q,
 // so that their rotations J leave V = Q J, the left singular vectors of T (the
-// permutation only acts on the right).  R and cols are work blocks as large as T.
+// permutation only acts on the right).  R and cols are work blocks as large as T.  On
+// clusters, or one CTA per patch where the patches keep all SMs busy.
 msp_status patch_qrcp(const PatchClasses& C, const PatchBlock* blocks, const double* T, double* W, double* Q, double* R,
                       double* cols, cudaStream_t s);
 
