@@ -612,8 +612,8 @@ msp_status svd_bases(const double* snaps, long long snap_elems, const std::vecto
             MSP_CUDA(cudaGetLastError());
         }
         MSP_TRY(phase_mark(marks, s));
-        // a cluster per patch; the blocks too large for one (above about 450 columns) on
-        // one CTA each
+        // a cluster per patch; one CTA each for the blocks too large for one (above about 450
+        // columns) and for batches that end sooner so
         std::vector<PatchBlock> rest_blocks;
         std::vector<PatchBlock> sorted(classes.blocks);
         std::stable_sort(sorted.begin(), sorted.end(), [](const PatchBlock& a, const PatchBlock& b) { return a.c > b.c; });

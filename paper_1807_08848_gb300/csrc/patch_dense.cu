@@ -10,7 +10,11 @@
 #include "device_util.cuh"
 
 #include <algorithm>
+#include <cmath>
 #include <cooperative_groups.h>
+#include <functional>
+#include <queue>
+#include <utility>
 
 namespace cg = cooperative_groups;
 
@@ -1112,6 +1116,31 @@ static int jac_cluster(int c, double share, size_t room, int max_nc) {
     return best;
 }
 
+// Time at which the last of `jobs` (CTAs that start together, work of each) ends when they are
+// started in order as CTA slots of the device come free.  A slot is 1 / per_sm of an SM, so
+// launches of different shared memory share the device in sixths of an SM.
+struct JacJob {
+    int ctas, sixths;
+    double work;
+};
+static double jac_makespan(const std::vector<JacJob>& jobs) {
+    long long room = 6LL * num_sms();
+    double now = 0.0, last = 0.0;
+    std::priority_queue<std::pair<double, int>, std::vector<std::pair<double, int>>, std::greater<>> running;   // end, sixths
+    for (const JacJob& j : jobs) {
+        const int need = j.ctas * j.sixths;
+        while (room < need && !running.empty()) {
+            now = running.top().first;
+            room += running.top().second;
+            running.pop();
+        }
+        running.push({now + j.work, need});
+        room -= need;
+        last = std::max(last, now + j.work);
+    }
+    return last;
+}
+
 // Streams beside the caller's for launches that may overlap; on every way out the
 // caller's stream waits for them.
 struct ForkedStreams {
@@ -1193,6 +1222,31 @@ msp_status patch_jacobi(const std::vector<PatchBlock>& all, double* W, double* V
         }
     }
     first[kJacSizes] = (int)list.size();
+    // One CTA per patch (jacobi_svd_kernel) where that ends sooner.  A patch on one CTA of 16
+    // warps takes about c^2.5 (the dropped columns are skipped), a CTA of a cluster, of 8 warps
+    // and with a barrier per round, 2.1 c^2.5 / nc whether one, two or three share its SM.  Clusters win where patches are few or uneven, one CTA each where the
+    // clusters' shared memory leaves one or two CTAs per SM or their last wave is nearly empty.
+    // Sweeps on clusters against one CTA each: 64 patches of 128 to 289 columns 48.6 ms against
+    // 217, 196 of 100 to 221 40.7 against 105; 196 of 200 to 253 176 against 115, 484 of 150 to 219
+    // 157 against 127, 324 of 160 to 281 223 against 186.
+    {
+        std::vector<JacJob> cluster, one;
+        auto work = [](int c) { return c > 1 ? (double)c * c * std::sqrt((double)c) : 0.0; };
+        for (int q = 0; q < kJacSizes; ++q) {
+            if (first[q] == first[q + 1]) continue;
+            int per_sm = 0;
+            MSP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, patch_jacobi_kernel, kJacThreads, bytes[q]));
+            per_sm = std::max(1, std::min(per_sm, 3));
+            for (int k = first[q]; k < first[q + 1]; ++k)
+                cluster.push_back(JacJob{kJacNc[q], 6 / per_sm, 2.1 * work(list[k].c) / kJacNc[q]});
+        }
+        for (const PatchBlock& b : rest) cluster.push_back(JacJob{1, 6, work(b.c)});   // they follow on one CTA
+        for (const PatchBlock& b : all) one.push_back(JacJob{1, 6, work(b.c)});
+        if (jac_makespan(one) < jac_makespan(cluster)) {
+            rest = all;
+            return MSP_OK;
+        }
+    }
     MSP_TRY(upload(d_blocks, list, s));
     // the largest patches first, the other sizes beside them
     ForkedStreams fs;

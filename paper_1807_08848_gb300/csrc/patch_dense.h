@@ -44,9 +44,9 @@ msp_status patch_qrcp(const PatchClasses& C, const PatchBlock* blocks, const dou
                       double* cols, cudaStream_t s);
 
 // FP64 one-sided Jacobi sweeps of every block (W rotated to U S, V accumulating) with
-// each patch on a cluster; `all` largest first.  Blocks whose columns a cluster's
-// shared memory does not hold are returned in `rest`.  d_blocks is read until the
-// stream has passed the launches.
+// each patch on a cluster; `all` largest first.  Returned in `rest`, for the sweeps on one CTA
+// each: the blocks whose columns a cluster's shared memory does not hold, or all of them where
+// that ends sooner.  d_blocks is read until the stream has passed the launches.
 msp_status patch_jacobi(const std::vector<PatchBlock>& all, double* W, double* V, int max_sweeps, double tol,
                         double small_rel, int* sweeps, DevBuf<PatchBlock>& d_blocks, std::vector<PatchBlock>& rest,
                         cudaStream_t s);

@@ -1,7 +1,7 @@
-"""The two forms of the pivoted QR (a cluster per patch, one CTA per patch) on the same blocks:
-one snapshot block extracted as a patch of a 2 x 2 partition, whose few patches take clusters,
-and as an inner patch of a 12 x 12 partition, whose many patches take a CTA each, in shared
-memory or beyond it (164 columns).  Every step's arithmetic is that of a patch by itself, so
+"""The two forms of the pivoted QR and of the Jacobi sweeps (a cluster per patch, one CTA per
+patch) on the same blocks: one snapshot block extracted as a patch of a 2 x 2 partition, whose
+few patches take clusters, and as an inner patch of a 12 x 12 partition, whose many patches
+take a CTA each, in shared memory or beyond it (164 columns).  Every step's arithmetic is that of a patch by itself, so
 singular values and bases are the same bits; the SVD of the block is checked against numpy as
 in test_gpu_patch_dense.py."""
 import numpy as np
