@@ -465,7 +465,7 @@ __global__ void __launch_bounds__(32 * kFormWarps) patch_form_q_kernel(const Pat
 // place, and the reflectors are applied to Q where they lie.  Every element takes the
 // operations of the two kernels above in their order.  Bound by FP64 issue: what a patch has
 // less of than on a cluster is SMs, so this form is for batches that keep them all busy; both
-// sides' times stand at the rule in patch_qrcp.
+// sides' times stand at the rule in classify_patches.
 constexpr int kQrMaxCols = 1024;    // the extraction's largest order
 __global__ void __launch_bounds__(kQrThreads) patch_qr_one_kernel(const PatchBlock* blocks, const double* Tm, double* W,
                                                                   double* Q, int smem_c) {
@@ -959,16 +959,30 @@ msp_status smem_room(size_t* room) {
 PatchClasses classify_patches(const std::vector<int>& cols, const std::vector<long long>& off) {
     PatchClasses C;
     double total = 0.0;
-    for (int c : cols) total += (double)c * c * c;
+    int cmax = 0;
+    for (int c : cols) {
+        total += (double)c * c * c;
+        cmax = std::max(cmax, c);
+    }
     const double share = total / num_sms();
+    // Clusters are for batches that one CTA per patch would leave waiting for the largest patch:
+    // where that one takes more than three times the batch's share of an SM, and more than 80
+    // columns (a cluster's step is two cluster barriers, longer than a smaller patch's step on
+    // one SM).  Clusters against one CTA each, ms (multiples of the share in brackets):
+    //   Cholesky and inverse   64 patches of 128 to 289 columns (8.2) 1.6 : 2.5, 256 of these (3.2)
+    //                          2.5 : 2.9; 64 of 96 (2.4) 0.52 : 0.37, 1024 of 128 to 289 (1.1)
+    //                          6.2 : 5.0, 152 of 160 (1.0) 2.1 : 1.1
+    //   QR and Q               64 of 128 to 289 (8.2) 7.7 : 25.9, 256 of these (3.2) 18.3 : 26.0;
+    //                          400 of 20 to 69 (4.0) 2.2 : 1.2, 1024 of 128 to 289 (1.1)
+    //                          45.8 : 36.5, 256 of 128 to 165 (1.1) 17.8 : 8.8
+    const bool clusters = cmax > 80 && (double)cmax * cmax * cmax > 3.0 * share;
     std::vector<PatchBlock> small;
     for (size_t m = 0; m < cols.size(); ++m) {
         const double w = (double)cols[m] * cols[m] * cols[m];
-        // A cluster for every patch that alone would keep one SM for more than half of
-        // the time in which the whole batch keeps all of them, and above the order
-        // whose columns one SM's shared memory holds; below 48 columns eight CTAs
-        // would spend their time in barriers.
-        const bool big = (w > 0.5 * share && cols[m] >= 48) || cols[m] > 160;
+        // then every patch that alone would keep one SM for more than half of the time in which
+        // the whole batch keeps all of them, and above the order whose columns one SM's
+        // shared memory holds; below 48 columns eight CTAs would spend their time in barriers
+        const bool big = clusters && ((w > 0.5 * share && cols[m] >= 48) || cols[m] > 160);
         const PatchBlock b{off[m], cols[m], (int)m};
         (big ? C.blocks : small).push_back(b);
     }
@@ -1040,19 +1054,7 @@ msp_status patch_qrcp(const PatchClasses& C, const PatchBlock* blocks, const dou
                       double* cols, cudaStream_t s) {
     size_t room = 0;
     MSP_TRY(smem_room(&room));
-    double total = 0.0;
-    for (const PatchBlock& b : C.blocks) total += (double)b.c * b.c * b.c;
-    const double share = total / num_sms();
-    // Clusters for the patches classified for them where the largest one alone would keep its SM
-    // for more than three times the batch's share of an SM, and above 80 columns (a cluster's
-    // step is two cluster barriers, longer than a smaller patch's step on one SM); else every
-    // patch on one CTA.  QR and Q, clusters against one CTA each: 64 patches of 128 to 289
-    // columns (9 times the share) 7.7 ms against 25.9; 256 of 128 to 289 (3.6) 18.3 against 26.0;
-    // 256 of 60 to 181 (4.5) 6.4 against 8.2.  The other way: 1024 of 128 to 289 (1.2) 45.8
-    // against 36.5; 576 of 100 to 177 (1.1) 16.6 against 11.4; 256 of 128 to 165 (1.1) 17.8
-    // against 8.8; 100 of 128 to 165 (2.7) 7.5 against 6.7; 400 of 20 to 69 (4.0) 2.2 against 1.2.
-    const int c0 = C.n_big > 0 ? C.max_c[0] : 0;
-    const int n_cluster = c0 > 80 && (double)c0 * c0 * c0 > 3.0 * share ? C.n_big : 0;
+    const int c0 = C.max_c[0], n_cluster = C.n_big;
     const int n_one = (int)C.blocks.size() - n_cluster;
     if (n_cluster > 0) {
         const size_t own = sizeof(double) * ((size_t)(c0 + kPatchCluster - 1) / kPatchCluster) * (c0 | 1),
@@ -1070,7 +1072,7 @@ msp_status patch_qrcp(const PatchClasses& C, const PatchBlock* blocks, const dou
         MSP_CUDA(cudaGetLastError());
     }
     if (n_one > 0) {
-        const int c = std::max(n_cluster > 0 ? 0 : C.max_c[0], C.max_c[1]);
+        const int c = C.max_c[1];
         cudaFuncAttributes fa{};
         MSP_CUDA(cudaFuncGetAttributes(&fa, patch_qr_one_kernel));
         room += 3072;                                        // all but the 1 KB a block reserves
