@@ -357,12 +357,49 @@ __global__ void __launch_bounds__(256) tile_inverse_kernel(const T* D, int n, T*
 // Panel of the block Cholesky: P <- P L^{-T} for the m x nb panel P (ld ldp) under
 // the factored diagonal tile L (nb x nb lower, ld ldl): every row x solves
 // L x^T = p^T by column-oriented forward substitution, x_j = x_j / L[j][j], then
-// x_l -= L[l][j] x_j for l > j.  Eight lanes per row, lane s holding x_s, x_{s+8}, ... in
-// registers and four rows per warp: a column costs one product for four rows and only the
-// FMAs right of it (a warp per row spends a product and two FMAs per column on one row,
-// most lanes idle; FP64-bound either way), x_j passed by one shuffle.  L is shared by the
-// CTA's rows.
-constexpr int kTrsmWarps = 4;            // 150 CTAs, a warp per quarter of an SM, for 2400 rows
+// x_l -= L[l][j] x_j for l > j.  Two forms of the same operations; L is shared by the CTA's rows.
+//
+// One warp per row, lane l holding x_l and x_{l+32} in registers, x_j passed by one shuffle,
+// so the chain of a column is one product, one shuffle and one FMA: latency-bound while every
+// CTA of eight rows has an SM.
+constexpr int kTrsmRowWarps = 8;
+template <class T>
+__global__ void __launch_bounds__(32 * kTrsmRowWarps) trsm_rows_kernel(const T* Lkk, int ldl, T* P, int ldp, int m, int nb) {
+    __shared__ T L[kTile][kTile + 1];
+    __shared__ T rd[kTile];
+    const int tid = threadIdx.x, lane = tid & 31;
+    for (int e = tid; e < nb * nb; e += blockDim.x) {
+        const int i = e % nb, j = e / nb;
+        L[i][j] = (i >= j) ? Lkk[i + (long long)j * ldl] : T(0);
+    }
+    __syncthreads();
+    for (int i = tid; i < nb; i += blockDim.x) rd[i] = T(1) / L[i][i];
+    __syncthreads();
+    const int row = blockIdx.x * kTrsmRowWarps + (tid >> 5);
+    if (row >= m) return;   // warp-uniform; no barrier follows
+    T* pr = P + row;
+    const int l1 = lane + 32;
+    T x0 = lane < nb ? pr[(long long)lane * ldp] : T(0);
+    T x1 = l1 < nb ? pr[(long long)l1 * ldp] : T(0);
+    for (int j = 0; j < nb; ++j) {
+        T v = j < 32 ? x0 : x1;
+        if (lane == (j & 31)) {
+            v *= rd[j];
+            if (j < 32) x0 = v;
+            else x1 = v;
+        }
+        const T xj = __shfl_sync(0xffffffffu, v, j & 31);
+        if (lane > j && lane < nb) x0 = fma(-L[lane][j], xj, x0);
+        if (l1 > j && l1 < nb) x1 = fma(-L[l1][j], xj, x1);
+    }
+    if (lane < nb) pr[(long long)lane * ldp] = x0;
+    if (l1 < nb) pr[(long long)l1 * ldp] = x1;
+}
+
+// Eight lanes per row, lane s holding x_s, x_{s+8}, ... and four rows per warp: a column costs
+// one product for four rows and only the FMAs right of it (a warp per row spends a product and
+// two FMAs per column on one row, most lanes idle), on a longer chain per row.  FP64-bound.
+constexpr int kTrsmWarps = 4;            // a warp per quarter of an SM
 constexpr int kTrsmRows = 4 * kTrsmWarps;
 template <class T>
 __global__ void __launch_bounds__(32 * kTrsmWarps) trsm_panel_kernel(const T* Lkk, int ldl, T* P, int ldp, int m, int nb) {
@@ -975,6 +1012,7 @@ msp_status factorize(Basis& B, const double* Hs64p, long long total, double shif
         } side;
         MSP_CUDA(cudaStreamCreateWithFlags(&side.st, cudaStreamNonBlocking));
         for (cudaEvent_t& e : side.ev) MSP_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+        const int sms = num_sms();
         for (size_t si = 0; si < steps.size(); ++si) {
             const Step& st = steps[si];
             const cudaStream_t ss = st.stream ? side.st : s;
@@ -1021,8 +1059,15 @@ msp_status factorize(Basis& B, const double* Hs64p, long long total, double shif
                 potrf_tile_kernel<T><<<1, 256, 0, s>>>(st.ptr, st.ld, st.nb, fail.p);
                 count_launches(1);
             } else if (st.kind == 6) {
-                trsm_panel_kernel<T><<<(st.nr + kTrsmRows - 1) / kTrsmRows, 32 * kTrsmWarps, 0, s>>>(
-                    st.src, st.lds, st.ptr, st.ld, st.nr, st.nb);
+                // a warp per row up to one CTA per SM (FP64; 20.5 us a launch of 64 columns at 16 to
+                // 1216 rows, four rows per warp 26.7; at 1232 rows 35.0 against 28.7) or two (FP32;
+                // 10.3 against 14.4 at 1216 rows, 12.3 against 14.4 at 2432, 16.4 against 14.4 at 4096)
+                const int row_ctas = (st.nr + kTrsmRowWarps - 1) / kTrsmRowWarps;
+                if (row_ctas <= (sizeof(T) == 8 ? 1 : 2) * sms)
+                    trsm_rows_kernel<T><<<row_ctas, 32 * kTrsmRowWarps, 0, s>>>(st.src, st.lds, st.ptr, st.ld, st.nr, st.nb);
+                else
+                    trsm_panel_kernel<T><<<(st.nr + kTrsmRows - 1) / kTrsmRows, 32 * kTrsmWarps, 0, s>>>(
+                        st.src, st.lds, st.ptr, st.ld, st.nr, st.nb);
                 count_launches(1);
             } else if (st.kind == 7) {
                 tile_inverse_kernel<T><<<st.nr, 256, 0, s>>>(st.ptr, st.nb, st.inv);
