@@ -12,7 +12,8 @@
 //   backward  x_m = L_m^{-T} y_m - (L_m^{-T} C_m^T) x_{m+1}.
 // As one CTA for the whole factor and one per data set, with the triangular solves on
 // one thread, the 8192-cell slab of 64 patches took 44 ms to factor and 124 ms to solve;
-// now 7.2 ms of chain, 1.2 of sweeps and 0.6 of the rest.
+// now 7.2 ms of chain, 1.2 of sweeps and 0.6 of the rest.  The smallest slabs keep one CTA
+// for the factor's chain, and one per data set for a whole solve.
 #include "kinetic_online.h"
 #include "device_util.cuh"
 #include "patch_dense.h"
@@ -190,7 +191,7 @@ __global__ void __launch_bounds__(kKfThreads) kinetic_chain_kernel(KOnArgs A, do
     if (rank == 0 && tid == 0) *fail = s_ok ? 0 : 1;
 }
 
-// The chain on one CTA out of global memory, for blocks beyond kKfMaxK
+// The chain on one CTA out of global memory, for blocks beyond kKfMaxK and for the smallest
 __global__ void __launch_bounds__(kKfThreads) kinetic_chain_global_kernel(KOnArgs A, double* Lf, double* Cf, int* fail) {
     __shared__ int s_ok;
     if (threadIdx.x == 0) s_ok = 1;
@@ -270,13 +271,14 @@ __device__ __forceinline__ double kval(const KOnArgs& A, int m, int node, int l,
     return a;
 }
 
-// residual rows r = d - P c (c = 0 on the first pass); blockIdx (data set, row tile)
-__global__ void __launch_bounds__(128) kinetic_residual_kernel(KOnArgs A, KVec W, const double* inflow, int first) {
-    const int b = blockIdx.x, nv = A.nv, M = A.M, rows = M * nv;
+// residual rows r = d - P c (c = 0 on the first pass): rows t0, t0 + step, ... of data set b
+__device__ __forceinline__ void residual_rows(const KOnArgs& A, const KVec& W, const double* inflow, int first, int b,
+                                              int t0, int step) {
+    const int nv = A.nv, M = A.M, rows = M * nv;
     const double* inl = inflow + (long long)b * 2 * nv;
     const double* inr = inl + nv;
     const double* c = W.c(b);
-    for (int t = blockIdx.y * 128 + threadIdx.x; t < rows; t += 128 * gridDim.y) {
+    for (int t = t0; t < rows; t += step) {
         double v;
         if (t < (M - 1) * nv) {
             const int m = t / nv, l = t - m * nv, last = A.patches[m].x1 - A.patches[m].x0;
@@ -292,15 +294,14 @@ __global__ void __launch_bounds__(128) kinetic_residual_kernel(KOnArgs A, KVec W
     }
 }
 
-// g = P^T r, then t = L^{-1} g, patch by patch; blockIdx (data set, patch)
-__global__ void __launch_bounds__(256) kinetic_rhs_kernel(KOnArgs A, KVec W) {
-    extern __shared__ double gs[];
-    const int b = blockIdx.x, nv = A.nv, M = A.M, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+// g = P^T r, then t = L^{-1} g: patches m0, m0 + step, ... of data set b, g in gs
+__device__ __forceinline__ void rhs_patches(const KOnArgs& A, const KVec& W, int b, int m0, int step, double* gs) {
+    const int nv = A.nv, M = A.M, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     const double* r = W.r(b);
-    for (int m = blockIdx.y; m < M; m += gridDim.y) {
+    for (int m = m0; m < M; m += step) {
         const KPatchDev P = A.patches[m];
         const int km = A.k[m], last = P.x1 - P.x0;
-        for (int j = warp; j < km; j += 8) {
+        for (int j = warp; j < km; j += nw) {
             const double* q0 = A.Q + A.q_off[m] + (long long)j * P.n_k;
             const double* q1 = q0 + (long long)last * nv;
             double a = 0.0;
@@ -315,7 +316,7 @@ __global__ void __launch_bounds__(256) kinetic_rhs_kernel(KOnArgs A, KVec W) {
         }
         __syncthreads();
         const double* Fi = A.Fi + A.l_off[m];            // L^{-T}: column i holds row i of L^{-1}
-        for (int i = warp; i < km; i += 8) {
+        for (int i = warp; i < km; i += nw) {
             double a = 0.0;
             for (int q = lane; q <= i; q += 32) a += Fi[q + (long long)i * km] * gs[q];
             a = warp_sum(a);
@@ -325,16 +326,14 @@ __global__ void __launch_bounds__(256) kinetic_rhs_kernel(KOnArgs A, KVec W) {
     }
 }
 
-// w = L^{-T} y, patch by patch (y in t, w into g); blockIdx (data set, patch)
-__global__ void __launch_bounds__(256) kinetic_lit_kernel(KOnArgs A, KVec W) {
-    extern __shared__ double ys[];
-    const int b = blockIdx.x;
-    for (int m = blockIdx.y; m < A.M; m += gridDim.y) {
+// w = L^{-T} y (y in t, w into g): patches m0, m0 + step, ... of data set b, y in ys
+__device__ __forceinline__ void lit_patches(const KOnArgs& A, const KVec& W, int b, int m0, int step, double* ys) {
+    for (int m = m0; m < A.M; m += step) {
         const int km = A.k[m];
         const double* Fi = A.Fi + A.l_off[m];
-        for (int i = threadIdx.x; i < km; i += 256) ys[i] = W.t(b)[A.c_off[m] + i];
+        for (int i = threadIdx.x; i < km; i += blockDim.x) ys[i] = W.t(b)[A.c_off[m] + i];
         __syncthreads();
-        for (int i = threadIdx.x; i < km; i += 256) {
+        for (int i = threadIdx.x; i < km; i += blockDim.x) {
             double a = 0.0;
 #pragma unroll 8
             for (int q = i; q < km; ++q) a += Fi[i + (long long)q * km] * ys[q];
@@ -344,13 +343,12 @@ __global__ void __launch_bounds__(256) kinetic_lit_kernel(KOnArgs A, KVec W) {
     }
 }
 
-// One chain: z_m = s_m - T_m z_{m -+ 1} along the patches (T_m: k_m x k_{m -+ 1}), one CTA per
-// data set; the rows' sums are split over the threads that share a row.  The next
-// patch's matrix is brought into the L2 meanwhile.  Forward: in place in t.  Backward:
-// s in g, and c += z.
-__global__ void __launch_bounds__(kKfThreads) kinetic_sweep_kernel(KOnArgs A, KVec W, int backward) {
-    extern __shared__ double zs[];                       // z of two patches, partial sums
-    const int b = blockIdx.x, tid = threadIdx.x, M = A.M;
+// One chain: z_m = s_m - T_m z_{m -+ 1} along the patches (T_m: k_m x k_{m -+ 1}), one CTA of
+// kKfThreads per data set; the rows' sums are split over the threads that share a row.  The
+// next patch's matrix is brought into the L2 meanwhile.  Forward: in place in t.
+// Backward: s in g, and c += z.  zs: z of two patches, partial sums.
+__device__ __forceinline__ void chain_sweep(const KOnArgs& A, const KVec& W, int b, int backward, double* zs) {
+    const int tid = threadIdx.x, M = A.M;
     const int kx = A.k_max;
     double* part = zs + 2 * kx;                          // kKfThreads
     double* src = backward ? W.g(b) : W.t(b);
@@ -368,7 +366,7 @@ __global__ void __launch_bounds__(kKfThreads) kinetic_sweep_kernel(KOnArgs A, KV
             const long long n = (long long)A.k[mn] * km;
             for (long long e = 16LL * tid; e < n; e += 16LL * kKfThreads) asm volatile("prefetch.global.L2 [%0];" ::"l"(Tn + e));
         }
-        const int rows = (km + 31) / 32 * 32;            // 32 <= rows <= kKfThreads where km > 0
+        const int rows = (km + 31) / 32 * 32;            // beyond kKfThreads rows: one part, several rounds
         const int parts = rows > 0 ? max(1, kKfThreads / rows) : 1;
         const int p = rows > 0 ? tid / rows : 0;
         for (int i0 = 0; i0 < km; i0 += kKfThreads) {
@@ -392,17 +390,17 @@ __global__ void __launch_bounds__(kKfThreads) kinetic_sweep_kernel(KOnArgs A, KV
     }
 }
 
-// reconstruction: patch interiors, interface averages, incoming data at the ends;
-// blockIdx (data set, tile of (node, velocity))
-__global__ void __launch_bounds__(256) kinetic_recon_kernel(KOnArgs A, KVec W, const double* inflow, double* f_out,
-                                                            double* c_out) {
-    const int b = blockIdx.x, nv = A.nv, M = A.M, N = A.N;
+// reconstruction: patch interiors, interface averages, incoming data at the ends; values
+// (node, velocity) t0, t0 + step, ... of data set b
+__device__ __forceinline__ void recon_values(const KOnArgs& A, const KVec& W, const double* inflow, double* f_out,
+                                             double* c_out, int b, long long t0, long long step) {
+    const int nv = A.nv, M = A.M, N = A.N;
     const double* inl = inflow + (long long)b * 2 * nv;
     const double* inr = inl + nv;
     const double* c = W.c(b);
     const long long total = (long long)(N + 1) * nv;
     const int Wd = A.patches[0].x1 - A.patches[0].x0;
-    for (long long t = blockIdx.y * 256LL + threadIdx.x; t < total; t += 256LL * gridDim.y) {
+    for (long long t = t0; t < total; t += step) {
         const int i = (int)(t / nv), l = (int)(t % nv);
         const int m = min(i / Wd, M - 1);
         double val;
@@ -415,7 +413,47 @@ __global__ void __launch_bounds__(256) kinetic_recon_kernel(KOnArgs A, KVec W, c
         f_out[b * total + t] = val;
     }
     if (c_out)
-        for (int j = blockIdx.y * 256 + threadIdx.x; j < W.Np; j += 256 * gridDim.y) c_out[(long long)b * W.Np + j] = c[j];
+        for (long long j = t0; j < W.Np; j += step) c_out[(long long)b * W.Np + j] = c[j];
+}
+
+// The phases by themselves: blockIdx (data set, tile or patch)
+__global__ void __launch_bounds__(128) kinetic_residual_kernel(KOnArgs A, KVec W, const double* inflow, int first) {
+    residual_rows(A, W, inflow, first, blockIdx.x, blockIdx.y * 128 + threadIdx.x, 128 * gridDim.y);
+}
+__global__ void __launch_bounds__(256) kinetic_rhs_kernel(KOnArgs A, KVec W) {
+    extern __shared__ double ksv[];
+    rhs_patches(A, W, blockIdx.x, blockIdx.y, gridDim.y, ksv);
+}
+__global__ void __launch_bounds__(kKfThreads) kinetic_sweep_kernel(KOnArgs A, KVec W, int backward) {
+    extern __shared__ double ksv[];
+    chain_sweep(A, W, blockIdx.x, backward, ksv);
+}
+__global__ void __launch_bounds__(256) kinetic_lit_kernel(KOnArgs A, KVec W) {
+    extern __shared__ double ksv[];
+    lit_patches(A, W, blockIdx.x, blockIdx.y, gridDim.y, ksv);
+}
+__global__ void __launch_bounds__(256) kinetic_recon_kernel(KOnArgs A, KVec W, const double* inflow, double* f_out,
+                                                            double* c_out) {
+    recon_values(A, W, inflow, f_out, c_out, blockIdx.x, blockIdx.y * 256LL + threadIdx.x, 256LL * gridDim.y);
+}
+
+// All of them, one CTA per data set, for slabs so small that sixteen launches take longer
+// than the work
+__global__ void __launch_bounds__(kKfThreads) kinetic_small_kernel(KOnArgs A, KVec W, const double* inflow, double* f_out,
+                                                                   double* c_out) {
+    extern __shared__ double ksv[];
+    const int b = blockIdx.x;
+    for (int pass = 0; pass < 3; ++pass) {
+        residual_rows(A, W, inflow, pass == 0, b, threadIdx.x, blockDim.x);
+        __syncthreads();
+        rhs_patches(A, W, b, 0, 1, ksv);
+        chain_sweep(A, W, b, 0, ksv);
+        __syncthreads();
+        lit_patches(A, W, b, 0, 1, ksv);
+        chain_sweep(A, W, b, 1, ksv);
+        __syncthreads();
+    }
+    recon_values(A, W, inflow, f_out, c_out, b, threadIdx.x, blockDim.x);
 }
 
 }  // namespace
@@ -431,7 +469,9 @@ msp_status kinetic_factor(const KOnArgs& A, const std::vector<int>& k, const std
     }
     DevBuf<int> fail;
     MSP_TRY(fail.alloc(1, s));
-    if (A.k_max <= kKfMaxK) {
+    // Below eight columns a block's barriers on a cluster take longer than its work by one CTA: 1024
+    // patches of 2 or 4 columns 6.9 and 8.7 ms against 3.4 and 6.4 (256 of 8: 3.06 against 3.36)
+    if (A.k_max >= 8 && A.k_max <= kKfMaxK) {
         const size_t smem = sizeof(double) * std::max<size_t>((size_t)A.k_max * (A.k_max | 1), kKfChunk + A.k_max);
         MSP_TRY(allow_smem(kinetic_chain_kernel, smem));
         cudaLaunchConfig_t cfg{};
@@ -480,6 +520,15 @@ msp_status kinetic_factor(const KOnArgs& A, const std::vector<int>& k, const std
     return MSP_OK;
 }
 
+// One launch in place of sixteen: up to 64 columns over the patches and 2^17 terms of the
+// reconstruction.  A call for one data set, one launch against sixteen: 1 patch of 2 columns 54 us
+// against 107, 3 of 2 85 against 134, 4 of 16 138 against 171, 8 of 8 183 against 191; beyond it
+// 16 of 8 326 against 289, 4 of 32 250 against 192; 4 of 8 with 2049 nodes (2^17 terms) 152
+// against 154.
+static bool small_slab(const KOnArgs& A) {
+    return (long long)A.M * A.k_max <= 64 && (long long)(A.N + 1) * A.nv * std::max(A.k_max, 1) <= 1 << 17;
+}
+
 msp_status kinetic_online(const KOnArgs& A, int Np, const double* inflow, int batch, double* f_out, double* c_out,
                           cudaStream_t s) {
     const int M = A.M, nv = A.nv, n1 = std::max(Np, 1);
@@ -493,6 +542,14 @@ msp_status kinetic_online(const KOnArgs& A, int Np, const double* inflow, int ba
     const size_t vec = sizeof(double) * std::max(A.k_max, 1);
     const size_t chain = 2 * vec + sizeof(double) * kKfThreads;
     const unsigned pm = (unsigned)std::min(M, 65535);
+    const long long total = (long long)(A.N + 1) * nv;
+    if (small_slab(A)) {
+        kinetic_small_kernel<<<batch, kKfThreads, chain, s>>>(A, W, inflow, f_out, c_out);
+        count_launches(1);
+        MSP_CUDA(cudaGetLastError());
+        MSP_CUDA(cudaStreamSynchronize(s));   // the work buffer is released on return
+        return MSP_OK;
+    }
     for (int pass = 0; pass < 3; ++pass) {
         kinetic_residual_kernel<<<dim3(batch, std::min(1024, (M * nv + 127) / 128)), 128, 0, s>>>(A, W, inflow, pass == 0);
         kinetic_rhs_kernel<<<dim3(batch, pm), 256, vec, s>>>(A, W);
@@ -501,7 +558,6 @@ msp_status kinetic_online(const KOnArgs& A, int Np, const double* inflow, int ba
         kinetic_sweep_kernel<<<batch, kKfThreads, chain, s>>>(A, W, 1);
         count_launches(5);
     }
-    const long long total = (long long)(A.N + 1) * nv;
     kinetic_recon_kernel<<<dim3(batch, (unsigned)std::min<long long>(16384, (total + 255) / 256)), 256, 0, s>>>(
         A, W, inflow, f_out, c_out);
     count_launches(1);
