@@ -947,7 +947,3 @@ extern "C" msp_status msp_medium_direct_timing(msp_medium m, double* ms_host, in
     }
     return MSP_OK;
 }
-
-namespace msp {
-
-}  // namespace msp
