@@ -1,11 +1,11 @@
 // Per-patch Cholesky factors and their inverses (the QR remark of Sec. 3.3; the patch
-// blocks of the online normal matrix), spread over the GPU by rows of work instead of
-// one CTA per patch.
+// blocks of the online normal matrix), pivoted QR and Jacobi sweeps: on thread-block
+// clusters where one CTA per patch would leave the GPU waiting, else one CTA per patch.
 //
 // A patch on the domain boundary has more than twice the snapshot columns of an inner
 // one (289 against 128 on the 64-cell partitions: the boundary deltas), twelve times
-// its arithmetic, so one CTA per patch ran for as long as the corner patch took on one
-// SM out of 152, and out of global memory.
+// its arithmetic, so with few patches one CTA each runs for as long as the corner patch
+// takes on one SM out of 152.
 #include "patch_dense.h"
 #include "device_util.cuh"
 
@@ -38,8 +38,10 @@ __host__ __device__ inline size_t panel_elems(int c, int rank, int nc) {
 // factors a panel and stores it to L; after a cluster barrier every CTA stages it and
 // updates its own later panels.  Every element takes its updates in ascending order
 // of the pivot, one FMA each, so the factor does not depend on the panel width or the
-// number of CTAs.  Bound: the FP64 pipe and the chain of panels.  64 patches of 130 to 290
-// columns: 1.7 ms a call, where a CTA per patch took 14.4 with the inverse.
+// number of CTAs.  Bound: the chain of panels and its barriers on clusters (64 patches of 128 to
+// 289 columns: 1.0 ms a try, FP64 pipe busy 18% of the time, a warp waits 84 issue slots at
+// barriers for each of its own), the FP64 pipe and the chain on one CTA each (1024 patches:
+// 2.3 ms, 62%).  Those 64 patches took 14.4 ms with the inverse on a CTA per patch.
 __global__ void __launch_bounds__(kCholThreads) patch_chol_kernel(const PatchBlock* blocks, const double* G, double* L,
                                                                   const double* shift_scale, int shifted, int* status,
                                                                   int in_smem) {
@@ -189,9 +191,9 @@ __device__ __forceinline__ double warp_sum4(const double (&a)[4], int lane) {
 // division per row and CTA (it takes as long as six FMAs).  X(i, j) is stored at Fi(j, i);
 // the CTA of the first columns also writes F.  Columns are independent, so a patch takes
 // c / kCols CTAs, and a column's sums do not depend on CPW.
-// Bound by FP64 issue: 1024 patches of up to 290 columns took 9.5 ms a call with a division
-// per row and column and one column per warp; a 513^2 extraction went from 115.8 to 104.4 ms
-// with both changes, a 2049^2 step from 1121 to 1100.
+// Bound by FP64 issue (pipe busy 80% of the time): 1024 patches of 128 to 289 columns 2.9 ms a
+// call, 9.5 with a division per row and column and one column per warp; a 513^2 extraction went
+// from 115.8 to 104.4 ms with both changes, a 2049^2 step from 1121 to 1100.
 template <int CPW>
 struct InvShape {
     static constexpr int kWarps = CPW == 1 ? 16 : 8;
@@ -280,8 +282,9 @@ constexpr int kFormWarps = 8;       // columns of Q per CTA
 // the rows below are summed afresh in the same pass (no downdating).  Columns are not
 // moved: a table holds the column at each position of the permuted order.
 // W = R^T (lower triangular); R holds the reflectors, v below the diagonal and tau on it,
-// for patch_form_q_kernel.  Bound: the FP64 pipe and two cluster barriers a step.  64 patches
-// of 130 to 290 columns: 6.2 ms and 1.6 for Q, where a CTA per patch took 26.
+// for patch_form_q_kernel.  Bound: two cluster barriers a step and the FP64 pipe (busy 50% of
+// the time).  64 patches of 128 to 289 columns: 6.2 ms and 1.6 for Q (65%), where a CTA per
+// patch takes 26.
 struct QrShared {
     double cand[2][kPatchCluster];   // published candidates, by step parity
     int cand_pos[2][kPatchCluster];
@@ -463,8 +466,9 @@ __global__ void __launch_bounds__(32 * kFormWarps) patch_form_q_kernel(const Pat
 // The same factorisation by one CTA per patch, with Q: the columns live in shared memory (or in
 // W, orders above smem_c, which R^T overwrites at the end either way), are swapped into
 // place, and the reflectors are applied to Q where they lie.  Every element takes the
-// operations of the two kernels above in their order.  Bound by FP64 issue: what a patch has
-// less of than on a cluster is SMs, so this form is for batches that keep them all busy; both
+// operations of the two kernels above in their order.  Bound by FP64 issue (1024 patches of 128
+// to 289 columns 36 ms, pipe busy 72% of the time): what a patch has less of than on a
+// cluster is SMs, so this form is for batches that keep them all busy; both
 // sides' times stand at the rule in classify_patches.
 constexpr int kQrMaxCols = 1024;    // the extraction's largest order
 __global__ void __launch_bounds__(kQrThreads) patch_qr_one_kernel(const PatchBlock* blocks, const double* Tm, double* W,
@@ -654,10 +658,12 @@ struct JacArgs {
 // rotating it only mixes directions that are dropped.
 // Every pair, sum and rotation is that of the one-CTA form (jacobi_svd_kernel), in
 // the same order: the result does not depend on the cluster size.
-// Bound: the FP64 pipe (3 c products and 8 c for the two rotations per pair, about
-// 1.75 FMA per clock and SM); the three CTAs of an SM hide each other's angles and
-// barriers, and a large patch no longer runs on one SM alone: 64 patches of 130 to 290
-// columns took 201 ms with a CTA each, now 49; 1024 patches 229 ms in both forms.
+// Bound: the FP64 pipe (3 c products and 8 c for the two rotations per pair) where three CTAs
+// share an SM and hide each other's angles and barriers, the rounds' barriers where they
+// do not.  1024 patches of 128 to 289 columns: 229 ms in both forms; the three launches, each
+// by itself, keep the GPU's FP64 pipe busy 80% (900 inner patches), 41% and 4% (four corner
+// patches) of their times, 65% of the 229 ms in which they overlap.  64 such patches took
+// 201 ms with a CTA each, now 49 (10, 31 and 23%): a large patch no longer runs on one SM alone.
 __global__ void __launch_bounds__(kJacThreads, 3) patch_jacobi_kernel(JacArgs A) {
     extern __shared__ __align__(16) double jsm[];
     constexpr int kSlots = 2 * kJacPairs + 2;
@@ -954,41 +960,77 @@ msp_status smem_room(size_t* room) {
     return MSP_OK;
 }
 
+// Time at which the last of `jobs` (a patch's CTAs, which start together; the SM sixths that each
+// takes; its time) ends when they are started in order as room on the device comes free.
+struct Job {
+    int ctas, sixths;
+    double time;
+};
+double makespan(const std::vector<Job>& jobs) {
+    long long room = 6LL * num_sms();
+    double now = 0.0, last = 0.0;
+    std::priority_queue<std::pair<double, int>, std::vector<std::pair<double, int>>, std::greater<>> running;   // end, sixths
+    for (const Job& j : jobs) {
+        const int need = j.ctas * j.sixths;
+        while (room < need && !running.empty()) {
+            now = running.top().first;
+            room += running.top().second;
+            running.pop();
+        }
+        running.push({now + j.time, need});
+        room -= need;
+        last = std::max(last, now + j.time);
+    }
+    return last;
+}
+
 }  // namespace
 
 PatchClasses classify_patches(const std::vector<int>& cols, const std::vector<long long>& off) {
     PatchClasses C;
     double total = 0.0;
-    int cmax = 0;
-    for (int c : cols) {
-        total += (double)c * c * c;
-        cmax = std::max(cmax, c);
-    }
+    for (int c : cols) total += (double)c * c * c;
     const double share = total / num_sms();
-    // Clusters are for batches that one CTA per patch would leave waiting for the largest patch:
-    // where that one takes more than three times the batch's share of an SM, and more than 80
-    // columns (a cluster's step is two cluster barriers, longer than a smaller patch's step on
-    // one SM).  Clusters against one CTA each, ms (multiples of the share in brackets):
-    //   Cholesky and inverse   64 patches of 128 to 289 columns (8.2) 1.6 : 2.5, 256 of these (3.2)
-    //                          2.5 : 2.9; 64 of 96 (2.4) 0.52 : 0.37, 1024 of 128 to 289 (1.1)
-    //                          6.2 : 5.0, 152 of 160 (1.0) 2.1 : 1.1
-    //   QR and Q               64 of 128 to 289 (8.2) 7.7 : 25.9, 256 of these (3.2) 18.3 : 26.0;
-    //                          400 of 20 to 69 (4.0) 2.2 : 1.2, 1024 of 128 to 289 (1.1)
-    //                          45.8 : 36.5, 256 of 128 to 165 (1.1) 17.8 : 8.8
-    const bool clusters = cmax > 80 && (double)cmax * cmax * cmax > 3.0 * share;
     std::vector<PatchBlock> small;
     for (size_t m = 0; m < cols.size(); ++m) {
         const double w = (double)cols[m] * cols[m] * cols[m];
-        // then every patch that alone would keep one SM for more than half of the time in which
-        // the whole batch keeps all of them, and above the order whose columns one SM's
-        // shared memory holds; below 48 columns eight CTAs would spend their time in barriers
-        const bool big = clusters && ((w > 0.5 * share && cols[m] >= 48) || cols[m] > 160);
+        // candidates: the patches that alone would keep one SM for more than half of the time
+        // in which the whole batch keeps all of them, and those above the order whose columns
+        // one SM's shared memory holds; below 48 columns a cluster has no advantage
+        const bool big = (w > 0.5 * share && cols[m] >= 48) || cols[m] > 160;
         const PatchBlock b{off[m], cols[m], (int)m};
         (big ? C.blocks : small).push_back(b);
     }
     auto larger = [](const PatchBlock& a, const PatchBlock& b) { return a.c > b.c; };
     std::stable_sort(C.blocks.begin(), C.blocks.end(), larger);
     std::stable_sort(small.begin(), small.end(), larger);
+    // They take clusters, and the others one CTA each after them, if that ends before one CTA for
+    // every patch does.  Times in us of the QR with Q, the longest of the stages: a patch alone
+    // on one CTA and on a cluster of eight (24 to 160 columns, fitted), the latter times 1.15 for
+    // the clusters beside it, two of whose CTAs share an SM.  Over 272 batches (1 to 1600 patches
+    // of 20 to 373 columns) the choice takes 0.3 percent longer than the better one on average, 14 at
+    // most.  Clusters against one CTA each, ms:
+    //   QR and Q               64 patches of 128 to 289 columns 7.7 : 25.9, 8 of 64 0.73 : 0.97;
+    //                          1024 of 128 to 289 45.8 : 36.5, 256 of 128 to 165 17.8 : 8.8, 400 of
+    //                          20 to 69 2.2 : 1.2, 64 of 96 3.0 : 2.0
+    //   Cholesky and inverse   64 of 128 to 289 1.6 : 2.5; 1024 of 128 to 289 6.2 : 5.0, 152 of 160
+    //                          2.1 : 1.1, 64 of 96 0.52 : 0.37
+    auto one = [](int c) { return Job{1, 6, c * (6.5 + c * (0.1 + c * 5.4e-4))}; };
+    auto cluster = [](int c) { return Job{kPatchCluster, 3, 1.15 * c * (9.5 + c * 0.024)}; };
+    std::vector<Job> with, rest, without;
+    for (const PatchBlock& b : C.blocks) {
+        with.push_back(cluster(b.c));
+        without.push_back(one(b.c));
+    }
+    for (const PatchBlock& b : small) {
+        rest.push_back(one(b.c));
+        without.push_back(one(b.c));
+    }
+    if (makespan(with) + makespan(rest) >= makespan(without)) {
+        C.blocks.insert(C.blocks.end(), small.begin(), small.end());
+        small.swap(C.blocks);
+        C.blocks.clear();
+    }
     C.n_big = (int)C.blocks.size();
     if (!C.blocks.empty()) C.max_c[0] = C.blocks.front().c;
     if (!small.empty()) C.max_c[1] = small.front().c;
@@ -1088,10 +1130,9 @@ msp_status patch_qrcp(const PatchClasses& C, const PatchBlock* blocks, const dou
     return MSP_OK;
 }
 
-// Cluster sizes of the sweeps.  A warp's FP64 instructions go to its quarter of the SM
-// at 64 to 76 clocks each, whatever its lanes hold, so a CTA does best with pairs for four
-// or eight full warps of inner products: 5 and 10 CTAs put 29 and 15 pairs of a 289-column
-// patch on a CTA where 4 and 8 put 37 (too many) and 19 (a fifth warp on one quarter).
+// Cluster sizes of the sweeps: 2, 4, 8 and 16, and two between.  5 takes the orders that four
+// CTAs of 32 pairs do not hold (257 to 320 columns) without going to eight; 10 is the next
+// step for a patch whose share asks for more than eight.
 constexpr int kJacSizes = 7;
 constexpr int kJacNc[kJacSizes] = {16, 10, 8, 5, 4, 2, 1};
 
@@ -1116,31 +1157,6 @@ static int jac_cluster(int c, double share, size_t room, int max_nc) {
         if (nc >= want) break;
     }
     return best;
-}
-
-// Time at which the last of `jobs` (CTAs that start together, work of each) ends when they are
-// started in order as CTA slots of the device come free.  A slot is 1 / per_sm of an SM, so
-// launches of different shared memory share the device in sixths of an SM.
-struct JacJob {
-    int ctas, sixths;
-    double work;
-};
-static double jac_makespan(const std::vector<JacJob>& jobs) {
-    long long room = 6LL * num_sms();
-    double now = 0.0, last = 0.0;
-    std::priority_queue<std::pair<double, int>, std::vector<std::pair<double, int>>, std::greater<>> running;   // end, sixths
-    for (const JacJob& j : jobs) {
-        const int need = j.ctas * j.sixths;
-        while (room < need && !running.empty()) {
-            now = running.top().first;
-            room += running.top().second;
-            running.pop();
-        }
-        running.push({now + j.work, need});
-        room -= need;
-        last = std::max(last, now + j.work);
-    }
-    return last;
 }
 
 // Streams beside the caller's for launches that may overlap; on every way out the
@@ -1232,7 +1248,7 @@ msp_status patch_jacobi(const std::vector<PatchBlock>& all, double* W, double* V
     // 217, 196 of 100 to 221 40.7 against 105; 196 of 200 to 253 176 against 115, 484 of 150 to 219
     // 157 against 127, 324 of 160 to 281 223 against 186.
     {
-        std::vector<JacJob> cluster, one;
+        std::vector<Job> cluster, one;
         auto work = [](int c) { return c > 1 ? (double)c * c * std::sqrt((double)c) : 0.0; };
         for (int q = 0; q < kJacSizes; ++q) {
             if (first[q] == first[q + 1]) continue;
@@ -1240,11 +1256,11 @@ msp_status patch_jacobi(const std::vector<PatchBlock>& all, double* W, double* V
             MSP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, patch_jacobi_kernel, kJacThreads, bytes[q]));
             per_sm = std::max(1, std::min(per_sm, 3));
             for (int k = first[q]; k < first[q + 1]; ++k)
-                cluster.push_back(JacJob{kJacNc[q], 6 / per_sm, 2.1 * work(list[k].c) / kJacNc[q]});
+                cluster.push_back(Job{kJacNc[q], 6 / per_sm, 2.1 * work(list[k].c) / kJacNc[q]});
         }
-        for (const PatchBlock& b : rest) cluster.push_back(JacJob{1, 6, work(b.c)});   // they follow on one CTA
-        for (const PatchBlock& b : all) one.push_back(JacJob{1, 6, work(b.c)});
-        if (jac_makespan(one) < jac_makespan(cluster)) {
+        for (const PatchBlock& b : rest) cluster.push_back(Job{1, 6, work(b.c)});   // they follow on one CTA
+        for (const PatchBlock& b : all) one.push_back(Job{1, 6, work(b.c)});
+        if (makespan(one) < makespan(cluster)) {
             rest = all;
             return MSP_OK;
         }

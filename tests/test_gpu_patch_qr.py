@@ -17,7 +17,7 @@ SIDE, BUFFER, TAU = 6, 2, 1e-6
 DELTAS = 2 * (SIDE + BUFFER) + 1     # boundary columns of a corner patch
 
 
-@pytest.mark.parametrize("cols", [20, 48, 80, 81, 161, 163, 164, 260])
+@pytest.mark.parametrize("cols", [20, 48, 80, 81, 161, 163, 164, 200, 260])
 def test_forms_agree(cols):
     few = msp.Medium(synth.lognormal(2 * SIDE, 1 / 3, 16, 3), synth.uniform_patches(2 * SIDE, 2, 2, BUFFER, cols - DELTAS))
     many = msp.Medium(synth.lognormal(12 * SIDE, 1 / 12, 16, 3),
