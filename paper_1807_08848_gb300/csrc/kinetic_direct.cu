@@ -146,7 +146,8 @@ __device__ __forceinline__ void kd_product(T (&acc)[RA][RA], const T* L, const T
 
 // The serial part, one CTA per patch: E_i, its inverse and P_i of every node, written to the
 // - columns of W.  Thread (ty, tx) of the 16 x 16 grid owns the entries (ty + 16 a,
-// tx + 16 b), a, b < RA, of each h x h block (h <= 16 RA).  Bound by FP64 issue: a warp's
+// tx + 16 b), a, b < RA, of each h x h block (h <= 16 RA).  Bound by FP64 issue of the SMs that
+// hold a patch (their pipe is busy 74% of the time, 31% over the GPU at 64 patches): a warp's
 // instruction holds its quarter of the SM for 64 clocks, a division for about 380, so only
 // the thread that finishes the next pivot divides and publishes the reciprocal.  8193
 // nodes, 64 velocities, 64 patches: the factor as one n_v x n_v inverse per node took

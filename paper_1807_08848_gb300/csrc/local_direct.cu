@@ -296,7 +296,7 @@ __global__ void __launch_bounds__(kDirThreads) direct_init_kernel(DirArgs A) {
 // along the row, rows ascending.  first: |b| = |r| of the initial iterate.  A column stays
 // active while |r| > tol |b|.  A CTA takes 8 warps' columns of a chunk, 32 of them or 8
 // (blockIdx.y) when the chunks alone would leave SMs idle.
-// Bound: the FP64 pipe.  A difference across a face is formed once: the one to the left
+// Bound: the FP64 pipe (busy 82% of the time at 2049^2).  A difference across a face is formed once: the one to the left
 // is the left lane's to the right, negated, and the one below is the row below's upward,
 // kept in a register; with them a node costs 8 FP64 operations in place of 10.  At 1023^2
 // with 169 uneven patches all passes take 27.3 ms, 34.7 with every difference by itself.
@@ -437,10 +437,12 @@ __global__ void __launch_bounds__(kDirThreads) direct_residual_kernel(DirArgs A,
 // ahead, one barrier per slab); the product reads it four terms at a time (16-byte loads,
 // conflict-free) against broadcast loads of y, 4 G CPW FMAs for G + CPW loads, each output
 // one chain of FMAs over the terms in order.  R of the next row (forward) or w_j (backward)
-// is read before the product that hides it.  Bound: the FP32 pipe (2 nx^2 FMA per row and
-// column) with the shared-memory loads close behind; a warp whose columns have all
-// converged skips its products.  143356 columns on 1024 patches (2049^2): 66 ms for all
-// passes, 16.5 TFLOP/s; with W_j by plain loads and 32 columns per CTA 93 ms.
+// is read before the product that hides it.  Bound: issue slots and the latency of the row
+// chain (2 nx^2 FMA per row and column): with 32 columns per CTA on 64 patches 54% of the issue
+// slots and 38% of the FP32 pipe are busy, shared and global loads the first stalls; a warp
+// whose columns have all converged skips its products.  143356 columns on 1024 patches
+// (2049^2): 64 ms for all passes, 17 TFLOP/s, 24% of the FP32 rate; with W_j by plain loads and
+// 32 columns per CTA 93 ms.
 constexpr int kSlabRows = 32;
 constexpr int kSlabs = 4;
 

@@ -211,10 +211,12 @@ __global__ void __launch_bounds__(256) patch_post_kernel(const double* F, const 
 // At the end the columns are scaled, L[i][j] / sqrt(d_j) below the diagonal and sqrt(d_j)
 // on it.  Every element takes its updates in ascending order of k, one FMA each.  A
 // non-positive pivot sets *fail (and continues with d = 1).  The inverse of the factor is
-// left to tile_inverse_kernel, off the critical path.  Bound: the pivot chain (reciprocal,
-// product, FMA: about 510 clocks a column); with its inputs in cache a tile takes 71 us,
-// panels of eight over two warps took 85.  The whole factorisation of a 2049^2 basis went
-// from 401 to 324 ms with this, the panel solve and the shorter chain of launches.
+// left to tile_inverse_kernel, off the critical path.  A 64 x 64 tile takes 58 us in FP64 (73 as
+// one column and barrier at a time) and 30 in FP32 (42), launches back to back.  16 of the 58
+// are the pivot chain (reciprocal, product, FMA: about 510 clocks a column); the rest is the
+// panel before, longer than the corner beside it while many columns are left, then B and C,
+// and three barriers a panel.  The whole factorisation of a 2049^2 basis went from 401 to
+// 324 ms with this, the panel solve and the shorter chain of launches.
 constexpr int kPotPanel = 4;
 template <class T>
 __global__ void __launch_bounds__(256) potrf_tile_kernel(T* A, int lda, int nb, int* fail) {
