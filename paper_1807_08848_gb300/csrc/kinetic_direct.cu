@@ -366,9 +366,10 @@ __device__ __forceinline__ double kd_datum(const KdArgs& A, int m, int s, int l,
 // lane of the half = sample, so that an FP64 instruction (as long for 16 lanes as for 32)
 // carries two rows and a patch spreads over twice as many CTAs: with 32 samples each the
 // 192 CTAs of 64 patches x 96 samples gave 40 of 152 SMs two and the others one (8193
-// nodes, 64 velocities: offline + online 127.4 ms, now 114.2).  y (in T) shares the f
-// layout: [node][velocity][sample]; it holds the residual after the residual sweep and y_i
-// after the forward sweep.
+// nodes, 64 velocities: offline + online 127.4 ms, now 114.2; the solves 35.6 ms with the chunks
+// in a second grid dimension, 29.3 in most runs numbered in one and 35.6 in the others, by how
+// the 384 CTAs land on the SMs).  y (in T) shares the f layout: [node][velocity][sample]; it
+// holds the residual after the residual sweep and y_i after the forward sweep.
 template <class T, int RJ>
 __global__ void __launch_bounds__(kKdThreads) kd_solve_kernel(KdArgs A, int M, const T* W, T* y) {
     extern __shared__ __align__(16) unsigned char kd_dyn[];
