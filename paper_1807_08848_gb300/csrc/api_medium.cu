@@ -44,6 +44,7 @@ void clear_error() { g_err.clear(); }
 
 msp_status cuda_fail(cudaError_t e, const char* what, const char* file, int line) {
     set_error(std::string(what) + " failed: " + cudaGetErrorString(e) + " (" + file + ":" + std::to_string(line) + ")");
+    wait_before_release();
     return MSP_ERR_CUDA;
 }
 

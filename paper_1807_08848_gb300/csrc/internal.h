@@ -43,6 +43,12 @@ void destroy_handle(Handle* h, int device, const char* who) {
                   cudaGetErrorString(e));
 }
 
+// Before a call returns early on a failed runtime call or a refused allocation: its other
+// buffers are released on the way out, and kernels that it has enqueued may be using them.
+inline void wait_before_release() {
+    if (cudaDeviceSynchronize() != cudaSuccess) (void)cudaGetLastError();
+}
+
 // Lets launches of `kernel` ask for `bytes` of dynamic shared memory on the current device.
 // The limit is the process's, not the launch's: it is only ever raised, so that no call
 // takes it from another thread's launch between that thread's call and its launch.
@@ -76,6 +82,7 @@ struct DevBuf {
         const size_t bytes = count * sizeof(T);
         const cudaError_t e = pool_alloc((void**)&p, bytes, s);
         if (e != cudaSuccess) {
+            wait_before_release();
             p = nullptr;
             set_error(std::string("device allocation of ") + std::to_string(bytes) + " bytes failed: " +
                       cudaGetErrorString(e));

@@ -1,7 +1,8 @@
-"""The order of the runtime's calls when a handle is given back (csrc/handle.h): compiled for
-the host against stand-ins of the CUDA runtime's device calls, with a handle of device 1
-dropped while device 0 is current.  The handle's buffers may go only after device 1 was
-waited for and while it is current, and not at all when the wait fails."""
+"""The order of the runtime's calls when device memory is given back, compiled for the host
+against stand-ins of the CUDA runtime.  Handles (csrc/handle.h), one of device 1 dropped while
+device 0 is current: the buffers may go only after device 1 was waited for and while it is
+current, and not at all when the wait fails.  Buffers (DevBuf, csrc/internal.h): one that grows,
+and the others of a call whose allocation is refused, go only after a wait."""
 import os
 import shutil
 import subprocess
@@ -79,3 +80,75 @@ def test_failed_wait_keeps_the_memory(program):
 
 def test_unusable_device_keeps_the_memory(program):
     assert run(program, 0, set_=101) == ["clear", "status 101 current 0"]
+
+
+BUFFERS = r"""
+#include "internal.h"
+#include <cstdio>
+#include <cstring>
+
+static bool refuse = false;
+
+extern "C" {
+cudaError_t cudaDeviceSynchronize() { std::printf("sync\n"); return cudaSuccess; }
+cudaError_t cudaGetLastError() { return cudaSuccess; }
+cudaError_t cudaFree(void*) { std::printf("free\n"); return cudaSuccess; }
+const char* cudaGetErrorString(cudaError_t) { return "refused"; }
+}
+namespace msp {
+void set_error(const std::string&) {}
+msp_status cuda_fail(cudaError_t, const char*, const char*, int) { return MSP_ERR_CUDA; }
+cudaError_t pool_alloc(void** p, size_t, cudaStream_t) {
+    if (refuse) return cudaErrorMemoryAllocation;
+    std::printf("alloc\n");
+    *p = (void*)8;
+    return cudaSuccess;
+}
+}  // namespace msp
+
+static msp_status call() {
+    msp::DevBuf<double> a, b;
+    MSP_TRY(a.alloc(10, nullptr));
+    refuse = true;
+    MSP_TRY(b.alloc(10, nullptr));
+    return MSP_OK;
+}
+
+int main(int, char** argv) {
+    if (!std::strcmp(argv[1], "grow")) {
+        msp::DevBuf<double> a;
+        a.alloc(10, nullptr);
+        a.alloc(20, nullptr);
+        std::printf("end\n");
+    } else {
+        std::printf("status %d\n", (int)call());
+    }
+    return 0;
+}
+"""
+
+
+@pytest.fixture(scope="module")
+def buffers(tmp_path_factory):
+    cxx = shutil.which("g++")
+    if cxx is None or not os.path.exists(os.path.join(CUDA, "include", "cuda_runtime.h")):
+        pytest.skip("needs g++ and the CUDA headers")
+    d = tmp_path_factory.mktemp("buffers")
+    src, exe = str(d / "main.cpp"), str(d / "main")
+    with open(src, "w") as f:
+        f.write(BUFFERS)
+    subprocess.run([cxx, "-std=c++17", "-w", "-O1", "-I", CSRC, "-I", os.path.join(CUDA, "include"), src, "-o", exe],
+                   check=True)
+    return exe
+
+
+def lines(exe, arg):
+    return subprocess.run([exe, arg], capture_output=True, text=True, check=True).stdout.split("\n")[:-1]
+
+
+def test_growing_buffer_waits(buffers):
+    assert lines(buffers, "grow") == ["alloc", "sync", "free", "alloc", "end", "free"]
+
+
+def test_refused_allocation_waits(buffers):
+    assert lines(buffers, "refuse") == ["alloc", "sync", "free", "status -2"]
